@@ -181,7 +181,10 @@ kde_status kde_pack_positions(kde_ctx *ctx, const double *x, int64_t N, double L
  * Flags: KDE_F64.  In FP32 the per-particle normalisations come from a table of
  * I0e built in FP64 when the context is created (relative error below 5e-7), and
  * chunks whose widths are all at most 32 use the form 2^(K cos(theta_g - theta_i) - K),
- * K = kappa log2(e), whose exponent carries about K 2^-24 of rounding error. */
+ * K = kappa log2(e), whose exponent carries about K 2^-24 of rounding error.  At the
+ * default truncation, chunks with many particles sum them into a few proxy particles at
+ * Chebyshev points of position and width first (interpolation error below 2e-8 of a
+ * kernel's peak in each). */
 kde_status kde_deposit(kde_ctx *ctx, const uint32_t *u, const void *kappa, double kappa_uniform,
                        const void *weight, int64_t N, int32_t Ng, double L, void *rho_out,
                        uint32_t flags);

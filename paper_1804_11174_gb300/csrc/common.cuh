@@ -75,6 +75,7 @@ enum WsSlot {
     WS_PIC_E,
     WS_PIC_LOO,
     WS_PIC_KS,
+    WS_PIC_RANGE,  // float bits of the largest and smallest width of an FP32 PIC state
     WS_SP_PART,
     WS_SP_S,
     WS_SP_A,
@@ -123,6 +124,7 @@ struct kde_ctx {
     // Anderson-Darling per-bin logarithms (one table per context)
     void *ad_tab = nullptr;
     float2 *norm_tab = nullptr;  // FP32 width-normalisation table (kde_norm_tab), built at creation
+    float *pxy_tab = nullptr;    // interpolation matrices (proxy.cuh), built at creation
     unsigned wait_polls = 1u << 26;         // polls of a bounded device wait (kde_set_wait_limit)
     bool count_flip = false;                // which sort count table the next counted sort reads (sort.cu)
     bool autotune = false;                  // kde_set_autotune
@@ -297,6 +299,22 @@ __device__ __forceinline__ kde_f2 kde_ex22(kde_f2 x)
     return kde_pk(kde_ex2(a), kde_ex2(b));
 }
 
+// butterfly over 32 values: afterwards lane l holds the warp sum of v[l]
+__device__ __forceinline__ float warp_transpose_sum32(float (&v)[32], int lane)
+{
+#pragma unroll
+    for (int o = 16; o >= 1; o >>= 1) {
+        const bool up = (lane & o) != 0;
+#pragma unroll
+        for (int i = 0; i < o; ++i) {
+            float send = up ? v[i] : v[i + o];
+            float keep = up ? v[i + o] : v[i];
+            v[i] = keep + __shfl_xor_sync(0xffffffffu, send, o);
+        }
+    }
+    return v[0];
+}
+
 // largest width for the cosine form of the FP32 kernel value,
 // 2^(K cos x_j cos x_g + K sin x_j sin x_g - K) with K = kappa log2(e): three
 // multiply-adds per pair instead of the half-angle form's four, at the price of an
@@ -461,7 +479,8 @@ kde_status kde_deposit_reserve(kde_ctx *ctx, int64_t N, int Ng);
 // the FP32 deposit of cell-sorted particles (uniform weight w_u, N >= 1) left as its
 // per-CTA int64 rows (workspace, valid until the next deposit on the context):
 // node g of row k is rows[k Ng + ((g - hdr[k].x) mod Ng)] when that index is below
-// hdr[k].y, else 0; fixed-point scale kde_acc_scale(bound)
+// hdr[k].y, else 0; fixed-point scale kde_acc_scale(bound).  krange: float bits of the
+// largest and smallest width on the device, which spare the kernel a pass over the widths
 struct DepRows {
     const long long *rows;
     const int2 *hdr;
@@ -469,7 +488,7 @@ struct DepRows {
 };
 kde_status kde_deposit_rows_f32(kde_ctx *ctx, const uint32_t *u, const float *kappa, float kappa_u, const float *norm,
                                 float norm_u, int64_t N, int Ng, double coef, float w_u, double bound, DepRows *out,
-                                float xcut = 0.f);
+                                float xcut = 0.f, const unsigned int *krange = nullptr);
 // the PIC step's field from those rows: rho_total = background + charge * rho with its
 // mean removed (so the constant background drops out), E by the spectral or
 // finite-difference Green's function (FP32 output)
@@ -547,4 +566,23 @@ kde_status kde_cv_spectral_device(kde_ctx *ctx, const uint32_t *u, int64_t N, do
 // as float or double.
 kde_status kde_adapt_device(kde_ctx *ctx, const float *loo, int64_t N, double L, const double *kstar_dev,
                             double kstar_host, double alpha, double kmin, double kmax, void *kappa_out,
-                            void *norm_out, bool f64);
+                            void *norm_out, bool f64, unsigned int *krange = nullptr);
+
+// float bits of the largest and smallest of many widths: kde_krange_reset on the stream,
+// then kde_krange_add by every warp of the kernel that writes the widths (all lanes; a lane
+// without a width passes lo = 3e38, hi = 0)
+inline cudaError_t kde_krange_reset(unsigned int *krange, cudaStream_t stream)
+{
+    const cudaError_t e = cudaMemsetAsync(krange, 0, 4, stream);
+    return e != cudaSuccess ? e : cudaMemsetAsync(krange + 1, 0x7f, 4, stream);
+}
+__device__ __forceinline__ void kde_krange_add(unsigned int *krange, float lo, float hi)
+{
+    const unsigned int h = __reduce_max_sync(0xffffffffu, __float_as_uint(hi));
+    const unsigned int l = __reduce_min_sync(0xffffffffu, __float_as_uint(lo));
+    if ((threadIdx.x & 31) == 0) {
+        // most warps find the range as wide already and add nothing
+        if (h > __ldcg(&krange[0])) atomicMax(&krange[0], h);
+        if (l < __ldcg(&krange[1])) atomicMin(&krange[1], l);
+    }
+}

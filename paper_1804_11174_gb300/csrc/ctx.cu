@@ -4,6 +4,7 @@
 #include <cstring>
 
 #include "common.cuh"
+#include "proxy.cuh"
 
 kde_status kde_fail(kde_ctx *ctx, kde_status code, const char *fmt, ...)
 {
@@ -181,6 +182,17 @@ __global__ void norm_tab_kernel(float2 *tab)
     tab[i] = make_float2((float)q(t), (float)((q(t + d) - q(t - d)) / (2.0 * d) / KDE_NTAB_INVH));
 }
 
+// the interpolation matrices of proxy.cuh: entry (p, a) of every degree D, in FP64
+__global__ void pxy_tab_kernel(float *tab)
+{
+    const int D = blockIdx.x + 1;
+    float *c = tab + pxy_tab_off(D);
+    for (int i = threadIdx.x; i < D * D; i += blockDim.x) {
+        const int p = i / D, a = i - p * D;
+        c[i] = (float)((p ? 2.0 : 1.0) / D * cospi((double)((p * (2 * a + 1)) % (4 * D)) / (2.0 * D)));
+    }
+}
+
 // ---------------------------------------------------------------------------
 // C ABI: context
 // ---------------------------------------------------------------------------
@@ -200,11 +212,17 @@ extern "C" kde_status kde_create(kde_ctx **out, int device, void *stream)
         norm_tab_kernel<<<(KDE_NTAB_N + 255) / 256, 256, 0, ctx->stream>>>(ctx->norm_tab);
         e = cudaGetLastError();
     }
+    if (e == cudaSuccess) e = cudaMalloc(&ctx->pxy_tab, PXY_TAB_N * sizeof(float));
+    if (e == cudaSuccess) {
+        pxy_tab_kernel<<<PXY_MAXQ, 128, 0, ctx->stream>>>(ctx->pxy_tab);
+        e = cudaGetLastError();
+    }
     if (e == cudaSuccess) e = cudaStreamSynchronize(ctx->stream);
     if (e != cudaSuccess) {
         cudaGetLastError();
         if (ctx->d_status) cudaFree(ctx->d_status);
         if (ctx->norm_tab) cudaFree(ctx->norm_tab);
+        if (ctx->pxy_tab) cudaFree(ctx->pxy_tab);
         delete ctx;
         return KDE_ECUDA;
     }
@@ -223,6 +241,7 @@ extern "C" kde_status kde_destroy(kde_ctx *ctx)
     for (auto &kv : ctx->green_tab) cudaFree(kv.second);
     if (ctx->ad_tab) cudaFree(ctx->ad_tab);
     if (ctx->norm_tab) cudaFree(ctx->norm_tab);
+    if (ctx->pxy_tab) cudaFree(ctx->pxy_tab);
     if (ctx->d_status) cudaFree(ctx->d_status);
     for (auto &p : ctx->prof) {
         cudaEventDestroy(p.second.first);

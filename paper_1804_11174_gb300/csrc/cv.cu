@@ -448,22 +448,6 @@ __device__ __forceinline__ void cvf_dispatch(int ng, const float2 *t, int ncol, 
     }
 }
 
-// butterfly over 32 values: afterwards lane l holds the warp sum of v[l]
-__device__ __forceinline__ float warp_transpose_sum32(float (&v)[32], int lane)
-{
-#pragma unroll
-    for (int o = 16; o >= 1; o >>= 1) {
-        const bool up = (lane & o) != 0;
-#pragma unroll
-        for (int i = 0; i < o; ++i) {
-            float send = up ? v[i] : v[i + o];
-            float keep = up ? v[i + o] : v[i];
-            v[i] = keep + __shfl_xor_sync(0xffffffffu, send, o);
-        }
-    }
-    return v[0];
-}
-
 __global__ void __launch_bounds__(CV_T, 2)
     cv_pairs_fast_kernel(const float2 *__restrict__ sc, int64_t N, int NT, const uint2 *__restrict__ tile_u,
                          int *counter, double *part, unsigned int *status, unsigned wait_polls,
@@ -1061,10 +1045,14 @@ __global__ void __launch_bounds__(256) adapt_mean_kernel(const double *part, int
 
 template <typename T>
 __global__ void adapt_apply_kernel(const float *loo, int64_t N, const AdaptPar *__restrict__ P, double alpha,
-                                   double kmin, double kmax, T *kappa_out, T *norm_out, const float2 *ntab)
+                                   double kmin, double kmax, T *kappa_out, T *norm_out, const float2 *ntab,
+                                   unsigned int *krange)
 {
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= N) return;
+    if (i >= N) {
+        if (krange) kde_krange_add(krange, 3.0e38f, 0.f);
+        return;
+    }
     // lambda = (f/g)^-alpha, kappa = kappa* / lambda^2; FP32 widths in FP32 with base-2
     // logarithms (the log-mean of adapt_logsum_dev_kernel<true> is in the same base), FP64
     // widths in FP64 with natural ones
@@ -1082,6 +1070,7 @@ __global__ void adapt_apply_kernel(const float *loo, int64_t N, const AdaptPar *
         k = kd;
     }
     kappa_out[i] = k;
+    if (krange) kde_krange_add(krange, (float)k, (float)k);
     if (norm_out) {
         // FP32 widths take the tabulated norm, FP64 widths the FP64 Bessel series
         if constexpr (sizeof(T) == 4) norm_out[i] = (T)kde_norm_tab(ntab, (float)k);
@@ -1124,7 +1113,7 @@ __global__ void adapt_logsum_dev_kernel(const float *loo, int64_t N, const Adapt
 
 kde_status kde_adapt_device(kde_ctx *ctx, const float *loo, int64_t N, double L, const double *kstar_dev,
                             double kstar_host, double alpha, double kmin, double kmax, void *kappa_out,
-                            void *norm_out, bool f64)
+                            void *norm_out, bool f64, unsigned int *krange)
 {
     double *part = (double *)kde_ws(ctx, WS_CV_RED, AD_BLOCKS * 8 + sizeof(AdaptPar) + 64);
     if (!part) return KDE_ENOMEM;
@@ -1140,10 +1129,12 @@ kde_status kde_adapt_device(kde_ctx *ctx, const float *loo, int64_t N, double L,
     unsigned grid = (unsigned)((N + 255) / 256);
     if (f64)
         adapt_apply_kernel<double><<<grid, 256, 0, ctx->stream>>>(loo, N, P, alpha, kmin, kmax, (double *)kappa_out,
-                                                                   (double *)norm_out, ctx->norm_tab);
-    else
+                                                                   (double *)norm_out, ctx->norm_tab, nullptr);
+    else {
+        if (krange) KDE_CUDA(ctx, kde_krange_reset(krange, ctx->stream), "width range memset");
         adapt_apply_kernel<float><<<grid, 256, 0, ctx->stream>>>(loo, N, P, alpha, kmin, kmax, (float *)kappa_out,
-                                                                  (float *)norm_out, ctx->norm_tab);
+                                                                  (float *)norm_out, ctx->norm_tab, krange);
+    }
     KDE_LAUNCHED(ctx, "adapt_apply_kernel");
     return KDE_OK;
 }

@@ -14,6 +14,7 @@
 // and added with integer atomics, so the grid sum is exact and independent of
 // the order in which chunks finish: results are bitwise reproducible.
 #include "common.cuh"
+#include "proxy.cuh"
 
 #define DEP_THREADS 256
 #define DEP_WARPS (DEP_THREADS / 32)
@@ -50,6 +51,9 @@ template <typename T> struct DepSrc {
     int scale_exp;  // KDE_ES_FROM_BOUND, or the exponent es of the fixed-point scale 2^es
     const float2 *ntab;  // FP32 norm table (kde_norm_tab) for per-particle widths without norms, or nullptr
     float xcut = (float)KDE_XCUT;  // FP32 packed kernels: truncation cut exponent (kde_fp32_cut)
+    PxyGrid grid;                    // the nodes as position codes
+    const float *pxt;                // interpolation matrices (proxy.cuh)
+    const unsigned int *krange;      // float bits of the largest and smallest width, or null
 };
 
 #define KDE_ES_FROM_BOUND (-100000)
@@ -725,6 +729,337 @@ __device__ __forceinline__ void depp_sweep_pairs(const DepSrc<float> &S, int n, 
     }
 }
 
+// ---------------------------------------------------------------------------
+// Compressed form of a CTA's deposit (proxy.cuh): its particles, an interval of whole
+// cells with widths in [kmin, kmax], become P Q proxy particles, and only the proxies sweep
+// the node window.  Moments M_pq = sum_i w_i T_p(x_i) T_q(s_i), three ways:
+//  * one width (Q = 1): P sums a thread in registers;
+//  * a narrow range of widths and P <= 8: a thread's products in registers too (the
+//    normalisation is interpolated with the kernel, so no norm is read);
+//  * otherwise a small matrix product: a warp stages the T_p (times weight and norm) of 16
+//    particles and their T_q, and its lanes own 4 x 4 tiles of the P x Q sums.
+// Warp and CTA sums follow in a fixed order.
+//
+// What bounds it: the direct sweep spends one exp2 and three or four multiply-adds on every
+// (particle, node) pair, 256 a particle for whole-grid windows; here a particle costs the
+// Chebyshev values and 28 to 48 multiply-adds (a few hundred in the matrix form) whatever the
+// window, and is bound by instruction issue and load latency.  Measured (event-free launch
+// times): 2^20 particles, 256 nodes, widths near 14 43.2 -> 16.3 us; 4,000,037 particles, 4096
+// nodes, widths log-uniform in [5, 5e3] 2389 -> 298 us.
+// ---------------------------------------------------------------------------
+#define PXY_STAGE 16  // particles a warp stages at a time
+
+__device__ __forceinline__ float depp_kappa(const DepSrc<float> &S, float k, int64_t j)
+{
+    if (!(k > 0.f && k <= (float)KDE_KAPPA_MAX)) {
+        kde_flag(S.status, KDE_DEV_KAPPA_RANGE, (unsigned)j);
+        k = (float)KDE_KAPPA_MAX;
+    }
+    return k;
+}
+
+// the moments kept by the register form: all of PM x QM, or with TRI those with
+// p / PM + q / QM < 1 (the coefficients of the joint interpolant fall off in p and q together)
+template <int PM, int QM, bool TRI>
+__host__ __device__ constexpr bool depp_kept(int p, int q)
+{
+    return !TRI || p * QM + q * PM < PM * QM;
+}
+template <int PM, int QM, bool TRI> __host__ __device__ constexpr int depp_count(int upto)
+{
+    int n = 0;
+    for (int i = 0; i < upto; ++i) n += depp_kept<PM, QM, TRI>(i / QM, i % QM) ? 1 : 0;
+    return n;
+}
+
+template <int PM, int QM, bool TRI>
+__device__ __forceinline__ void depp_moments_reg(const DepSrc<float> &S, int64_t i0, int n, const PxyBox &B,
+                                                 float *part, float *M)
+{
+    constexpr int NM = depp_count<PM, QM, TRI>(PM * QM), QB = 4;
+    constexpr int NR = (NM + 31) / 32;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const uint32_t *u = S.u + i0;
+    const float *kap = S.kappa ? S.kappa + i0 : nullptr, *w = S.w ? S.w + i0 : nullptr;
+    float acc[NM];
+#pragma unroll
+    for (int i = 0; i < NM; ++i) acc[i] = 0.f;
+#pragma unroll 1
+    for (int b0 = tid; b0 < n; b0 += QB * DEPP_THREADS) {
+        uint32_t ru[QB];
+        float rk[QB], rw[QB];
+#pragma unroll
+        for (int q = 0; q < QB; ++q) {
+            const int t = b0 + q * DEPP_THREADS;
+            const int j = t < n ? t : 0;
+            ru[q] = u[j];
+            rk[q] = QM > 1 ? kap[j] : 0.f;
+            rw[q] = t < n ? (w ? w[j] : S.w_u) : 0.f;
+        }
+#pragma unroll
+        for (int q = 0; q < QB; ++q) {
+            const float x = pxy_x(B, ru[q]), x2 = x + x;
+            float tp[PM];
+            tp[0] = rw[q];
+            tp[1] = tp[0] * x;
+#pragma unroll
+            for (int p = 2; p < PM; ++p) tp[p] = fmaf(x2, tp[p - 1], -tp[p - 2]);
+            if constexpr (QM == 1) {
+#pragma unroll
+                for (int p = 0; p < PM; ++p) acc[p] += tp[p];
+            } else {
+                float k = rk[q];
+                if (!(k > 0.f && k <= (float)KDE_KAPPA_MAX)) k = depp_kappa(S, k, i0 + b0 + q * DEPP_THREADS);
+                const float sv = (k - B.kc) * B.inv_kh, s2 = sv + sv;
+                // t0 = T_{r-1}(s), t1 = T_r(s)
+                float t0 = 1.f, t1 = sv;
+#pragma unroll
+                for (int p = 0; p < PM; ++p) acc[depp_count<PM, QM, TRI>(p * QM)] += tp[p];
+#pragma unroll
+                for (int r = 1; r < QM; ++r) {
+#pragma unroll
+                    for (int p = 0; p < PM; ++p)
+                        if (depp_kept<PM, QM, TRI>(p, r)) {
+                            const int m = depp_count<PM, QM, TRI>(p * QM + r);
+                            acc[m] = fmaf(tp[p], t1, acc[m]);
+                        }
+                    const float t2 = fmaf(s2, t1, -t0);
+                    t0 = t1;
+                    t1 = t2;
+                }
+            }
+        }
+    }
+    // lane l of a warp ends with the warp's sums of moments l, l + 32, ...
+    float *pw = part + warp * 64;
+    if (NM <= 8) {
+#pragma unroll
+        for (int i = 0; i < NM; ++i) {
+            float v = acc[i];
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+            if (lane == 0) pw[i] = v;
+        }
+    } else {
+#pragma unroll
+        for (int h = 0; h < NR; ++h) {
+            float v[32];
+#pragma unroll
+            for (int i = 0; i < 32; ++i) v[i] = h * 32 + i < NM ? acc[h * 32 + i < NM ? h * 32 + i : 0] : 0.f;
+            pw[h * 32 + lane] = warp_transpose_sum32(v, lane);
+        }
+    }
+    __syncthreads();
+    for (int i = tid; i < PM * QM; i += DEPP_THREADS) {
+        float a = 0.f;
+        int m = i;  // position of moment (p, q) among the kept ones
+        bool kept = true;
+        if (TRI) {
+            kept = depp_kept<PM, QM, TRI>(i / QM, i % QM);
+            m = 0;
+            for (int p = 0; p < i / QM; ++p) m += (QM * (PM - p) + PM - 1) / PM;
+            m += i % QM;
+        }
+        if (kept) {
+#pragma unroll
+            for (int k = 0; k < DEPP_WARPS; ++k) a += part[k * 64 + m];
+        }
+        M[i] = a * S.coef;
+    }
+}
+
+// moments of any degrees (P <= 16, Q <= 40) as a matrix product; stage: the warp's rows of
+// RS = 4 (LP + LQ) floats (an odd number of 16-byte words)
+__device__ __forceinline__ void depp_moments_mm(const DepSrc<float> &S, int64_t i0, int64_t i1, const PxyBox &B,
+                                                float *stage, float *part, float *M)
+{
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int LP = (B.P + 3) >> 2, LQ = (B.Q + 3) >> 2;
+    const int RS = 4 * ((LP + LQ) | 1);
+    const int tiles = LP * LQ;
+    int KS = 1;  // particles taken at once (power of two, KS tiles <= 32)
+    while (2 * KS * tiles <= 32 && 2 * KS <= PXY_STAGE) KS *= 2;
+    const int ks = lane / tiles, tile = lane - ks * tiles, lp = tile / LQ, lq = tile - lp * LQ;
+    const bool on = ks < KS;
+    const int row = lane & (PXY_STAGE - 1);  // the particle this lane stages
+    const bool roleB = lane >= PXY_STAGE;    // lanes 0..15 the T_p, lanes 16..31 the T_q
+    float acc[4][4];
+#pragma unroll
+    for (int a = 0; a < 4; ++a)
+#pragma unroll
+        for (int b = 0; b < 4; ++b) acc[a][b] = 0.f;
+    constexpr int QB = 4;
+    const int64_t step = (int64_t)DEPP_WARPS * PXY_STAGE;
+#pragma unroll 1
+    for (int64_t g0 = i0 + warp * PXY_STAGE; g0 < i1; g0 += QB * step) {
+        uint32_t ru[QB];
+        float rk[QB], rn[QB], rw[QB];
+#pragma unroll
+        for (int q = 0; q < QB; ++q) {
+            const int64_t t = g0 + q * step + row;
+            const int64_t j = t < i1 ? t : i0;
+            ru[q] = S.u[j];
+            rk[q] = S.kappa[j];
+            rn[q] = S.norm ? S.norm[j] : 0.f;
+            rw[q] = S.w ? S.w[j] : S.w_u;
+        }
+#pragma unroll 1
+        for (int q = 0; q < QB; ++q) {
+            const int64_t t0 = g0 + q * step;
+            if (t0 >= i1) break;
+            const int64_t t = t0 + row;
+            const bool ok = t < i1;
+            const float k = ok ? depp_kappa(S, rk[0], t) : 1.f;
+            // the first of the recurrence: the weight (0 past the end) or 1
+            float z, y0 = 1.f;
+            if (roleB) {
+                z = pxy_s(B, k);
+            } else {
+                z = pxy_x(B, ru[0]);
+                y0 = ok ? rw[0] * S.coef * (S.norm ? rn[0] : kde_norm_tab(S.ntab, k)) : 0.f;
+            }
+#pragma unroll
+            for (int i = 0; i + 1 < QB; ++i) {
+                ru[i] = ru[i + 1];
+                rk[i] = rk[i + 1];
+                rn[i] = rn[i + 1];
+                rw[i] = rw[i + 1];
+            }
+            float y1 = y0 * z;
+            const float z2 = z + z;
+            float4 *dst = (float4 *)(stage + row * RS) + (roleB ? LP : 0);
+            const int n4 = roleB ? LQ : LP;
+            for (int i = 0; i < n4; ++i) {
+                const float y2 = fmaf(z2, y1, -y0), y3 = fmaf(z2, y2, -y1);
+                dst[i] = make_float4(y0, y1, y2, y3);
+                y0 = fmaf(z2, y3, -y2);
+                y1 = fmaf(z2, y0, -y3);
+            }
+            __syncwarp();
+            if (on) {
+#pragma unroll 4
+                for (int r = ks; r < PXY_STAGE; r += KS) {
+                    const float4 A = *(const float4 *)(stage + r * RS + 4 * lp);
+                    const float4 Q4 = *(const float4 *)(stage + r * RS + 4 * (LP + lq));
+                    const float av[4] = {A.x, A.y, A.z, A.w}, bv[4] = {Q4.x, Q4.y, Q4.z, Q4.w};
+#pragma unroll
+                    for (int a = 0; a < 4; ++a)
+#pragma unroll
+                        for (int b = 0; b < 4; ++b) acc[a][b] = fmaf(av[a], bv[b], acc[a][b]);
+                }
+            }
+            __syncwarp();
+        }
+    }
+    // part[warp][lane][16], then moment (p, q) over the warps and their particle groups
+    float4 *pw = (float4 *)part + (warp * 32 + lane) * 4;
+#pragma unroll
+    for (int a = 0; a < 4; ++a) pw[a] = make_float4(acc[a][0], acc[a][1], acc[a][2], acc[a][3]);
+    __syncthreads();
+    for (int i = tid; i < B.P * B.Q; i += DEPP_THREADS) {
+        const int p = i / B.Q, q = i - p * B.Q;
+        const int off = ((p >> 2) * LQ + (q >> 2)) * 16 + (p & 3) * 4 + (q & 3);
+        float a = 0.f;
+        for (int w = 0; w < DEPP_WARPS; ++w)
+            for (int g = 0; g < KS; ++g) a += part[(w * 32 + g * tiles) * 16 + off];
+        M[i] = a;
+    }
+}
+
+// moments -> proxies -> node window: flush(r, a) receives the sum at window node r.
+// normed: the proxies carry their width's normalisation (the particles' weights did not).
+// mem: at least 2 P Q + 2 P + Q floats; part: DEPP_WARPS DEPP_PART floats
+template <typename F>
+__device__ __forceinline__ void depp_proxies(const DepSrc<float> &S, const PxyBox &B, bool normed, int g_lo, int R,
+                                             const float *M, float *mem, float *part, F &&flush)
+{
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int P = B.P, Q = B.Q, PQ = P * Q, Ng = S.Ng;
+    const float *cp = S.pxt + pxy_tab_off(P), *cq = S.pxt + pxy_tab_off(Q);
+    float *U = mem, *W = U + PQ, *fr = W + PQ, *k2 = fr + P;
+    uint32_t *cd = (uint32_t *)(k2 + Q);
+    // proxy positions and exponent factors -2 kappa_b log2 e (the Chebyshev points are
+    // the matrices' second rows times D / 2)
+    if (tid < P) pxy_pos(B, P > 1 ? cp[P + tid] * (0.5f * (float)P) : 0.f, cd[tid], fr[tid]);
+    if (tid >= 64 && tid < 64 + Q) {
+        const int b = tid - 64;
+        k2[b] = (float)(-2.0 * KDE_LOG2E) * (Q > 1 ? pxy_kappa(B, cq[Q + b] * (0.5f * (float)Q)) : B.kc);
+    }
+    __syncthreads();  // also: the moments are written
+    for (int i = tid; i < PQ; i += DEPP_THREADS) {
+        const int a = i / Q, q = i - a * Q;
+        float s = 0.f;
+        for (int p = 0; p < P; ++p) s = fmaf(cp[p * P + a], M[p * Q + q], s);
+        U[i] = s;
+    }
+    __syncthreads();
+    for (int i = tid; i < PQ; i += DEPP_THREADS) {
+        const int a = i / Q, b = i - a * Q;
+        float s = 0.f;
+        for (int q = 0; q < Q; ++q) s = fmaf(cq[q * Q + b], U[a * Q + q], s);
+        if (normed) s *= S.kappa ? kde_norm_tab(S.ntab, k2[b] * (float)(-0.5 * KDE_LN2)) : S.norm_u;
+        W[i] = s;
+    }
+    __syncthreads();
+    // a thread takes a node and every SL-th proxy position; the widest kernels (last b)
+    // come first, and a kernel below 2^-32 of its peak ends the row
+    const int ng = (R + 31) >> 5;  // node groups of a warp
+    const int SL = ng >= DEPP_WARPS ? 1 : DEPP_WARPS / ng;
+    auto node = [&](int r, int a0, int da) -> float {
+        int g = g_lo + r;
+        g = g < 0 ? g + Ng : (g >= Ng ? g - Ng : g);
+        uint32_t nc;
+        float nf;
+        pxy_node(S.grid, g, nc, nf);
+        float acc = 0.f;
+#pragma unroll 1
+        for (int a = a0; a < P; a += da) {
+            const float s2 = pxy_sin2(nc, nf, cd[a], fr[a]);
+            const float *w = W + a * Q;
+            int b = Q - 1;
+            for (; b >= 3; b -= 4) {  // four at a time: the first has the largest value
+                const float e = s2 * k2[b];
+                if (e < -32.f) break;
+                const float e0 = kde_ex2(e) * w[b], e1 = kde_ex2(s2 * k2[b - 1]) * w[b - 1];
+                const float e2 = kde_ex2(s2 * k2[b - 2]) * w[b - 2], e3 = kde_ex2(s2 * k2[b - 3]) * w[b - 3];
+                acc += (e0 + e1) + (e2 + e3);
+            }
+            if (b < 3)
+                for (; b >= 0; --b) acc = fmaf(kde_ex2(s2 * k2[b]), w[b], acc);
+        }
+        return acc;
+    };
+    if (SL == 1) {
+#pragma unroll 1
+        for (int r = tid; r < R; r += DEPP_THREADS) flush(r, node(r, 0, 1));
+        return;
+    }
+    const int gi = warp % ng, sl = warp / ng, r = gi * 32 + lane;
+    if (sl < SL) part[sl * DEPP_PART + r] = r < R ? node(r, sl, SL) : 0.f;
+    __syncthreads();
+    for (int q = tid; q < R; q += DEPP_THREADS) {
+        float a = 0.f;
+        for (int k = 0; k < SL; ++k) a += part[k * DEPP_PART + q];
+        flush(q, a);
+    }
+}
+
+// whether the compressed form costs less than the direct sweep: instructions of a lane,
+// direct about 3.2 a (particle, node) pair and 48 a particle; compressed 55 a particle plus
+// its Chebyshev values and moments (shared by the lanes of a warp), then 16 a (node, proxy
+// position), 3 a (node, proxy), the interpolation matrices and a CTA's fixed steps.  Near the
+// line: 658 particles a CTA in windows of 27 nodes with P = 11 (300,007 particles, 512 nodes,
+// width 2000) take 10.5 us direct and 13.5 compressed, so they stay direct
+__device__ __forceinline__ bool depp_compress_pays(const PxyBox &B, int n, int R)
+{
+    // the moment tiles of the matrix product have to fit a warp
+    if (B.P > PXY_MAXP || B.Q > PXY_MAXQ || ((B.P + 3) >> 2) * ((B.Q + 3) >> 2) > 32) return false;
+    const float fn = (float)n, fR = (float)R, P = (float)B.P, Q = (float)B.Q, PQ = P * Q;
+    const float direct = fn * (3.2f * fR + 48.f);
+    const float comp = fn * (55.f + 3.f * (P + Q) + 1.6f * PQ) + fR * P * (16.f + 3.f * Q) + PQ * (P + Q) * 4.f + 40000.f;
+    return comp < direct;
+}
+
 // acc[g] = sum over the rows whose window covers node g of that row's entry; CTA b
 // takes nodes [32 b, 32 b + 32), lane l node 32 b + l, warp w rows w, w + 32, ...
 __global__ void __launch_bounds__(DEPP_RED_THREADS) deposit_rows_kernel(const long long *__restrict__ rows,
@@ -782,12 +1117,18 @@ __global__ void __launch_bounds__(DEPP_THREADS, DEPP_MINB) deposit_persist_kerne
     // smallest and largest width of the CTA's particles (the window and the form): a pass
     // over the widths, PER loads in flight per thread
     float kmin = (float)KDE_KAPPA_MAX, kmax = 0.f;
+    if (S.krange) {
+        kmax = __uint_as_float(S.krange[0]);
+        kmin = __uint_as_float(S.krange[1]);
+    } else if (!S.kappa) {
+        kmin = kmax = S.kappa_u;
+    } else
     for (int64_t j0 = i0; j0 < i1; j0 += (int64_t)PER * DEPP_THREADS) {
         float kk[PER];
 #pragma unroll
         for (int p = 0; p < PER; ++p) {
             const int64_t j = j0 + tid + p * DEPP_THREADS;
-            kk[p] = j < i1 ? (S.kappa ? S.kscale * S.kappa[j] : S.kappa_u) : -1.f;
+            kk[p] = j < i1 ? S.kappa[j] : -1.f;
         }
 #pragma unroll
         for (int p = 0; p < PER; ++p)
@@ -843,6 +1184,42 @@ __global__ void __launch_bounds__(DEPP_THREADS, DEPP_MINB) deposit_persist_kerne
                   : (2 * n128 == n64 && (n128 >= DEPP_WARPS || n128 * 128 <= DEPP_PART)) ? 2
                                                                                           : 1;
     long long *row = Pl.rows + (size_t)c * Ng;
+    if (S.xcut == (float)KDE_XCUT && c_last >= c_first) {
+        // the default cut: compressed where that is less work (a cut the caller has set keeps
+        // the sweep over the particles that it is defined for)
+        PxyBox B;
+        pxy_box_pos(B, S.grid, c_first, c_last, kmax);
+        pxy_box_width(B, kmin, kmax);
+        const int n = (int)(i1 - i0);
+        if (depp_compress_pays(B, n, R)) {
+            __shared__ float M[PXY_MAXP * PXY_MAXQ];
+            bool normed = true;
+            if (B.Q == 1) {
+                if (B.P <= 8) {
+                    B.P = 8;
+                    depp_moments_reg<8, 1, false>(S, i0, n, B, part, M);
+                } else {
+                    B.P = 16;
+                    depp_moments_reg<16, 1, false>(S, i0, n, B, part, M);
+                }
+            } else if (B.lin && B.P <= 6) {
+                B.P = B.Q = 7;
+                depp_moments_reg<7, 7, true>(S, i0, n, B, part, M);
+            } else if (B.lin && B.P <= 8) {
+                B.P = 8;
+                depp_moments_reg<8, 6, false>(S, i0, n, B, part, M);
+            } else {
+                normed = false;
+                depp_moments_mm(S, i0, i1, B, (float *)rec + warp * (DEPP_SUB * 4 / DEPP_WARPS), part, M);
+            }
+            auto flush = [&](int r, float a) {
+                row[r] = (es >= -100 && es <= 100) ? fix_pow2(a, es) : __double2ll_rn(ldexp((double)a, es));
+            };
+            depp_proxies(S, B, normed, g_lo, R, M, (float *)rec, part, flush);
+            if (tid == 0) Pl.hdr[c] = make_int2(g_lo, R);
+            return;
+        }
+    }
 
     for (int64_t b0 = i0; b0 < i1; b0 += DEPP_SUB) {
         const int n = (int)(i1 - b0 < DEPP_SUB ? i1 - b0 : DEPP_SUB);
@@ -983,7 +1360,7 @@ template <typename T>
 static kde_status deposit_sorted_impl(kde_ctx *ctx, const uint32_t *u, const T *kappa, T kappa_u, const T *norm,
                                       T norm_u, const T *w, T w_u, int64_t N, int Ng, double coef, long long *acc,
                                       double bound, const unsigned int *wmax_bits, double norm_bound, DepRows *rows_out,
-                                      float xcut = 0.f)
+                                      float xcut = 0.f, const unsigned int *krange = nullptr)
 {
     // the persistent FP32 kernel writes every node; the others add into zeroed accumulators
     if (!(sizeof(T) == 4 && N > 0))
@@ -1019,6 +1396,9 @@ static kde_status deposit_sorted_impl(kde_ctx *ctx, const uint32_t *u, const T *
     }
     S.ntab = ctx->norm_tab;
     S.xcut = xcut > 0.f ? xcut : kde_fp32_cut(ctx);
+    S.grid = pxy_grid(Ng);
+    S.pxt = ctx->pxy_tab;
+    S.krange = krange;
     if constexpr (sizeof(T) == 4) {
         DepPlan Pl{};
         KDE_TRY(depp_plan(ctx, N, Ng, acc, Pl));
@@ -1063,11 +1443,11 @@ kde_status kde_deposit_sorted(kde_ctx *ctx, const uint32_t *u, const T *kappa, T
 
 kde_status kde_deposit_rows_f32(kde_ctx *ctx, const uint32_t *u, const float *kappa, float kappa_u, const float *norm,
                                 float norm_u, int64_t N, int Ng, double coef, float w_u, double bound, DepRows *out,
-                                float xcut)
+                                float xcut, const unsigned int *krange)
 {
     if (N < 1) return kde_fail(ctx, KDE_EINVAL, "deposit rows: need N >= 1");
     return deposit_sorted_impl<float>(ctx, u, kappa, kappa_u, norm, norm_u, nullptr, w_u, N, Ng, coef, nullptr, bound,
-                                      nullptr, 0.0, out, xcut);
+                                      nullptr, 0.0, out, xcut, krange);
 }
 
 template <typename T>

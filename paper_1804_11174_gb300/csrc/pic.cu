@@ -13,15 +13,21 @@
 #include "common.cuh"
 
 template <typename T>
-__global__ void norm_from_kappa_kernel(const T *kappa, int64_t N, T *norm, unsigned int *status, const float2 *ntab)
+__global__ void norm_from_kappa_kernel(const T *kappa, int64_t N, T *norm, unsigned int *status, const float2 *ntab,
+                                       unsigned int *krange)
 {
     int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= N) return;
+    if (i >= N) {
+        if (krange) kde_krange_add(krange, 3.0e38f, 0.f);
+        return;
+    }
     double k = (double)kappa[i];
     if (!(k > 0 && k <= KDE_KAPPA_MAX)) {
         kde_flag(status, KDE_DEV_KAPPA_RANGE, (unsigned)i);
         k = KDE_KAPPA_MAX;
     }
+    // the range of the widths as the deposit and the gather use them
+    if (krange) kde_krange_add(krange, (float)k, (float)k);
     // FP32 state: the tabulated norm; FP64 state: the FP64 Bessel series
     if constexpr (sizeof(T) == 4) norm[i] = (T)kde_norm_tab(ntab, (float)k);
     else norm[i] = (T)kde_norm(k);
@@ -229,9 +235,16 @@ static kde_status pic_run(kde_ctx *ctx, pic_state *st, int n_steps)
     // the AD schedule smooths h = kappa^{-1/2}, carried across the steps of this call
     double h_ad = adsched ? 1.0 / sqrt(st->kappa_uniform) : 0.0;
 
+    // FP32 particle-wise widths: their range, kept on the device beside them
+    unsigned int *krange = nullptr;
+    if (per && sizeof(T) == 4) {
+        krange = (unsigned int *)kde_ws(ctx, WS_PIC_RANGE, 64);
+        if (!krange) return KDE_ENOMEM;
+        KDE_CUDA(ctx, kde_krange_reset(krange, ctx->stream), "width range memset");
+    }
     if (per) {
         norm_from_kappa_kernel<T><<<(unsigned)((N + 255) / 256), 256, 0, ctx->stream>>>(
-            (const T *)st->kappa, N, norm_arr, ctx->d_status, ctx->norm_tab);
+            (const T *)st->kappa, N, norm_arr, ctx->d_status, ctx->norm_tab, krange);
         KDE_LAUNCHED(ctx, "norm_from_kappa_kernel");
     }
     const double coef = KDE_TWO_PI / L;
@@ -256,7 +269,7 @@ static kde_status pic_run(kde_ctx *ctx, pic_state *st, int n_steps)
                 KDE_TRY(kde_cv_device(ctx, st->u, nullptr, N, L, st->cand, st->n_cand, false, cv_dev, amin_dev, loo,
                                       ks_dev));
             KDE_TRY(kde_adapt_device(ctx, loo, N, L, ks_dev, 0.0, st->alpha, st->kappa_min, st->kappa_max, st->kappa,
-                                     norm_arr, sizeof(T) == 8));
+                                     norm_arr, sizeof(T) == 8, krange));
             k_cur = (const T *)st->kappa;  // the new widths and norms are in the state's arrays
             n_cur = (const T *)norm_arr;
             if (!fetch_ws()) return KDE_ENOMEM;
@@ -345,7 +358,7 @@ static kde_status pic_run(kde_ctx *ctx, pic_state *st, int n_steps)
             {
                 KdeRange r_("kdepic deposit");
                 KDE_TRY(kde_deposit_rows_f32(ctx, us, ks, (float)st->kappa_uniform, ns, (float)norm_u, N, Ng, coef,
-                                             (float)w_u, bound, &dr, cut));
+                                             (float)w_u, bound, &dr, cut, krange));
             }
             {
                 KdeRange r_("kdepic field (row sums + Poisson)");

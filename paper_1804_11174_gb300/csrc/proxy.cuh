@@ -1,0 +1,158 @@
+// proxy.cuh -- compression of many particles into few proxy particles.
+//
+// A kernel value f(theta_g; theta, kappa) = exp(-2 kappa sin^2((theta_g - theta)/2)), and
+// norm(kappa) f as well, is a smooth function of the particle's position and width, so over
+// an interval of positions of half-width a and widths in [kmin, kmax] it equals its
+// Chebyshev interpolant
+//     f(theta_g; theta, kappa) = sum_{a<P, b<Q} l_a(x) l_b(s) f(theta_g; theta_a, kappa_b),
+// x in [-1, 1] the position in the interval and s that of the width in its range, theta_a
+// and kappa_b the Chebyshev points (first kind).  A deposit sums its particles' weights into
+// P Q moments, turns these into P Q proxy particles (theta_a, kappa_b) with signed weights
+// and sweeps the nodes with the proxies alone; a gather evaluates the field at the proxies
+// and interpolates it at the particles.
+//
+// Degrees.  With y = a sqrt(kmax + 1.5) the interpolation error in position is below
+// 2 (y/2)^P / sqrt(P!) of the kernel's peak (derivatives of a Gaussian of variance 1/kappa;
+// the 1.5 covers small widths, where the cosine and not kappa sets the scale).  In the width
+// it depends on the range alone and holds for every distance: a linear map of kappa for
+// narrow ranges (by r = (kmax - kmin) / (kmax + kmin)), a linear map of ln kappa for wide
+// ones (by ln(kmax / kmin)).  P and Q are the smallest that keep each error below 2e-8 of
+// the peak: below one FP32 rounding, and below the 2^-24 at which kernels are truncated.
+#pragma once
+
+#include "common.cuh"
+
+#define PXY_MAXP 16
+#define PXY_MAXQ 40
+
+// interpolation matrices of degree D, c[p][a] = (2 - [p = 0]) / D cos(pi p (2a + 1) / (2D)),
+// D = 1 .. PXY_MAXQ one after another (built in FP64 when the context is created)
+__host__ __device__ constexpr int pxy_tab_off(int D) { return (D - 1) * D * (2 * D - 1) / 6; }
+#define PXY_TAB_N pxy_tab_off(PXY_MAXQ + 1)
+
+// smallest P with 2 (y/2)^P / sqrt(P!) <= 2e-8; PXY_MAXP + 1 when there is none up to PXY_MAXP
+__device__ __forceinline__ int pxy_degree_pos(float y)
+{
+    return 3 + (y > 0.0058f) + (y > 0.0298f) + (y > 0.0811f) + (y > 0.1606f) + (y > 0.2646f) + (y > 0.3880f) +
+           (y > 0.5260f) + (y > 0.6746f) + (y > 0.8304f) + (y > 0.9909f) + (y > 1.1544f) + (y > 1.3193f) +
+           (y > 1.4845f) + (y > 1.6493f);
+}
+// the linear map of kappa reaches 2e-8 with six points up to this r
+#define PXY_LIN_R 0.12f
+// smallest Q whose interpolant of e^{-s e^t} in t has an error of at most 2e-8 for every
+// s >= 0 over a range of length l = ln(kmax / kmin) (measured; 4.5 + 4.86 l bounds it above
+// l = 0.379); above PXY_MAXQ when the range is too wide
+__device__ __forceinline__ int pxy_degree_log(float l)
+{
+    if (l <= 0.379f) return 3 + (l > 0.0208f) + (l > 0.0861f) + (l > 0.2077f);
+    return (int)fminf(ceilf(fmaf(4.86f, l, 4.5f)), 1000.f);
+}
+
+// an Ng-node grid in position codes: node g is at code g step + (g rem) / Ng, with
+// 2^32 = step Ng + rem (g rem < 2^24)
+struct PxyGrid {
+    int Ng;
+    uint32_t step, rem;
+};
+inline PxyGrid pxy_grid(int Ng)
+{
+    PxyGrid g;
+    g.Ng = Ng;
+    g.step = (uint32_t)((1ull << 32) / (uint64_t)Ng);  // Ng = 1: 2^32 wraps to 0, and the only node is 0
+    g.rem = (uint32_t)((1ull << 32) % (uint64_t)Ng);
+    return g;
+}
+__device__ __forceinline__ void pxy_node(const PxyGrid &G, int g, uint32_t &code, float &frac)
+{
+    code = (uint32_t)g * G.step;
+    frac = 0.f;
+    if (G.rem) {
+        const uint32_t m = (uint32_t)g * G.rem, q = m / (uint32_t)G.Ng;
+        code += q;
+        frac = (float)(m - q * (uint32_t)G.Ng) / (float)G.Ng;
+    }
+}
+
+// interval of positions and range of widths
+struct PxyBox {
+    uint32_t mid;  // middle position (code)
+    float hw;      // half-width in codes
+    float inv_hw;
+    float kc, kh, inv_kh;  // middle and half-length of the range of kappa (linear) or ln kappa
+    int P, Q;              // degrees (Q = 1: one width)
+    bool lin;
+};
+
+// positions of the whole cells [c_first, c_last], 0 <= c_first <= c_last < Ng
+__device__ __forceinline__ void pxy_box_pos(PxyBox &B, const PxyGrid &G, int c_first, int c_last, float kmax)
+{
+    uint32_t lo, hi;
+    float f;
+    pxy_node(G, c_first, lo, f);
+    pxy_node(G, c_last + 1, hi, f);  // the end of the grid, 2^32, wraps to 0
+    if (c_last + 1 == G.Ng) hi = 0u;
+    const uint32_t len = hi - lo;  // 0: the whole circle
+    const uint32_t half = len ? (len >> 1) + (len & 1u) : 0x80000000u;
+    B.mid = lo + half;
+    B.hw = (float)half;
+    B.inv_hw = 1.f / B.hw;
+    B.P = pxy_degree_pos(B.hw * (float)(KDE_TWO_PI / 4294967296.0) * sqrtf(kmax + 1.5f));
+}
+__device__ __forceinline__ void pxy_box_width(PxyBox &B, float kmin, float kmax)
+{
+    B.lin = kmax - kmin <= PXY_LIN_R * (kmax + kmin);
+    if (kmin == kmax) {
+        B.Q = 1;
+        B.kc = kmin;
+        B.kh = B.inv_kh = 0.f;
+    } else if (B.lin) {
+        B.Q = 6;
+        B.kc = 0.5f * (kmin + kmax);
+        B.kh = 0.5f * (kmax - kmin);
+        B.inv_kh = 1.f / B.kh;
+    } else {
+        const float l0 = logf(kmin), l1 = logf(kmax);
+        B.Q = pxy_degree_log(l1 - l0);
+        B.kc = 0.5f * (l0 + l1);
+        B.kh = 0.5f * (l1 - l0);
+        B.inv_kh = 1.f / B.kh;
+    }
+}
+
+// position in the box, [-1, 1]: the code difference is exact
+__device__ __forceinline__ float pxy_x(const PxyBox &B, uint32_t u) { return (float)(int32_t)(u - B.mid) * B.inv_hw; }
+__device__ __forceinline__ float pxy_s(const PxyBox &B, float kappa)
+{
+    return ((B.lin ? kappa : logf(kappa)) - B.kc) * B.inv_kh;
+}
+// proxy a of P at Chebyshev point x: code and fraction of a code (the rounding of the
+// product is carried exactly)
+__device__ __forceinline__ void pxy_pos(const PxyBox &B, float x, uint32_t &code, float &frac)
+{
+    const float p = B.hw * x, e = fmaf(B.hw, x, -p), r = rintf(p);
+    code = B.mid + (uint32_t)__float2int_rn(r);
+    frac = (p - r) + e;
+}
+// proxy width at Chebyshev point s
+__device__ __forceinline__ float pxy_kappa(const PxyBox &B, float s)
+{
+    const float k = fmaf(B.kh, s, B.kc);
+    return B.lin ? k : expf(k);
+}
+
+// sin^2 of half the angle between two positions given as codes and fractions.  The code
+// difference is exact, so near pairs keep full relative accuracy; sin(pi f) for
+// f in [-1/2, 1/2] by its Taylor series (the first term left out is below 7e-10 relative)
+__device__ __forceinline__ float pxy_sin2(uint32_t na, float fa, uint32_t nb, float fb)
+{
+    const float f = ((float)(int32_t)(na - nb) + (fa - fb)) * (1.f / 4294967296.f), t = f * f;
+    float s = (float)(0.00046630280576761256);  // pi^13 / 13!
+    s = fmaf(s, t, (float)(-0.0073704309457143504));
+    s = fmaf(s, t, (float)(0.082145886611128228));
+    s = fmaf(s, t, (float)(-0.59926452932079208));
+    s = fmaf(s, t, (float)(2.5501640398773454));
+    s = fmaf(s, t, (float)(-5.1677127800499701));
+    s = fmaf(s, t, (float)(3.1415926535897932));
+    s *= f;
+    return s * s;
+}
