@@ -230,7 +230,9 @@ kde_status kde_poisson(kde_ctx *ctx, const void *rho, int32_t Ng, double L, doub
 /* Gather through the deposit's kernels:
  *   out_i = sum_g (2 pi / Ng) K_{kappa_i}(theta_g - theta_i) field_g.
  * u: uint32[N] (any order); kappa: real[N] or NULL (kappa_uniform); field:
- * real[Ng]; out: real[N] in the order of u.  Flags: KDE_F64. */
+ * real[Ng]; out: real[N] in the order of u.  Flags: KDE_F64.  FP32 calls at the
+ * default truncation interpolate the smoothed field from tables (error below 5e-8 of
+ * a kernel's peak); a cut set by kde_set_truncation sweeps the nodes. */
 kde_status kde_gather(kde_ctx *ctx, const uint32_t *u, const void *kappa, double kappa_uniform,
                       int64_t N, const void *field, int32_t Ng, double L, void *out,
                       uint32_t flags);

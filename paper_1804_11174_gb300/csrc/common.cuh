@@ -96,6 +96,7 @@ enum WsSlot {
     WS_HOST_NORM,
     WS_HOST_ID,
     WS_HOST_HIST,  // energy, kappa* and ln p histories
+    WS_GTAB,       // tables of the smoothed field (plain FP32 gather)
     WS_TUNE,       // truncation tuner: reference and candidate fields and their error sums
     WS_NSLOTS
 };
@@ -522,11 +523,17 @@ struct PushArgs {
     unsigned int *counts;    // FP32 gather: count table of the next cell sort (kde_sort_counts_table), or null
     int cnt_nblk, cnt_shift;
     float xcut;              // FP32 truncation cut exponent (kde_fp32_cut), 0: the context's default
+    const unsigned int *krange;  // FP32: float bits of the largest and smallest width, or null
 };
 template <typename T>
 kde_status kde_gather_sorted(kde_ctx *ctx, const uint32_t *u, const T *kappa, T kappa_u, const T *norm, T norm_u,
                              int64_t N, const T *field, int Ng, double coef, T *out, const uint32_t *perm,
-                             const PushArgs *push, float xcut = 0.f);
+                             const PushArgs *push, float xcut = 0.f, const unsigned int *krange = nullptr);
+
+// the plain FP32 gather of particles in any order, at the default truncation (gtable.cu)
+kde_status kde_gather_table(kde_ctx *ctx, const uint32_t *u, const float *kappa, double kappa_u, int64_t N,
+                            const float *field, int Ng, float *out);
+kde_status kde_gather_table_reserve(kde_ctx *ctx);  // grows its workspace (kde_reserve)
 
 // candidate widths (or scale factors) for the CV kernels, passed by value
 struct CandList {

@@ -551,6 +551,7 @@ struct DepPlan {
     long long *rows;  // [G][Ng] per-CTA node sums over its window
     int2 *hdr;        // [G] (first node, node count) of every row
     long long *acc;   // [Ng] output accumulators (every node written by the row reduction)
+    float fixed;      // cost of the compressed form's fixed steps (depp_compress_pays)
 };
 // node pairs of the persistent deposit: each lane owns P pairs of nodes (64 P
 // consecutive nodes a warp pass) of the window [g_lo, g_lo + R); the n records of
@@ -976,11 +977,11 @@ __device__ __forceinline__ void depp_proxies(const DepSrc<float> &S, const PxyBo
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int P = B.P, Q = B.Q, PQ = P * Q, Ng = S.Ng;
     const float *cp = S.pxt + pxy_tab_off(P), *cq = S.pxt + pxy_tab_off(Q);
-    float *U = mem, *W = U + PQ, *fr = W + PQ, *k2 = fr + P;
-    uint32_t *cd = (uint32_t *)(k2 + Q);
-    // proxy positions and exponent factors -2 kappa_b log2 e (the Chebyshev points are
+    float *U = mem, *W = U + PQ, *sd = W + PQ, *cd = sd + P, *k2 = cd + P;
+    // sine and cosine of half the proxies' angles from the box's middle, and exponent factors -2 kappa_b log2 e (the Chebyshev points are
     // the matrices' second rows times D / 2)
-    if (tid < P) pxy_pos(B, P > 1 ? cp[P + tid] * (0.5f * (float)P) : 0.f, cd[tid], fr[tid]);
+    if (tid < P)
+        sincospif((P > 1 ? cp[P + tid] * (0.5f * (float)P) : 0.f) * (B.hw * (1.f / 4294967296.f)), &sd[tid], &cd[tid]);
     if (tid >= 64 && tid < 64 + Q) {
         const int b = tid - 64;
         k2[b] = (float)(-2.0 * KDE_LOG2E) * (Q > 1 ? pxy_kappa(B, cq[Q + b] * (0.5f * (float)Q)) : B.kc);
@@ -1011,10 +1012,13 @@ __device__ __forceinline__ void depp_proxies(const DepSrc<float> &S, const PxyBo
         uint32_t nc;
         float nf;
         pxy_node(S.grid, g, nc, nf);
-        float acc = 0.f;
+        float acc = 0.f, sn, cn;
+        pxy_sincos(nc, nf, B.mid, 0.f, sn, cn);
 #pragma unroll 1
         for (int a = a0; a < P; a += da) {
-            const float s2 = pxy_sin2(nc, nf, cd[a], fr[a]);
+            // the box is at most 1.65 standard deviations of its narrowest kernel wide on either
+            // side, so the angle difference keeps 1e-7 of that width
+            const float sa = fmaf(sn, cd[a], -cn * sd[a]), s2 = sa * sa;
             const float *w = W + a * Q;
             int b = Q - 1;
             for (; b >= 3; b -= 4) {  // four at a time: the first has the largest value
@@ -1047,16 +1051,18 @@ __device__ __forceinline__ void depp_proxies(const DepSrc<float> &S, const PxyBo
 // whether the compressed form costs less than the direct sweep: instructions of a lane,
 // direct about 3.2 a (particle, node) pair and 48 a particle; compressed 55 a particle plus
 // its Chebyshev values and moments (shared by the lanes of a warp), then 16 a (node, proxy
-// position), 3 a (node, proxy), the interpolation matrices and a CTA's fixed steps.  Near the
-// line: 658 particles a CTA in windows of 27 nodes with P = 11 (300,007 particles, 512 nodes,
-// width 2000) take 10.5 us direct and 13.5 compressed, so they stay direct
-__device__ __forceinline__ bool depp_compress_pays(const PxyBox &B, int n, int R)
+// position), 3 a (node, proxy), the interpolation matrices and the fixed steps -- barriers and
+// table loads, which other CTAs cover where an SM has three but not where it has one.  Near
+// the lines: 658 particles a CTA in windows of 27 nodes with P = 11 (300,007 particles, 512
+// nodes, width 2000) take 10.5 us direct and 13.5 compressed; a PIC step of 3202 particles on
+// 118 nodes 39 us direct and 44 compressed
+__device__ __forceinline__ bool depp_compress_pays(const PxyBox &B, int n, int R, float fixed)
 {
     // the moment tiles of the matrix product have to fit a warp
     if (B.P > PXY_MAXP || B.Q > PXY_MAXQ || ((B.P + 3) >> 2) * ((B.Q + 3) >> 2) > 32) return false;
     const float fn = (float)n, fR = (float)R, P = (float)B.P, Q = (float)B.Q, PQ = P * Q;
     const float direct = fn * (3.2f * fR + 48.f);
-    const float comp = fn * (55.f + 3.f * (P + Q) + 1.6f * PQ) + fR * P * (16.f + 3.f * Q) + PQ * (P + Q) * 4.f + 40000.f;
+    const float comp = fn * (55.f + 3.f * (P + Q) + 1.6f * PQ) + fR * P * (16.f + 3.f * Q) + PQ * (P + Q) * 4.f + fixed;
     return comp < direct;
 }
 
@@ -1100,6 +1106,8 @@ __global__ void __launch_bounds__(DEPP_RED_THREADS) deposit_rows_kernel(const lo
     }
 }
 
+// COMP: with the compressed form, chosen per CTA; without it where no CTA would take it
+template <bool COMP>
 __global__ void __launch_bounds__(DEPP_THREADS, DEPP_MINB) deposit_persist_kernel(DepSrc<float> S, DepPlan Pl)
 {
     __shared__ float4 rec[DEPP_SUB];
@@ -1184,14 +1192,15 @@ __global__ void __launch_bounds__(DEPP_THREADS, DEPP_MINB) deposit_persist_kerne
                   : (2 * n128 == n64 && (n128 >= DEPP_WARPS || n128 * 128 <= DEPP_PART)) ? 2
                                                                                           : 1;
     long long *row = Pl.rows + (size_t)c * Ng;
-    if (S.xcut == (float)KDE_XCUT && c_last >= c_first) {
+    if constexpr (COMP) {
+    if (c_last >= c_first) {
         // the default cut: compressed where that is less work (a cut the caller has set keeps
         // the sweep over the particles that it is defined for)
         PxyBox B;
         pxy_box_pos(B, S.grid, c_first, c_last, kmax);
         pxy_box_width(B, kmin, kmax);
         const int n = (int)(i1 - i0);
-        if (depp_compress_pays(B, n, R)) {
+        if (depp_compress_pays(B, n, R, Pl.fixed)) {
             __shared__ float M[PXY_MAXP * PXY_MAXQ];
             bool normed = true;
             if (B.Q == 1) {
@@ -1219,6 +1228,7 @@ __global__ void __launch_bounds__(DEPP_THREADS, DEPP_MINB) deposit_persist_kerne
             if (tid == 0) Pl.hdr[c] = make_int2(g_lo, R);
             return;
         }
+    }
     }
 
     for (int64_t b0 = i0; b0 < i1; b0 += DEPP_SUB) {
@@ -1347,6 +1357,7 @@ static kde_status depp_plan(kde_ctx *ctx, int64_t N, int Ng, long long *acc, Dep
     Pl.rows = (long long *)w;
     Pl.hdr = (int2 *)(w + rows_b);
     Pl.acc = acc;
+    Pl.fixed = Pl.G <= ctx->sm_count ? 3.0e5f : 6.0e4f;
     return KDE_OK;
 }
 
@@ -1404,7 +1415,14 @@ static kde_status deposit_sorted_impl(kde_ctx *ctx, const uint32_t *u, const T *
         KDE_TRY(depp_plan(ctx, N, Ng, acc, Pl));
         {
             KdeProfScope _ps(ctx, PROF_DEPOSIT);
-            KDE_CUDA(ctx, kde_launch(ctx, true, deposit_persist_kernel, dim3(Pl.G), dim3(DEPP_THREADS), 0, S, Pl),
+            // the compressed form is for the default cut (one the caller has set keeps the sweep
+            // over the particles that it is defined for), and for CTAs whose sweep of the whole
+            // grid would cost more than its fixed steps
+            const double n = (double)N / Pl.G;
+            const bool comp = S.xcut == (float)KDE_XCUT && n * (3.2 * Ng + 48.0) > (double)Pl.fixed;
+            KDE_CUDA(ctx,
+                     kde_launch(ctx, true, comp ? deposit_persist_kernel<true> : deposit_persist_kernel<false>,
+                                dim3(Pl.G), dim3(DEPP_THREADS), 0, S, Pl),
                      "deposit_persist_kernel");
         }
         KDE_LAUNCHED(ctx, "deposit_persist_kernel");

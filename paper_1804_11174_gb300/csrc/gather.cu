@@ -10,6 +10,7 @@
 // push, the write-back of the particle state and (block 0) the field energy
 // ride in the same kernel.
 #include "common.cuh"
+#include "proxy.cuh"
 
 #define GAT_THREADS 256
 
@@ -59,6 +60,10 @@ template <typename T> struct GatherArgs {
     unsigned int *counts;
     int cnt_nblk, cnt_shift;
     float xcut = (float)KDE_XCUT;  // FP32 packed gather: truncation cut exponent
+    PxyGrid grid;                    // the nodes as position codes
+    const float *pxt;                // interpolation matrices (proxy.cuh)
+    const unsigned int *krange;      // float bits of the largest and smallest width, or null
+    int tile;                        // particles of a CTA of gather_tile_kernel
 };
 
 __device__ __forceinline__ int window_nodes_g(float kappa, int Ng, float xcut)
@@ -222,6 +227,67 @@ __device__ __forceinline__ void gat2_nodes(const float4 *SC, const float2 *FF, i
     for (int g = 0; g < e2; ++g) node(g);
 }
 
+// the end of a warp's gather of NP particles a lane (particle base + 32 h + lane) with codes
+// uu and fields ea: the push and the write-back of the state, or the plain output.  VIN: the
+// velocities are in vin already
+template <bool VIN, int NP>
+__device__ __forceinline__ void gat_finish(const GatherArgs<float> &A, int64_t base, int lane, const uint32_t (&uu)[NP],
+                                           const float (&ea)[NP], const float *vpre)
+{
+    const int Ng = A.Ng;
+    if (A.u_out) {
+        // the push's inputs of four particles at a time first (one load latency per group;
+        // the stores below alias nothing the loads read, but the compiler cannot know
+        // that), then the stores
+        constexpr int HB = NP % 4 == 0 ? 4 : (NP % 3 == 0 ? 3 : 2);
+#pragma unroll
+        for (int h0 = 0; h0 < NP; h0 += HB) {
+            float vin[HB], kin[HB], nin[HB];
+            uint32_t idin[HB];
+#pragma unroll
+            for (int hh = 0; hh < HB; ++hh) {
+                const int64_t j = base + (h0 + hh) * 32 + lane;
+                const bool ok = j < A.N;
+                vin[hh] = VIN ? vpre[h0 + hh] : (ok ? A.v_in[j] : 0.f);
+                kin[hh] = (ok && A.kappa_out) ? (A.kappa ? A.kappa[j] : A.kappa_u) : 0.f;
+                nin[hh] = (ok && A.norm_out) ? A.norm_in[j] : 0.f;
+                idin[hh] = (ok && A.id_out) ? A.id_in[j] : 0u;
+            }
+#pragma unroll
+            for (int hh = 0; hh < HB; ++hh) {
+                const int h = h0 + hh;
+                const int64_t j = base + h * 32 + lane;
+                int key = -1;
+                if (j < A.N) {
+                    const float v = vin[hh] + A.kick_qm_dt * ea[h];
+                    A.v_out[j] = v;
+                    const uint32_t nu = advance_position(uu[h], v * A.dt_scale);
+                    A.u_out[j] = nu;
+                    if (A.kappa_out) {
+                        const float k = kin[hh];
+                        A.kappa_out[j] = (k > 0.f && k <= (float)KDE_KAPPA_MAX) ? k : (float)KDE_KAPPA_MAX;
+                    }
+                    if (A.norm_out) A.norm_out[j] = nin[hh];
+                    if (A.id_out) A.id_out[j] = idin[hh];
+                    key = kde_cell(nu, Ng);
+                }
+                if (A.counts) {  // warp-uniform; the 32 particles of a round share one sort tile
+                    const unsigned int peers = __match_any_sync(0xffffffffu, key);
+                    if (key >= 0 && lane == __ffs(peers) - 1)
+                        atomicAdd(&A.counts[(size_t)key * A.cnt_nblk + (size_t)(j >> A.cnt_shift)],
+                                  (unsigned int)__popc(peers));
+                }
+            }
+        }
+    } else {
+#pragma unroll
+        for (int h = 0; h < NP; ++h) {
+            const int64_t j = base + h * 32 + lane;
+            if (j < A.N) A.out[A.perm ? A.perm[j] : j] = ea[h];
+        }
+    }
+}
+
 template <int NP, int UD, int US, int MINB>
 __global__ void __launch_bounds__(GAT2_WARPS * 32, MINB) gather2_kernel(GatherArgs<float> A)
 {
@@ -362,55 +428,443 @@ __global__ void __launch_bounds__(GAT2_WARPS * 32, MINB) gather2_kernel(GatherAr
     float ea[GAT2_NP];
 #pragma unroll
     for (int q = 0; q < NPP; ++q) kde_upk(acc[q], ea[2 * q], ea[2 * q + 1]);
-    if (A.u_out) {
-        // the push's inputs of four particles at a time first (one load latency per group;
-        // the stores below alias nothing the loads read, but the compiler cannot know
-        // that), then the stores
-        constexpr int HB = GAT2_NP % 4 == 0 ? 4 : (GAT2_NP % 3 == 0 ? 3 : 2);
 #pragma unroll
-        for (int h0 = 0; h0 < GAT2_NP; h0 += HB) {
-        float vin[HB], kin[HB], nin[HB];
-        uint32_t idin[HB];
+    for (int h = 0; h < GAT2_NP; ++h) ea[h] *= nm[h] * A.coef;
+    gat_finish<false>(A, base, lane, uu, ea, nullptr);
+}
+
+// ---------------------------------------------------------------------------
+// Gather + push of cell-sorted particles through proxies (proxy.cuh): a CTA takes
+// A.tile consecutive particles -- an interval of whole cells, widths in [kmin, kmax] --
+// evaluates the field at P Q proxy particles from the nodes, turns these values into the
+// coefficients of the joint Chebyshev interpolant and evaluates that at its particles.  A
+// particle then costs its Chebyshev values and P (one width) or 28 to 48 multiply-adds
+// (packed for two particles) whatever the window, and no norm is read: the normalisation is
+// interpolated with the kernel.  Tiles whose range of widths is too wide, or whose windows are short
+// beside P Q, sweep the nodes particle by particle as gather2_kernel does (GATT_WARPS
+// warps, 128 particles each at a time).
+// Everything before kde_pdl_wait() -- the box, the proxies -- overlaps the field kernel.
+// Bound by instruction issue and fetch (a tile runs straight through its code) and latency.
+// Measured: 2^20 particles on 256 nodes, widths near 14, 38.6 us swept, 22.8 in tiles; a step of
+// 32 realisations of 2^14 to 2^20 particles 824 -> 590 us.
+// ---------------------------------------------------------------------------
+#define GATT_THREADS 256
+#define GATT_WARPS 8
+#define GATT_UNIT 1024  // particles the CTA's warps take in a round, 4 a lane
+
+// sums over the warp of v[0..7] (lane l ends with the sum of v[(l >> 2) & 7])
+__device__ __forceinline__ float warp_sum8(float (&v)[8], int lane)
+{
 #pragma unroll
-        for (int hh = 0; hh < HB; ++hh) {
-            const int64_t j = base + (h0 + hh) * 32 + lane;
-            const bool ok = j < A.N;
-            vin[hh] = ok ? A.v_in[j] : 0.f;
-            kin[hh] = (ok && A.kappa_out) ? (A.kappa ? A.kappa[j] : A.kappa_u) : 0.f;
-            nin[hh] = (ok && A.norm_out) ? A.norm_in[j] : 0.f;
-            idin[hh] = (ok && A.id_out) ? A.id_in[j] : 0u;
+    for (int o = 4; o >= 1; o >>= 1) {
+        const bool up = (lane & (o * 4)) != 0;
+#pragma unroll
+        for (int i = 0; i < o; ++i) {
+            const float send = up ? v[i] : v[i + o], keep = up ? v[i + o] : v[i];
+            v[i] = keep + __shfl_xor_sync(0xffffffffu, send, o * 4);
+        }
+    }
+    float r = v[0];
+    r += __shfl_xor_sync(0xffffffffu, r, 1);
+    r += __shfl_xor_sync(0xffffffffu, r, 2);
+    return r;
+}
+
+// field at the PM x QM proxies of the box from the window nodes, then coefficients
+// C[p QM + q] (the normalisation and coef included), each stored twice for the packed
+// evaluation.  s2: sin^2 of the thread's first node (r = tid) and every proxy position, known
+// before the field; tabs: the interpolation matrices of PM and QM in shared memory;
+// part: GATT_WARPS x PM x QM floats; F: 2 PM QM floats
+template <int PM, int QM>
+__device__ __forceinline__ void gatt_coefs(const GatherArgs<float> &A, int g_lo, int R, const float *s2a,
+                                           const uint32_t *cd, const float *fr, const float *k2, const float *nk,
+                                           const float *tabs, float *part, float *F, float2 *C)
+{
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, Ng = A.Ng;
+    constexpr int PQ = PM * QM;
+    auto wrap = [&](int r) {
+        const int g = g_lo + r;
+        return g < 0 ? g + Ng : (g >= Ng ? g - Ng : g);
+    };
+    const float e0 = tid < R ? A.field[wrap(tid)] : 0.f;
+    float kk[QM];
+#pragma unroll
+    for (int b = 0; b < QM; ++b) kk[b] = k2[b];
+#pragma unroll(QM == 1 ? PM : 1)
+    for (int a = 0; a < PM; ++a) {
+        float v[8];
+        const float s2 = s2a[a * GATT_THREADS + tid];
+#pragma unroll
+        for (int b = 0; b < 8; ++b) v[b] = b < QM ? kde_ex2(s2 * kk[b < QM ? b : 0]) * e0 : 0.f;
+        if (R > GATT_THREADS) {
+            const uint32_t ca = cd[a];
+            const float fa = fr[a];
+#pragma unroll 1
+            for (int r = tid + GATT_THREADS; r < R; r += GATT_THREADS) {
+                const int g = wrap(r);
+                uint32_t nc;
+                float nf;
+                pxy_node(A.grid, g, nc, nf);
+                const float s2r = pxy_sin2(nc, nf, ca, fa), e = A.field[g];
+#pragma unroll
+                for (int b = 0; b < QM; ++b) v[b] = fmaf(kde_ex2(s2r * kk[b]), e, v[b]);
+            }
+        }
+        if (QM == 1) {
+            float w = v[0];
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) w += __shfl_xor_sync(0xffffffffu, w, o);
+            if (lane == 0) part[warp * PM + a] = w;
+        } else {
+            const float w = warp_sum8(v, lane);
+            if ((lane & 3) == 0 && (lane >> 2) < QM) part[(warp * PM + a) * QM + (lane >> 2)] = w;
+        }
+    }
+    __syncthreads();
+    const float *cp = tabs, *cq = tabs + PM * PM;
+    for (int i = tid; i < PQ; i += GATT_THREADS) {
+        float f = 0.f;
+#pragma unroll
+        for (int w = 0; w < GATT_WARPS; ++w) f += part[w * PQ + i];
+        F[i] = f * nk[i % QM];
+    }
+    __syncthreads();
+    float *U = F + PQ;
+    for (int i = tid; i < PQ; i += GATT_THREADS) {
+        const int p = i / QM, b = i % QM;
+        float f = 0.f;
+#pragma unroll
+        for (int a = 0; a < PM; ++a) f = fmaf(cp[p * PM + a], F[a * QM + b], f);
+        U[i] = f;
+    }
+    if (QM > 1) __syncthreads();
+    for (int i = tid; i < PQ; i += GATT_THREADS) {
+        const int p = i / QM, q = i % QM;
+        float f = 0.f;
+#pragma unroll
+        for (int b = 0; b < QM; ++b) f = fmaf(cq[q * QM + b], U[p * QM + b], f);
+        C[i] = make_float2(f, f);
+    }
+    __syncthreads();
+}
+
+// the interpolant at four particles a lane (two packed pairs); TRI: the coefficients with
+// p / PM + q / QM < 1 alone
+template <int PM, int QM, bool TRI>
+__device__ __forceinline__ void gatt_eval(const GatherArgs<float> &A, const PxyBox &B, const float2 *C, int64_t base,
+                                          int lane, const uint32_t (&uu)[4], const float (&kap)[4], float (&ea)[4])
+{
+    float xs[4], ss[4];
+#pragma unroll
+    for (int h = 0; h < 4; ++h) {
+        const int64_t j = base + h * 32 + lane;
+        xs[h] = pxy_x(B, uu[h]);
+        ss[h] = 0.f;
+        if (QM > 1) {
+            float k = kap[h];
+            if (!(k > 0.f && k <= (float)KDE_KAPPA_MAX)) {
+                if (j < A.N) kde_flag(A.status, KDE_DEV_KAPPA_RANGE, (unsigned)j);
+                k = (float)KDE_KAPPA_MAX;
+            }
+            ss[h] = (k - B.kc) * B.inv_kh;
+        }
+    }
+    const kde_f2 one = kde_pk(1.f, 1.f), neg = kde_pk(-1.f, -1.f);
+    kde_f2 x[2], x2[2], s[2], t0[2], t1[2], acc[2], tq[QM][2];
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+        x[h] = kde_pk(xs[2 * h], xs[2 * h + 1]);
+        x2[h] = kde_pk(2.f * xs[2 * h], 2.f * xs[2 * h + 1]);
+        s[h] = kde_pk(ss[2 * h], ss[2 * h + 1]);
+        tq[0][h] = one;
+        if (QM > 1) tq[1 % QM][h] = s[h];
+#pragma unroll
+        for (int q = 2; q < QM; ++q) {
+            const kde_f2 sq = kde_fma2(s[h], tq[q - 1][h], kde_pk(0.f, 0.f));
+            tq[q][h] = kde_fma2(kde_pk(2.f, 2.f), sq, kde_mul2(neg, tq[q - 2][h]));
+        }
+        t0[h] = one;
+        t1[h] = x[h];
+    }
+#pragma unroll
+    for (int p = 0; p < PM; ++p) {
+        kde_f2 row[2];
+#pragma unroll
+        for (int q = 0; q < QM; ++q) {
+            if (TRI && p * QM + q * PM >= PM * QM) continue;
+            const float2 c2 = C[p * QM + q];
+            const kde_f2 c = kde_pk(c2.x, c2.y);
+#pragma unroll
+            for (int h = 0; h < 2; ++h) row[h] = q == 0 ? c : kde_fma2(c, tq[q][h], row[h]);
         }
 #pragma unroll
-        for (int hh = 0; hh < HB; ++hh) {
-            const int h = h0 + hh;
+        for (int h = 0; h < 2; ++h) {
+            if (p == 0) {
+                acc[h] = row[h];
+            } else {
+                acc[h] = kde_fma2(row[h], t1[h], acc[h]);
+                const kde_f2 t2 = kde_fma2(x2[h], t1[h], kde_mul2(neg, t0[h]));
+                t0[h] = t1[h];
+                t1[h] = t2;
+            }
+        }
+    }
+#pragma unroll
+    for (int h = 0; h < 2; ++h) kde_upk(acc[h], ea[2 * h], ea[2 * h + 1]);
+}
+
+// the direct sweep of one warp's 128 particles: node tables SC and FF of the whole grid in
+// shared memory, in the form cosf
+__device__ __forceinline__ void gatt_direct(const GatherArgs<float> &A, const float4 *SC, const float2 *FF, bool cosf,
+                                            int64_t base, int lane, const uint32_t (&uu)[4], const float (&kap)[4],
+                                            float (&ea)[4])
+{
+    const int Ng = A.Ng;
+    float ps[4], pc[4], nm[4];
+    int lo = 0x3fffffff, hi = -0x3fffffff;
+    float kmin = (float)KDE_KAPPA_MAX;
+#pragma unroll
+    for (int h = 0; h < 4; ++h) {
+        const int64_t j = base + h * 32 + lane;
+        const bool valid = j < A.N;
+        float k = kap[h];
+        if (!(k > 0.f && k <= (float)KDE_KAPPA_MAX)) {
+            if (valid) kde_flag(A.status, KDE_DEV_KAPPA_RANGE, (unsigned)j);
+            k = (float)KDE_KAPPA_MAX;
+        }
+        nm[h] = A.norm ? (valid ? A.norm[j] : 0.f) : (A.kappa ? kde_norm_tab(A.ntab, k) : A.norm_u);
+        if (valid) {
+            kmin = fminf(kmin, k);
+            const int cell = kde_cell(uu[h], Ng);
+            lo = min(lo, cell);
+            hi = max(hi, cell);
+        }
+        float sh, ch;
+        kde_half_sincos(uu[h], sh, ch);
+        if (cosf) {
+            const float K = (float)KDE_LOG2E * k;
+            ps[h] = K * (2.f * sh * ch);
+            pc[h] = K * ((ch - sh) * (ch + sh));
+            nm[h] *= kde_ex2(-K);
+        } else {
+            const float beta = sqrtf((float)(2.0 * KDE_LOG2E) * k);
+            ps[h] = beta * ch;
+            pc[h] = beta * sh;
+        }
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        lo = min(lo, __shfl_xor_sync(0xffffffffu, lo, o));
+        hi = max(hi, __shfl_xor_sync(0xffffffffu, hi, o));
+        kmin = fminf(kmin, __shfl_xor_sync(0xffffffffu, kmin, o));
+    }
+    if (lo <= hi) {
+        const int W = window_nodes_g(kmin, Ng, A.xcut);
+        lo -= W;
+        hi += W;
+    }
+    int len = hi - lo + 1;
+    if (len >= Ng) {
+        lo = 0;
+        len = Ng;
+    }
+    kde_f2 psP[2], pcP[2], acc[2];
+#pragma unroll
+    for (int q = 0; q < 2; ++q) {
+        psP[q] = kde_pk(ps[2 * q], ps[2 * q + 1]);
+        pcP[q] = kde_pk(pc[2 * q], pc[2 * q + 1]);
+        acc[q] = kde_pk(0.f, 0.f);
+    }
+    if (len > 0) {
+        int g0 = lo % Ng;
+        if (g0 < 0) g0 += Ng;
+        const int e1 = g0 + len < Ng ? g0 + len : Ng, e2 = len - (e1 - g0);
+        const bool deep = len >= GAT2_DEEP_LEN;
+        if (cosf) {
+            if (deep) gat2_nodes<8, true, 2>(SC, FF, g0, e1, e2, psP, pcP, acc);
+            else gat2_nodes<4, true, 2>(SC, FF, g0, e1, e2, psP, pcP, acc);
+        } else {
+            if (deep) gat2_nodes<8, false, 2>(SC, FF, g0, e1, e2, psP, pcP, acc);
+            else gat2_nodes<4, false, 2>(SC, FF, g0, e1, e2, psP, pcP, acc);
+        }
+    }
+#pragma unroll
+    for (int q = 0; q < 2; ++q) kde_upk(acc[q], ea[2 * q], ea[2 * q + 1]);
+#pragma unroll
+    for (int h = 0; h < 4; ++h) ea[h] *= nm[h] * A.coef;
+}
+
+// C of the compressed forms: degrees (P, Q) as evaluated
+#define GATT_FORM_P(f) ((f) == 1 ? 8 : ((f) == 2 ? 16 : ((f) == 3 ? 7 : 8)))
+#define GATT_FORM_Q(f) ((f) <= 2 ? 1 : ((f) == 3 ? 7 : 6))
+
+__global__ void __launch_bounds__(GATT_THREADS, 3) gather_tile_kernel(GatherArgs<float> A)
+{
+    extern __shared__ __align__(16) unsigned char sm[];
+    __shared__ uint32_t cd[PXY_MAXP];
+    __shared__ float fr[PXY_MAXP], k2[8], nk[8];
+    __shared__ float tabs[PXY_MAXP * PXY_MAXP + 8], part[GATT_WARPS * 49], F[2 * 49];
+    __shared__ float s2a[PXY_MAXP * GATT_THREADS];
+    __shared__ __align__(16) float2 C[50];
+    __shared__ float kred[2 * GATT_WARPS];
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, Ng = A.Ng;
+    if (A.energy && blockIdx.x == gridDim.x - 1) {
+        // the last CTA of the grid has the field energy alone
+        double *red = (double *)s2a;
+        kde_pdl_wait();
+        kde_pdl_trigger();
+        double sum = 0.0;
+        for (int g = tid; g < Ng; g += GATT_THREADS) sum += (double)A.field[g] * (double)A.field[g];
+        red[tid] = sum;
+        __syncthreads();
+        for (int o = GATT_THREADS / 2; o > 0; o >>= 1) {
+            if (tid < o) red[tid] += red[tid + o];
+            __syncthreads();
+        }
+        if (tid == 0) {
+            A.energy[0] = 0.5 * red[0] * A.dx;
+            if (A.kstar_out) A.kstar_out[0] = A.kstar_in ? A.kstar_in[0] : (double)A.kappa_u;
+        }
+        return;
+    }
+    const int64_t t0 = (int64_t)blockIdx.x * A.tile;
+    const int64_t t1 = t0 + A.tile < A.N ? t0 + A.tile : A.N;  // not empty
+    // the warp's first particles, in flight over everything up to the field
+    uint32_t uu[4];
+    float kap[4], vin[4];
+    auto load = [&](int64_t base, uint32_t (&lu)[4], float (&lk)[4], float (&lv)[4]) {
+#pragma unroll
+        for (int h = 0; h < 4; ++h) {
             const int64_t j = base + h * 32 + lane;
-            int key = -1;
-            if (j < A.N) {
-                const float v = vin[hh] + A.kick_qm_dt * (ea[h] * nm[h] * A.coef);
-                A.v_out[j] = v;
-                const uint32_t nu = advance_position(uu[h], v * A.dt_scale);
-                A.u_out[j] = nu;
-                if (A.kappa_out) {
-                    const float k = kin[hh];
-                    A.kappa_out[j] = (k > 0.f && k <= (float)KDE_KAPPA_MAX) ? k : (float)KDE_KAPPA_MAX;
-                }
-                if (A.norm_out) A.norm_out[j] = nin[hh];
-                if (A.id_out) A.id_out[j] = idin[hh];
-                key = kde_cell(nu, Ng);
-            }
-            if (A.counts) {  // warp-uniform; the 32 particles of a round share one sort tile
-                const unsigned int peers = __match_any_sync(0xffffffffu, key);
-                if (key >= 0 && lane == __ffs(peers) - 1)
-                    atomicAdd(&A.counts[(size_t)key * A.cnt_nblk + (size_t)(j >> A.cnt_shift)],
-                              (unsigned int)__popc(peers));
-            }
+            const int64_t jj = j < A.N ? j : A.N - 1;
+            lu[h] = A.u[jj];
+            lk[h] = A.kappa ? A.kappa[jj] : A.kappa_u;
+            lv[h] = A.u_out ? ((const float *)A.v_in)[jj] : 0.f;
         }
-        }
+    };
+    load(t0 + warp * 128, uu, kap, vin);
+    float kmin, kmax;
+    if (!A.kappa) {
+        kmin = kmax = A.kappa_u;
+    } else if (A.krange) {
+        kmax = __uint_as_float(A.krange[0]);
+        kmin = __uint_as_float(A.krange[1]);
     } else {
+        kmin = (float)KDE_KAPPA_MAX;
+        kmax = 0.f;
+        for (int64_t j = t0 + tid; j < t1; j += GATT_THREADS) {
+            float k = A.kappa[j];
+            if (!(k > 0.f && k <= (float)KDE_KAPPA_MAX)) k = (float)KDE_KAPPA_MAX;
+            kmin = fminf(kmin, k);
+            kmax = fmaxf(kmax, k);
+        }
 #pragma unroll
-        for (int h = 0; h < GAT2_NP; ++h) {
-            const int64_t j = base + h * 32 + lane;
-            if (j < A.N) A.out[A.perm ? A.perm[j] : j] = ea[h] * nm[h] * A.coef;
+        for (int o = 16; o > 0; o >>= 1) {
+            kmin = fminf(kmin, __shfl_xor_sync(0xffffffffu, kmin, o));
+            kmax = fmaxf(kmax, __shfl_xor_sync(0xffffffffu, kmax, o));
+        }
+        if (lane == 0) {
+            kred[warp] = kmin;
+            kred[GATT_WARPS + warp] = kmax;
+        }
+        __syncthreads();
+#pragma unroll
+        for (int w = 0; w < GATT_WARPS; ++w) {
+            kmin = fminf(kmin, kred[w]);
+            kmax = fmaxf(kmax, kred[GATT_WARPS + w]);
+        }
+    }
+    const int c_first = kde_cell(A.u[t0], Ng), c_last = kde_cell(A.u[t1 - 1], Ng);
+    const int W = window_nodes_g(kmin, Ng, A.xcut);
+    int g_lo = c_first - W, R = c_last + W - g_lo + 1;
+    if (R >= Ng || R < 1 || c_last < c_first) {
+        g_lo = 0;
+        R = Ng;
+    }
+    PxyBox B;
+    pxy_box_pos(B, A.grid, c_first, max(c_first, c_last), kmax);
+    pxy_box_width(B, kmin, kmax);
+    // the form of the tile: one width, P <= 8 or 16; a narrow range of widths, P <= 6 or 8;
+    // else direct.  In instructions of a lane: compressed about 20 a particle and 0.8 a
+    // coefficient, 5 a (node, proxy) and the tile's fixed steps; direct 2.6 a (particle, node)
+    int form = 0;
+    if (c_last >= c_first && A.xcut == (float)KDE_XCUT) {
+        if (B.Q == 1) form = B.P <= 8 ? 1 : (B.P <= 16 ? 2 : 0);
+        else if (B.lin) form = B.P <= 6 ? 3 : (B.P <= 8 ? 4 : 0);
+        if (form) {
+            const float n = (float)(t1 - t0), PQ = form == 1 ? 8.f : (form == 2 ? 16.f : (form == 3 ? 28.f : 48.f));
+            const float comp = n * (20.f + 0.8f * PQ) + (float)R * PQ * 5.f + 60000.f;
+            if (comp >= n * 2.6f * (float)R) form = 0;
+        }
+    }
+    // what does not depend on the field, while the kernel before may still run
+    float4 *SC = (float4 *)sm;
+    float2 *FF = (float2 *)(SC + Ng);
+    bool cosf = false;
+    if (form) {
+        const int P = GATT_FORM_P(form), Q = GATT_FORM_Q(form);
+        const float *cp = A.pxt + pxy_tab_off(P), *cq = A.pxt + pxy_tab_off(Q);
+        for (int i = tid; i < P * P; i += GATT_THREADS) tabs[i] = cp[i];
+        if (tid < Q * Q) tabs[P * P + tid] = cq[tid];
+        if (tid < P) pxy_pos(B, cp[P + tid] * (0.5f * (float)P), cd[tid], fr[tid]);
+        if (tid >= 32 && tid < 32 + Q) {
+            const int b = tid - 32;
+            const float k = Q > 1 ? pxy_kappa(B, cq[Q + b] * (0.5f * (float)Q)) : kmin;
+            k2[b] = (float)(-2.0 * KDE_LOG2E) * k;
+            nk[b] = A.coef * (A.kappa ? kde_norm_tab(A.ntab, k) : A.norm_u);
+        }
+        __syncthreads();
+        int g = g_lo + (tid < R ? tid : 0);
+        g = g < 0 ? g + Ng : (g >= Ng ? g - Ng : g);
+        uint32_t nc;
+        float nf;
+        pxy_node(A.grid, g, nc, nf);
+        for (int a = 0; a < P; ++a) s2a[a * GATT_THREADS + tid] = pxy_sin2(nc, nf, cd[a], fr[a]);
+    } else {
+        cosf = kmax <= KDE_COSFORM_KMAX;
+        for (int g = tid; g < Ng; g += GATT_THREADS) {
+            const float2 sc = A.nodes[g];
+            if (cosf) {
+                const float sf = 2.f * sc.x * sc.y, cf = (sc.y - sc.x) * (sc.y + sc.x);
+                SC[g] = make_float4(sf, sf, cf, cf);
+            } else {
+                SC[g] = make_float4(sc.x, sc.x, -sc.y, -sc.y);
+            }
+        }
+    }
+    kde_pdl_wait();  // the field from here on
+    kde_pdl_trigger();
+    switch (form) {
+    case 1: gatt_coefs<8, 1>(A, g_lo, R, s2a, cd, fr, k2, nk, tabs, part, F, C); break;
+    case 2: gatt_coefs<16, 1>(A, g_lo, R, s2a, cd, fr, k2, nk, tabs, part, F, C); break;
+    case 3: gatt_coefs<7, 7>(A, g_lo, R, s2a, cd, fr, k2, nk, tabs, part, F, C); break;
+    case 4: gatt_coefs<8, 6>(A, g_lo, R, s2a, cd, fr, k2, nk, tabs, part, F, C); break;
+    default:
+        for (int g = tid; g < Ng; g += GATT_THREADS) {
+            const float f = A.field[g];
+            FF[g] = make_float2(f, f);
+        }
+        __syncthreads();
+    }
+#pragma unroll 1
+    for (int64_t base = t0 + warp * 128; base < t1; base += GATT_UNIT) {
+        uint32_t nu[4];
+        float nkap[4], nv[4];
+        load(base + GATT_UNIT < t1 ? base + GATT_UNIT : base, nu, nkap, nv);  // the next round's
+        float ea[4];
+        switch (form) {
+        case 1: gatt_eval<8, 1, false>(A, B, C, base, lane, uu, kap, ea); break;
+        case 2: gatt_eval<16, 1, false>(A, B, C, base, lane, uu, kap, ea); break;
+        case 3: gatt_eval<7, 7, true>(A, B, C, base, lane, uu, kap, ea); break;
+        case 4: gatt_eval<8, 6, false>(A, B, C, base, lane, uu, kap, ea); break;
+        default: gatt_direct(A, SC, FF, cosf, base, lane, uu, kap, ea);
+        }
+        gat_finish<true>(A, base, lane, uu, ea, vin);
+#pragma unroll
+        for (int h = 0; h < 4; ++h) {
+            uu[h] = nu[h];
+            kap[h] = nkap[h];
+            vin[h] = nv[h];
         }
     }
 }
@@ -457,6 +911,50 @@ static kde_status gat2_variant(kde_ctx *ctx, const GatherArgs<float> &A, int v)
     }
 }
 
+// the gather through proxies: at the default truncation, in the PIC step (and its truncation
+// tuner).  The rest -- plain gathers with particle-wise widths and cuts the caller has
+// set -- sweeps the nodes (gather2_kernel)
+// For one width the host knows the outcome: where the tiles would sweep the nodes anyway,
+// gather2_kernel does it.
+static int gatt_tile(kde_ctx *ctx, const GatherArgs<float> &A)
+{
+    // one wave of three CTAs an SM, whole rounds of 1024 particles, which spread the tile's
+    // fixed steps (a warp's 128 particles stay in one tile of the sort)
+    const int64_t slots = 3LL * (ctx->sm_count > 0 ? ctx->sm_count : 1);
+    const int64_t units = (A.N + GATT_UNIT - 1) / GATT_UNIT;
+    return (int)((units + slots - 1) / slots * GATT_UNIT);
+}
+static bool gatt_applies(kde_ctx *ctx, GatherArgs<float> &A)
+{
+    if (A.xcut != (float)KDE_XCUT || !(A.kappa ? A.krange != nullptr : A.u_out != nullptr)) return false;
+    A.tile = gatt_tile(ctx, A);
+    // particle-wise widths: a range is given for those of a width schedule (Silverman's rule
+    // around one width, a narrow range unless the density varies much); a few tiles are
+    // better swept by four times as many blocks
+    if (A.kappa) return A.N >= 64 * GATT_UNIT;
+    const double n = (double)(A.N < A.tile ? A.N : A.tile), share = n / (double)A.N;
+    const double a = KDE_PI * std::min(1.0, share + 2.0 / A.Ng), y = a * sqrt((double)A.kappa_u + 1.5);
+    const double R = std::min((double)A.Ng, 2.0 * kde_window_nodes(A.kappa_u, A.Ng) + share * A.Ng + 2.0);
+    return y < 1.6 && n * (y < 0.38 ? 26.0 : 33.0) + R * (y < 0.38 ? 40.0 : 80.0) + 60000.0 < n * 2.6 * R;
+}
+
+static kde_status gatt_launch(kde_ctx *ctx, GatherArgs<float> &A)
+{
+    static bool attr = false;
+    if (!attr) {
+        KDE_CUDA(ctx, cudaFuncSetAttribute(gather_tile_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                           KDE_MAX_NG * (int)(sizeof(float4) + sizeof(float2))),
+                 "gather_tile attribute");
+        attr = true;
+    }
+    const unsigned grid = (unsigned)((A.N + A.tile - 1) / A.tile) + (A.energy ? 1u : 0u);
+    const size_t smem = (size_t)A.Ng * (sizeof(float4) + sizeof(float2));
+    KDE_CUDA(ctx, kde_launch(ctx, A.u_out != nullptr, gather_tile_kernel, dim3(grid), dim3(GATT_THREADS), smem, A),
+             "gather_tile_kernel");
+    KDE_LAUNCHED(ctx, "gather_tile_kernel");
+    return KDE_OK;
+}
+
 static uint64_t gat2_key(const GatherArgs<float> &A)
 {
     return kde_width_key(A.N, A.Ng, A.kappa != nullptr, (double)A.kappa_u);
@@ -473,7 +971,15 @@ static kde_status launch_gather2(kde_ctx *ctx, GatherArgs<float> &A)
     A.nodes = (const float2 *)nodes;
     A.status = ctx->d_status;
     A.ntab = ctx->norm_tab;
+    A.grid = pxy_grid(A.Ng);
+    A.pxt = ctx->pxy_tab;
     const uint64_t key = gat2_key(A);
+    if (gatt_applies(ctx, A)) {
+        // one shape: nothing to tune, and the key counts as tuned with the default
+        if (ctx->autotune) ctx->gat2_tuned.insert({key, 0});
+        KdeProfScope _ps(ctx, PROF_GATHER);
+        return gatt_launch(ctx, A);
+    }
     auto it = ctx->gat2_tuned.find(key);
     int v = it != ctx->gat2_tuned.end() ? it->second : 0;
     bool tune = false;
@@ -548,7 +1054,7 @@ static kde_status launch_gather(kde_ctx *ctx, GatherArgs<T> &A)
 template <typename T>
 kde_status kde_gather_sorted(kde_ctx *ctx, const uint32_t *u, const T *kappa, T kappa_u, const T *norm, T norm_u,
                              int64_t N, const T *field, int Ng, double coef, T *out, const uint32_t *perm,
-                             const PushArgs *push, float xcut)
+                             const PushArgs *push, float xcut, const unsigned int *krange)
 {
     GatherArgs<T> A{};
     A.u = u;
@@ -563,6 +1069,7 @@ kde_status kde_gather_sorted(kde_ctx *ctx, const uint32_t *u, const T *kappa, T 
     A.out = out;
     A.perm = perm;
     A.xcut = xcut > 0.f ? xcut : (push && push->xcut > 0.f ? push->xcut : kde_fp32_cut(ctx));
+    A.krange = push ? push->krange : krange;
     if (push) {
         A.v_in = (const T *)push->v_in;
         A.u_out = push->u_out;
@@ -588,10 +1095,10 @@ kde_status kde_gather_sorted(kde_ctx *ctx, const uint32_t *u, const T *kappa, T 
 
 template kde_status kde_gather_sorted<float>(kde_ctx *, const uint32_t *, const float *, float, const float *, float,
                                              int64_t, const float *, int, double, float *, const uint32_t *,
-                                             const PushArgs *, float);
+                                             const PushArgs *, float, const unsigned int *);
 template kde_status kde_gather_sorted<double>(kde_ctx *, const uint32_t *, const double *, double, const double *,
                                               double, int64_t, const double *, int, double, double *,
-                                              const uint32_t *, const PushArgs *, float);
+                                              const uint32_t *, const PushArgs *, float, const unsigned int *);
 
 // ---------------------------------------------------------------------------
 template <typename T>
@@ -599,6 +1106,15 @@ static kde_status gather_api(kde_ctx *ctx, const uint32_t *u, const T *kappa, do
                              const T *field, int Ng, double L, T *out)
 {
     cudaSetDevice(ctx->device);
+    if constexpr (sizeof(T) == 4) {
+        // at the default truncation from tables of the smoothed field, without a sort; a cut
+        // the caller has set keeps the sweep over the nodes that it is defined for
+        if (kde_fp32_cut(ctx) == (float)KDE_XCUT) {
+            // no tile shapes to tune: the key counts as tuned with the default
+            if (ctx->autotune) ctx->gat2_tuned.insert({kde_width_key(N, Ng, kappa != nullptr, kappa_u), 0});
+            return kde_gather_table(ctx, u, kappa, kappa_u, N, field, Ng, out);
+        }
+    }
     uint32_t *us = (uint32_t *)kde_ws(ctx, WS_SORT_U, (size_t)N * 4);
     uint32_t *perm = (uint32_t *)kde_ws(ctx, WS_SORT_PERM, (size_t)N * 4);
     T *ks = kappa ? (T *)kde_ws(ctx, WS_SORT_P0, (size_t)N * sizeof(T)) : nullptr;

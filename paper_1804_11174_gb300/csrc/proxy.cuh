@@ -140,6 +140,29 @@ __device__ __forceinline__ float pxy_kappa(const PxyBox &B, float s)
     return B.lin ? k : expf(k);
 }
 
+// sine and cosine of half the angle between two positions: sin(pi f), cos(pi f), f in
+// [-1/2, 1/2] the difference in turns, by their Taylor series (the first terms left out are
+// below 7e-10 relative to the sine and 6e-9 of the cosine's unit)
+__device__ __forceinline__ void pxy_sincos(uint32_t na, float fa, uint32_t nb, float fb, float &s, float &c)
+{
+    const float f = ((float)(int32_t)(na - nb) + (fa - fb)) * (1.f / 4294967296.f), t = f * f;
+    s = (float)(0.00046630280576761256);  // pi^13 / 13!
+    s = fmaf(s, t, (float)(-0.0073704309457143504));
+    s = fmaf(s, t, (float)(0.082145886611128228));
+    s = fmaf(s, t, (float)(-0.59926452932079208));
+    s = fmaf(s, t, (float)(2.5501640398773454));
+    s = fmaf(s, t, (float)(-5.1677127800499701));
+    s = fmaf(s, t, (float)(3.1415926535897932));
+    s *= f;
+    c = (float)(0.0019295743094039231);  // pi^12 / 12!
+    c = fmaf(c, t, (float)(-0.025806891390014061));
+    c = fmaf(c, t, (float)(0.23533063035889321));
+    c = fmaf(c, t, (float)(-1.3352627688545895));
+    c = fmaf(c, t, (float)(4.0587121264167682));
+    c = fmaf(c, t, (float)(-4.9348022005446793));
+    c = fmaf(c, t, 1.f);
+}
+
 // sin^2 of half the angle between two positions given as codes and fractions.  The code
 // difference is exact, so near pairs keep full relative accuracy; sin(pi f) for
 // f in [-1/2, 1/2] by its Taylor series (the first term left out is below 7e-10 relative)

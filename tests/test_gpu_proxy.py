@@ -63,3 +63,55 @@ def test_deposit_compressed(ctx, oracle, N, Ng, kap, where, weights):
     finally:
         ctx.set_truncation(0.0)
     assert rel_l2(rho, direct) <= 2 * TOL
+
+
+@pytest.mark.parametrize("N,Ng,kap,where", CASES + [(20000, 4096, 2e5, "box"), (1, 64, 30.0, "box"),
+                                                    (1025, 300, "extreme", "spike")])
+def test_gather_from_tables(ctx, oracle, N, Ng, kap, where):
+    u = positions(N + Ng, N, where)
+    k = None
+    if kap == "extreme":  # every band, the widths below 1/2 and those beyond the bands
+        k = np.exp(np.linspace(math.log(1e-6), math.log(1e6), N)).astype(np.float32)
+        k[-1] = 1e6
+    elif isinstance(kap, str):
+        k = widths(kap, Ng, N)
+    g = 2 * math.pi * np.arange(Ng) / Ng
+    f = (np.sin(g) + 0.3 * np.cos(3 * g) + 0.2 * (I.uniforms(5, 3, Ng) - 0.5)).astype(np.float32)
+    kw = dict(kappa=to_dev(k)) if k is not None else dict(kappa_uniform=kap)
+    ud, fd = to_dev_u(u), to_dev(f)
+    out = ctx.gather(ud, fd, L, **kw).cpu().numpy()
+    okw = dict(kappa=k.astype(np.float64)) if k is not None else dict(kappa_u=kap)
+    assert rel_l2(out, oracle.gather(I.from_fixed(u, L), f.astype(np.float64), L, **okw)) <= TOL
+    try:
+        ctx.set_truncation(25.0)
+        direct = ctx.gather(ud, fd, L, **kw).cpu().numpy()
+    finally:
+        ctx.set_truncation(0.0)
+    # the direct sweep's half-angle form has its own error, about sqrt(8 kappa x) 6e-8 e^-x per value
+    kmax = float(k.max()) if k is not None else kap
+    assert rel_l2(out, direct) <= 2 * TOL + 6e-8 * math.sqrt(kmax)
+
+
+@pytest.mark.parametrize("N,Ng,kap", [(20000, 256, "one"), (70001, 256, "narrow"), (130, 256, "narrow"),
+                                      (70001, 1000, "ten"), (20000, 300, "wide"), (70001, 33, 2.0), (70001, 512, 300.0),
+                                      (40000, 1024, 40.0), (33, 64, 5.0), (3000, 4096, 3.0), (300, 2, 4.0)])
+def test_pic_step_through_proxies(ctx, kp, oracle, N, Ng, kap):
+    # deposit and gather + push of two steps, every form of their tiles
+    dt = 0.1
+    u, v = I.landau_load(N + Ng, N, L, 0.05, 1.0)
+    v32 = v.astype(np.float32)
+    k = widths(kap, Ng, N) if isinstance(kap, str) else None
+    import torch
+    st = kp.PicState(to_dev_u(u), to_dev(v32), L, Ng, dt, kappa=None if k is None else to_dev(k),
+                     kappa_uniform=0.0 if k is not None else kap, max_steps=2,
+                     ids=torch.arange(N, dtype=torch.int32, device="cuda:0"))
+    ctx.pic_step(st, 2)
+    ctx.sync()
+    r = oracle.pic_run(I.from_fixed(u, L), v32, L, Ng, dt, 2, kappa=None if k is None else k.astype(np.float64),
+                       kappa_u=0.0 if k is not None else kap)
+    e = st.energy.cpu().numpy()[:2]
+    np.testing.assert_allclose(e, r["energy"], rtol=1e-5, atol=1e-12 * max(1.0, float(np.max(r["energy"]))))
+    at = np.argsort(st.id.cpu().numpy())
+    x = I.from_fixed(st.u.cpu().numpy().view(np.uint32), L)[at]
+    assert np.max(np.abs((x - r["x"] + L / 2) % L - L / 2)) <= 1e-6 * L
+    assert rel_l2(st.v.cpu().numpy()[at], r["v"]) <= 1e-5
