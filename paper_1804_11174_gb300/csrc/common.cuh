@@ -125,6 +125,7 @@ struct kde_ctx {
     // Anderson-Darling per-bin logarithms (one table per context)
     void *ad_tab = nullptr;
     float2 *norm_tab = nullptr;  // FP32 width-normalisation table (kde_norm_tab), built at creation
+    double *f64_tab = nullptr;   // 2^(j / 2048) for the FP64 kernels (fp64.cuh), built at creation
     float *pxy_tab = nullptr;    // interpolation matrices (proxy.cuh), built at creation
     unsigned wait_polls = 1u << 26;         // polls of a bounded device wait (kde_set_wait_limit)
     bool count_flip = false;                // which sort count table the next counted sort reads (sort.cu)
@@ -463,8 +464,8 @@ kde_status kde_bspline_gather_push(kde_ctx *ctx, uint32_t *u, float *v, int64_t 
 // tmp: N-element scratch; u may alias neither out nor tmp
 kde_status kde_radix_sort_u32(kde_ctx *ctx, const uint32_t *u, int64_t N, uint32_t *out, uint32_t *tmp);
 
-// deposit of cell-sorted particles into int64 accumulators acc[Ng] (zeroed
-// here).  Particle j contributes w_j * coef * norm_j * exp(-2 kappa_j sin^2(..)).
+// deposit of cell-sorted particles into int64 accumulators (zeroed here): acc[Ng], and in FP64
+// a second acc[Ng .. 2 Ng) of remainders in units of 2^-24 of the first's.  Particle j contributes w_j * coef * norm_j * exp(-2 kappa_j sin^2(..)).
 // Arrays may be null (then the uniform scalar is used; norm null with a kappa
 // array means "compute the norm from the width").  `bound` is the largest
 // possible node value; with wmax_bits it is N * coef * norm_bound * w_max.
@@ -497,7 +498,8 @@ kde_status kde_field_from_rows(kde_ctx *ctx, const long long *rows, const int2 *
                                double acc_inv, double charge, bool fd, float *E_out);
 
 // Poisson solve of rho_total = background + charge * rho, rho given as a real
-// array or as int64 accumulators (value = acc * acc_inv)
+// array or as int64 accumulators (value = acc * acc_inv; in FP64 with the remainders of the
+// FP64 deposit behind them)
 template <typename T>
 kde_status kde_poisson_impl(kde_ctx *ctx, const T *rho, const long long *acc, double acc_inv, int Ng, double L,
                             double charge, double background, bool fd, T *E_out);

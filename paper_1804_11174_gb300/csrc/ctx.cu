@@ -4,6 +4,7 @@
 #include <cstring>
 
 #include "common.cuh"
+#include "fp64.cuh"
 #include "proxy.cuh"
 
 kde_status kde_fail(kde_ctx *ctx, kde_status code, const char *fmt, ...)
@@ -193,6 +194,12 @@ __global__ void pxy_tab_kernel(float *tab)
     }
 }
 
+__global__ void f64_tab_kernel(double *tab)
+{
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i < F64_TAB) tab[i] = exp2((double)i / F64_TAB);
+}
+
 // ---------------------------------------------------------------------------
 // C ABI: context
 // ---------------------------------------------------------------------------
@@ -217,9 +224,15 @@ extern "C" kde_status kde_create(kde_ctx **out, int device, void *stream)
         pxy_tab_kernel<<<PXY_MAXQ, 128, 0, ctx->stream>>>(ctx->pxy_tab);
         e = cudaGetLastError();
     }
+    if (e == cudaSuccess) e = cudaMalloc(&ctx->f64_tab, F64_TAB * sizeof(double));
+    if (e == cudaSuccess) {
+        f64_tab_kernel<<<F64_TAB / 256, 256, 0, ctx->stream>>>(ctx->f64_tab);
+        e = cudaGetLastError();
+    }
     if (e == cudaSuccess) e = cudaStreamSynchronize(ctx->stream);
     if (e != cudaSuccess) {
         cudaGetLastError();
+        if (ctx->f64_tab) cudaFree(ctx->f64_tab);
         if (ctx->d_status) cudaFree(ctx->d_status);
         if (ctx->norm_tab) cudaFree(ctx->norm_tab);
         if (ctx->pxy_tab) cudaFree(ctx->pxy_tab);
@@ -242,6 +255,7 @@ extern "C" kde_status kde_destroy(kde_ctx *ctx)
     if (ctx->ad_tab) cudaFree(ctx->ad_tab);
     if (ctx->norm_tab) cudaFree(ctx->norm_tab);
     if (ctx->pxy_tab) cudaFree(ctx->pxy_tab);
+    if (ctx->f64_tab) cudaFree(ctx->f64_tab);
     if (ctx->d_status) cudaFree(ctx->d_status);
     for (auto &p : ctx->prof) {
         cudaEventDestroy(p.second.first);

@@ -22,6 +22,7 @@
 // Integral term: exact trapezoid sum of fhat^2 on a power-of-two grid fine
 // enough for each candidate (deposit.cu).  Combination and argmin in FP64.
 #include "common.cuh"
+#include "fp64.cuh"
 
 #define CV_T 256
 #define CV_WARPS (CV_T / 32)
@@ -1074,7 +1075,7 @@ __global__ void adapt_apply_kernel(const float *loo, int64_t N, const AdaptPar *
     if (norm_out) {
         // FP32 widths take the tabulated norm, FP64 widths the FP64 Bessel series
         if constexpr (sizeof(T) == 4) norm_out[i] = (T)kde_norm_tab(ntab, (float)k);
-        else norm_out[i] = (T)kde_norm((double)k);
+        else norm_out[i] = (T)f64_norm((double)k);
     }
 }
 

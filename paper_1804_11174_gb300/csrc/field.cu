@@ -22,9 +22,14 @@ __global__ void __launch_bounds__(POI_THREADS)
     T *rt = (T *)sm;
     T *Gs = rt + Ng;
     __shared__ double red[POI_THREADS];
+    auto value = [&](int l) -> double {
+        if (!acc) return (double)rho[l];
+        if (sizeof(T) == 8) return ((double)acc[l] + (double)acc[Ng + l] * (1.0 / 16777216.0)) * acc_inv;
+        return (double)acc[l] * acc_inv;
+    };
     double local = 0.0;
     for (int l = threadIdx.x; l < Ng; l += POI_THREADS) {
-        double r = acc ? (double)acc[l] * acc_inv : (double)rho[l];
+        double r = value(l);
         local += background + charge * r;
     }
     red[threadIdx.x] = local;
@@ -35,7 +40,7 @@ __global__ void __launch_bounds__(POI_THREADS)
     }
     const double mean = red[0] / Ng;
     for (int l = threadIdx.x; l < Ng; l += POI_THREADS) {
-        double r = acc ? (double)acc[l] * acc_inv : (double)rho[l];
+        double r = value(l);
         rt[l] = (T)(background + charge * r - mean);
         Gs[l] = G[l];
     }

@@ -11,6 +11,7 @@
 //   Poisson solve straight from the accumulators (mean removed in FP64)
 //   gather + leap-frog push + write-back + field energy (one kernel)
 #include "common.cuh"
+#include "fp64.cuh"
 
 template <typename T>
 __global__ void norm_from_kappa_kernel(const T *kappa, int64_t N, T *norm, unsigned int *status, const float2 *ntab,
@@ -30,7 +31,7 @@ __global__ void norm_from_kappa_kernel(const T *kappa, int64_t N, T *norm, unsig
     if (krange) kde_krange_add(krange, (float)k, (float)k);
     // FP32 state: the tabulated norm; FP64 state: the FP64 Bessel series
     if constexpr (sizeof(T) == 4) norm[i] = (T)kde_norm_tab(ntab, (float)k);
-    else norm[i] = (T)kde_norm(k);
+    else norm[i] = (T)f64_norm(k);
 }
 
 // ---------------------------------------------------------------------------
@@ -169,7 +170,7 @@ static kde_status pic_run_bspline(kde_ctx *ctx, pic_state *st, int n_steps)
     const double L = st->L;
     const double h = st->shape_h > 0 ? st->shape_h : L / Ng;
     const bool fd = (st->flags & KDE_POISSON_FD) != 0;
-    long long *acc = (long long *)kde_ws(ctx, WS_ACC, (size_t)Ng * 8);
+    long long *acc = (long long *)kde_ws(ctx, WS_ACC, (size_t)Ng * 16);
     float *E = (float *)kde_ws(ctx, WS_GRID0, (size_t)Ng * sizeof(float));
     if (!acc || !E) return KDE_ENOMEM;
     for (int s = 0; s < n_steps; ++s) {
@@ -224,7 +225,7 @@ static kde_status pic_run(kde_ctx *ctx, pic_state *st, int n_steps)
         return ok;
     };
     if (!fetch_ws()) return KDE_ENOMEM;
-    long long *acc = (long long *)kde_ws(ctx, WS_ACC, (size_t)Ng * 8);
+    long long *acc = (long long *)kde_ws(ctx, WS_ACC, (size_t)Ng * 16);
     T *E = (T *)kde_ws(ctx, WS_GRID0, (size_t)Ng * sizeof(T));
     float *loo = sched ? (float *)kde_ws(ctx, WS_PIC_LOO, (size_t)N * 4) : nullptr;
     double *ks_dev = sched ? (double *)kde_ws(ctx, WS_PIC_KS, 64) : nullptr;

@@ -115,3 +115,29 @@ def test_pic_step_through_proxies(ctx, kp, oracle, N, Ng, kap):
     x = I.from_fixed(st.u.cpu().numpy().view(np.uint32), L)[at]
     assert np.max(np.abs((x - r["x"] + L / 2) % L - L / 2)) <= 1e-6 * L
     assert rel_l2(st.v.cpu().numpy()[at], r["v"]) <= 1e-5
+
+
+@pytest.mark.parametrize("N,Ng,kap", [(1, 64, 30.0), (15, 33, 5.0), (17, 100, 200.0), (33, 1, 2.0), (700, 2, 40.0),
+                                      (5000, 300, "ten"), (3000, 1030, "wide"), (1300, 4096, 3.0), (90000, 64, 100.0),
+                                      (2000, 129, "extreme")])
+def test_fp64_deposit_and_gather(ctx, oracle, N, Ng, kap):
+    # tolerance: a few FP64 roundings a value (the exponential within 2e-16, exponents up to
+    # 2 kappa sin^2 log2 e with kappa to 1e6 known to 1e-16 of 1e6: 1e-10 there, else 1e-12)
+    import torch
+    u = positions(N + Ng, N, "box")
+    k = None
+    if kap == "extreme":
+        k = np.exp(np.linspace(math.log(1e-6), math.log(1e6), N))
+        k[-1] = 1e6
+    elif isinstance(kap, str):
+        k = widths(kap, Ng, N).astype(np.float64)
+    tol = 1e-10 if kap == "extreme" else 1e-12
+    x, ud = I.from_fixed(u, L), to_dev_u(u)
+    w = 0.5 + I.uniforms(7, 9, N)
+    kw = dict(kappa=to_dev(k, torch.float64)) if k is not None else dict(kappa_uniform=kap)
+    okw = dict(kappa=k) if k is not None else dict(kappa_u=kap)
+    rho = ctx.deposit(ud, Ng, L, weight=to_dev(w, torch.float64), dtype=torch.float64, **kw).cpu().numpy()
+    assert rel_l2(rho, oracle.deposit(x, Ng, L, w=w, **okw)) <= tol
+    f = np.cos(2 * math.pi * np.arange(Ng) / Ng) + 0.3 * I.uniforms(5, 3, Ng)
+    out = ctx.gather(ud, to_dev(f, torch.float64), L, **kw).cpu().numpy()
+    assert rel_l2(out, oracle.gather(x, f, L, **okw)) <= tol
