@@ -250,6 +250,9 @@ kde_status kde_gather(kde_ctx *ctx, const uint32_t *u, const void *kappa, double
  * accumulation; the integral term is an exact trapezoid sum on a grid fine
  * enough for the narrowest candidate; the final combination is FP64.  Pairs
  * whose kernel value is below 2^-24 of the peak may be skipped.  Synchronises.
+ * KDE_CV_SCALE calls on large samples evaluate the same objective from Fourier sums
+ * of the particle-wise kernels (error below the pair sums'), by a cost rule that
+ * KDE_CV_PAIRS switches off; they wait once for the range of the widths.
  * KDE_CV_SPECTRAL (uniform widths only) evaluates the same objective by the
  * identity K(t) = (1/2pi) sum_m A_m e^{imt}, A_m = I_m/I_0: with the structure
  * factor S_m = sum_j e^{i m theta_j} (exact integer phases, FP64 combination),

@@ -96,6 +96,7 @@ enum WsSlot {
     WS_HOST_NORM,
     WS_HOST_ID,
     WS_HOST_HIST,  // energy, kappa* and ln p histories
+    WS_LTAB,       // table of the density series (leave-one-out densities)
     WS_GTAB,       // tables of the smoothed field (plain FP32 gather)
     WS_TUNE,       // truncation tuner: reference and candidate fields and their error sums
     WS_NSLOTS
@@ -129,6 +130,7 @@ struct kde_ctx {
     float *pxy_tab = nullptr;    // interpolation matrices (proxy.cuh), built at creation
     unsigned wait_polls = 1u << 26;         // polls of a bounded device wait (kde_set_wait_limit)
     bool count_flip = false;                // which sort count table the next counted sort reads (sort.cu)
+    int64_t cv_fourier_bytes = 1ll << 30;   // workspace the Fourier form of a scale-mode CV may take
     bool autotune = false;                  // kde_set_autotune
     bool overlap = true;                    // kde_set_launch_overlap: PDL launches in the step chain
     std::map<uint64_t, int> gat2_tuned;     // packed-gather tile shape per key (gather.cu)
@@ -136,6 +138,8 @@ struct kde_ctx {
     std::map<uint64_t, float> cut_tuned;    // FP32 PIC truncation cut exponent per key (pic.cu)
     void *sp_atab = nullptr;                // workspace holding the Bessel ratios of sp_atab_cands (spectral.cu)
     std::vector<double> sp_atab_cands;
+    cudaStream_t aux = nullptr;             // second stream of the scale-mode CV (kde_aux_stream)
+    cudaEvent_t aux_ev[2] = {};
 };
 
 // ---------------------------------------------------------------------------
@@ -146,6 +150,9 @@ kde_status kde_cuda_check(kde_ctx *ctx, cudaError_t e, const char *what);
 void *kde_ws(kde_ctx *ctx, WsSlot slot, size_t bytes);  // grows the slot; nullptr + error on failure
 const void *kde_node_table(kde_ctx *ctx, int Ng, bool f64);
 const void *kde_green_table(kde_ctx *ctx, int Ng, double L, bool fd, bool f64);
+// the context's second stream, with events to fork it from the context's stream ([0]) and to
+// join it ([1]); made on first use
+kde_status kde_aux_stream(kde_ctx *ctx);
 double kde_host_i0e(double x);  // scaled Bessel I0e in FP64 on the host (uniform widths)
 
 #define KDE_TRY(expr)                       \
@@ -393,6 +400,15 @@ __host__ __device__ inline double kde_i0e(double x)
     return sum / sqrt(KDE_TWO_PI * x);
 }
 
+// Fourier modes the exact form of the CV keeps for a width: A_m = I_m / I_0 ~
+// exp(-m^2 / (2 kappa)) < 1e-17 beyond sqrt(78.4 kappa)
+#define KDE_SPEC_MAXM 16384
+__host__ __device__ inline int kde_spec_modes(double kappa)
+{
+    const int M = (int)ceil(sqrt(78.4 * kappa)) + 8;
+    return M > KDE_SPEC_MAXM ? KDE_SPEC_MAXM : M;
+}
+
 // von Mises normalisation 1 / (2 pi I0e(kappa))
 __host__ __device__ inline double kde_norm(double kappa) { return 1.0 / (KDE_TWO_PI * kde_i0e(kappa)); }
 
@@ -562,7 +578,17 @@ kde_status kde_ad_device(kde_ctx *ctx, const uint32_t *u, int64_t N, double *out
 // exact Fourier form: the same values as the pair-sum pass, O(N M(kappa*)) work
 kde_status kde_loo_spectral_device(kde_ctx *ctx, const uint32_t *u, int64_t N, double L, const double *cand_host,
                                    int n_cand, const int *argmin_dev, float *loo);
-int kde_spec_modes(double kappa);  // Fourier modes the exact form keeps for a width
+// S_m = sum_j e^{i m theta_j}, m = 1 .. M, in the structure-factor workspace
+kde_status kde_spec_structure(kde_ctx *ctx, const uint32_t *u, int64_t N, int M, double2 **S_out);
+// the CV of particle-wise widths cand[c] kr[j] by its Fourier form (scalecv.cu), where its cost
+// rule prefers that to the pair sums: *taken says whether it did.  Waits for the stream once.
+kde_status kde_cv_scale_fourier(kde_ctx *ctx, const uint32_t *u, const float *kr, int64_t N, double L,
+                                const double *cand_host, int n_cand, double *cv_dev, int *argmin_dev, float *loo,
+                                bool *taken);
+// leave-one-out densities of that form: F[c Mst + m - 1] = sum_j A_m(cand_c kr_j) e^{i m theta_j},
+// at the candidate *argmin_dev; kappa_max: the largest width of any candidate
+kde_status kde_loo_series(kde_ctx *ctx, const uint32_t *u, const float *kr, int64_t N, double L, const double2 *F,
+                          int Mst, const CandList &cl, const int *argmin_dev, double kappa_max, float *loo);
 // the cost rule between the exact forms of a uniform-width CV curve (true: Fourier form)
 bool kde_cv_prefer_spectral(int64_t N, const double *cand, int n_cand);
 

@@ -61,6 +61,15 @@ void *kde_ws(kde_ctx *ctx, WsSlot slot, size_t bytes)
 
 double kde_host_i0e(double x) { return kde_i0e(x); }
 
+kde_status kde_aux_stream(kde_ctx *ctx)
+{
+    if (ctx->aux) return KDE_OK;
+    for (auto &e : ctx->aux_ev)
+        if (!e) KDE_CUDA(ctx, cudaEventCreateWithFlags(&e, cudaEventDisableTiming), "second stream's event");
+    KDE_CUDA(ctx, cudaStreamCreateWithFlags(&ctx->aux, cudaStreamNonBlocking), "second stream");
+    return KDE_OK;
+}
+
 // ---------------------------------------------------------------------------
 // cached tables
 // ---------------------------------------------------------------------------
@@ -248,6 +257,12 @@ extern "C" kde_status kde_destroy(kde_ctx *ctx)
     if (!ctx) return KDE_EINVAL;
     cudaSetDevice(ctx->device);
     cudaStreamSynchronize(ctx->stream);
+    if (ctx->aux) {
+        cudaStreamSynchronize(ctx->aux);
+        cudaStreamDestroy(ctx->aux);
+    }
+    for (auto &e : ctx->aux_ev)
+        if (e) cudaEventDestroy(e);
     for (int i = 0; i < WS_NSLOTS; ++i)
         if (ctx->ws[i]) cudaFree(ctx->ws[i]);
     for (auto &kv : ctx->node_tab) cudaFree(kv.second);

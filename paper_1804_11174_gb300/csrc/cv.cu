@@ -991,7 +991,10 @@ extern "C" kde_status kde_cv(kde_ctx *ctx, const uint32_t *u, const float *kappa
     double *cvd = (double *)kde_ws(ctx, WS_CV_OUT, (size_t)n_cand * 8 + 64);
     if (!cvd) return KDE_ENOMEM;
     int *amin = (int *)(cvd + n_cand);
-    if (spectral) KDE_TRY(kde_cv_spectral_device(ctx, u, N, L, cand, n_cand, cvd, amin, loo_out, nullptr));
+    bool taken = false;
+    if (scale && !pairs) KDE_TRY(kde_cv_scale_fourier(ctx, u, kappa_rel, N, L, cand, n_cand, cvd, amin, loo_out, &taken));
+    if (taken) {
+    } else if (spectral) KDE_TRY(kde_cv_spectral_device(ctx, u, N, L, cand, n_cand, cvd, amin, loo_out, nullptr));
     else
         KDE_TRY(kde_cv_device(ctx, u, scale ? kappa_rel : nullptr, N, L, cand, n_cand, scale, cvd, amin, loo_out,
                               nullptr));

@@ -45,6 +45,7 @@ struct Ticket {
     bool cancelled = false;
     int64_t io = 0;  // transient device buffers
     int64_t ws = 0;  // workspace the request needs in its slot's context
+    int64_t cv_extra = 0;  // part of it that the Fourier form of a scale-mode CV may use
     double dev_start = -1.0, dev_end = -1.0;  // device clock, ms since the server's epoch event
     std::string err;
 };
@@ -123,9 +124,10 @@ static void ctx_trim(kde_ctx *c)
     c->sp_atab_cands.clear();
 }
 
-static kde_status run_request(kde_server *S, kde_ctx *ctx, cudaStream_t st, const kde_request &r, cudaEvent_t ev0,
-                              cudaEvent_t ev1)
+static kde_status run_request(kde_server *S, kde_ctx *ctx, cudaStream_t st, const kde_request &r, int64_t cv_extra,
+                              cudaEvent_t ev0, cudaEvent_t ev1)
 {
+    ctx->cv_fourier_bytes = cv_extra;
     const int64_t N = r.N;
     cudaEventRecord(ev0, st);
     void *bufs[6] = {nullptr, nullptr, nullptr, nullptr, nullptr, nullptr};
@@ -265,7 +267,7 @@ static void worker_main(kde_server *S, int slot)
     cudaEventCreate(&ev0);
     cudaEventCreate(&ev1);
     for (;;) {
-        int64_t id;
+        int64_t id, cv_extra;
         kde_request req;
         {
             std::unique_lock<std::mutex> lk(S->mu);
@@ -284,8 +286,9 @@ static void worker_main(kde_server *S, int slot)
             S->busy[slot] = 1;
             t.t_start = clk::now();
             req = t.req;
+            cv_extra = t.cv_extra;
         }
-        kde_status rc = run_request(S, ctx, st, req, ev0, ev1);
+        kde_status rc = run_request(S, ctx, st, req, cv_extra, ev0, ev1);
         float a = -1.f, b = -1.f;
         if (cudaEventElapsedTime(&a, S->epoch, ev0) != cudaSuccess || cudaEventElapsedTime(&b, S->epoch, ev1) != cudaSuccess) {
             cudaGetLastError();
@@ -361,7 +364,13 @@ extern "C" kde_status kde_server_submit(kde_server *S, const kde_request *req, i
     default: ok = false;
     }
     if (!ok) return KDE_EINVAL;
-    const int64_t io = request_io_bytes(r), ws = request_ws_bytes(r);
+    const int64_t io = request_io_bytes(r);
+    int64_t ws = request_ws_bytes(r);
+    // a CV with particle-wise widths may take its Fourier form in up to a 64th of the budget,
+    // unless that would keep the request out
+    int64_t extra = r.kind == KDE_REQ_CV && r.kappa ? std::min<int64_t>(S->budget / 64, 512ll << 20) : 0;
+    if (io + ws + extra + (1 << 20) > S->budget) extra = 0;
+    ws += extra;
     if (io + ws + (1 << 20) > S->budget) return KDE_EINVAL;  // could never be admitted (1 MiB for tables)
     {
         std::lock_guard<std::mutex> lk(S->mu);
@@ -370,6 +379,7 @@ extern "C" kde_status kde_server_submit(kde_server *S, const kde_request *req, i
         t.req = r;
         t.io = io;
         t.ws = ws;
+        t.cv_extra = extra;
         t.t_submit = clk::now();
         S->queue.push_back(id);
         *ticket = id;

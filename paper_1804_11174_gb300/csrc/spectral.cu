@@ -18,20 +18,14 @@
 // combined in FP64 in a fixed order; the CV combination and the leave-one-out
 // sums are FP64.  Particles may come in any order (no sort).
 #include "common.cuh"
+#include "fp64.cuh"
+#include "proxy.cuh"
 
 #define SP_THREADS 256
 #define SP_SUB 256
-#define SP_MAXM 16384
 #define SP_MAXCHUNK 16384
 #define SP_Q 8         // consecutive modes a thread in the structure factor
 #define SP_SF_THREADS 128  // threads of a structure-factor block (SP_Q SP_SF_THREADS modes)
-
-// modes needed for a width: A_m ~ exp(-m^2 / (2 kappa)) < 1e-17 beyond sqrt(78.4 kappa)
-__host__ __device__ inline int spec_modes(double kappa)
-{
-    int M = (int)ceil(sqrt(78.4 * kappa)) + 8;
-    return M > SP_MAXM ? SP_MAXM : M;
-}
 
 // A_m(kappa), m = 0..M, into A[0..M]; r scratch of M + tail + 1 doubles.
 // Backward recurrence r_m = 1 / (2m/kappa + r_{m+1}) for r_m = I_m / I_{m-1},
@@ -172,7 +166,7 @@ __global__ void __launch_bounds__(SP_THREADS)
     const int c = blockIdx.x;
     const double n = (double)N;
     const double kappa = cl.k[c];
-    const int M = spec_modes(kappa);
+    const int M = kde_spec_modes(kappa);
     double *A = Atab + (size_t)c * Astride;
     if (threadIdx.x == 0 && !ratios_ready) spec_ratios(kappa, M, A);
     __syncthreads();
@@ -204,38 +198,74 @@ __global__ void __launch_bounds__(SP_THREADS)
     }
 }
 
-// argmin (smallest index on ties) and the selected width
-__global__ void spec_argmin_kernel(const double *cv, CandList cl, int *argmin, double *kstar)
+// the density table of the leave-one-out densities (below)
+#define LT_P 7
+#define LT_IV 4        // intervals of a block, LT_P lanes each
+#define LT_GROUPS 8    // warps that share the modes of its points
+#define LT_CH 512      // modes staged at a time
+
+__host__ __device__ inline int lt_intervals(double kappa)
 {
-    int best = 0;
-    for (int q = 1; q < cl.n; ++q)
-        if (cv[q] < cv[best]) best = q;
-    *argmin = best;
-    if (kstar) *kstar = cl.k[best];
+    const int C = (int)ceil(KDE_PI / 0.2646 * sqrt(kappa + 1.5));
+    return C < 4 ? 4 : C;
 }
 
 // the selected width kappa* = cand[*argmin]: its mode count, Bessel ratios A[0..M]
 // and normalisation 1 / (2 pi I0e(kappa*)), for the leave-one-out pass
 struct SpecSel {
     int M;
+    int C;         // intervals of the density table (lt_intervals)
+    double kappa;  // the width (for particle-wise widths the factor on them)
     double norm;
     const double *A;  // the ratios A[0..M]: a row of the candidates' table, or the kernel's own output
 };
-// Atab: the candidates' ratio table (row stride Astride) when the caller has it, else
-// nullptr and the ratios are worked out into A
-__global__ void spec_select_kernel(CandList cl, const int *argmin, SpecSel *sel, double *A, const double *Atab,
-                                   int Astride)
+// argmin (smallest index on ties) over the first n of cv, by a warp; every lane has it
+__device__ __forceinline__ int spec_argmin(const double *cv, int n, int lane)
 {
-    const double kappa = cl.k[*argmin];
-    const int M = spec_modes(kappa);
+    double v = 1.0e300;
+    int at = 0x7fffffff;
+    for (int q = lane; q < n; q += 32) {
+        const double x = cv[q];
+        if (at == 0x7fffffff || x < v) {
+            v = x;
+            at = q;
+        }
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        const double w = __shfl_xor_sync(0xffffffffu, v, o);
+        const int k = __shfl_xor_sync(0xffffffffu, at, o);
+        if (k != 0x7fffffff && (at == 0x7fffffff || w < v || (w == v && k < at))) {
+            v = w;
+            at = k;
+        }
+    }
+    return at;
+}
+
+// the selected candidate: its index and width, and (sel given) what the leave-one-out pass
+// needs of it.  cv: the curve, or nullptr when *argmin is known.  Atab: the candidates' ratio
+// table (row stride Astride) when the caller has it, else the ratios are worked out into A
+__global__ void __launch_bounds__(32) spec_select_kernel(const double *cv, CandList cl, int *argmin, double *kstar,
+                                                         SpecSel *sel, double *A, const double *Atab, int Astride)
+{
+    const int best = cv ? spec_argmin(cv, cl.n, threadIdx.x) : *argmin;
+    if (threadIdx.x != 0) return;
+    if (cv) *argmin = best;
+    const double kappa = cl.k[best];
+    if (kstar) *kstar = kappa;
+    if (!sel) return;
+    const int M = kde_spec_modes(kappa);
     if (Atab) {
-        sel->A = Atab + (size_t)*argmin * Astride;
+        sel->A = Atab + (size_t)best * Astride;
     } else {
         spec_ratios(kappa, M, A);
         sel->A = A;
     }
     sel->M = M;
-    sel->norm = kde_norm(kappa);
+    sel->C = lt_intervals(kappa);
+    sel->kappa = kappa;
+    sel->norm = f64_norm(kappa);
 }
 
 // A_m S_m in FP32 for the leave-one-out sums
@@ -248,72 +278,192 @@ __global__ void spec_as_kernel(const double2 *S, const SpecSel *sel, float2 *AS)
     AS[m - 1] = make_float2((float)(A[m] * s.x), (float)(A[m] * s.y));
 }
 
-// leave-one-out density at the selected width for every particle (input order):
-// sum_j K(theta_i - theta_j) = (1/2pi)(n + 2 sum_m Re(e^{i m theta_i} conj(A_m S_m))),
-// minus the particle's own K(0).  Exact integer phases, FP32 terms with compensated
-// (Kahan) summation over the modes; the combination in FP64 once per particle.
-#define SP_LOO_CH 1024
-__global__ void __launch_bounds__(SP_THREADS)
-    spec_loo_kernel(const uint32_t *__restrict__ u, int64_t N, const float2 *__restrict__ AS,
-                    const SpecSel *__restrict__ sel, double xs, float *loo)
+// ---------------------------------------------------------------------------
+// Leave-one-out densities from a density series sum_j K(theta - theta_j) = (1/2pi)(n + 2 f(theta)),
+// f(theta) = sum_{m=1}^{M} Re(e^{i m theta} conj(c_m)).  f is smooth on the scale of the narrowest
+// kernel, so it is tabulated: C equal intervals, chosen on the device from the largest width in
+// force, with seven Chebyshev points each (proxy.cuh, y <= 0.2646), and every particle reads its
+// interval's seven coefficients, the first in FP64 (the density is nearly constant over an
+// interval, so the others need FP32 only).  M sines a point instead of M a particle: 2^18
+// particles at kappa* = 450 83 -> 12 us.
+// ---------------------------------------------------------------------------
+// row of an interval's coefficients of f / n
+struct __align__(32) LtRow {
+    double c0;
+    float c[6];
+};
+
+// lanes are points, warps take blocks of eight modes in turn: exact integer phases (a sincospi a
+// mode: rotations would triple the error of the densities), compensated sums
+__global__ void __launch_bounds__(32 * LT_GROUPS)
+    spec_table_kernel(const float2 *__restrict__ AS, const SpecSel *__restrict__ sel, const float *__restrict__ cp,
+                      double inv_n, LtRow *tab)
 {
-    __shared__ float2 sAS[SP_LOO_CH];
-    const int M = sel->M;
-    const int64_t i = (int64_t)blockIdx.x * SP_THREADS + threadIdx.x;
-    const uint32_t ui = i < N ? u[i] : 0u;
+    __shared__ float2 sAS[LT_CH];
+    __shared__ double val[LT_GROUPS][32];
+    const int M = sel->M, C = sel->C;
+    if (blockIdx.x * LT_IV >= C) return;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int iv = lane / LT_P, a = lane - iv * LT_P, i = blockIdx.x * LT_IV + iv;
+    // the point: interval middle and Chebyshev point, to a code (2^-33 of the circle)
+    const float x = cp[LT_P + a] * (0.5f * (float)LT_P);
+    const double pos = ((double)i + 0.5 + 0.5 * (double)x) * (4294967296.0 / (double)C);
+    const uint32_t code = (uint32_t)(unsigned long long)__double2ll_rn(pos);
     float acc = 0.f, comp = 0.f;
-    for (int m0 = 1; m0 <= M; m0 += SP_LOO_CH) {
-        const int cnt = M - m0 + 1 < SP_LOO_CH ? M - m0 + 1 : SP_LOO_CH;
+    for (int m0 = 1; m0 <= M; m0 += LT_CH) {
+        const int cnt = min(LT_CH, M - m0 + 1);
         __syncthreads();
-        for (int k = threadIdx.x; k < cnt; k += SP_THREADS) sAS[k] = AS[m0 - 1 + k];
+        for (int k = threadIdx.x; k < LT_CH; k += 32 * LT_GROUPS)
+            sAS[k] = k < cnt ? AS[m0 - 1 + k] : make_float2(0.f, 0.f);
         __syncthreads();
-#pragma unroll 4
-        for (int k = 0; k < cnt; ++k) {
-            const uint32_t ph = (uint32_t)(m0 + k) * ui;
-            float s, co;
-            sincospif((float)(int32_t)ph * (1.0f / 2147483648.0f), &s, &co);
-            const float2 q = sAS[k];
-            // Re(e^{i m theta_i} conj(A_m S_m)) = cos * Re + sin * Im, added with compensation
-            const float y = fmaf(co, q.x, s * q.y) - comp;
-            const float t = acc + y;
-            comp = (t - acc) - y;
-            acc = t;
+        for (int k = warp * 8; k < cnt; k += LT_GROUPS * 8) {
+#pragma unroll
+            for (int h = 0; h < 8; ++h) {
+                const uint32_t ph = (uint32_t)(m0 + k + h) * code;
+                float s, c;
+                sincospif((float)(int32_t)ph * (1.0f / 2147483648.0f), &s, &c);
+                const float2 q = sAS[k + h];
+                // Re(e^{i m theta} conj(c_m)) = cos * Re + sin * Im
+                const float y = fmaf(c, q.x, s * q.y) - comp;
+                const float t = acc + y;
+                comp = (t - acc) - y;
+                acc = t;
+            }
         }
     }
-    if (i >= N) return;
-    const double n = (double)N;
-    const double all = (n + 2.0 * ((double)acc - (double)comp)) / KDE_TWO_PI;
-    loo[i] = (float)(xs * (all - sel->norm) / (n - 1.0));
+    val[warp][lane] = (double)acc - (double)comp;
+    __syncthreads();
+    if (warp == 0) {
+        double v = 0.0;
+#pragma unroll
+        for (int w = 0; w < LT_GROUPS; ++w) v += val[w][lane];
+        val[0][lane] = v * inv_n;
+        __syncwarp();
+        if (iv < LT_IV && i < C) {
+            const double *f = &val[0][iv * LT_P];
+            if (a == 0) {
+                double t = 0.0;
+                for (int q = 0; q < LT_P; ++q) t += f[q];
+                tab[i].c0 = t * (1.0 / LT_P);
+            } else {
+                // the points' differences from the first: the sum of a row of the matrix is 0
+                float t = 0.f;
+                for (int q = 1; q < LT_P; ++q) t = fmaf(cp[a * LT_P + q], (float)(f[q] - f[0]), t);
+                tab[i].c[a - 1] = t;
+            }
+        }
+    }
 }
 
-// leave-one-out densities at cand[*argmin] from the structure factor S (modes
-// 1..M(kappa*) present)
+// loo_i = (2 pi / L) (sum_j K - own kernel) / (n - 1) from the table; own kernel: sel->norm, or
+// norm(sel->kappa kr_i) for particle-wise widths
+// (fa = xs n / (2 pi (n - 1)), fb = xs / (n - 1))
+__global__ void __launch_bounds__(SP_THREADS)
+    spec_loo_kernel(const uint32_t *__restrict__ u, const float *__restrict__ kr, int64_t N,
+                    const LtRow *__restrict__ tab, const SpecSel *__restrict__ sel, double fa, double fb,
+                    const float2 *__restrict__ ntab, float *loo)
+{
+    const int C = sel->C;
+    const double base = kr ? fa : fma(-fb, sel->norm, fa), fa2 = 2.0 * fa;
+    const float kap = (float)sel->kappa;
+    for (int64_t i = (int64_t)blockIdx.x * SP_THREADS + threadIdx.x; i < N; i += (int64_t)gridDim.x * SP_THREADS) {
+        const uint32_t ui = u[i];
+        const float x = (float)(int32_t)((ui * (uint32_t)C) ^ 0x80000000u) * (1.f / 2147483648.f);
+        const uint4 *r = (const uint4 *)(tab + __umulhi(ui, (uint32_t)C));
+        const uint4 a = __ldg(r), b = __ldg(r + 1);
+        const float x2 = x + x;
+        float b1 = __uint_as_float(b.w), b2 = 0.f, t;
+#define LT_STEP(w) t = fmaf(x2, b1, __uint_as_float(w) - b2); b2 = b1; b1 = t
+        LT_STEP(b.z);
+        LT_STEP(b.y);
+        LT_STEP(b.x);
+        LT_STEP(a.w);
+        LT_STEP(a.z);
+#undef LT_STEP
+        const double g = __hiloint2double((int)a.y, (int)a.x) + (double)fmaf(x, b1, -b2);
+        double v = fma(fa2, g, base);
+        if (kr) v = fma(-fb, (double)kde_norm_tab(ntab, kap * kr[i]), v);
+        loo[i] = (float)v;
+    }
+}
+
+// table and densities from the series coefficients AS (modes 1..sel->M) of a sample whose
+// widths are at most kappa_max
+static kde_status spec_loo_table(kde_ctx *ctx, const uint32_t *u, const float *kr, int64_t N, double L,
+                                 const float2 *AS, const SpecSel *sel, double kappa_max, float *loo)
+{
+    const int C = lt_intervals(kappa_max);
+    LtRow *tab = (LtRow *)kde_ws(ctx, WS_LTAB, (size_t)C * sizeof(LtRow));
+    if (!tab) return KDE_ENOMEM;
+    KdeProfScope _ps(ctx, PROF_CV_LOO);
+    spec_table_kernel<<<(C + LT_IV - 1) / LT_IV, 32 * LT_GROUPS, 0, ctx->stream>>>(
+        AS, sel, ctx->pxy_tab + pxy_tab_off(LT_P), 1.0 / (double)N, tab);
+    KDE_LAUNCHED(ctx, "spec_table_kernel");
+    const int64_t want = (N + SP_THREADS - 1) / SP_THREADS, cap = 8LL * (ctx->sm_count > 0 ? ctx->sm_count : 1);
+    spec_loo_kernel<<<(unsigned)(want < cap ? want : cap), SP_THREADS, 0, ctx->stream>>>(
+        u, kr, N, tab, sel, (double)N / (L * (double)(N - 1)), KDE_TWO_PI / (L * (double)(N - 1)), ctx->norm_tab, loo);
+    KDE_LAUNCHED(ctx, "spec_loo_kernel");
+    return KDE_OK;
+}
+
+// the selected candidate's row of F in FP32, and its limits, for particle-wise widths
+__global__ void __launch_bounds__(256) spec_as_scale_kernel(const double2 *F, int Mst, CandList cl, const int *argmin,
+                                                            double kr_max, float2 *AS, SpecSel *sel)
+{
+    const int c = *argmin, m = blockIdx.x * 256 + threadIdx.x;
+    if (m < Mst) {
+        const double2 f = F[(size_t)c * Mst + m];
+        AS[m] = make_float2((float)f.x, (float)f.y);
+    }
+    if (m == 0) {
+        const double k = cl.k[c] * kr_max;
+        sel->M = min(Mst, kde_spec_modes(k));
+        sel->C = lt_intervals(k);
+        sel->kappa = cl.k[c];
+        sel->norm = 0.0;
+    }
+}
+
+kde_status kde_loo_series(kde_ctx *ctx, const uint32_t *u, const float *kr, int64_t N, double L, const double2 *F,
+                          int Mst, const CandList &cl, const int *argmin_dev, double kappa_max, float *loo)
+{
+    double smax = 0.0;
+    for (int c = 0; c < cl.n; ++c) smax = cl.k[c] > smax ? cl.k[c] : smax;
+    float2 *AS = (float2 *)kde_ws(ctx, WS_SP_AS, (size_t)Mst * sizeof(float2) + 64);
+    SpecSel *sel = (SpecSel *)kde_ws(ctx, WS_SP_SEL, sizeof(SpecSel));
+    if (!AS || !sel) return KDE_ENOMEM;
+    spec_as_scale_kernel<<<(Mst + 255) / 256, 256, 0, ctx->stream>>>(F, Mst, cl, argmin_dev, kappa_max / smax, AS, sel);
+    KDE_LAUNCHED(ctx, "spec_as_scale_kernel");
+    return spec_loo_table(ctx, u, kr, N, L, AS, sel, kappa_max, loo);
+}
+
+// leave-one-out densities at cand[*argmin] from the structure factor S (modes 1..M(kappa*)
+// present); with cv_dev the argmin (and *kstar_dev) of that curve is found on the way
 static kde_status spec_loo_from_S(kde_ctx *ctx, const uint32_t *u, int64_t N, double L, const double2 *S,
-                                  const CandList &cl, int Mmax, const int *argmin_dev, float *loo,
+                                  const CandList &cl, int Mmax, int *argmin_dev, float *loo,
+                                  const double *cv_dev = nullptr, double *kstar_dev = nullptr,
                                   const double *Atab = nullptr, int Astride = 0)
 {
     double *Asel = (double *)kde_ws(ctx, WS_SP_ASEL, (size_t)(Mmax + 1) * 8 + 64);
     float2 *AS = (float2 *)kde_ws(ctx, WS_SP_AS, (size_t)Mmax * sizeof(float2) + 64);
     SpecSel *sel = (SpecSel *)kde_ws(ctx, WS_SP_SEL, sizeof(SpecSel));
     if (!Asel || !AS || !sel) return KDE_ENOMEM;
-    spec_select_kernel<<<1, 1, 0, ctx->stream>>>(cl, argmin_dev, sel, Asel, Atab, Astride);
+    spec_select_kernel<<<1, 32, 0, ctx->stream>>>(cv_dev, cl, argmin_dev, kstar_dev, sel, Asel, Atab, Astride);
     KDE_LAUNCHED(ctx, "spec_select_kernel");
     spec_as_kernel<<<(Mmax + 255) / 256, 256, 0, ctx->stream>>>(S, sel, AS);
     KDE_LAUNCHED(ctx, "spec_as_kernel");
-    {
-        KdeProfScope _ps(ctx, PROF_CV_LOO);
-        spec_loo_kernel<<<(unsigned)((N + SP_THREADS - 1) / SP_THREADS), SP_THREADS, 0, ctx->stream>>>(
-            u, N, AS, sel, KDE_TWO_PI / L, loo);
-    }
-    KDE_LAUNCHED(ctx, "spec_loo_kernel");
-    return KDE_OK;
+    double kmax = 0.0;
+    for (int c = 0; c < cl.n; ++c) kmax = cl.k[c] > kmax ? cl.k[c] : kmax;
+    return spec_loo_table(ctx, u, nullptr, N, L, AS, sel, kmax, loo);
 }
 
 // structure factor for modes 1..M (or up to *mlim) into S
 static kde_status spec_structure(kde_ctx *ctx, const uint32_t *u, int64_t N, int M, const int *mlim, double2 **S_out)
 {
-    // about a thousand chunks keep every SM busy; the partials stay under 2^22 entries (64 MB)
-    int64_t chunk = 1024;
+    // about a thousand chunks keep every SM busy (2^18 particles and 893 modes: 124 us in 256
+    // chunks of 1024, 91 in 1024 of 256; 50,021 and 1724 modes: 101 and 45 us); the partials stay
+    // under 2^22 entries (64 MB)
+    int64_t chunk = 256;
     while (((N + chunk - 1) / chunk > 1024 || (N + chunk - 1) / chunk * M > (1 << 22)) && chunk < SP_MAXCHUNK)
         chunk *= 2;
     const int nchunks = (int)((N + chunk - 1) / chunk);
@@ -343,8 +493,13 @@ static kde_status spec_structure(kde_ctx *ctx, const uint32_t *u, int64_t N, int
     return KDE_OK;
 }
 
+kde_status kde_spec_structure(kde_ctx *ctx, const uint32_t *u, int64_t N, int M, double2 **S_out)
+{
+    return spec_structure(ctx, u, N, M, nullptr, S_out);
+}
+
 // selected width's mode count, for the structure factor of the leave-one-out pass
-__global__ void spec_mlim_kernel(CandList cl, const int *argmin, int *mlim) { *mlim = spec_modes(cl.k[*argmin]); }
+__global__ void spec_mlim_kernel(CandList cl, const int *argmin, int *mlim) { *mlim = kde_spec_modes(cl.k[*argmin]); }
 
 kde_status kde_loo_spectral_device(kde_ctx *ctx, const uint32_t *u, int64_t N, double L, const double *cand_host,
                                    int n_cand, const int *argmin_dev, float *loo)
@@ -356,17 +511,15 @@ kde_status kde_loo_spectral_device(kde_ctx *ctx, const uint32_t *u, int64_t N, d
         cl.k[c] = cand_host[c];
         kmax = cand_host[c] > kmax ? cand_host[c] : kmax;
     }
-    const int Mmax = spec_modes(kmax);
+    const int Mmax = kde_spec_modes(kmax);
     int *mlim = (int *)kde_ws(ctx, WS_SP_MLIM, 64);
     if (!mlim) return KDE_ENOMEM;
     spec_mlim_kernel<<<1, 1, 0, ctx->stream>>>(cl, argmin_dev, mlim);
     KDE_LAUNCHED(ctx, "spec_mlim_kernel");
     double2 *S = nullptr;
     KDE_TRY(spec_structure(ctx, u, N, Mmax, mlim, &S));
-    return spec_loo_from_S(ctx, u, N, L, S, cl, Mmax, argmin_dev, loo);
+    return spec_loo_from_S(ctx, u, N, L, S, cl, Mmax, const_cast<int *>(argmin_dev), loo);
 }
-
-int kde_spec_modes(double kappa) { return spec_modes(kappa); }
 
 kde_status kde_cv_spectral_device(kde_ctx *ctx, const uint32_t *u, int64_t N, double L, const double *cand_host,
                                   int n_cand, double *cv_dev, int *argmin_dev, float *loo, double *kstar_dev)
@@ -379,7 +532,7 @@ kde_status kde_cv_spectral_device(kde_ctx *ctx, const uint32_t *u, int64_t N, do
         cl.k[c] = cand_host[c];
         kmax = cand_host[c] > kmax ? cand_host[c] : kmax;
     }
-    const int M = spec_modes(kmax);
+    const int M = kde_spec_modes(kmax);
     const int Astride = M + 1;
     double *Atab = (double *)kde_ws(ctx, WS_SP_A, (size_t)n_cand * Astride * 8 + 64 * 1024 * 8);
     if (!Atab) return KDE_ENOMEM;
@@ -393,8 +546,8 @@ kde_status kde_cv_spectral_device(kde_ctx *ctx, const uint32_t *u, int64_t N, do
     ctx->sp_atab = (void *)Atab;
     ctx->sp_atab_cands = key;
     KDE_LAUNCHED(ctx, "spec_cv_kernel");
-    spec_argmin_kernel<<<1, 1, 0, ctx->stream>>>(cv_dev, cl, argmin_dev, kstar_dev);
-    KDE_LAUNCHED(ctx, "spec_argmin_kernel");
-    if (loo) KDE_TRY(spec_loo_from_S(ctx, u, N, L, S, cl, M, argmin_dev, loo, Atab, Astride));
+    if (loo) return spec_loo_from_S(ctx, u, N, L, S, cl, M, argmin_dev, loo, cv_dev, kstar_dev, Atab, Astride);
+    spec_select_kernel<<<1, 32, 0, ctx->stream>>>(cv_dev, cl, argmin_dev, kstar_dev, nullptr, nullptr, nullptr, 0);
+    KDE_LAUNCHED(ctx, "spec_select_kernel");
     return KDE_OK;
 }

@@ -268,3 +268,38 @@ def test_cv_cost_rule_picks_an_exact_form(ctx, oracle, kp):
         check_curve(auto, am, ref, label="cost rule N=%d (%s)" % (N, form))
     with pytest.raises(kp.KdeError):
         ctx.cv(ud, L, cand, spectral=True, pairs=True)
+
+
+@pytest.mark.parametrize("N,lo,hi,n_cand", [(20000, 5.0, 5e3, 16), (16384, 40.0, 40.0, 8), (30001, 0.2, 90.0, 5),
+                                            (25000, 300.0, 700.0, 33)])
+def test_cv_scale_fourier_form(ctx, oracle, N, lo, hi, n_cand):
+    # particle-wise widths by the Fourier form (large samples) against the pair sums the same
+    # call makes when asked for them, and a few candidates and densities against the oracle.
+    # Tolerances: the curve within the pair sums' 2e-6 of its maximum (the Fourier form itself
+    # within 1e-7: structure factors of FP32 phases, random over the particles), densities 1e-5
+    L = 4 * math.pi
+    u, _ = I.landau_load(N, N, L, 0.05, 1.0)
+    x = I.from_fixed(u, L)
+    kr = I.log_uniform(N, I.STREAM_KAPPA, N, lo, hi).astype(np.float32)
+    scales = 10.0 ** (np.linspace(-1.0, 0.8, n_cand))
+    ud, kd = to_dev_u(u), to_dev(kr)
+    cv, am, loo = ctx.cv(ud, L, scales, kappa_rel=kd, want_loo=True)
+    cp, ap, lp = ctx.cv(ud, L, scales, kappa_rel=kd, want_loo=True, pairs=True)
+    check_curve(cv, am, cp, label="scale mode N=%d" % N)
+    np.testing.assert_allclose(loo.cpu().numpy(), lp.cpu().numpy(), rtol=2e-5, atol=1e-7 * float(lp.max()))
+    for c in (0, n_cand - 1):
+        ref, _, _, lref = oracle.cv_dense(x, L, kappa=scales[c] * kr.astype(np.float64), want_loo=True)
+        assert abs(cv[c] - ref) <= 1e-7 * np.max(np.abs(cv))
+        if c == am:
+            np.testing.assert_allclose(loo.cpu().numpy(), lref, rtol=1e-5, atol=1e-7 * np.max(lref))
+
+
+def test_cv_scale_out_of_range_width_is_reported(ctx, kp):
+    N = 20000
+    u, _ = I.landau_load(1, N, 4 * math.pi, 0.05, 1.0)
+    kr = np.full(N, 50.0, np.float32)
+    kr[7] = -1.0
+    with pytest.raises(kp.KdeError):
+        ctx.cv(to_dev_u(u), 4 * math.pi, [0.5, 1.0], kappa_rel=to_dev(kr))
+    kr[7] = 50.0
+    ctx.cv(to_dev_u(u), 4 * math.pi, [0.5, 1.0], kappa_rel=to_dev(kr))
