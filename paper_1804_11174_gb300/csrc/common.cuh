@@ -481,14 +481,15 @@ kde_status kde_bspline_gather_push(kde_ctx *ctx, uint32_t *u, float *v, int64_t 
 kde_status kde_radix_sort_u32(kde_ctx *ctx, const uint32_t *u, int64_t N, uint32_t *out, uint32_t *tmp);
 
 // deposit of cell-sorted particles into int64 accumulators (zeroed here): acc[Ng], and in FP64
-// a second acc[Ng .. 2 Ng) of remainders in units of 2^-24 of the first's.  Particle j contributes w_j * coef * norm_j * exp(-2 kappa_j sin^2(..)).
+// a second acc[Ng .. 2 Ng) of remainders in units of 2^-24 of the first's.
+// Particle j contributes w_j * coef * norm_j * exp(-2 kappa_j sin^2(..)).
 // Arrays may be null (then the uniform scalar is used; norm null with a kappa
 // array means "compute the norm from the width").  `bound` is the largest
 // possible node value; with wmax_bits it is N * coef * norm_bound * w_max.
-template <typename T>
-kde_status kde_deposit_sorted(kde_ctx *ctx, const uint32_t *u, const T *kappa, T kappa_u, const T *norm, T norm_u,
-                              const T *w, T w_u, int64_t N, int Ng, double coef, long long *acc, double bound,
-                              const unsigned int *wmax_bits, double norm_bound);
+kde_status kde_deposit_sorted_f64(kde_ctx *ctx, const uint32_t *u, const double *kappa, double kappa_u,
+                                  const double *norm, double norm_u, const double *w, double w_u, int64_t N, int Ng,
+                                  double coef, long long *acc, double bound, const unsigned int *wmax_bits,
+                                  double norm_bound);
 template <typename T>
 kde_status kde_acc_to_real(kde_ctx *ctx, const long long *acc, int Ng, double bound, const unsigned int *wmax_bits,
                            double wscale, T *out);

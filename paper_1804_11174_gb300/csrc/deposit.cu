@@ -52,6 +52,7 @@ template <typename T> struct DepSrc {
     int scale_exp;  // KDE_ES_FROM_BOUND, or the exponent es of the fixed-point scale 2^es
     const float2 *ntab;  // FP32 norm table (kde_norm_tab) for per-particle widths without norms, or nullptr
     float xcut = (float)KDE_XCUT;  // FP32 packed kernels: truncation cut exponent (kde_fp32_cut)
+    int nbins = 0;                   // sort bins of the particles: 0 the cells, -1 not sorted at all
     PxyGrid grid;                    // the nodes as position codes
     const float *pxt;                // interpolation matrices (proxy.cuh)
     const unsigned int *krange;      // float bits of the largest and smallest width, or null
@@ -631,13 +632,12 @@ __global__ void __launch_bounds__(DEP_THREADS) deposit64_kernel(DepSrc<double> S
 #define DEPP_SUB 2304  // records a sub-chunk: a 2^20-particle run has one sub-chunk a CTA
 #define DEPP_PART 512
 #define DEPP_RED_THREADS 1024
-#define DEPP_RED_NODES 32
+#define DEPP_RED_NODES 8
 
 struct DepPlan {
     int G;            // CTAs
     long long *rows;  // [G][Ng] per-CTA node sums over its window
     int2 *hdr;        // [G] (first node, node count) of every row
-    long long *acc;   // [Ng] output accumulators (every node written by the row reduction)
     float fixed;      // cost of the compressed form's fixed steps (depp_compress_pays)
 };
 // node pairs of the persistent deposit: each lane owns P pairs of nodes (64 P
@@ -1153,23 +1153,28 @@ __device__ __forceinline__ bool depp_compress_pays(const PxyBox &B, int n, int R
     return comp < direct;
 }
 
-// acc[g] = sum over the rows whose window covers node g of that row's entry; CTA b
-// takes nodes [32 b, 32 b + 32), lane l node 32 b + l, warp w rows w, w + 32, ...
+// out[g] = 2^-es times the sum over the rows whose window covers node g of that row's entry;
+// CTA b takes nodes [8 b, 8 b + 8), eight lanes a row (64 bytes), the CTA's 128 row slots rows
+// s, s + 128, ...  es: from the host's bound, or from the device's largest weight
 __global__ void __launch_bounds__(DEPP_RED_THREADS) deposit_rows_kernel(const long long *__restrict__ rows,
                                                                        const int2 *__restrict__ hdr, int G, int Ng,
-                                                                       long long *acc)
+                                                                       double bound, const unsigned int *wmax_bits,
+                                                                       double wscale, float *out)
 {
     __shared__ long long wsum[DEPP_RED_THREADS / 32][DEPP_RED_NODES];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    constexpr int NW = DEPP_RED_THREADS / 32;
-    const int g = blockIdx.x * DEPP_RED_NODES + lane;
+    constexpr int NW = DEPP_RED_THREADS / DEPP_RED_NODES;
+    const int slot = threadIdx.x / DEPP_RED_NODES;
+    const int g = blockIdx.x * DEPP_RED_NODES + (lane & (DEPP_RED_NODES - 1));
+    kde_pdl_wait();
+    kde_pdl_trigger();
     long long sum = 0;
     if (g < Ng) {
-        // rows in batches of 8 per warp, every load of a batch issued before any is used
-        for (int k0 = warp; k0 < G; k0 += 8 * NW) {
-            long long v[8];
+        // rows in batches of 4 a slot, every load of a batch issued before any is used
+        for (int k0 = slot; k0 < G; k0 += 4 * NW) {
+            long long v[4];
 #pragma unroll
-            for (int q = 0; q < 8; ++q) {
+            for (int q = 0; q < 4; ++q) {
                 const int k = k0 + q * NW;
                 v[q] = 0;
                 if (k < G) {
@@ -1180,16 +1185,19 @@ __global__ void __launch_bounds__(DEPP_RED_THREADS) deposit_rows_kernel(const lo
                 }
             }
 #pragma unroll
-            for (int q = 0; q < 8; ++q) sum += v[q];
+            for (int q = 0; q < 4; ++q) sum += v[q];
         }
     }
-    wsum[warp][lane] = sum;
+#pragma unroll
+    for (int o = DEPP_RED_NODES; o < 32; o <<= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
+    if (lane < DEPP_RED_NODES) wsum[warp][lane] = sum;
     __syncthreads();
-    if (warp == 0 && g < Ng) {
+    if (threadIdx.x < DEPP_RED_NODES && g < Ng) {
         long long t = 0;
 #pragma unroll
-        for (int w = 0; w < NW; ++w) t += wsum[w][lane];
-        acc[g] = t;
+        for (int w = 0; w < DEPP_RED_THREADS / 32; ++w) t += wsum[w][lane];
+        const double b = wmax_bits ? wscale * (double)__uint_as_float(*wmax_bits) : bound;
+        out[g] = (float)((double)t / kde_acc_scale(b));
     }
 }
 
@@ -1261,7 +1269,15 @@ __global__ void __launch_bounds__(DEPP_THREADS, DEPP_MINB) deposit_persist_kerne
     const int es = s_es;
     const bool cosf = kmax <= KDE_COSFORM_KMAX;
     const int W = window_nodes_f(kmin, Ng, S.xcut);
-    const int c_first = kde_cell(S.u[i0], Ng), c_last = kde_cell(S.u[i1 - 1], Ng);
+    // the CTA's cells: those of its first and last sort bin (unsorted particles: all)
+    int c_first = 0, c_last = Ng - 1;
+    if (S.nbins == 0) {
+        c_first = kde_cell(S.u[i0], Ng);
+        c_last = kde_cell(S.u[i1 - 1], Ng);
+    } else if (S.nbins > 0) {
+        c_first = kde_cell(S.u[i0], S.nbins) * Ng / S.nbins;
+        c_last = ((kde_cell(S.u[i1 - 1], S.nbins) + 1) * Ng - 1) / S.nbins;
+    }
     int g_lo = c_first - W;
     int R = c_last + W - g_lo + 1;
     if (R >= Ng || R < 1 || c_last < c_first) {
@@ -1425,26 +1441,33 @@ __global__ void wmax_kernel(const T *w, int64_t N, unsigned int *wmax_bits, unsi
         if (!(v >= 0.f) || isinf(v)) kde_flag(status, KDE_DEV_BAD_ARG, (unsigned)i);
         else m = fmaxf(m, v);
     }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
-    // round the maximum up by one ulp so that the float bound of a double weight still bounds it
-    if ((threadIdx.x & 31) == 0 && m > 0.f) atomicMax(wmax_bits, __float_as_uint(m) + 1u);
+    __shared__ unsigned int red[8];
+    const unsigned int h = __reduce_max_sync(0xffffffffu, __float_as_uint(m));
+    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = h;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        unsigned int b = red[0];
+        for (int w = 1; w < 8; ++w) b = b > red[w] ? b : red[w];
+        // the maximum rounded up by one ulp so that the float bound of a double weight still
+        // bounds it; most blocks find a larger one already
+        if (b > 0u && b + 1u > *(volatile unsigned int *)wmax_bits) atomicMax(wmax_bits, b + 1u);
+    }
 }
 
 // ---------------------------------------------------------------------------
 // workspace of the persistent FP32 deposit for N particles on Ng nodes: the CTAs'
 // rows and their headers
-static kde_status depp_plan(kde_ctx *ctx, int64_t N, int Ng, long long *acc, DepPlan &Pl)
+static kde_status depp_plan(kde_ctx *ctx, int64_t N, int Ng, bool flat, DepPlan &Pl)
 {
     const int64_t gmax = (int64_t)DEPP_MINB * ctx->sm_count;
-    const int64_t gn = (N + 255) / 256;
+    // unsorted particles sweep the whole grid: shorter shares, so that small calls reach more SMs
+    const int64_t gn = flat ? (N + 63) / 64 : (N + 255) / 256;
     Pl.G = (int)(gn < gmax ? gn : gmax);
     const size_t rows_b = (size_t)Pl.G * Ng * 8;
     unsigned char *w = (unsigned char *)kde_ws(ctx, WS_DEP_ROWS, rows_b + (size_t)Pl.G * 8);
     if (!w) return KDE_ENOMEM;
     Pl.rows = (long long *)w;
     Pl.hdr = (int2 *)(w + rows_b);
-    Pl.acc = acc;
     Pl.fixed = Pl.G <= ctx->sm_count ? 3.0e5f : 6.0e4f;
     return KDE_OK;
 }
@@ -1452,17 +1475,17 @@ static kde_status depp_plan(kde_ctx *ctx, int64_t N, int Ng, long long *acc, Dep
 kde_status kde_deposit_reserve(kde_ctx *ctx, int64_t N, int Ng)
 {
     DepPlan Pl{};
-    return depp_plan(ctx, N, Ng, nullptr, Pl);
+    return depp_plan(ctx, N, Ng, true, Pl);
 }
 
 template <typename T>
 static kde_status deposit_sorted_impl(kde_ctx *ctx, const uint32_t *u, const T *kappa, T kappa_u, const T *norm,
                                       T norm_u, const T *w, T w_u, int64_t N, int Ng, double coef, long long *acc,
                                       double bound, const unsigned int *wmax_bits, double norm_bound, DepRows *rows_out,
-                                      float xcut = 0.f, const unsigned int *krange = nullptr)
+                                      float xcut = 0.f, const unsigned int *krange = nullptr, int nbins = 0)
 {
-    // the persistent FP32 kernel writes every node; the others add into zeroed accumulators
-    if (!(sizeof(T) == 4 && N > 0))
+    // the persistent FP32 kernel writes rows; the FP64 one adds into zeroed accumulators
+    if (sizeof(T) == 8)
         KDE_CUDA(ctx, cudaMemsetAsync(acc, 0, (size_t)2 * Ng * sizeof(long long), ctx->stream), "acc memset");
     if (N == 0) return KDE_OK;
     const void *nodes = kde_node_table(ctx, Ng, sizeof(T) == 8);
@@ -1498,35 +1521,28 @@ static kde_status deposit_sorted_impl(kde_ctx *ctx, const uint32_t *u, const T *
     S.grid = pxy_grid(Ng);
     S.pxt = ctx->pxy_tab;
     S.krange = krange;
+    S.nbins = nbins;
     if constexpr (sizeof(T) == 4) {
         DepPlan Pl{};
-        KDE_TRY(depp_plan(ctx, N, Ng, acc, Pl));
+        KDE_TRY(depp_plan(ctx, N, Ng, nbins < 0, Pl));
         {
             KdeProfScope _ps(ctx, PROF_DEPOSIT);
             // the compressed form is for the default cut (one the caller has set keeps the sweep
             // over the particles that it is defined for), and for CTAs whose sweep of the whole
             // grid would cost more than its fixed steps
             const double n = (double)N / Pl.G;
-            const bool comp = S.xcut == (float)KDE_XCUT && n * (3.2 * Ng + 48.0) > (double)Pl.fixed;
+            const bool comp = nbins >= 0 && S.xcut == (float)KDE_XCUT && n * (3.2 * Ng + 48.0) > (double)Pl.fixed;
             KDE_CUDA(ctx,
                      kde_launch(ctx, true, comp ? deposit_persist_kernel<true> : deposit_persist_kernel<false>,
                                 dim3(Pl.G), dim3(DEPP_THREADS), 0, S, Pl),
                      "deposit_persist_kernel");
         }
         KDE_LAUNCHED(ctx, "deposit_persist_kernel");
-        if (rows_out) {
-            // the caller sums the rows itself (the PIC step's field kernel)
-            rows_out->rows = Pl.rows;
-            rows_out->hdr = Pl.hdr;
-            rows_out->G = Pl.G;
-            return KDE_OK;
-        }
-        {
-            KdeProfScope _ps(ctx, PROF_DEPOSIT_ROWS);
-            deposit_rows_kernel<<<(Ng + DEPP_RED_NODES - 1) / DEPP_RED_NODES, DEPP_RED_THREADS, 0, ctx->stream>>>(
-                Pl.rows, Pl.hdr, Pl.G, Ng, acc);
-        }
-        KDE_LAUNCHED(ctx, "deposit_rows_kernel");
+        // the caller sums the rows (the PIC step's field kernel, deposit_rows_f32)
+        rows_out->rows = Pl.rows;
+        rows_out->hdr = Pl.hdr;
+        rows_out->G = Pl.G;
+        return KDE_OK;
     } else {
         // four chunks an SM where that leaves them 16 particles or more, 256 at most
         const int64_t per = N / (4LL * (ctx->sm_count > 0 ? ctx->sm_count : 1)) + 1;
@@ -1540,13 +1556,13 @@ static kde_status deposit_sorted_impl(kde_ctx *ctx, const uint32_t *u, const T *
     return KDE_OK;
 }
 
-template <typename T>
-kde_status kde_deposit_sorted(kde_ctx *ctx, const uint32_t *u, const T *kappa, T kappa_u, const T *norm, T norm_u,
-                              const T *w, T w_u, int64_t N, int Ng, double coef, long long *acc, double bound,
-                              const unsigned int *wmax_bits, double norm_bound)
+kde_status kde_deposit_sorted_f64(kde_ctx *ctx, const uint32_t *u, const double *kappa, double kappa_u,
+                                  const double *norm, double norm_u, const double *w, double w_u, int64_t N, int Ng,
+                                  double coef, long long *acc, double bound, const unsigned int *wmax_bits,
+                                  double norm_bound)
 {
-    return deposit_sorted_impl<T>(ctx, u, kappa, kappa_u, norm, norm_u, w, w_u, N, Ng, coef, acc, bound, wmax_bits,
-                                  norm_bound, nullptr);
+    return deposit_sorted_impl<double>(ctx, u, kappa, kappa_u, norm, norm_u, w, w_u, N, Ng, coef, acc, bound, wmax_bits,
+                                       norm_bound, nullptr);
 }
 
 kde_status kde_deposit_rows_f32(kde_ctx *ctx, const uint32_t *u, const float *kappa, float kappa_u, const float *norm,
@@ -1568,12 +1584,6 @@ kde_status kde_acc_to_real(kde_ctx *ctx, const long long *acc, int Ng, double bo
     return KDE_OK;
 }
 
-template kde_status kde_deposit_sorted<float>(kde_ctx *, const uint32_t *, const float *, float, const float *, float,
-                                              const float *, float, int64_t, int, double, long long *, double,
-                                              const unsigned int *, double);
-template kde_status kde_deposit_sorted<double>(kde_ctx *, const uint32_t *, const double *, double, const double *,
-                                               double, const double *, double, int64_t, int, double, long long *,
-                                               double, const unsigned int *, double);
 template kde_status kde_acc_to_real<float>(kde_ctx *, const long long *, int, double, const unsigned int *, double,
                                            float *);
 template kde_status kde_acc_to_real<double>(kde_ctx *, const long long *, int, double, const unsigned int *, double,
@@ -1705,44 +1715,105 @@ kde_status kde_cv_integral_term(kde_ctx *ctx, const uint32_t *u_sorted, int64_t 
 // ---------------------------------------------------------------------------
 // C ABI
 // ---------------------------------------------------------------------------
+// largest weight into the workspace's word (float bits), or nullptr without weights
 template <typename T>
-static kde_status deposit_api(kde_ctx *ctx, const uint32_t *u, const T *kappa, double kappa_u, const T *weight,
-                              int64_t N, int Ng, double L, T *rho_out)
+static kde_status deposit_wmax(kde_ctx *ctx, const T *weight, int64_t N, unsigned int **out)
+{
+    *out = nullptr;
+    if (!weight) return KDE_OK;
+    unsigned int *wmax = (unsigned int *)kde_ws(ctx, WS_WMAX, 64);
+    if (!wmax) return KDE_ENOMEM;
+    KDE_CUDA(ctx, cudaMemsetAsync(wmax, 0, 4, ctx->stream), "wmax memset");
+    int blocks = (int)((N + 255) / 256);
+    blocks = blocks > ctx->sm_count * 4 ? ctx->sm_count * 4 : blocks;
+    wmax_kernel<T><<<blocks, 256, 0, ctx->stream>>>(weight, N, wmax, ctx->d_status);
+    KDE_LAUNCHED(ctx, "wmax_kernel");
+    *out = wmax;
+    return KDE_OK;
+}
+
+static kde_status deposit_api_f64(kde_ctx *ctx, const uint32_t *u, const double *kappa, double kappa_u,
+                                  const double *weight, int64_t N, int Ng, double L, double *rho_out)
 {
     cudaSetDevice(ctx->device);
     long long *acc = (long long *)kde_ws(ctx, WS_ACC, (size_t)2 * Ng * sizeof(long long));
     if (!acc) return KDE_ENOMEM;
     if (N == 0) {
-        KDE_CUDA(ctx, cudaMemsetAsync(rho_out, 0, (size_t)Ng * sizeof(T), ctx->stream), "rho memset");
+        KDE_CUDA(ctx, cudaMemsetAsync(rho_out, 0, (size_t)Ng * 8, ctx->stream), "rho memset");
         return KDE_OK;
     }
     uint32_t *us = (uint32_t *)kde_ws(ctx, WS_SORT_U, (size_t)N * 4);
-    T *ks = kappa ? (T *)kde_ws(ctx, WS_SORT_P0, (size_t)N * sizeof(T)) : nullptr;
-    T *ws = weight ? (T *)kde_ws(ctx, WS_SORT_P1, (size_t)N * sizeof(T)) : nullptr;
+    double *ks = kappa ? (double *)kde_ws(ctx, WS_SORT_P0, (size_t)N * 8) : nullptr;
+    double *ws = weight ? (double *)kde_ws(ctx, WS_SORT_P1, (size_t)N * 8) : nullptr;
     if (!us || (kappa && !ks) || (weight && !ws)) return KDE_ENOMEM;
     SortPayload pl[2];
     int npl = 0;
-    if (kappa) pl[npl++] = SortPayload{kappa, ks, (int)sizeof(T)};
-    if (weight) pl[npl++] = SortPayload{weight, ws, (int)sizeof(T)};
+    if (kappa) pl[npl++] = SortPayload{kappa, ks, 8};
+    if (weight) pl[npl++] = SortPayload{weight, ws, 8};
     KDE_TRY(kde_sort_by_bin(ctx, u, N, Ng, us, pl, npl, nullptr));
     const double coef = KDE_TWO_PI / L;
-    double norm_u = kappa ? 0.0 : kde_norm(kappa_u);
-    double norm_bound = kappa ? kde_norm(KDE_KAPPA_MAX) : norm_u;
-    double w_u = L / (double)N;
+    const double norm_u = kappa ? 0.0 : kde_norm(kappa_u);
+    const double norm_bound = kappa ? kde_norm(KDE_KAPPA_MAX) : norm_u;
+    const double w_u = L / (double)N;
+    const double bound = (double)N * w_u * coef * norm_bound;
     unsigned int *wmax = nullptr;
-    double bound = (double)N * w_u * coef * norm_bound;
-    if (weight) {
-        wmax = (unsigned int *)kde_ws(ctx, WS_WMAX, 64);
-        if (!wmax) return KDE_ENOMEM;
-        KDE_CUDA(ctx, cudaMemsetAsync(wmax, 0, 4, ctx->stream), "wmax memset");
-        int blocks = (int)((N + 255) / 256);
-        blocks = blocks > ctx->sm_count * 8 ? ctx->sm_count * 8 : blocks;
-        wmax_kernel<T><<<blocks, 256, 0, ctx->stream>>>(weight, N, wmax, ctx->d_status);
-        KDE_LAUNCHED(ctx, "wmax_kernel");
+    KDE_TRY(deposit_wmax<double>(ctx, weight, N, &wmax));
+    KDE_TRY(kde_deposit_sorted_f64(ctx, us, ks, kappa_u, nullptr, norm_u, ws, w_u, N, Ng, coef, acc, bound, wmax, norm_bound));
+    return kde_acc_to_real<double>(ctx, acc, Ng, bound, wmax, (double)N * coef * norm_bound, rho_out);
+}
+
+static kde_status deposit_api_f32(kde_ctx *ctx, const uint32_t *u, const float *kappa, double kappa_u,
+                                  const float *weight, int64_t N, int Ng, double L, float *rho_out)
+{
+    cudaSetDevice(ctx->device);
+    if (N == 0) {
+        KDE_CUDA(ctx, cudaMemsetAsync(rho_out, 0, (size_t)Ng * 4, ctx->stream), "rho memset");
+        return KDE_OK;
     }
-    KDE_TRY(kde_deposit_sorted<T>(ctx, us, ks, (T)kappa_u, nullptr, (T)norm_u, ws, (T)w_u, N, Ng, coef, acc, bound,
-                                  wmax, norm_bound));
-    return kde_acc_to_real<T>(ctx, acc, Ng, bound, wmax, (double)N * coef * norm_bound, rho_out);
+    // few (particle, node) pairs: the particles as they are over the whole grid, at the default
+    // truncation (a cut the caller has set keeps its windows).  2^25 pairs take about 8 us, the
+    // sort they spare 16 to 20
+    const bool flat = (double)N * Ng <= 33554432.0 && kde_fp32_cut(ctx) == (float)KDE_XCUT;
+    // the sort groups the particles for the CTAs' windows, which have at most a few hundred
+    // CTAs' worth of resolution: 1024 bins at most (4,000,037 particles on 4096 nodes: 255 us
+    // sorted by cells)
+    const int nbins = flat ? -1 : (Ng > 1024 ? 1024 : Ng);
+    const uint32_t *us = u;
+    const float *ks = kappa, *ws = weight;
+    if (!flat) {
+        uint32_t *uo = (uint32_t *)kde_ws(ctx, WS_SORT_U, (size_t)N * 4);
+        float *ko = kappa ? (float *)kde_ws(ctx, WS_SORT_P0, (size_t)N * 4) : nullptr;
+        float *wo = weight ? (float *)kde_ws(ctx, WS_SORT_P1, (size_t)N * 4) : nullptr;
+        if (!uo || (kappa && !ko) || (weight && !wo)) return KDE_ENOMEM;
+        SortPayload pl[2];
+        int npl = 0;
+        if (kappa) pl[npl++] = SortPayload{kappa, ko, 4};
+        if (weight) pl[npl++] = SortPayload{weight, wo, 4};
+        KDE_TRY(kde_sort_by_bin(ctx, u, N, nbins, uo, pl, npl, nullptr));
+        us = uo;
+        ks = ko;
+        ws = wo;
+    }
+    const double coef = KDE_TWO_PI / L;
+    const double norm_u = kappa ? 0.0 : kde_norm(kappa_u);
+    const double norm_bound = kappa ? kde_norm(KDE_KAPPA_MAX) : norm_u;
+    const double w_u = L / (double)N;
+    const double bound = (double)N * w_u * coef * norm_bound;
+    unsigned int *wmax = nullptr;
+    KDE_TRY(deposit_wmax<float>(ctx, weight, N, &wmax));
+    DepRows dr{};
+    KDE_TRY(deposit_sorted_impl<float>(ctx, us, ks, (float)kappa_u, nullptr, (float)norm_u, ws, (float)w_u, N, Ng, coef,
+                                       nullptr, bound, wmax, norm_bound, &dr, 0.f, nullptr, nbins == Ng ? 0 : nbins));
+    {
+        KdeProfScope _ps(ctx, PROF_DEPOSIT_ROWS);
+        KDE_CUDA(ctx,
+                 kde_launch(ctx, true, deposit_rows_kernel, dim3((Ng + DEPP_RED_NODES - 1) / DEPP_RED_NODES),
+                            dim3(DEPP_RED_THREADS), 0, dr.rows, dr.hdr, dr.G, Ng, bound, (const unsigned int *)wmax,
+                            (double)N * coef * norm_bound, rho_out),
+                 "deposit_rows_kernel");
+    }
+    KDE_LAUNCHED(ctx, "deposit_rows_kernel");
+    return KDE_OK;
 }
 
 extern "C" kde_status kde_deposit(kde_ctx *ctx, const uint32_t *u, const void *kappa, double kappa_uniform,
@@ -1757,10 +1828,9 @@ extern "C" kde_status kde_deposit(kde_ctx *ctx, const uint32_t *u, const void *k
     if (N > 0xFFFFFFFFll) return kde_fail(ctx, KDE_EINVAL, "kde_deposit: N must be below 2^32");
     if (flags & ~KDE_F64) return kde_fail(ctx, KDE_ENOTSUP, "kde_deposit: unsupported flags 0x%x", flags);
     if (flags & KDE_F64)
-        return deposit_api<double>(ctx, u, (const double *)kappa, kappa_uniform, (const double *)weight, N, Ng, L,
-                                   (double *)rho_out);
-    return deposit_api<float>(ctx, u, (const float *)kappa, kappa_uniform, (const float *)weight, N, Ng, L,
-                              (float *)rho_out);
+        return deposit_api_f64(ctx, u, (const double *)kappa, kappa_uniform, (const double *)weight, N, Ng, L,
+                               (double *)rho_out);
+    return deposit_api_f32(ctx, u, (const float *)kappa, kappa_uniform, (const float *)weight, N, Ng, L, (float *)rho_out);
 }
 
 // ---------------------------------------------------------------------------

@@ -370,8 +370,8 @@ static kde_status pic_run(kde_ctx *ctx, pic_state *st, int n_steps)
         } else {
             {
                 KdeRange r_("kdepic deposit");
-                KDE_TRY(kde_deposit_sorted<T>(ctx, us, ks, (T)st->kappa_uniform, ns, (T)norm_u, nullptr, (T)w_u, N,
-                                              Ng, coef, acc, bound, nullptr, norm_bound));
+                KDE_TRY(kde_deposit_sorted_f64(ctx, us, ks, st->kappa_uniform, ns, norm_u, nullptr, w_u, N, Ng, coef,
+                                               acc, bound, nullptr, norm_bound));
             }
             {
                 KdeRange r_("kdepic Poisson");
