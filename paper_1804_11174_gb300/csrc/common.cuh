@@ -89,7 +89,7 @@ enum WsSlot {
     WS_AD_OUT,
     WS_CV_GPAR,
     WS_GREEN,
-    WS_DEP_ROWS,   // persistent FP32 deposit: per-CTA node rows and their headers
+    WS_DEP_SUMS,   // grids of int64 node sums of the FP32 deposits
     WS_HOST_U,     // device copies of a host-resident PIC state (pic_step_host)
     WS_HOST_V,
     WS_HOST_K,
@@ -129,6 +129,8 @@ struct kde_ctx {
     double *f64_tab = nullptr;   // 2^(j / 2048) for the FP64 kernels (fp64.cuh), built at creation
     float *pxy_tab = nullptr;    // interpolation matrices (proxy.cuh), built at creation
     unsigned wait_polls = 1u << 26;         // polls of a bounded device wait (kde_set_wait_limit)
+    bool sums_zero = false;                 // kde_deposit's grid of node sums is zero
+    bool sums_flip = false;                 // which grid of node sums the next FP32 deposit adds to
     bool count_flip = false;                // which sort count table the next counted sort reads (sort.cu)
     int64_t cv_fourier_bytes = 1ll << 30;   // workspace the Fourier form of a scale-mode CV may take
     bool autotune = false;                  // kde_set_autotune
@@ -493,26 +495,26 @@ kde_status kde_deposit_sorted_f64(kde_ctx *ctx, const uint32_t *u, const double 
 template <typename T>
 kde_status kde_acc_to_real(kde_ctx *ctx, const long long *acc, int Ng, double bound, const unsigned int *wmax_bits,
                            double wscale, T *out);
-// grows the workspace of the FP32 deposit for N particles on Ng nodes (kde_reserve)
-kde_status kde_deposit_reserve(kde_ctx *ctx, int64_t N, int Ng);
-// the FP32 deposit of cell-sorted particles (uniform weight w_u, N >= 1) left as its
-// per-CTA int64 rows (workspace, valid until the next deposit on the context):
-// node g of row k is rows[k Ng + ((g - hdr[k].x) mod Ng)] when that index is below
-// hdr[k].y, else 0; fixed-point scale kde_acc_scale(bound).  krange: float bits of the
-// largest and smallest width on the device, which spare the kernel a pass over the widths
-struct DepRows {
-    const long long *rows;
-    const int2 *hdr;
-    int G;
+// grows the workspace of the FP32 deposit (kde_reserve)
+kde_status kde_deposit_reserve(kde_ctx *ctx);
+// the FP32 deposit of cell-sorted particles (uniform weight w_u, N >= 1) left as int64 node sums
+// (fixed-point scale kde_acc_scale(bound)) for the field kernel.  Two grids of sums are used in
+// turn: the field kernel that reads one zeroes the other, which the next deposit adds to.
+// kde_deposit_sums_reset zeroes both and comes before the first deposit of a call; every deposit
+// is followed by one kde_field_from_sums.  krange: float bits of the largest and smallest width
+// on the device, which spare the kernel a pass over the widths
+struct DepSums {
+    long long *acc, *next;
 };
-kde_status kde_deposit_rows_f32(kde_ctx *ctx, const uint32_t *u, const float *kappa, float kappa_u, const float *norm,
-                                float norm_u, int64_t N, int Ng, double coef, float w_u, double bound, DepRows *out,
+kde_status kde_deposit_sums_reset(kde_ctx *ctx);
+kde_status kde_deposit_sums_f32(kde_ctx *ctx, const uint32_t *u, const float *kappa, float kappa_u, const float *norm,
+                                float norm_u, int64_t N, int Ng, double coef, float w_u, double bound, DepSums *out,
                                 float xcut = 0.f, const unsigned int *krange = nullptr);
-// the PIC step's field from those rows: rho_total = background + charge * rho with its
+// the PIC step's field from those sums: rho_total = background + charge * rho with its
 // mean removed (so the constant background drops out), E by the spectral or
 // finite-difference Green's function (FP32 output)
-kde_status kde_field_from_rows(kde_ctx *ctx, const long long *rows, const int2 *hdr, int G, int Ng, double L,
-                               double acc_inv, double charge, bool fd, float *E_out);
+kde_status kde_field_from_sums(kde_ctx *ctx, const DepSums &ds, int Ng, double L, double acc_inv, double charge, bool fd,
+                               float *E_out);
 
 // Poisson solve of rho_total = background + charge * rho, rho given as a real
 // array or as int64 accumulators (value = acc * acc_inv; in FP64 with the remainders of the
@@ -604,6 +606,8 @@ kde_status kde_adapt_device(kde_ctx *ctx, const float *loo, int64_t N, double L,
                             double kstar_host, double alpha, double kmin, double kmax, void *kappa_out,
                             void *norm_out, bool f64, unsigned int *krange = nullptr);
 
+// the norms of the proxy widths (proxy.cuh) of a finished range, behind its two words
+kde_status kde_krange_norms(kde_ctx *ctx, unsigned int *krange);
 // float bits of the largest and smallest of many widths: kde_krange_reset on the stream,
 // then kde_krange_add by every warp of the kernel that writes the widths (all lanes; a lane
 // without a width passes lo = 3e38, hi = 0)

@@ -404,11 +404,11 @@ extern "C" kde_status kde_reserve(kde_ctx *ctx, int64_t N, int32_t Ng, int32_t n
         {WS_SORT_P3B, (size_t)Np * 4}, {WS_SORT_PERM, (size_t)Np * 4}, {WS_NORM, (size_t)Np * 8},
         {WS_ACC, (size_t)(n_cand > 0 ? n_cand : 1) * 8192 * 8 + 64}, {WS_GRID0, KDE_MAX_NG * 8},
         {WS_GRID1, KDE_MAX_NG * 8}, {WS_GREEN, 2 * KDE_MAX_NG * 8}, {WS_WMAX, 64}, {WS_PIC_E, (size_t)Np * 4}, {WS_PIC_LOO, (size_t)Np * 4},
-        {WS_PIC_KS, 64}, {WS_PIC_RANGE, 64}};
+        {WS_PIC_KS, 64}, {WS_PIC_RANGE, 256}};
     for (auto &b : big)
         if (!kde_ws(ctx, (WsSlot)b[0], b[1])) return KDE_ENOMEM;
     if (!kde_node_table(ctx, Ng, false) || !kde_node_table(ctx, Ng, true)) return KDE_ENOMEM;
-    if (N > 0) KDE_TRY(kde_deposit_reserve(ctx, N, Ng));
+    KDE_TRY(kde_deposit_reserve(ctx));
     KDE_TRY(kde_gather_table_reserve(ctx));
     return KDE_OK;
 }

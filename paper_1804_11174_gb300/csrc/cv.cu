@@ -1138,6 +1138,10 @@ kde_status kde_adapt_device(kde_ctx *ctx, const float *loo, int64_t N, double L,
         if (krange) KDE_CUDA(ctx, kde_krange_reset(krange, ctx->stream), "width range memset");
         adapt_apply_kernel<float><<<grid, 256, 0, ctx->stream>>>(loo, N, P, alpha, kmin, kmax, (float *)kappa_out,
                                                                   (float *)norm_out, ctx->norm_tab, krange);
+        if (krange) {
+            KDE_LAUNCHED(ctx, "adapt_apply_kernel");
+            return kde_krange_norms(ctx, krange);
+        }
     }
     KDE_LAUNCHED(ctx, "adapt_apply_kernel");
     return KDE_OK;

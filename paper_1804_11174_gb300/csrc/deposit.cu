@@ -607,8 +607,7 @@ __global__ void __launch_bounds__(DEP_THREADS) deposit64_kernel(DepSrc<double> S
 }
 
 // ---------------------------------------------------------------------------
-// FP32 deposit of cell-sorted particles over a balanced persistent grid, without
-// global atomics.
+// FP32 deposit of cell-sorted particles over a balanced persistent grid.
 //
 // G = min(3 x SMs, ceil(N / 256)) CTAs (one wave); CTA c owns the contiguous
 // particles [c N / G, (c + 1) N / G), so every CTA carries the same number of
@@ -619,25 +618,20 @@ __global__ void __launch_bounds__(DEP_THREADS) deposit64_kernel(DepSrc<double> S
 // a Landau-size run of 2^20 particles has one sub-chunk a CTA), the inputs of a
 // sub-chunk loaded in batches of register loads, and swept by node-owner lanes as
 // in the chunk kernel (f32x2 pairs of nodes, fixed-order combination of particle
-// slices).  After every sub-chunk the FP32 node sums become int64 fixed point in
-// the CTA's row of the workspace (each node always by the same thread: plain
-// loads and stores).  A second kernel sums the rows: one CTA per 32 nodes, its
-// warps taking the rows in turn with all their loads in flight, the warps'
-// integer sums combined in shared memory, every output node written with a plain
-// store.  Integer sums make the result exact and independent of any order.
+// slices).  After every sub-chunk the FP32 node sums become int64 fixed point and are
+// added to the grid's sums by integer reductions in the L2, at most Ng a CTA (456 x 256
+// at Landau size, about 1 us), exact and independent of any order.  Rows per CTA and a
+// second pass over them took 8 us a step of the field kernel.
 // ---------------------------------------------------------------------------
 #define DEPP_THREADS 256
 #define DEPP_WARPS 8
 #define DEPP_MINB 3  // CTAs an SM (80 registers a thread): 7% faster than 4 at 64 registers
 #define DEPP_SUB 2304  // records a sub-chunk: a 2^20-particle run has one sub-chunk a CTA
 #define DEPP_PART 512
-#define DEPP_RED_THREADS 1024
-#define DEPP_RED_NODES 8
 
 struct DepPlan {
     int G;            // CTAs
-    long long *rows;  // [G][Ng] per-CTA node sums over its window
-    int2 *hdr;        // [G] (first node, node count) of every row
+    long long *acc;   // [Ng] node sums, zero before
     float fixed;      // cost of the compressed form's fixed steps (depp_compress_pays)
 };
 // node pairs of the persistent deposit: each lane owns P pairs of nodes (64 P
@@ -832,8 +826,9 @@ __device__ __forceinline__ void depp_sweep_pairs(const DepSrc<float> &S, int n, 
 // (particle, node) pair, 256 a particle for whole-grid windows; here a particle costs the
 // Chebyshev values and 28 to 48 multiply-adds (a few hundred in the matrix form) whatever the
 // window, and is bound by instruction issue and load latency.  Measured (event-free launch
-// times): 2^20 particles, 256 nodes, widths near 14 43.2 -> 16.3 us; 4,000,037 particles, 4096
-// nodes, widths log-uniform in [5, 5e3] 2389 -> 298 us.
+// times): 2^20 particles, 256 nodes, widths near 14 43.2 -> 12.8 us (16.3 before the register
+// forms' proxies were unrolled); 4,000,037 particles, 4096 nodes, widths log-uniform in [5, 5e3]
+// 2389 -> 306 us.
 // ---------------------------------------------------------------------------
 #define PXY_STAGE 16  // particles a warp stages at a time
 
@@ -886,6 +881,7 @@ __device__ __forceinline__ void depp_moments_reg(const DepSrc<float> &S, int64_t
         }
 #pragma unroll
         for (int q = 0; q < QB; ++q) {
+            if (b0 - tid + q * DEPP_THREADS >= n) break;  // the CTA has no particle left
             const float x = pxy_x(B, ru[q]), x2 = x + x;
             float tp[PM];
             tp[0] = rw[q];
@@ -1055,10 +1051,9 @@ __device__ __forceinline__ void depp_moments_mm(const DepSrc<float> &S, int64_t 
 }
 
 // moments -> proxies -> node window: flush(r, a) receives the sum at window node r.
-// normed: the proxies carry their width's normalisation (the particles' weights did not).
 // mem: at least 2 P Q + 2 P + Q floats; part: DEPP_WARPS DEPP_PART floats
 template <typename F>
-__device__ __forceinline__ void depp_proxies(const DepSrc<float> &S, const PxyBox &B, bool normed, int g_lo, int R,
+__device__ __forceinline__ void depp_proxies(const DepSrc<float> &S, const PxyBox &B, int g_lo, int R,
                                              const float *M, float *mem, float *part, F &&flush)
 {
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -1068,10 +1063,10 @@ __device__ __forceinline__ void depp_proxies(const DepSrc<float> &S, const PxyBo
     // sine and cosine of half the proxies' angles from the box's middle, and exponent factors -2 kappa_b log2 e (the Chebyshev points are
     // the matrices' second rows times D / 2)
     if (tid < P)
-        sincospif((P > 1 ? cp[P + tid] * (0.5f * (float)P) : 0.f) * (B.hw * (1.f / 4294967296.f)), &sd[tid], &cd[tid]);
+        sincospif(cp[P + tid] * (0.5f * (float)P) * (B.hw * (1.f / 4294967296.f)), &sd[tid], &cd[tid]);
     if (tid >= 64 && tid < 64 + Q) {
         const int b = tid - 64;
-        k2[b] = (float)(-2.0 * KDE_LOG2E) * (Q > 1 ? pxy_kappa(B, cq[Q + b] * (0.5f * (float)Q)) : B.kc);
+        k2[b] = (float)(-2.0 * KDE_LOG2E) * pxy_kappa(B, cq[Q + b] * (0.5f * (float)Q));
     }
     __syncthreads();  // also: the moments are written
     for (int i = tid; i < PQ; i += DEPP_THREADS) {
@@ -1085,7 +1080,6 @@ __device__ __forceinline__ void depp_proxies(const DepSrc<float> &S, const PxyBo
         const int a = i / Q, b = i - a * Q;
         float s = 0.f;
         for (int q = 0; q < Q; ++q) s = fmaf(cq[q * Q + b], U[a * Q + q], s);
-        if (normed) s *= S.kappa ? kde_norm_tab(S.ntab, k2[b] * (float)(-0.5 * KDE_LN2)) : S.norm_u;
         W[i] = s;
     }
     __syncthreads();
@@ -1135,6 +1129,87 @@ __device__ __forceinline__ void depp_proxies(const DepSrc<float> &S, const PxyBo
     }
 }
 
+// the same for the degrees of the register forms, unrolled (the proxies carry the widths'
+// norms); mem: 2 PM QM + 2 PM + QM + PM PM + QM QM floats
+template <int PM, int QM, typename F>
+__device__ __forceinline__ void depp_proxies_reg(const DepSrc<float> &S, const PxyBox &B, int g_lo, int R, const float *M,
+                                                 const float *tabs, float *mem, float *part, F &&flush)
+{
+    constexpr int PQ = PM * QM;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, Ng = S.Ng;
+    const float *cp = tabs, *cq = tabs + PM * PM;
+    float *U = mem, *W = U + PQ + (PQ & 1), *k2 = W + PQ, *nk = k2 + QM;
+    float2 *sc = (float2 *)(nk + QM + (PQ & 1));  // an even number of floats from mem
+    static_assert((PQ + (PQ & 1) + PQ + 2 * QM + (PQ & 1)) % 2 == 0, "float2 alignment");
+    if (tid < PM) {
+        const float x = cp[PM + tid] * (0.5f * (float)PM);
+        float sn, cs;
+        sincospif(x * (B.hw * (1.f / 4294967296.f)), &sn, &cs);
+        sc[tid] = make_float2(sn, cs);
+    }
+    if (tid >= 32 && tid < 32 + QM) {
+        const int b = tid - 32;
+        const float k = QM > 1 ? pxy_lin_kappa(B.kc, B.kh, cq[QM + b], QM) : B.kc;
+        k2[b] = (float)(-2.0 * KDE_LOG2E) * k;
+        if (!S.kappa) nk[b] = S.norm_u;
+        else if (QM > 1 && S.krange) nk[b] = __uint_as_float(S.krange[(QM == 7 ? PXY_NORM7 : PXY_NORM6) + b]);
+        else nk[b] = kde_norm_tab(S.ntab, k);
+    }
+    __syncthreads();  // also: the moments are written
+    if (tid < PQ) {
+        const int a = tid / QM, q = tid % QM;
+        float s = 0.f;
+#pragma unroll
+        for (int p = 0; p < PM; ++p) s = fmaf(cp[p * PM + a], M[p * QM + q], s);
+        U[tid] = s;
+    }
+    __syncthreads();
+    if (tid < PQ) {
+        const int a = tid / QM, b = tid % QM;
+        float s = 0.f;
+#pragma unroll
+        for (int q = 0; q < QM; ++q) s = fmaf(cq[q * QM + b], U[a * QM + q], s);
+        W[tid] = s * nk[b];
+    }
+    __syncthreads();
+    float kk[QM];
+#pragma unroll
+    for (int b = 0; b < QM; ++b) kk[b] = k2[b];
+    // a thread takes a node and every SL-th proxy position
+    const int ng = (R + 31) >> 5;
+    const int SL = ng >= DEPP_WARPS ? 1 : DEPP_WARPS / ng;
+    auto node = [&](int r, int a0) -> float {
+        int g = g_lo + r;
+        g = g < 0 ? g + Ng : (g >= Ng ? g - Ng : g);
+        uint32_t nc;
+        float nf, sn, cn, acc = 0.f;
+        pxy_node(S.grid, g, nc, nf);
+        pxy_sincos(nc, nf, B.mid, 0.f, sn, cn);
+#pragma unroll 1
+        for (int a = a0; a < PM; a += SL) {
+            const float2 p = sc[a];
+            const float sa = fmaf(sn, p.y, -cn * p.x), s2 = sa * sa;
+            const float *w = W + a * QM;
+#pragma unroll
+            for (int b = 0; b < QM; ++b) acc = fmaf(kde_ex2(s2 * kk[b]), w[b], acc);
+        }
+        return acc;
+    };
+    if (SL == 1) {
+#pragma unroll 1
+        for (int r = tid; r < R; r += DEPP_THREADS) flush(r, node(r, 0));
+        return;
+    }
+    const int gi = warp % ng, sl = warp / ng, r = gi * 32 + lane;
+    if (sl < SL) part[sl * DEPP_PART + r] = r < R ? node(r, sl) : 0.f;
+    __syncthreads();
+    for (int q = tid; q < R; q += DEPP_THREADS) {
+        float a = 0.f;
+        for (int k = 0; k < SL; ++k) a += part[k * DEPP_PART + q];
+        flush(q, a);
+    }
+}
+
 // whether the compressed form costs less than the direct sweep: instructions of a lane,
 // direct about 3.2 a (particle, node) pair and 48 a particle; compressed 55 a particle plus
 // its Chebyshev values and moments (shared by the lanes of a warp), then 16 a (node, proxy
@@ -1151,54 +1226,6 @@ __device__ __forceinline__ bool depp_compress_pays(const PxyBox &B, int n, int R
     const float direct = fn * (3.2f * fR + 48.f);
     const float comp = fn * (55.f + 3.f * (P + Q) + 1.6f * PQ) + fR * P * (16.f + 3.f * Q) + PQ * (P + Q) * 4.f + fixed;
     return comp < direct;
-}
-
-// out[g] = 2^-es times the sum over the rows whose window covers node g of that row's entry;
-// CTA b takes nodes [8 b, 8 b + 8), eight lanes a row (64 bytes), the CTA's 128 row slots rows
-// s, s + 128, ...  es: from the host's bound, or from the device's largest weight
-__global__ void __launch_bounds__(DEPP_RED_THREADS) deposit_rows_kernel(const long long *__restrict__ rows,
-                                                                       const int2 *__restrict__ hdr, int G, int Ng,
-                                                                       double bound, const unsigned int *wmax_bits,
-                                                                       double wscale, float *out)
-{
-    __shared__ long long wsum[DEPP_RED_THREADS / 32][DEPP_RED_NODES];
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    constexpr int NW = DEPP_RED_THREADS / DEPP_RED_NODES;
-    const int slot = threadIdx.x / DEPP_RED_NODES;
-    const int g = blockIdx.x * DEPP_RED_NODES + (lane & (DEPP_RED_NODES - 1));
-    kde_pdl_wait();
-    kde_pdl_trigger();
-    long long sum = 0;
-    if (g < Ng) {
-        // rows in batches of 4 a slot, every load of a batch issued before any is used
-        for (int k0 = slot; k0 < G; k0 += 4 * NW) {
-            long long v[4];
-#pragma unroll
-            for (int q = 0; q < 4; ++q) {
-                const int k = k0 + q * NW;
-                v[q] = 0;
-                if (k < G) {
-                    const int2 h = hdr[k];
-                    int r = g - h.x;
-                    r = r < 0 ? r + Ng : (r >= Ng ? r - Ng : r);
-                    if (r < h.y) v[q] = rows[(size_t)k * Ng + r];
-                }
-            }
-#pragma unroll
-            for (int q = 0; q < 4; ++q) sum += v[q];
-        }
-    }
-#pragma unroll
-    for (int o = DEPP_RED_NODES; o < 32; o <<= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
-    if (lane < DEPP_RED_NODES) wsum[warp][lane] = sum;
-    __syncthreads();
-    if (threadIdx.x < DEPP_RED_NODES && g < Ng) {
-        long long t = 0;
-#pragma unroll
-        for (int w = 0; w < DEPP_RED_THREADS / 32; ++w) t += wsum[w][lane];
-        const double b = wmax_bits ? wscale * (double)__uint_as_float(*wmax_bits) : bound;
-        out[g] = (float)((double)t / kde_acc_scale(b));
-    }
 }
 
 // COMP: with the compressed form, chosen per CTA; without it where no CTA would take it
@@ -1294,7 +1321,15 @@ __global__ void __launch_bounds__(DEPP_THREADS, DEPP_MINB) deposit_persist_kerne
     const int P = (4 * n256 == n64 && (n256 >= DEPP_WARPS || n256 * 256 <= DEPP_PART))   ? 4
                   : (2 * n128 == n64 && (n128 >= DEPP_WARPS || n128 * 128 <= DEPP_PART)) ? 2
                                                                                           : 1;
-    long long *row = Pl.rows + (size_t)c * Ng;
+    // node sums of a sub-chunk into the grid's int64 sums: reductions without a return value,
+    // exact, so the result does not depend on their order
+    auto flush = [&](int r, float a) {
+        int g = g_lo + r;
+        g = g < 0 ? g + Ng : (g >= Ng ? g - Ng : g);
+        // x 2^es in integer arithmetic; the FP64 product only for extreme bounds
+        const long long v = (es >= -100 && es <= 100) ? fix_pow2(a, es) : __double2ll_rn(ldexp((double)a, es));
+        if (v) atomicAdd((unsigned long long *)&Pl.acc[g], (unsigned long long)v);
+    };
     if constexpr (COMP) {
     if (c_last >= c_first) {
         // the default cut: compressed where that is less work (a cut the caller has set keeps
@@ -1305,30 +1340,33 @@ __global__ void __launch_bounds__(DEPP_THREADS, DEPP_MINB) deposit_persist_kerne
         const int n = (int)(i1 - i0);
         if (depp_compress_pays(B, n, R, Pl.fixed)) {
             __shared__ float M[PXY_MAXP * PXY_MAXQ];
-            bool normed = true;
-            if (B.Q == 1) {
-                if (B.P <= 8) {
-                    B.P = 8;
-                    depp_moments_reg<8, 1, false>(S, i0, n, B, part, M);
-                } else {
-                    B.P = 16;
-                    depp_moments_reg<16, 1, false>(S, i0, n, B, part, M);
-                }
-            } else if (B.lin && B.P <= 6) {
-                B.P = B.Q = 7;
-                depp_moments_reg<7, 7, true>(S, i0, n, B, part, M);
-            } else if (B.lin && B.P <= 8) {
-                B.P = 8;
-                depp_moments_reg<8, 6, false>(S, i0, n, B, part, M);
-            } else {
-                normed = false;
-                depp_moments_mm(S, i0, i1, B, (float *)rec + warp * (DEPP_SUB * 4 / DEPP_WARPS), part, M);
-            }
-            auto flush = [&](int r, float a) {
-                row[r] = (es >= -100 && es <= 100) ? fix_pow2(a, es) : __double2ll_rn(ldexp((double)a, es));
+            // the register forms' interpolation matrices, beside the records' space
+            float *tabs = (float *)rec, *mem = tabs + PXY_MAXP * PXY_MAXP + 64;
+            auto load_tabs = [&](int P, int Q) {
+                const float *cp = S.pxt + pxy_tab_off(P), *cq = S.pxt + pxy_tab_off(Q);
+                for (int i = tid; i < P * P; i += DEPP_THREADS) tabs[i] = cp[i];
+                if (tid < Q * Q) tabs[P * P + tid] = cq[tid];
             };
-            depp_proxies(S, B, normed, g_lo, R, M, (float *)rec, part, flush);
-            if (tid == 0) Pl.hdr[c] = make_int2(g_lo, R);
+            if (B.Q == 1 && B.P <= 8) {
+                load_tabs(8, 1);
+                depp_moments_reg<8, 1, false>(S, i0, n, B, part, M);
+                depp_proxies_reg<8, 1>(S, B, g_lo, R, M, tabs, mem, part, flush);
+            } else if (B.Q == 1) {
+                load_tabs(16, 1);
+                depp_moments_reg<16, 1, false>(S, i0, n, B, part, M);
+                depp_proxies_reg<16, 1>(S, B, g_lo, R, M, tabs, mem, part, flush);
+            } else if (B.lin && B.P <= 6) {
+                load_tabs(7, 7);
+                depp_moments_reg<7, 7, true>(S, i0, n, B, part, M);
+                depp_proxies_reg<7, 7>(S, B, g_lo, R, M, tabs, mem, part, flush);
+            } else if (B.lin && B.P <= 8) {
+                load_tabs(8, 6);
+                depp_moments_reg<8, 6, false>(S, i0, n, B, part, M);
+                depp_proxies_reg<8, 6>(S, B, g_lo, R, M, tabs, mem, part, flush);
+            } else {
+                depp_moments_mm(S, i0, i1, B, (float *)rec + warp * (DEPP_SUB * 4 / DEPP_WARPS), part, M);
+                depp_proxies(S, B, g_lo, R, M, (float *)rec, part, flush);
+            }
             return;
         }
     }
@@ -1400,11 +1438,6 @@ __global__ void __launch_bounds__(DEPP_THREADS, DEPP_MINB) deposit_persist_kerne
             ((float *)recW)[n] = 0.f;
         }
         __syncthreads();
-        auto flush = [&](int r, float a) {
-            // x 2^es in integer arithmetic; the FP64 product only for extreme bounds
-            const long long v = (es >= -100 && es <= 100) ? fix_pow2(a, es) : __double2ll_rn(ldexp((double)a, es));
-            row[r] = first ? v : __ldcg(&row[r]) + v;
-        };
         if (pairs) {
             if (R <= 8) depp_sweep_pairs<8, 1>(S, n, g_lo, R, cosf, recAB, recW, part, flush);
             else if (R <= 16) depp_sweep_pairs<16, 1>(S, n, g_lo, R, cosf, recAB, recW, part, flush);
@@ -1415,7 +1448,6 @@ __global__ void __launch_bounds__(DEPP_THREADS, DEPP_MINB) deposit_persist_kerne
         else if (P == 2) depp_sweep<2>(S, n, g_lo, R, cosf, rec, part, flush);
         else depp_sweep<1>(S, n, g_lo, R, cosf, rec, part, flush);
     }
-    if (tid == 0) Pl.hdr[c] = make_int2(g_lo, R);
 }
 
 // acc -> real values
@@ -1455,36 +1487,63 @@ __global__ void wmax_kernel(const T *w, int64_t N, unsigned int *wmax_bits, unsi
 }
 
 // ---------------------------------------------------------------------------
-// workspace of the persistent FP32 deposit for N particles on Ng nodes: the CTAs'
-// rows and their headers
-static kde_status depp_plan(kde_ctx *ctx, int64_t N, int Ng, bool flat, DepPlan &Pl)
+__global__ void krange_norms_kernel(unsigned int *krange, const float *pxt)
 {
-    const int64_t gmax = (int64_t)DEPP_MINB * ctx->sm_count;
-    // unsorted particles sweep the whole grid: shorter shares, so that small calls reach more SMs
-    const int64_t gn = flat ? (N + 63) / 64 : (N + 255) / 256;
-    Pl.G = (int)(gn < gmax ? gn : gmax);
-    const size_t rows_b = (size_t)Pl.G * Ng * 8;
-    unsigned char *w = (unsigned char *)kde_ws(ctx, WS_DEP_ROWS, rows_b + (size_t)Pl.G * 8);
-    if (!w) return KDE_ENOMEM;
-    Pl.rows = (long long *)w;
-    Pl.hdr = (int2 *)(w + rows_b);
-    Pl.fixed = Pl.G <= ctx->sm_count ? 3.0e5f : 6.0e4f;
+    const float kmax = __uint_as_float(krange[0]), kmin = __uint_as_float(krange[1]);
+    const float kc = 0.5f * (kmin + kmax), kh = 0.5f * (kmax - kmin);
+    const int i = threadIdx.x, Q = i < 16 ? 7 : 6, b = i & 15;
+    if (b >= Q) return;
+    const float k = pxy_lin_kappa(kc, kh, pxt[pxy_tab_off(Q) + Q + b], Q);
+    krange[(Q == 7 ? PXY_NORM7 : PXY_NORM6) + b] = __float_as_uint((float)f64_norm((double)k));
+}
+
+kde_status kde_krange_norms(kde_ctx *ctx, unsigned int *krange)
+{
+    krange_norms_kernel<<<1, 32, 0, ctx->stream>>>(krange, ctx->pxy_tab);
+    KDE_LAUNCHED(ctx, "krange_norms_kernel");
     return KDE_OK;
 }
 
-kde_status kde_deposit_reserve(kde_ctx *ctx, int64_t N, int Ng)
+// grids of int64 node sums: two for the PIC step's deposits (see DepSums), and one for
+// kde_deposit, which every call leaves zero
+static long long *depp_sums(kde_ctx *ctx)
 {
-    DepPlan Pl{};
-    return depp_plan(ctx, N, Ng, true, Pl);
+    if (ctx->ws_bytes[WS_DEP_SUMS] == 0) ctx->sums_zero = false;
+    return (long long *)kde_ws(ctx, WS_DEP_SUMS, (size_t)3 * KDE_MAX_NG * 8);
+}
+
+// out = sums 2^-es, and the sums back to zero
+__global__ void __launch_bounds__(256) sums_to_real_kernel(long long *acc, int Ng, double bound, const unsigned int *wmax_bits,
+                                                           double wscale, float *out)
+{
+    const int g = blockIdx.x * 256 + threadIdx.x;
+    kde_pdl_wait();
+    kde_pdl_trigger();
+    if (g >= Ng) return;
+    const double b = wmax_bits ? wscale * (double)__uint_as_float(*wmax_bits) : bound;
+    const long long a = __ldcg(&acc[g]);
+    acc[g] = 0;
+    out[g] = (float)((double)a / kde_acc_scale(b));
+}
+
+kde_status kde_deposit_reserve(kde_ctx *ctx) { return depp_sums(ctx) ? KDE_OK : KDE_ENOMEM; }
+
+kde_status kde_deposit_sums_reset(kde_ctx *ctx)
+{
+    long long *s = depp_sums(ctx);
+    if (!s) return KDE_ENOMEM;
+    ctx->sums_flip = false;
+    KDE_CUDA(ctx, cudaMemsetAsync(s, 0, (size_t)2 * KDE_MAX_NG * 8, ctx->stream), "node sums memset");
+    return KDE_OK;
 }
 
 template <typename T>
 static kde_status deposit_sorted_impl(kde_ctx *ctx, const uint32_t *u, const T *kappa, T kappa_u, const T *norm,
                                       T norm_u, const T *w, T w_u, int64_t N, int Ng, double coef, long long *acc,
-                                      double bound, const unsigned int *wmax_bits, double norm_bound, DepRows *rows_out,
+                                      double bound, const unsigned int *wmax_bits, double norm_bound,
                                       float xcut = 0.f, const unsigned int *krange = nullptr, int nbins = 0)
 {
-    // the persistent FP32 kernel writes rows; the FP64 one adds into zeroed accumulators
+    // (the FP32 callers zero their sums)
     if (sizeof(T) == 8)
         KDE_CUDA(ctx, cudaMemsetAsync(acc, 0, (size_t)2 * Ng * sizeof(long long), ctx->stream), "acc memset");
     if (N == 0) return KDE_OK;
@@ -1524,7 +1583,12 @@ static kde_status deposit_sorted_impl(kde_ctx *ctx, const uint32_t *u, const T *
     S.nbins = nbins;
     if constexpr (sizeof(T) == 4) {
         DepPlan Pl{};
-        KDE_TRY(depp_plan(ctx, N, Ng, nbins < 0, Pl));
+        // unsorted particles sweep the whole grid: shorter shares, so that small calls reach more SMs
+        const int64_t gmax = (int64_t)DEPP_MINB * ctx->sm_count;
+        const int64_t gn = nbins < 0 ? (N + 63) / 64 : (N + 255) / 256;
+        Pl.G = (int)(gn < gmax ? gn : gmax);
+        Pl.acc = acc;
+        Pl.fixed = Pl.G <= ctx->sm_count ? 3.0e5f : 6.0e4f;
         {
             KdeProfScope _ps(ctx, PROF_DEPOSIT);
             // the compressed form is for the default cut (one the caller has set keeps the sweep
@@ -1538,11 +1602,6 @@ static kde_status deposit_sorted_impl(kde_ctx *ctx, const uint32_t *u, const T *
                      "deposit_persist_kernel");
         }
         KDE_LAUNCHED(ctx, "deposit_persist_kernel");
-        // the caller sums the rows (the PIC step's field kernel, deposit_rows_f32)
-        rows_out->rows = Pl.rows;
-        rows_out->hdr = Pl.hdr;
-        rows_out->G = Pl.G;
-        return KDE_OK;
     } else {
         // four chunks an SM where that leaves them 16 particles or more, 256 at most
         const int64_t per = N / (4LL * (ctx->sm_count > 0 ? ctx->sm_count : 1)) + 1;
@@ -1562,16 +1621,21 @@ kde_status kde_deposit_sorted_f64(kde_ctx *ctx, const uint32_t *u, const double 
                                   double norm_bound)
 {
     return deposit_sorted_impl<double>(ctx, u, kappa, kappa_u, norm, norm_u, w, w_u, N, Ng, coef, acc, bound, wmax_bits,
-                                       norm_bound, nullptr);
+                                       norm_bound);
 }
 
-kde_status kde_deposit_rows_f32(kde_ctx *ctx, const uint32_t *u, const float *kappa, float kappa_u, const float *norm,
-                                float norm_u, int64_t N, int Ng, double coef, float w_u, double bound, DepRows *out,
+kde_status kde_deposit_sums_f32(kde_ctx *ctx, const uint32_t *u, const float *kappa, float kappa_u, const float *norm,
+                                float norm_u, int64_t N, int Ng, double coef, float w_u, double bound, DepSums *out,
                                 float xcut, const unsigned int *krange)
 {
-    if (N < 1) return kde_fail(ctx, KDE_EINVAL, "deposit rows: need N >= 1");
-    return deposit_sorted_impl<float>(ctx, u, kappa, kappa_u, norm, norm_u, nullptr, w_u, N, Ng, coef, nullptr, bound,
-                                      nullptr, 0.0, out, xcut, krange);
+    if (N < 1) return kde_fail(ctx, KDE_EINVAL, "deposit sums: need N >= 1");
+    long long *s = depp_sums(ctx);
+    if (!s) return KDE_ENOMEM;
+    out->acc = s + (ctx->sums_flip ? KDE_MAX_NG : 0);
+    out->next = s + (ctx->sums_flip ? 0 : KDE_MAX_NG);
+    ctx->sums_flip = !ctx->sums_flip;
+    return deposit_sorted_impl<float>(ctx, u, kappa, kappa_u, norm, norm_u, nullptr, w_u, N, Ng, coef, out->acc, bound,
+                                      nullptr, 0.0, xcut, krange);
 }
 
 template <typename T>
@@ -1801,18 +1865,24 @@ static kde_status deposit_api_f32(kde_ctx *ctx, const uint32_t *u, const float *
     const double bound = (double)N * w_u * coef * norm_bound;
     unsigned int *wmax = nullptr;
     KDE_TRY(deposit_wmax<float>(ctx, weight, N, &wmax));
-    DepRows dr{};
+    // the sums are zero from the call before, unless it failed half-way; a captured call, whose
+    // replays may come after such a one, zeroes them itself
+    long long *acc = depp_sums(ctx);
+    if (!acc) return KDE_ENOMEM;
+    acc += 2 * KDE_MAX_NG;
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    cudaStreamIsCapturing(ctx->stream, &cap);
+    if (!ctx->sums_zero || cap != cudaStreamCaptureStatusNone)
+        KDE_CUDA(ctx, cudaMemsetAsync(acc, 0, (size_t)KDE_MAX_NG * 8, ctx->stream), "node sums memset");
+    ctx->sums_zero = false;
     KDE_TRY(deposit_sorted_impl<float>(ctx, us, ks, (float)kappa_u, nullptr, (float)norm_u, ws, (float)w_u, N, Ng, coef,
-                                       nullptr, bound, wmax, norm_bound, &dr, 0.f, nullptr, nbins == Ng ? 0 : nbins));
-    {
-        KdeProfScope _ps(ctx, PROF_DEPOSIT_ROWS);
-        KDE_CUDA(ctx,
-                 kde_launch(ctx, true, deposit_rows_kernel, dim3((Ng + DEPP_RED_NODES - 1) / DEPP_RED_NODES),
-                            dim3(DEPP_RED_THREADS), 0, dr.rows, dr.hdr, dr.G, Ng, bound, (const unsigned int *)wmax,
-                            (double)N * coef * norm_bound, rho_out),
-                 "deposit_rows_kernel");
-    }
-    KDE_LAUNCHED(ctx, "deposit_rows_kernel");
+                                       acc, bound, wmax, norm_bound, 0.f, nullptr, nbins == Ng ? 0 : nbins));
+    KDE_CUDA(ctx,
+             kde_launch(ctx, true, sums_to_real_kernel, dim3((Ng + 255) / 256), dim3(256), 0, acc, Ng, bound,
+                        (const unsigned int *)wmax, (double)N * coef * norm_bound, rho_out),
+             "sums_to_real_kernel");
+    KDE_LAUNCHED(ctx, "sums_to_real_kernel");
+    ctx->sums_zero = cap == cudaStreamCaptureStatusNone;
     return KDE_OK;
 }
 

@@ -246,7 +246,7 @@ __device__ __forceinline__ void gat_finish(const GatherArgs<float> &A, int64_t b
                 const bool ok = j < A.N;
                 vin[hh] = VIN ? vpre[h0 + hh] : (ok ? A.v_in[j] : 0.f);
                 kin[hh] = (ok && A.kappa_out) ? (A.kappa ? A.kappa[j] : A.kappa_u) : 0.f;
-                nin[hh] = (ok && A.norm_out) ? A.norm_in[j] : 0.f;
+                nin[hh] = (ok && A.norm_out && A.norm_in) ? A.norm_in[j] : 0.f;
                 idin[hh] = (ok && A.id_out) ? A.id_in[j] : 0u;
             }
 #pragma unroll
@@ -255,15 +255,15 @@ __device__ __forceinline__ void gat_finish(const GatherArgs<float> &A, int64_t b
                 const int64_t j = base + h * 32 + lane;
                 int key = -1;
                 if (j < A.N) {
-                    const float v = vin[hh] + A.kick_qm_dt * ea[h];
+                    const float v = fmaf(A.kick_qm_dt, ea[h], vin[hh]);
                     A.v_out[j] = v;
                     const uint32_t nu = advance_position(uu[h], v * A.dt_scale);
                     A.u_out[j] = nu;
                     if (A.kappa_out) {
-                        const float k = kin[hh];
-                        A.kappa_out[j] = (k > 0.f && k <= (float)KDE_KAPPA_MAX) ? k : (float)KDE_KAPPA_MAX;
+                        const float k = (kin[hh] > 0.f && kin[hh] <= (float)KDE_KAPPA_MAX) ? kin[hh] : (float)KDE_KAPPA_MAX;
+                        A.kappa_out[j] = k;
+                        if (A.norm_out) A.norm_out[j] = A.norm_in ? nin[hh] : kde_norm_tab(A.ntab, k);
                     }
-                    if (A.norm_out) A.norm_out[j] = nin[hh];
                     if (A.id_out) A.id_out[j] = idin[hh];
                     key = kde_cell(nu, Ng);
                 }
@@ -441,8 +441,8 @@ __global__ void __launch_bounds__(GAT2_WARPS * 32, MINB) gather2_kernel(GatherAr
 // warps, 128 particles each at a time).
 // Everything before kde_pdl_wait() -- the box, the proxies -- overlaps the field kernel.
 // Bound by instruction issue and fetch (a tile runs straight through its code) and latency.
-// Measured: 2^20 particles on 256 nodes, widths near 14, 38.6 us swept, 22.8 in tiles; a step of
-// 32 realisations of 2^14 to 2^20 particles 824 -> 590 us.
+// Measured: 2^20 particles on 256 nodes, widths near 14, 38.6 us swept, 22.8 in tiles and 14.5
+// with gatt_run's loop without bounds checks.
 // ---------------------------------------------------------------------------
 #define GATT_THREADS 256
 #define GATT_WARPS 8
@@ -547,24 +547,8 @@ __device__ __forceinline__ void gatt_coefs(const GatherArgs<float> &A, int g_lo,
 // the interpolant at four particles a lane (two packed pairs); TRI: the coefficients with
 // p / PM + q / QM < 1 alone
 template <int PM, int QM, bool TRI>
-__device__ __forceinline__ void gatt_eval(const GatherArgs<float> &A, const PxyBox &B, const float2 *C, int64_t base,
-                                          int lane, const uint32_t (&uu)[4], const float (&kap)[4], float (&ea)[4])
+__device__ __forceinline__ void gatt_eval(const float2 *C, const float (&xs)[4], const float (&ss)[4], float (&ea)[4])
 {
-    float xs[4], ss[4];
-#pragma unroll
-    for (int h = 0; h < 4; ++h) {
-        const int64_t j = base + h * 32 + lane;
-        xs[h] = pxy_x(B, uu[h]);
-        ss[h] = 0.f;
-        if (QM > 1) {
-            float k = kap[h];
-            if (!(k > 0.f && k <= (float)KDE_KAPPA_MAX)) {
-                if (j < A.N) kde_flag(A.status, KDE_DEV_KAPPA_RANGE, (unsigned)j);
-                k = (float)KDE_KAPPA_MAX;
-            }
-            ss[h] = (k - B.kc) * B.inv_kh;
-        }
-    }
     const kde_f2 one = kde_pk(1.f, 1.f), neg = kde_pk(-1.f, -1.f);
     kde_f2 x[2], x2[2], s[2], t0[2], t1[2], acc[2], tq[QM][2];
 #pragma unroll
@@ -607,6 +591,95 @@ __device__ __forceinline__ void gatt_eval(const GatherArgs<float> &A, const PxyB
     }
 #pragma unroll
     for (int h = 0; h < 2; ++h) kde_upk(acc[h], ea[2 * h], ea[2 * h + 1]);
+}
+
+// the places xs, ss of four particles a lane (base + 32 h + lane) in the box
+template <int QM>
+__device__ __forceinline__ void gatt_place(const GatherArgs<float> &A, const PxyBox &B, int64_t base, int lane,
+                                           const uint32_t (&uu)[4], const float (&kap)[4], float (&xs)[4], float (&ss)[4])
+{
+    bool ok = true;
+#pragma unroll
+    for (int h = 0; h < 4; ++h) {
+        xs[h] = pxy_x(B, uu[h]);
+        ss[h] = QM > 1 ? (kap[h] - B.kc) * B.inv_kh : 0.f;
+        ok = ok && kap[h] > 0.f && kap[h] <= (float)KDE_KAPPA_MAX;
+    }
+    if (QM > 1 && !ok) {
+#pragma unroll
+        for (int h = 0; h < 4; ++h) {
+            if (kap[h] > 0.f && kap[h] <= (float)KDE_KAPPA_MAX) continue;
+            const int64_t j = base + h * 32 + lane;
+            if (j < A.N) kde_flag(A.status, KDE_DEV_KAPPA_RANGE, (unsigned)j);
+            ss[h] = ((float)KDE_KAPPA_MAX - B.kc) * B.inv_kh;
+        }
+    }
+}
+
+// the steps of a run but the last of a call (positions and velocities written, counts added,
+// nothing else), for whole groups of 128 particles: pointers once a group, no bounds checks;
+// returns the first group left.  Half the instructions of the general loop.
+template <int PM, int QM, bool TRI>
+__device__ __forceinline__ int64_t gatt_run(const GatherArgs<float> &A, const PxyBox &B, const float2 *C, int64_t base,
+                                            int64_t t1, int lane, uint32_t (&uu)[4], float (&kap)[4], float (&vin)[4])
+{
+#pragma unroll 1
+    while (base + 128 <= t1) {
+        const int64_t next = base + GATT_UNIT;
+        uint32_t nu[4];
+        float nk[4], nv[4];
+        if (next + 128 <= t1) {  // the next group's loads
+            const uint32_t *pu = A.u + next + lane;
+            const float *pk = A.kappa + next + lane, *pv = A.v_in + next + lane;
+#pragma unroll
+            for (int h = 0; h < 4; ++h) {
+                nu[h] = pu[32 * h];
+                nk[h] = QM > 1 ? pk[32 * h] : 0.f;
+                nv[h] = pv[32 * h];
+            }
+        } else {
+#pragma unroll
+            for (int h = 0; h < 4; ++h) {
+                nu[h] = 0u;
+                nk[h] = nv[h] = 0.f;
+            }
+        }
+        float xs[4], ss[4], ea[4];
+        gatt_place<QM>(A, B, base, lane, uu, kap, xs, ss);
+        gatt_eval<PM, QM, TRI>(C, xs, ss, ea);
+        float *vo = A.v_out + base + lane;
+        uint32_t *uo = A.u_out + base + lane;
+        unsigned int *pc = A.counts + (base >> A.cnt_shift);  // the group lies in one sort tile
+        float d[4];
+        bool small = true;
+#pragma unroll
+        for (int h = 0; h < 4; ++h) {
+            const float v = fmaf(A.kick_qm_dt, ea[h], vin[h]);
+            vo[32 * h] = v;
+            d[h] = v * A.dt_scale;
+            small = small && fabsf(d[h]) < 2147483520.0f;
+        }
+        uint32_t un[4];
+        if (small) {
+#pragma unroll
+            for (int h = 0; h < 4; ++h) un[h] = uu[h] + (uint32_t)__float2int_rn(d[h]);
+        } else {
+#pragma unroll
+            for (int h = 0; h < 4; ++h) un[h] = advance_position(uu[h], d[h]);
+        }
+#pragma unroll
+        for (int h = 0; h < 4; ++h) {
+            uo[32 * h] = un[h];
+            const unsigned int key = __umulhi(un[h], (unsigned int)A.Ng);
+            const unsigned int peers = __match_any_sync(0xffffffffu, key);
+            if (lane == 31 - __clz(peers)) atomicAdd(&pc[key * (unsigned int)A.cnt_nblk], (unsigned int)__popc(peers));
+            uu[h] = nu[h];
+            kap[h] = nk[h];
+            vin[h] = nv[h];
+        }
+        base = next;
+    }
+    return base;
 }
 
 // the direct sweep of one warp's 128 particles: node tables SC and FF of the whole grid in
@@ -805,9 +878,13 @@ __global__ void __launch_bounds__(GATT_THREADS, 3) gather_tile_kernel(GatherArgs
         if (tid < P) pxy_pos(B, cp[P + tid] * (0.5f * (float)P), cd[tid], fr[tid]);
         if (tid >= 32 && tid < 32 + Q) {
             const int b = tid - 32;
-            const float k = Q > 1 ? pxy_kappa(B, cq[Q + b] * (0.5f * (float)Q)) : kmin;
+            const float k = Q > 1 ? pxy_lin_kappa(B.kc, B.kh, cq[Q + b], Q) : kmin;
             k2[b] = (float)(-2.0 * KDE_LOG2E) * k;
-            nk[b] = A.coef * (A.kappa ? kde_norm_tab(A.ntab, k) : A.norm_u);
+            float nm = A.norm_u;
+            if (A.kappa)
+                nm = Q > 1 && A.krange ? __uint_as_float(A.krange[(Q == 7 ? PXY_NORM7 : PXY_NORM6) + b])
+                                       : kde_norm_tab(A.ntab, k);
+            nk[b] = A.coef * nm;
         }
         __syncthreads();
         int g = g_lo + (tid < R ? tid : 0);
@@ -842,26 +919,31 @@ __global__ void __launch_bounds__(GATT_THREADS, 3) gather_tile_kernel(GatherArgs
         }
         __syncthreads();
     }
-#pragma unroll 1
-    for (int64_t base = t0 + warp * 128; base < t1; base += GATT_UNIT) {
-        uint32_t nu[4];
-        float nkap[4], nv[4];
-        load(base + GATT_UNIT < t1 ? base + GATT_UNIT : base, nu, nkap, nv);  // the next round's
-        float ea[4];
+    int64_t base = t0 + warp * 128;
+    if (A.u_out && !A.kappa_out && !A.id_out && A.counts) {
         switch (form) {
-        case 1: gatt_eval<8, 1, false>(A, B, C, base, lane, uu, kap, ea); break;
-        case 2: gatt_eval<16, 1, false>(A, B, C, base, lane, uu, kap, ea); break;
-        case 3: gatt_eval<7, 7, true>(A, B, C, base, lane, uu, kap, ea); break;
-        case 4: gatt_eval<8, 6, false>(A, B, C, base, lane, uu, kap, ea); break;
+        case 1: base = gatt_run<8, 1, false>(A, B, C, base, t1, lane, uu, kap, vin); break;
+        case 2: base = gatt_run<16, 1, false>(A, B, C, base, t1, lane, uu, kap, vin); break;
+        case 3: base = gatt_run<7, 7, true>(A, B, C, base, t1, lane, uu, kap, vin); break;
+        case 4: base = gatt_run<8, 6, false>(A, B, C, base, t1, lane, uu, kap, vin); break;
+        default: break;
+        }
+    }
+    // the rest: a call's last step, plain gathers, the last particles, the direct sweep
+#pragma unroll 1
+    for (; base < t1; base += GATT_UNIT) {
+        load(base, uu, kap, vin);
+        float xs[4], ss[4], ea[4];
+        if (form >= 3) gatt_place<2>(A, B, base, lane, uu, kap, xs, ss);
+        else if (form) gatt_place<1>(A, B, base, lane, uu, kap, xs, ss);
+        switch (form) {
+        case 1: gatt_eval<8, 1, false>(C, xs, ss, ea); break;
+        case 2: gatt_eval<16, 1, false>(C, xs, ss, ea); break;
+        case 3: gatt_eval<7, 7, true>(C, xs, ss, ea); break;
+        case 4: gatt_eval<8, 6, false>(C, xs, ss, ea); break;
         default: gatt_direct(A, SC, FF, cosf, base, lane, uu, kap, ea);
         }
         gat_finish<true>(A, base, lane, uu, ea, vin);
-#pragma unroll
-        for (int h = 0; h < 4; ++h) {
-            uu[h] = nu[h];
-            kap[h] = nkap[h];
-            vin[h] = nv[h];
-        }
     }
 }
 

@@ -112,9 +112,9 @@ static kde_status tune_cut(kde_ctx *ctx, const uint32_t *us, const float *ks, fl
     kde_status st = KDE_OK;
     // one candidate: deposit + field into E, and a gather of the reference field into g
     auto run = [&](int c, float *E, float *g) -> kde_status {
-        DepRows dr{};
-        KDE_TRY(kde_deposit_rows_f32(ctx, us, ks, kappa_u, ns, norm_u, N, Ng, coef, w_u, bound, &dr, kCutCand[c], krange));
-        KDE_TRY(kde_field_from_rows(ctx, dr.rows, dr.hdr, dr.G, Ng, L, 1.0 / kde_acc_scale(bound), charge, fd, E));
+        DepSums ds{};
+        KDE_TRY(kde_deposit_sums_f32(ctx, us, ks, kappa_u, ns, norm_u, N, Ng, coef, w_u, bound, &ds, kCutCand[c], krange));
+        KDE_TRY(kde_field_from_sums(ctx, ds, Ng, L, 1.0 / kde_acc_scale(bound), charge, fd, E));
         return kde_gather_sorted<float>(ctx, us, ks, kappa_u, ns, norm_u, N, Eref, Ng, KDE_TWO_PI / Ng, g, nullptr,
                                         nullptr, kCutCand[c], gat_range);
     };
@@ -207,6 +207,9 @@ static kde_status pic_run(kde_ctx *ctx, pic_state *st, int n_steps)
     // the width update (CV) shares the sort slots; size them for it up front and
     // fetch the pointers again after every update, since a slot may be regrown
     const size_t npad = (size_t)((N + 255) / 256) * 256;
+    // FP64 norms move with the particles; FP32 ones are a table lookup of the width where a
+    // kernel needs them at all, and the state's come back from there on the call's last step
+    const bool norms = per && sizeof(T) == 8;
     // two sets of sorted widths, norms and labels, used in turn: within a call the push
     // writes them back to the state only on the call's last step, and each step sorts
     // them from wherever the previous step left them
@@ -218,9 +221,9 @@ static kde_status pic_run(kde_ctx *ctx, pic_state *st, int n_steps)
         bool ok = us && vs;
         for (int b = 0; b < 2; ++b) {
             ks2[b] = per ? (T *)kde_ws(ctx, b ? WS_SORT_P1B : WS_SORT_P1, npad * sizeof(T)) : nullptr;
-            ns2[b] = per ? (T *)kde_ws(ctx, b ? WS_SORT_P2B : WS_SORT_P2, npad * sizeof(T)) : nullptr;
+            ns2[b] = norms ? (T *)kde_ws(ctx, b ? WS_SORT_P2B : WS_SORT_P2, npad * sizeof(T)) : nullptr;
             ids2[b] = st->id ? (uint32_t *)kde_ws(ctx, b ? WS_SORT_P3B : WS_SORT_P3, npad * 4) : nullptr;
-            ok = ok && (!per || (ks2[b] && ns2[b])) && (!st->id || ids2[b]);
+            ok = ok && (!per || ks2[b]) && (!norms || ns2[b]) && (!st->id || ids2[b]);
         }
         return ok;
     };
@@ -240,7 +243,7 @@ static kde_status pic_run(kde_ctx *ctx, pic_state *st, int n_steps)
     // FP32 particle-wise widths: their range, kept on the device beside them
     unsigned int *krange = nullptr;
     if (per && sizeof(T) == 4) {
-        krange = (unsigned int *)kde_ws(ctx, WS_PIC_RANGE, 64);
+        krange = (unsigned int *)kde_ws(ctx, WS_PIC_RANGE, 256);
         if (!krange) return KDE_ENOMEM;
         KDE_CUDA(ctx, kde_krange_reset(krange, ctx->stream), "width range memset");
     }
@@ -248,7 +251,9 @@ static kde_status pic_run(kde_ctx *ctx, pic_state *st, int n_steps)
         norm_from_kappa_kernel<T><<<(unsigned)((N + 255) / 256), 256, 0, ctx->stream>>>(
             (const T *)st->kappa, N, norm_arr, ctx->d_status, ctx->norm_tab, krange);
         KDE_LAUNCHED(ctx, "norm_from_kappa_kernel");
+        if (krange) KDE_TRY(kde_krange_norms(ctx, krange));
     }
+    if (sizeof(T) == 4 && n_steps > 0) KDE_TRY(kde_deposit_sums_reset(ctx));
     const double coef = KDE_TWO_PI / L;
     const double w_u = L / (double)N;
     // the FP32 gather + push adds the next step's sort counts; a step whose table was
@@ -257,7 +262,7 @@ static kde_status pic_run(kde_ctx *ctx, pic_state *st, int n_steps)
     // where the current widths, norms and labels are: the state's arrays, or one of the
     // two sorted sets
     const T *k_cur = per ? (const T *)st->kappa : nullptr;
-    const T *n_cur = per ? (const T *)norm_arr : nullptr;
+    const T *n_cur = norms ? (const T *)norm_arr : nullptr;
     const uint32_t *id_cur = st->id;
     for (int s = 0; s < n_steps; ++s) {
         const int64_t step = st->step;
@@ -273,7 +278,7 @@ static kde_status pic_run(kde_ctx *ctx, pic_state *st, int n_steps)
             KDE_TRY(kde_adapt_device(ctx, loo, N, L, ks_dev, 0.0, st->alpha, st->kappa_min, st->kappa_max, st->kappa,
                                      norm_arr, sizeof(T) == 8, krange));
             k_cur = (const T *)st->kappa;  // the new widths and norms are in the state's arrays
-            n_cur = (const T *)norm_arr;
+            n_cur = norms ? (const T *)norm_arr : nullptr;
             if (!fetch_ws()) return KDE_ENOMEM;
         }
         if (adsched) {
@@ -313,7 +318,7 @@ static kde_status pic_run(kde_ctx *ctx, pic_state *st, int n_steps)
         }
         // this step's sorted set: the one the current arrays are not in
         auto holds = [&](int b) {
-            return (per && (k_cur == ks2[b] || n_cur == ns2[b])) || (st->id && id_cur == ids2[b]);
+            return (per && k_cur == ks2[b]) || (norms && n_cur == ns2[b]) || (st->id && id_cur == ids2[b]);
         };
         const int wsel = holds(0) ? 1 : 0;
         T *ks = ks2[wsel], *ns = ns2[wsel];
@@ -322,10 +327,8 @@ static kde_status pic_run(kde_ctx *ctx, pic_state *st, int n_steps)
         SortPayload pl[4];
         int npl = 0;
         pl[npl++] = SortPayload{st->v, vs, (int)sizeof(T)};
-        if (per) {
-            pl[npl++] = SortPayload{k_cur, ks, (int)sizeof(T)};
-            pl[npl++] = SortPayload{n_cur, ns, (int)sizeof(T)};
-        }
+        if (per) pl[npl++] = SortPayload{k_cur, ks, (int)sizeof(T)};
+        if (norms) pl[npl++] = SortPayload{n_cur, ns, (int)sizeof(T)};
         if (st->id) pl[npl++] = SortPayload{id_cur, ids, 4};
         {
             KdeRange r_("kdepic sort by cell");
@@ -355,17 +358,16 @@ static kde_status pic_run(kde_ctx *ctx, pic_state *st, int n_steps)
                     }
                 }
             }
-            // FP32: per-CTA rows, summed inside the field kernel (no accumulator round trip)
-            DepRows dr{};
+            // FP32: int64 node sums, from which the field kernel works
+            DepSums ds{};
             {
                 KdeRange r_("kdepic deposit");
-                KDE_TRY(kde_deposit_rows_f32(ctx, us, ks, (float)st->kappa_uniform, ns, (float)norm_u, N, Ng, coef,
-                                             (float)w_u, bound, &dr, cut, krange));
+                KDE_TRY(kde_deposit_sums_f32(ctx, us, ks, (float)st->kappa_uniform, ns, (float)norm_u, N, Ng, coef,
+                                             (float)w_u, bound, &ds, cut, krange));
             }
             {
-                KdeRange r_("kdepic field (row sums + Poisson)");
-                KDE_TRY(kde_field_from_rows(ctx, dr.rows, dr.hdr, dr.G, Ng, L, 1.0 / kde_acc_scale(bound), st->charge,
-                                            fd, (float *)E));
+                KdeRange r_("kdepic field (Poisson)");
+                KDE_TRY(kde_field_from_sums(ctx, ds, Ng, L, 1.0 / kde_acc_scale(bound), st->charge, fd, (float *)E));
             }
         } else {
             {

@@ -119,6 +119,17 @@ __device__ __forceinline__ void pxy_box_width(PxyBox &B, float kmin, float kmax)
     }
 }
 
+// norms of the proxy widths of a narrow range, behind the range's two words: PXY_NORM7 + b for
+// Q = 7, PXY_NORM6 + b for Q = 6, in FP64 and rounded (kde_krange_norms).  The proxies' norms
+// are a factor on the whole density, so the table's 5e-7 would be the field's.
+#define PXY_NORM7 4
+#define PXY_NORM6 12
+// width of proxy b (of Q) of a narrow range, c = c[1][b] of the matrix of degree Q
+__device__ __forceinline__ float pxy_lin_kappa(float kc, float kh, float c, int Q)
+{
+    return fmaf(kh, c * (0.5f * (float)Q), kc);
+}
+
 // position in the box, [-1, 1]: the code difference is exact
 __device__ __forceinline__ float pxy_x(const PxyBox &B, uint32_t u) { return (float)(int32_t)(u - B.mid) * B.inv_hw; }
 __device__ __forceinline__ float pxy_s(const PxyBox &B, float kappa)

@@ -94,8 +94,8 @@ static int64_t request_ws_bytes(const kde_request &r)
     // (workspace slots grow by a quarter beyond the request, hence the margins)
     if (r.kind == KDE_REQ_CV)
         return N * (32 + 5 * (int64_t)r.n_cand) + (int64_t)r.n_cand * 8192 * 10 + (4 << 20);
-    // sort slots (two sets of widths and norms for PIC runs), and the persistent deposit's
-    // int64 rows (an upper bound: 640 rows of Ng entries)
+    // sort slots (two sets of widths and norms for PIC runs); grids and the sort's count tables
+    // by Ng; the gather's tables in the constant
     return N * 56 + Ng * (64 + 640 * 8) + (16 << 20);
 }
 
