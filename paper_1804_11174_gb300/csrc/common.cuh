@@ -96,6 +96,7 @@ enum WsSlot {
     WS_HOST_NORM,
     WS_HOST_ID,
     WS_HOST_HIST,  // energy, kappa* and ln p histories
+    WS_SP_PX,      // moments of the structure factor and their transforms
     WS_LTAB,       // table of the density series (leave-one-out densities)
     WS_GTAB,       // tables of the smoothed field (plain FP32 gather)
     WS_TUNE,       // truncation tuner: reference and candidate fields and their error sums

@@ -9,11 +9,12 @@
 //   sum_j K(theta_i - theta_j)     = (1/2pi) (n + 2 sum_{m>=1} A_m Re(e^{i m theta_i} conj(S_m)))
 // These are identities; modes are cut where A_m < 1e-17.  The cost is
 // O(N M) for S_m (M ~ sqrt(78 kappa_max)) instead of O(N^2) pairs per
-// candidate, and all candidates share one S_m.
+// candidate, and all candidates share one S_m; large samples are sorted into
+// intervals, whose Chebyshev moments give all S_m at once (spec_moments).
 //
-// Phases are exact: m theta_j = 2 pi (m u_j mod 2^32) / 2^32 in integer
-// arithmetic, then one FP32 sincospi for the first of every four consecutive
-// modes and a rotation by e^{i theta_j} for the next three (an ulp or two each).
+// Particle by particle, phases are exact: m theta_j = 2 pi (m u_j mod 2^32) / 2^32 in integer
+// arithmetic, then one FP32 sincospi for the first of every SP_Q consecutive
+// modes and a rotation by e^{i theta_j} for the next ones (an ulp or two each).
 // Sub-chunk sums run in FP32 and are
 // combined in FP64 in a fixed order; the CV combination and the leave-one-out
 // sums are FP64.  Particles may come in any order (no sort).
@@ -457,6 +458,200 @@ static kde_status spec_loo_from_S(kde_ctx *ctx, const uint32_t *u, int64_t N, do
     return spec_loo_table(ctx, u, nullptr, N, L, AS, sel, kmax, loo);
 }
 
+// ---------------------------------------------------------------------------
+// Structure factor of a large sample from moments.  Over an interval of half-width a = pi / C the
+// phase e^{i m theta} is its Chebyshev interpolant with SM_P points to 2 (m a / 2)^P / P!, below
+// 1e-10 for m a <= 3.08.  So the particles, sorted into C intervals, leave SM_P Chebyshev moments
+// an interval; SM_P discrete Fourier transforms over the intervals take those to every mode at
+// once, and a mode is the sum of its SM_P values with the interpolant's coefficients:
+//   S_m = e^{i m a} sum_k c_k(m) sum_b M_{b,k} e^{2 pi i m b / C}.
+// Bound by launches and the sort.  2^20 particles and 893 modes took 348 us particle by particle,
+// 2^18 took 91: a CV call over 64 candidates and 2^18 particles went from 182 to 130 us, a 50-step
+// PIC period with one at 2^20 from 2292 to 2018 us.  Moments are summed as integers (FP32 values of at most 2^13 with steps
+// of 2^-30, so the sum is exact and in no order), and from there on all is FP64: the intervals'
+// phases and coefficients are few, and their rounding would not average out.
+// ---------------------------------------------------------------------------
+#define SM_P 16
+#define SM_THREADS 128
+#define SM_MAXRANGE 8192
+#define SM_LGC_MAX 13
+#define SM_LGC_MIN 8
+#define SM_SPLIT 8  // blocks a transform: the modes m = r mod SM_SPLIT
+
+// blocks below R: moments of `range` sorted particles, interval by interval; the rest: the table
+// E[j] = e^{i pi j / C}, j < 2 C
+__global__ void __launch_bounds__(SM_THREADS)
+    spec_moments_kernel(const uint32_t *__restrict__ us, int64_t N, int range, int R, int lgC, unsigned long long *mom,
+                        double2 *E)
+{
+    extern __shared__ uint32_t u[];
+    __shared__ float part[SM_THREADS / 32][32];
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, shift = 32 - lgC;
+    if ((int)blockIdx.x >= R) {
+        const int j = ((int)blockIdx.x - R) * SM_THREADS + tid;
+        if (j < 2 << lgC) {
+            double sn, cs;
+            sincospi(ldexp((double)j, -lgC), &sn, &cs);
+            E[j] = make_double2(cs, sn);
+        }
+        return;
+    }
+    const int64_t i0 = (int64_t)blockIdx.x * range;
+    const int n = (int)(N - i0 < range ? N - i0 : range);
+    for (int k = tid; k < n; k += SM_THREADS) u[k] = us[i0 + k];
+    __syncthreads();
+    for (int s = 0; s < n;) {
+        const uint32_t bin = u[s] >> shift;
+        int lo = s, hi = n;  // the interval's end: first particle of a later one
+        while (hi - lo > 1) {
+            const int mid = (lo + hi) >> 1;
+            if (u[mid] >> shift == bin) lo = mid;
+            else hi = mid;
+        }
+        float v[32];
+#pragma unroll
+        for (int p = 0; p < 32; ++p) v[p] = 0.f;
+        for (int k = s + tid; k < hi; k += SM_THREADS) {
+            const float x = (float)(int32_t)((u[k] << lgC) ^ 0x80000000u) * (1.f / 2147483648.f), x2 = x + x;
+            float t0 = 1.f, t1 = x;
+#pragma unroll
+            for (int p = 0; p < SM_P; ++p) {
+                v[p] += t0;
+                const float t2 = fmaf(x2, t1, -t0);
+                t0 = t1;
+                t1 = t2;
+            }
+        }
+        part[warp][lane] = warp_transpose_sum32(v, lane);
+        __syncthreads();
+        if (tid < SM_P) {
+            float m = 0.f;
+#pragma unroll
+            for (int w = 0; w < SM_THREADS / 32; ++w) m += part[w][tid];
+            atomicAdd(mom + ((size_t)tid << lgC) + bin, (unsigned long long)__double2ll_rn((double)m * 1073741824.0));
+        }
+        __syncthreads();
+        s = hi;
+    }
+}
+
+// modes m = r mod SM_SPLIT of the transform of moment k (k = blockIdx.y, r = blockIdx.x): one
+// step of decimation in frequency takes the C intervals to L = C / SM_SPLIT, then radix 2
+__global__ void __launch_bounds__(SM_THREADS)
+    spec_fft_kernel(const long long *__restrict__ mom, const double2 *__restrict__ E, int lgC, double2 *F)
+{
+    extern __shared__ double2 buf[];  // two of L
+    const int C = 1 << lgC, L = C / SM_SPLIT, mask = 2 * C - 1, r = blockIdx.x, tid = threadIdx.x;
+    const long long *x = mom + ((size_t)blockIdx.y << lgC);
+    double2 w[SM_SPLIT];  // e^{2 pi i r j / SM_SPLIT}
+#pragma unroll
+    for (int j = 0; j < SM_SPLIT; ++j) w[j] = E[(r * j * (2 * C / SM_SPLIT)) & mask];
+    for (int n = tid; n < L; n += SM_THREADS) {
+        double yr = 0.0, yi = 0.0;
+#pragma unroll
+        for (int j = 0; j < SM_SPLIT; ++j) {
+            const double v = (double)x[n + j * L];
+            yr = fma(v, w[j].x, yr);
+            yi = fma(v, w[j].y, yi);
+        }
+        const double2 e = E[(2 * r * n) & mask];
+        buf[n] = make_double2((yr * e.x - yi * e.y) * 0x1p-30, (yr * e.y + yi * e.x) * 0x1p-30);
+    }
+    __syncthreads();
+    double2 *a = buf, *b = buf + L;
+    for (int h = L / 2, s = 1, ls = 0; h >= 1; h >>= 1, s <<= 1, ++ls) {
+        for (int t = tid; t < L / 2; t += SM_THREADS) {
+            const int q = t & (s - 1), p = t >> ls;
+            const double2 c = a[q + s * p], d = a[q + s * (p + h)], e = E[(p * SM_SPLIT * 2) << ls];
+            const double2 g = make_double2(c.x - d.x, c.y - d.y);
+            b[q + s * 2 * p] = make_double2(c.x + d.x, c.y + d.y);
+            b[q + s * (2 * p + 1)] = make_double2(g.x * e.x - g.y * e.y, g.x * e.y + g.y * e.x);
+        }
+        __syncthreads();
+        double2 *o = a;
+        a = b;
+        b = o;
+    }
+    for (int q = tid; q < L; q += SM_THREADS) F[((size_t)blockIdx.y << lgC) + SM_SPLIT * q + r] = a[q];
+}
+
+// a mode from its SM_P values, eight lanes a mode: lane p has the points +-x_p, which share the
+// cosine (even moments) and the sine (odd ones); modes above *mlim (when given) are skipped
+__global__ void __launch_bounds__(SM_THREADS)
+    spec_modes_kernel(const double2 *__restrict__ F, const double2 *__restrict__ E, int lgC, int M, const int *mlim, double2 *S)
+{
+    __shared__ double ct[4 * SM_P];  // cos(pi j / (2 SM_P))
+    if (threadIdx.x < 4 * SM_P) ct[threadIdx.x] = cospi((double)threadIdx.x / (2 * SM_P));
+    __syncthreads();
+    const int Me = mlim ? min(M, *mlim) : M;
+    const int m = 1 + (int)(blockIdx.x * SM_THREADS + threadIdx.x) / (SM_P / 2), p = threadIdx.x & (SM_P / 2 - 1);
+    const int mc = m <= Me ? m : 0;
+    double er = 0.5 * F[mc].x, ei = 0.5 * F[mc].y, odr = 0.0, odi = 0.0;
+#pragma unroll
+    for (int k = 1; k < SM_P; ++k) {
+        const double t = ct[(k * (2 * p + 1)) & (4 * SM_P - 1)];
+        const double2 f = F[((size_t)k << lgC) + mc];
+        if (k & 1) {
+            odr = fma(t, f.x, odr);
+            odi = fma(t, f.y, odi);
+        } else {
+            er = fma(t, f.x, er);
+            ei = fma(t, f.y, ei);
+        }
+    }
+    double sn, cs;
+    sincospi(ldexp((double)mc * ct[2 * p + 1], -lgC), &sn, &cs);
+    double gr = fma(cs, er, -sn * odi), gi = fma(cs, ei, sn * odr);
+#pragma unroll
+    for (int o = SM_P / 4; o; o >>= 1) {
+        gr += __shfl_xor_sync(0xffffffffu, gr, o);
+        gi += __shfl_xor_sync(0xffffffffu, gi, o);
+    }
+    if (p == 0 && m <= Me) {
+        const double2 e = E[m];
+        const double f = 4.0 / SM_P;  // both points of a pair, and the 2 of the coefficients
+        S[m - 1] = make_double2(f * (gr * e.x - gi * e.y), f * (gr * e.y + gi * e.x));
+    }
+}
+
+// the structure factor so, where it pays; *taken is false where the particles go one by one
+static kde_status spec_moments(kde_ctx *ctx, const uint32_t *u, int64_t N, int M, const int *mlim, double2 *S, bool *taken)
+{
+    *taken = false;
+    int lgC = SM_LGC_MIN;
+    while (lgC < SM_LGC_MAX && (double)(1 << lgC) * 3.08 < KDE_PI * (double)M) ++lgC;
+    const int C = 1 << lgC;
+    if ((double)C * 3.08 < KDE_PI * (double)M) return KDE_OK;
+    int64_t range = (N + 511) / 512;
+    range = range < 512 ? 512 : (range > SM_MAXRANGE ? SM_MAXRANGE : range);
+    const int64_t R = (N + range - 1) / range;
+    // The sort, the transforms and the tables grow with the intervals, the particles one by one
+    // with N M.  CV calls of 16 candidates, so against one by one: 2^20 particles and 62 modes
+    // 112 against 184 us, 400,003 and 153 94 against 122, 150,000 and 279 90 against 97, 65,536
+    // and 883 100 against 99, 32,768 and 1530 128 against 97.
+    if ((double)N * M < 1e7 + 6e4 * C || N < 16 * (int64_t)C || R > 1 << 20) return KDE_OK;
+    uint32_t *us = (uint32_t *)kde_ws(ctx, WS_SORT_U, (size_t)N * 4);
+    const size_t momb = (size_t)SM_P * 8 << SM_LGC_MAX, tabb = (size_t)sizeof(double2) * 2 << SM_LGC_MAX;
+    char *ws = (char *)kde_ws(ctx, WS_SP_PX, 3 * momb + tabb);
+    if (!us || !ws) return KDE_OK;  // no room for them: one by one
+    unsigned long long *mom = (unsigned long long *)ws;
+    double2 *F = (double2 *)(ws + momb), *E = (double2 *)(ws + 3 * momb);
+    KDE_TRY(kde_sort_by_bin(ctx, u, N, C, us, nullptr, 0, nullptr));
+    KDE_CUDA(ctx, cudaMemsetAsync(mom, 0, (size_t)SM_P * C * 8, ctx->stream), "moments memset");
+    KdeProfScope _ps(ctx, PROF_SPECTRAL);
+    spec_moments_kernel<<<(unsigned)(R + 2 * C / SM_THREADS), SM_THREADS, (size_t)range * 4, ctx->stream>>>(
+        us, N, (int)range, (int)R, lgC, mom, E);
+    KDE_LAUNCHED(ctx, "spec_moments_kernel");
+    spec_fft_kernel<<<dim3(SM_SPLIT, SM_P), SM_THREADS, (size_t)2 * (C / SM_SPLIT) * sizeof(double2), ctx->stream>>>(
+        (const long long *)mom, E, lgC, F);
+    KDE_LAUNCHED(ctx, "spec_fft_kernel");
+    spec_modes_kernel<<<(unsigned)((M * (SM_P / 2) + SM_THREADS - 1) / SM_THREADS), SM_THREADS, 0, ctx->stream>>>(
+        F, E, lgC, M, mlim, S);
+    KDE_LAUNCHED(ctx, "spec_modes_kernel");
+    *taken = true;
+    return KDE_OK;
+}
+
 // structure factor for modes 1..M (or up to *mlim) into S
 static kde_status spec_structure(kde_ctx *ctx, const uint32_t *u, int64_t N, int M, const int *mlim, double2 **S_out)
 {
@@ -466,11 +661,16 @@ static kde_status spec_structure(kde_ctx *ctx, const uint32_t *u, int64_t N, int
     int64_t chunk = 256;
     while (((N + chunk - 1) / chunk > 1024 || (N + chunk - 1) / chunk * M > (1 << 22)) && chunk < SP_MAXCHUNK)
         chunk *= 2;
+    double2 *S = (double2 *)kde_ws(ctx, WS_SP_S, (size_t)M * sizeof(double2));
+    if (!S) return KDE_ENOMEM;
+    *S_out = S;
+    bool taken = false;
+    KDE_TRY(spec_moments(ctx, u, N, M, mlim, S, &taken));
+    if (taken) return KDE_OK;
     const int nchunks = (int)((N + chunk - 1) / chunk);
     double2 *part = (double2 *)kde_ws(ctx, WS_SP_PART, (size_t)(nchunks + SPR_G) * M * sizeof(double2));
     double2 *gpart = part + (size_t)nchunks * M;  // the chunk groups' sums
-    double2 *S = (double2 *)kde_ws(ctx, WS_SP_S, (size_t)M * sizeof(double2));
-    if (!part || !S) return KDE_ENOMEM;
+    if (!part) return KDE_ENOMEM;
     static bool attr = false;
     if (!attr) {
         KDE_CUDA(ctx, cudaFuncSetAttribute(spec_sf_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -489,7 +689,6 @@ static kde_status spec_structure(kde_ctx *ctx, const uint32_t *u, int64_t N, int
     KDE_LAUNCHED(ctx, "spec_reduce_kernel");
     spec_reduce2_kernel<<<(M + 255) / 256, 256, 0, ctx->stream>>>(gpart, M, mlim, S);
     KDE_LAUNCHED(ctx, "spec_reduce2_kernel");
-    *S_out = S;
     return KDE_OK;
 }
 

@@ -303,3 +303,27 @@ def test_cv_scale_out_of_range_width_is_reported(ctx, kp):
         ctx.cv(to_dev_u(u), 4 * math.pi, [0.5, 1.0], kappa_rel=to_dev(kr))
     kr[7] = 50.0
     ctx.cv(to_dev_u(u), 4 * math.pi, [0.5, 1.0], kappa_rel=to_dev(kr))
+
+
+@pytest.mark.parametrize("N,kmax,where", [(150_001, 1e3, "mix"), (300_000, 1e4, "mix"), (262_144, 1e4, "spike"),
+                                          (400_003, 3e2, "two"), (1 << 20, 1e4, "mix")])
+def test_cv_structure_factor_from_moments(ctx, oracle, N, kmax, where):
+    # large samples take the structure factor from the Chebyshev moments of sorted intervals; all
+    # particles in one place and in two give intervals with one and with many blocks.  The
+    # curve is held to the Fourier form's 1e-8 of its maximum (interpolation 1e-10, FP32 phases
+    # random over the points), checked at a few candidates
+    L = 2 * math.pi
+    u = I.cv_sweep_load(N, N)
+    if where == "spike":
+        u[:] = np.uint32(0xFFFFFF00) + (u >> np.uint32(25))
+    elif where == "two":
+        u = np.where(u & 1, u >> np.uint32(12), np.uint32(1 << 31) - (u >> np.uint32(13))).astype(np.uint32)
+    x = I.from_fixed(u, L)
+    cand = I.log_candidates(1.0, kmax, 24)
+    cv, am, loo = ctx.cv(to_dev_u(u), L, cand, want_loo=True, spectral=True)
+    sel = np.array([0, 9, 17, 23])
+    ref = np.array([oracle.cv_fourier(x, L, cand[c])[0] for c in sel])
+    assert np.max(np.abs(cv[sel] - ref)) <= 1e-8 * np.max(np.abs(ref))
+    _, _, _, lref = oracle.cv_fourier(x, L, cand[am], want_loo=True)
+    idx = np.arange(0, N, 97)
+    np.testing.assert_allclose(loo.cpu().numpy()[idx], lref[idx], rtol=1e-5, atol=1e-7 * np.max(lref))
