@@ -2,17 +2,19 @@
 //
 //   rho_g = sum_i w_i (2 pi / L) norm(kappa_i) exp(-2 kappa_i sin^2((theta_g - theta_i)/2))
 //
-// Layout: particles are counting-sorted by cell.  One CTA takes a chunk of
-// DEP_CHUNK consecutive sorted particles, stages (beta sin, beta cos, w*norm)
-// of each in shared memory, and finds the node range its particles' truncated
-// kernels can reach (first/last cell +- the widest window).  Lanes own nodes
-// (node-owner formulation): a warp sweeps 32 consecutive nodes over a slice of
-// the chunk, so every particle value is a shared-memory broadcast and each
-// lane accumulates in a register without atomics.  Slices are combined in a
-// fixed order in shared memory.  Chunk partials are converted to int64 fixed
-// point (an exact power-of-two scale below the largest possible node value)
-// and added with integer atomics, so the grid sum is exact and independent of
-// the order in which chunks finish: results are bitwise reproducible.
+// Layout: particles are counting-sorted by cell (small plain calls keep their
+// order).  One CTA takes a range of consecutive particles and finds the node
+// range their truncated kernels can reach.  FP32 ranges whose positions and
+// widths span a small box are compressed into interpolation points with signed
+// weights (proxy.cuh); the others stage (beta sin, beta cos, w*norm) of each
+// particle in shared memory.  Lanes own nodes (node-owner formulation): a warp
+// sweeps 32 consecutive nodes over a slice of the points, so every point is a
+// shared-memory broadcast and each lane accumulates in a register without
+// atomics.  Slices are combined in a fixed order in shared memory.  A CTA's
+// sums are converted to int64 fixed point (an exact power-of-two scale below
+// the largest possible node value) and added with integer atomics, so the grid
+// sum is exact and independent of the order in which CTAs finish: results are
+// bitwise reproducible.
 #include "common.cuh"
 #include "fp64.cuh"
 #include "proxy.cuh"
@@ -395,7 +397,7 @@ __device__ __forceinline__ void dep2_nodes(const DepSrc<float> &S, int n, int g_
 }
 
 __device__ void deposit_chunk_body_x2(const DepSrc<float> &S, int64_t chunk, float4 *rsc, float2 *rwn, float *part,
-                                      int *red, bool allow_cos)
+                                      int *red)
 {
     const int64_t i0 = chunk * DEP_CHUNK;
     if (i0 >= S.N) return;
@@ -403,11 +405,11 @@ __device__ void deposit_chunk_body_x2(const DepSrc<float> &S, int64_t chunk, flo
     const int Ng = S.Ng;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     // every input of the thread's particles loaded at once (one global-load latency per
-    // chunk); the smallest width sets the window, the largest the form
+    // chunk); the smallest width sets the window
     constexpr int PER = DEP_CHUNK / DEP_THREADS;
     uint32_t ru[PER];
     float rk[PER], rn[PER], rw[PER];
-    float kmin = (float)KDE_KAPPA_MAX, kmax = 0.f;
+    float kmin = (float)KDE_KAPPA_MAX;
 #pragma unroll
     for (int p = 0; p < PER; ++p) {
         const int t = tid + p * DEP_THREADS;
@@ -422,20 +424,11 @@ __device__ void deposit_chunk_body_x2(const DepSrc<float> &S, int64_t chunk, flo
             k = (float)KDE_KAPPA_MAX;
         }
         rk[p] = k;
-        if (ok) {
-            kmin = fminf(kmin, k);
-            kmax = fmaxf(kmax, k);
-        }
+        if (ok) kmin = fminf(kmin, k);
     }
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        kmin = fminf(kmin, __shfl_xor_sync(0xffffffffu, kmin, o));
-        kmax = fmaxf(kmax, __shfl_xor_sync(0xffffffffu, kmax, o));
-    }
-    if (lane == 0) {
-        red[warp] = __float_as_int(kmin);
-        red[DEP_WARPS + warp] = __float_as_int(kmax);
-    }
+    for (int o = 16; o > 0; o >>= 1) kmin = fminf(kmin, __shfl_xor_sync(0xffffffffu, kmin, o));
+    if (lane == 0) red[warp] = __float_as_int(kmin);
     // the fixed-point scale 2^es, worked out by one thread: FP64 stays off the other threads
     __shared__ int s_es;
     if (tid == 0) {
@@ -451,13 +444,9 @@ __device__ void deposit_chunk_body_x2(const DepSrc<float> &S, int64_t chunk, flo
     __syncthreads();
     const int es = s_es;
 #pragma unroll
-    for (int k = 0; k < DEP_WARPS; ++k) {
-        kmin = fminf(kmin, __int_as_float(red[k]));
-        kmax = fmaxf(kmax, __int_as_float(red[DEP_WARPS + k]));
-    }
+    for (int k = 0; k < DEP_WARPS; ++k) kmin = fminf(kmin, __int_as_float(red[k]));
     // the window shrinks as the width grows: the smallest width's window covers all
     const int W = window_nodes_f(kmin, Ng, S.xcut);
-    const bool cosf = allow_cos && kmax <= KDE_COSFORM_KMAX;
     // the particle records
 #pragma unroll
     for (int p = 0; p < PER; ++p) {
@@ -473,17 +462,9 @@ __device__ void deposit_chunk_body_x2(const DepSrc<float> &S, int64_t chunk, flo
         const float wn = rw[p] * S.coef * nm;
         float sh, ch;
         kde_half_sincos(uu, sh, ch);
-        if (cosf) {
-            const float K = (float)KDE_LOG2E * k;
-            const float cx = (ch - sh) * (ch + sh), sx = 2.f * sh * ch;
-            rsc[t] = make_float4(K * cx, K * cx, K * sx, K * sx);
-            const float wk = wn * kde_ex2(-K);
-            rwn[t] = make_float2(wk, wk);
-        } else {
-            const float beta = sqrtf((float)(2.0 * KDE_LOG2E) * k);
-            rsc[t] = make_float4(beta * sh, beta * sh, beta * ch, beta * ch);
-            rwn[t] = make_float2(wn, wn);
-        }
+        const float beta = sqrtf((float)(2.0 * KDE_LOG2E) * k);
+        rsc[t] = make_float4(beta * sh, beta * sh, beta * ch, beta * ch);
+        rwn[t] = make_float2(wn, wn);
     }
     __syncthreads();
     const int c_first = kde_cell(S.u[i0], Ng), c_last = kde_cell(S.u[i0 + n - 1], Ng);
@@ -497,18 +478,9 @@ __device__ void deposit_chunk_body_x2(const DepSrc<float> &S, int64_t chunk, flo
     // groups compute no extra nodes and their partial sums fit the buffer
     const int n64 = (R + 63) >> 6, n128 = (R + 127) >> 7;
     if (2 * n128 == n64 && (n128 >= DEP_WARPS || n128 * 128 <= DEP2_PART))
-        dep2_nodes<2>(S, n, g_lo, R, cosf, es, rsc, rwn, part);
+        dep2_nodes<2>(S, n, g_lo, R, false, es, rsc, rwn, part);
     else
-        dep2_nodes<1>(S, n, g_lo, R, cosf, es, rsc, rwn, part);
-}
-
-__global__ void __launch_bounds__(DEP_THREADS) deposit_chunk_x2_kernel(DepSrc<float> S)
-{
-    __shared__ float4 rsc[DEP_CHUNK];
-    __shared__ float2 rwn[DEP_CHUNK];
-    __shared__ float part[DEP_WARPS * DEP2_PART];
-    __shared__ int red[2 * DEP_WARPS];
-    deposit_chunk_body_x2(S, blockIdx.x, rsc, rwn, part, red, true);
+        dep2_nodes<1>(S, n, g_lo, R, false, es, rsc, rwn, part);
 }
 
 // ---------------------------------------------------------------------------
@@ -1729,7 +1701,7 @@ __global__ void __launch_bounds__(DEP_THREADS)
     S.scale_exp = p.es;
     S.Ng = p.M;
     // the CV integral term keeps the half-angle form: its sums carry the CV's accuracy
-    deposit_chunk_body_x2(S, blockIdx.x, rsc, rwn, part, red, false);
+    deposit_chunk_body_x2(S, blockIdx.x, rsc, rwn, part, red);
 }
 
 // FP64 trapezoid sum of fhat^2 on each candidate's grid: f2[c] = (2 pi / M) sum_g fhat_g^2
