@@ -180,9 +180,8 @@ const void *kde_green_table(kde_ctx *ctx, int Ng, double L, bool fd, bool f64)
 
 // the width-normalisation table of kde_norm_tab: q(t) = I0e(e^t) sqrt(1 + 2 pi e^t) and
 // h dq/dt (central difference of step 1e-4 in t, error ~1e-9) at t = T0 + i h, in FP64
-__global__ void norm_tab_kernel(float2 *tab)
+__device__ void norm_tab_entry(float2 *tab, int i)
 {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= KDE_NTAB_N) return;
     const double t = KDE_NTAB_T0 + i / KDE_NTAB_INVH, d = 1e-4;
     auto q = [](double tt) {
@@ -192,21 +191,31 @@ __global__ void norm_tab_kernel(float2 *tab)
     tab[i] = make_float2((float)q(t), (float)((q(t + d) - q(t - d)) / (2.0 * d) / KDE_NTAB_INVH));
 }
 
-// the interpolation matrices of proxy.cuh: entry (p, a) of every degree D, in FP64
-__global__ void pxy_tab_kernel(float *tab)
+// the interpolation matrices of proxy.cuh: entry (p, a) of every degree D, in FP64; PXY_TAB_BLOCKS
+// blocks a degree
+#define PXY_TAB_BLOCKS 4
+__device__ void pxy_tab_block(float *tab, int block)
 {
-    const int D = blockIdx.x + 1;
+    const int D = block / PXY_TAB_BLOCKS + 1;
     float *c = tab + pxy_tab_off(D);
-    for (int i = threadIdx.x; i < D * D; i += blockDim.x) {
+    for (int i = (block % PXY_TAB_BLOCKS) * blockDim.x + threadIdx.x; i < D * D; i += PXY_TAB_BLOCKS * blockDim.x) {
         const int p = i / D, a = i - p * D;
         c[i] = (float)((p ? 2.0 : 1.0) / D * cospi((double)((p * (2 * a + 1)) % (4 * D)) / (2.0 * D)));
     }
 }
 
-__global__ void f64_tab_kernel(double *tab)
+// the context's constant tables, in one launch and one allocation (three of each took 0.25 ms
+// more a context)
+#define NTAB_BLOCKS ((KDE_NTAB_N + 255) / 256)
+#define F64_BLOCKS (F64_TAB / 256)
+__global__ void __launch_bounds__(256) ctx_tables_kernel(float2 *norm, double *f64, float *pxy)
 {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < F64_TAB) tab[i] = exp2((double)i / F64_TAB);
+    const int b = blockIdx.x;
+    if (b < NTAB_BLOCKS) norm_tab_entry(norm, b * 256 + threadIdx.x);
+    else if (b < NTAB_BLOCKS + F64_BLOCKS) {
+        const int i = (b - NTAB_BLOCKS) * 256 + threadIdx.x;
+        f64[i] = exp2((double)i / F64_TAB);
+    } else pxy_tab_block(pxy, b - NTAB_BLOCKS - F64_BLOCKS);
 }
 
 // ---------------------------------------------------------------------------
@@ -223,19 +232,14 @@ extern "C" kde_status kde_create(kde_ctx **out, int device, void *stream)
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&ctx->sm_count, cudaDevAttrMultiProcessorCount, device);
     if (e == cudaSuccess) e = cudaMalloc(&ctx->d_status, 4 * sizeof(unsigned int));
     if (e == cudaSuccess) e = cudaMemset(ctx->d_status, 0, 4 * sizeof(unsigned int));
-    if (e == cudaSuccess) e = cudaMalloc(&ctx->norm_tab, KDE_NTAB_N * sizeof(float2));
+    // the constant tables lie behind one another
+    const size_t f64_b = F64_TAB * sizeof(double), norm_b = KDE_NTAB_N * sizeof(float2);
+    if (e == cudaSuccess) e = cudaMalloc(&ctx->f64_tab, f64_b + norm_b + PXY_TAB_N * sizeof(float));
     if (e == cudaSuccess) {
-        norm_tab_kernel<<<(KDE_NTAB_N + 255) / 256, 256, 0, ctx->stream>>>(ctx->norm_tab);
-        e = cudaGetLastError();
-    }
-    if (e == cudaSuccess) e = cudaMalloc(&ctx->pxy_tab, PXY_TAB_N * sizeof(float));
-    if (e == cudaSuccess) {
-        pxy_tab_kernel<<<PXY_MAXQ, 128, 0, ctx->stream>>>(ctx->pxy_tab);
-        e = cudaGetLastError();
-    }
-    if (e == cudaSuccess) e = cudaMalloc(&ctx->f64_tab, F64_TAB * sizeof(double));
-    if (e == cudaSuccess) {
-        f64_tab_kernel<<<F64_TAB / 256, 256, 0, ctx->stream>>>(ctx->f64_tab);
+        ctx->norm_tab = (float2 *)((char *)ctx->f64_tab + f64_b);
+        ctx->pxy_tab = (float *)((char *)ctx->norm_tab + norm_b);
+        ctx_tables_kernel<<<NTAB_BLOCKS + F64_BLOCKS + PXY_MAXQ * PXY_TAB_BLOCKS, 256, 0, ctx->stream>>>(
+            ctx->norm_tab, ctx->f64_tab, ctx->pxy_tab);
         e = cudaGetLastError();
     }
     if (e == cudaSuccess) e = cudaStreamSynchronize(ctx->stream);
@@ -243,8 +247,6 @@ extern "C" kde_status kde_create(kde_ctx **out, int device, void *stream)
         cudaGetLastError();
         if (ctx->f64_tab) cudaFree(ctx->f64_tab);
         if (ctx->d_status) cudaFree(ctx->d_status);
-        if (ctx->norm_tab) cudaFree(ctx->norm_tab);
-        if (ctx->pxy_tab) cudaFree(ctx->pxy_tab);
         delete ctx;
         return KDE_ECUDA;
     }
@@ -268,8 +270,6 @@ extern "C" kde_status kde_destroy(kde_ctx *ctx)
     for (auto &kv : ctx->node_tab) cudaFree(kv.second);
     for (auto &kv : ctx->green_tab) cudaFree(kv.second);
     if (ctx->ad_tab) cudaFree(ctx->ad_tab);
-    if (ctx->norm_tab) cudaFree(ctx->norm_tab);
-    if (ctx->pxy_tab) cudaFree(ctx->pxy_tab);
     if (ctx->f64_tab) cudaFree(ctx->f64_tab);
     if (ctx->d_status) cudaFree(ctx->d_status);
     for (auto &p : ctx->prof) {
