@@ -96,11 +96,13 @@ kde_status kde_sync(kde_ctx *ctx);
 
 /* Autotuner (no counterpart in the paper: a speed facility of this library).  Keys are
  * (grid size, log2 N, uniform width to a quarter octave, or "per-particle widths").
- *  - Tile shape of the FP32 gather.  The packed gather has several tile shapes
- *    (particles a lane, node-loop unrolling, launch bound) that give bitwise-identical
- *    results.  The first FP32 gather (kde_gather, or the gather and push of pic_step
+ *  - Tile shape of the FP32 gather.  The gather that sweeps each particle's nodes has
+ *    several tile shapes (node-loop unrolling, launch bound) that give bitwise-identical
+ *    results.  The first such gather (kde_gather, or the gather and push of pic_step
  *    and of the ensemble) of each key runs every shape twice on its own data, timed by
- *    CUDA events, and keeps the fastest for that key.
+ *    CUDA events, and keeps the fastest for that key.  Gathers that interpolate the
+ *    smoothed field (most of those at the default truncation) have no shapes: their keys
+ *    are stored with shape 0 and nothing is timed.
  *  - Truncation radius of the FP32 PIC step (see kde_set_truncation).  Unless a cut is
  *    fixed, the first FP32 pic_step of each key runs the deposit + field and a gather
  *    on the step's own sorted particles at the cuts 2^-24, 2^-20 and 2^-18 of each
@@ -132,7 +134,9 @@ kde_status kde_autotune_set(kde_ctx *ctx, int32_t n, const uint64_t *keys, const
  * gather evaluates each particle's kernel at least over the nodes where its weight is
  * 2^-c of its peak or more, c = log2_cut.  The kernel mass left outside is at most
  * 3.6e-8 (c = 24, the default), 5.8e-7 (20), 2.3e-6 (18) and 9.2e-6 (16) of the total,
- * over all widths (worst near kappa = 6-9; von Mises tail integrals).  log2_cut = 0
+ * over all widths (worst near kappa = 6-9; von Mises tail integrals).  At the default
+ * the deposit and the gather may evaluate a window through interpolation points of the
+ * kernel (error below 1e-7 of the result); any other cut sums pair by pair.  log2_cut = 0
  * returns to the default, with pic_step's cut chosen by the autotuner when it is on.
  * KDE_EINVAL unless log2_cut is 0 or in [16, 40].  FP64 paths always cut at 2^-64; the CV's
  * pair sums and kde_deposit_noalloc (which takes no context) keep 2^-24. */

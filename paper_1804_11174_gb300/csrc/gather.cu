@@ -3,12 +3,15 @@
 //
 //   E_i = (2 pi / Ng) norm(kappa_i) sum_g E_g exp(-2 kappa_i sin^2((theta_g - theta_i)/2))
 //
-// Layout: the whole grid (half-angle sine, cosine, field) sits in shared
-// memory.  Threads own particles (cell-sorted, so a warp's particles share a
-// few cells); each warp sweeps one node window covering all of its lanes'
-// truncated supports, so every node read is a shared-memory broadcast.  The
-// push, the write-back of the particle state and (block 0) the field energy
-// ride in the same kernel.
+// Forms.  gather_tile_kernel (FP32, default cut, sorted particles of a PIC
+// step): a CTA smooths the field at the interpolation points of its tile and
+// the particles take the interpolant.  gather2_kernel (FP32 otherwise): the
+// whole grid (half-angle sine, cosine, field) in shared memory, threads own
+// particles (a sorted warp's share a few cells), each warp sweeps one node
+// window covering all of its lanes' truncated supports, so every node read is
+// a broadcast.  gather64_kernel: the FP64 form.  The push, the write-back of
+// the particle state and the field energy ride in the same kernel.  Plain
+// FP32 calls at the default cut go through the tables of gtable.cu.
 #include "common.cuh"
 #include "fp64.cuh"
 #include "proxy.cuh"

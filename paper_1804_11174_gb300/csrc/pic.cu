@@ -2,13 +2,13 @@
 //
 // Per step (stream-ordered; no host synchronisation except in the AD schedule):
 //   [width update: CV over the uniform candidates, kappa* = argmin on the
-//    device, leave-one-out pilot densities, Silverman widths + norms]
+//    device, leave-one-out pilot densities, Silverman widths + their range]
 //   [or the Sec. II.D schedule on the uniform width: Anderson-Darling p-value
 //    read on the host, the update rule, CV on optimisation steps, smoothing
 //    of h = kappa^{-1/2}]
-//   counting sort by cell (positions, velocities, widths, norms, labels)
-//   deposit -> int64 grid accumulators
-//   Poisson solve straight from the accumulators (mean removed in FP64)
+//   counting sort by cell (positions, velocities, widths, labels; FP64: norms)
+//   deposit -> int64 node sums
+//   Poisson solve straight from the sums (mean removed in int64, FP64 states in FP64)
 //   gather + leap-frog push + write-back + field energy (one kernel)
 #include "common.cuh"
 #include "fp64.cuh"
