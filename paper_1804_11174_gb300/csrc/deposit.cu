@@ -1811,8 +1811,9 @@ static kde_status deposit_api_f32(kde_ctx *ctx, const uint32_t *u, const float *
     // sort they spare 16 to 20
     const bool flat = (double)N * Ng <= 33554432.0 && kde_fp32_cut(ctx) == (float)KDE_XCUT;
     // the sort groups the particles for the CTAs' windows, which have at most a few hundred
-    // CTAs' worth of resolution: 1024 bins at most (4,000,037 particles on 4096 nodes: 255 us
-    // sorted by cells)
+    // CTAs' worth of resolution: 1024 bins at most.  4,000,037 particles with widths of 5 to 5000
+    // on 4096 nodes: 470 us; 528 with 2048 bins and 540 sorted by cells (the count table and the
+    // scatter's short runs), 1712 with 512 (a bin is then too wide for proxies at the largest widths)
     const int nbins = flat ? -1 : (Ng > 1024 ? 1024 : Ng);
     const uint32_t *us = u;
     const float *ks = kappa, *ws = weight;
