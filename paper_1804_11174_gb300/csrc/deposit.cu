@@ -1566,8 +1566,11 @@ static kde_status deposit_sorted_impl(kde_ctx *ctx, const uint32_t *u, const T *
             // the compressed form is for the default cut (one the caller has set keeps the sweep
             // over the particles that it is defined for), and for CTAs whose sweep of the whole
             // grid would cost more than its fixed steps
+            // A width schedule's few CTAs sweep too: their proxies share seven widths, whose rounding
+            // few CTAs average (66 CTAs, 16,832 particles: field energies 1.0 to 1.6e-6 off, swept
+            // 0.3 to 1.0e-6; 157 CTAs: 0.1 to 1.0e-6 against 0.4 to 1.6e-6)
             const double n = (double)N / Pl.G;
-            const bool comp = nbins >= 0 && S.xcut == (float)KDE_XCUT && n * (3.2 * Ng + 48.0) > (double)Pl.fixed;
+            const bool comp = nbins >= 0 && !(krange && Pl.G < 128) && S.xcut == (float)KDE_XCUT && n * (3.2 * Ng + 48.0) > (double)Pl.fixed;
             KDE_CUDA(ctx,
                      kde_launch(ctx, true, comp ? deposit_persist_kernel<true> : deposit_persist_kernel<false>,
                                 dim3(Pl.G), dim3(DEPP_THREADS), 0, S, Pl),
