@@ -63,9 +63,9 @@ __global__ void __launch_bounds__(POI_THREADS)
 // a constant and drops out; so does the tiny remainder of the mean, which the zero-sum Green's
 // function annihilates) and convolves for its own nodes, a node a warp at a time.  No FP64,
 // which is slow on this part, and no exchange between CTAs.  CTA 0 zeroes the other grid of
-// sums for the next deposit.  The Green's function is loaded before the wait.  Bound by
-// latency: one round of loads, one block sum, Ng / 32 products a lane; 8.7 us when it summed
-// 456 rows in a cluster of eight CTAs, 3.9 us at 256 nodes now.
+// sums for the next deposit.  Bound by latency: one round of loads, one block sum, Ng / 32
+// products a lane; 8.7 us when it summed 456 rows in a cluster of eight CTAs, 3.9 us at 256
+// nodes now.
 // ---------------------------------------------------------------------------
 #define FIELD_THREADS 256
 #define FIELD_WARPS 8
@@ -79,22 +79,27 @@ __global__ void __launch_bounds__(FIELD_THREADS)
     __shared__ long long red[2 * FIELD_WARPS];
     constexpr int PT = KDE_MAX_NG / FIELD_THREADS;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    for (int g = tid; g < Ng; g += FIELD_THREADS) gs[g] = Gf[g];
-    kde_pdl_wait();  // the sums come from the deposit before
+    // the sums come from the deposit before, and on a grid's first use the Green's function from
+    // a kernel launched between the two
+    kde_pdl_wait();
     kde_pdl_trigger();
     long long n[PT];
+    float gv[PT];
     long long hi = 0, lo = 0;
 #pragma unroll
     for (int i = 0; i < PT; ++i) {
         const int g = tid + i * FIELD_THREADS;
         if (i * FIELD_THREADS >= Ng) break;
         n[i] = g < Ng ? __ldcg(&acc[g]) : 0;
+        gv[i] = g < Ng ? __ldcg(&Gf[g]) : 0.f;
     }
 #pragma unroll
     for (int i = 0; i < PT; ++i) {
         if (i * FIELD_THREADS >= Ng) break;
         hi += n[i] >> 32;
         lo += n[i] & 0xffffffffll;
+        const int g = tid + i * FIELD_THREADS;
+        if (g < Ng) gs[g] = gv[i];
     }
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) {

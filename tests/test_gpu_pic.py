@@ -426,3 +426,24 @@ def test_snapshot_restore_repeats_the_run(ctx, kp):
     ctx.pic_step(st, 3 * P)
     for t, x in first.items():
         assert torch.equal(getattr(st, t), x), t
+
+
+def test_first_step_on_a_new_grid(kp):
+    # the first step on a grid builds its Green's function on the way; its field has to be the one
+    # that the same step finds once the table is there, bit for bit
+    N, dt = 3001, 0.1
+    c = kp.Context(0)
+    try:
+        for i, Ng in enumerate([64, 256, 1000, 2048, 4096] * 4):
+            L = 4 * math.pi + 0.01 * i  # a grid of its own each time
+            u, v = I.landau_load(i, N, L, 0.05, 1.0)
+            runs = []
+            for _ in range(2):
+                st = make_state(kp, u, v.astype(np.float32), L, Ng, dt, 1, kappa_uniform=30.0)
+                c.pic_step(st, 1)
+                c.sync()
+                runs.append((st.energy.cpu().numpy().copy(), st.v.cpu().numpy().copy(), st.u.cpu().numpy().copy()))
+            for a, b in zip(*runs):
+                assert np.array_equal(a, b), (Ng, i)
+    finally:
+        c.close()
