@@ -64,9 +64,10 @@ __device__ __forceinline__ int gt_band(float k, float &s)
         return 0;
     }
     const float t = fmaf(2.f, log2f(k), 2.f);  // half octaves above 1/2
-    const float f = floorf(t);
+    // the last band ends at GT_KMAX, where t (rounded, from 65535.94 on) is a whole number already
+    const float f = fminf(floorf(t), (float)(GT_BANDS - 2));
     s = fmaf(2.f, t - f, -1.f);
-    return min(1 + (int)f, GT_BANDS - 1);
+    return 1 + (int)f;
 }
 __device__ __forceinline__ float gt_checked(const GtArgs &A, float k, int64_t j)
 {

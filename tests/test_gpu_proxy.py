@@ -141,3 +141,31 @@ def test_fp64_deposit_and_gather(ctx, oracle, N, Ng, kap):
     f = np.cos(2 * math.pi * np.arange(Ng) / Ng) + 0.3 * I.uniforms(5, 3, Ng)
     out = ctx.gather(ud, to_dev(f, torch.float64), L, **kw).cpu().numpy()
     assert rel_l2(out, oracle.gather(x, f, L, **okw)) <= tol
+
+
+@pytest.mark.parametrize("kind", ["top", "edges", "extreme"])
+def test_gather_tables_at_the_band_edges(ctx, oracle, kind):
+    # enough pairs for the tables (range, bands, evaluation: three launches), widths at the ends of
+    # the half-octave bands, in the band below 1/2 and beyond the last one.  Tolerance: TOL, per
+    # width group, since a wrong band is a wrong kernel for that group alone
+    N, Ng = 16500, 4096
+    if kind == "top":
+        ks = np.array([65535.0, 65535.93, 65535.95, 65535.96, 65535.996, 65536.0, 65536.01, 65537.0], np.float32)
+    elif kind == "edges":
+        e = 0.5 * 2.0 ** (0.5 * np.arange(0, 35))
+        ks = np.concatenate([e * (1 - 2e-7), e, e * (1 + 2e-7)]).astype(np.float32)
+    else:
+        ks = np.exp(np.linspace(math.log(1e-6), math.log(1e6), 97)).astype(np.float32)
+    k = ks[np.arange(N) % ks.size]
+    u = positions(77, N, "box")
+    g = 2 * math.pi * np.arange(Ng) / Ng
+    f = (1 + np.sin(g) + 0.3 * np.cos(3 * g) + 0.2 * (I.uniforms(5, 3, Ng) - 0.5)).astype(np.float32)
+    ctx.profile_enable(True)
+    out = ctx.gather(to_dev_u(u), to_dev(f), L, kappa=to_dev(k)).cpu().numpy()
+    launches = ctx.profile_read("all")[1]
+    ctx.profile_enable(False)
+    ref = oracle.gather(I.from_fixed(u, L), f.astype(np.float64), L, kappa=k.astype(np.float64))
+    for i, kv in enumerate(ks):
+        at = np.arange(i, N, ks.size)
+        assert rel_l2(out[at], ref[at]) <= TOL, kv
+    assert launches == 3
