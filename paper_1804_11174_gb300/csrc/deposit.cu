@@ -965,14 +965,13 @@ __device__ __forceinline__ void depp_moments_mm(const DepSrc<float> &S, int64_t 
             if (t0 >= i1) break;
             const int64_t t = t0 + row;
             const bool ok = t < i1;
-            const float k = ok ? depp_kappa(S, rk[0], t) : 1.f;
-            // the first of the recurrence: the weight (0 past the end) or 1
-            float z, y0 = 1.f;
-            if (roleB) {
-                z = pxy_s(B, k);
-            } else {
-                z = pxy_x(B, ru[0]);
-                y0 = ok ? rw[0] * S.coef * (S.norm ? rn[0] : kde_norm_tab(S.ntab, k)) : 0.f;
+            // the first of the recurrence: the weight or 1; rows past the end have no weight and sit
+            // in the middle of the box (values far outside it would overflow, and 0 inf is no 0)
+            float z = 0.f, y0 = roleB ? 1.f : 0.f;
+            if (ok) {
+                const float k = depp_kappa(S, rk[0], t);
+                z = roleB ? pxy_s(B, k) : pxy_x(B, ru[0]);
+                if (!roleB) y0 = rw[0] * S.coef * (S.norm ? rn[0] : kde_norm_tab(S.ntab, k));
             }
 #pragma unroll
             for (int i = 0; i + 1 < QB; ++i) {

@@ -169,3 +169,19 @@ def test_gather_tables_at_the_band_edges(ctx, oracle, kind):
         at = np.arange(i, N, ks.size)
         assert rel_l2(out[at], ref[at]) <= TOL, kv
     assert launches == 3
+
+
+@pytest.mark.parametrize("lo", [2047.9998])
+def test_deposit_of_nearly_equal_widths(ctx, lo):
+    # widths of two neighbouring floats: a CTA's range of widths is one rounding long, and a value
+    # from elsewhere mapped into it would be 1e7 half-lengths away.  Against one width for all:
+    # both deposits are within TOL of the exact one, whose own difference is below 1e-7
+    N, Ng = 1000003, 4096
+    u = positions(31, N, "box")
+    k = np.full(N, lo, np.float32)
+    k[::3] = np.nextafter(np.float32(lo), np.float32(1e6))
+    ud = to_dev_u(u)
+    rho = ctx.deposit(ud, Ng, L, kappa=to_dev(k)).cpu().numpy()
+    one = ctx.deposit(ud, Ng, L, kappa_uniform=float(k[0])).cpu().numpy()
+    ctx.sync()
+    assert np.all(np.isfinite(rho)) and rel_l2(rho, one) <= 2 * TOL
