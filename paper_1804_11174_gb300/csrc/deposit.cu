@@ -1461,7 +1461,8 @@ __global__ void wmax_kernel(const T *w, int64_t N, unsigned int *wmax_bits, unsi
 __global__ void krange_norms_kernel(unsigned int *krange, const float *pxt)
 {
     const float kmax = __uint_as_float(krange[0]), kmin = __uint_as_float(krange[1]);
-    const float kc = 0.5f * (kmin + kmax), kh = 0.5f * (kmax - kmin);
+    float kc, kh;
+    pxy_lin_range(kmin, kmax, kc, kh);
     const int i = threadIdx.x, Q = i < 16 ? 7 : 6, b = i & 15;
     if (b >= Q) return;
     const float k = pxy_lin_kappa(kc, kh, pxt[pxy_tab_off(Q) + Q + b], Q);

@@ -98,6 +98,15 @@ __device__ __forceinline__ void pxy_box_pos(PxyBox &B, const PxyGrid &G, int c_f
     B.inv_hw = 1.f / B.hw;
     B.P = pxy_degree_pos(B.hw * (float)(KDE_TWO_PI / 4294967296.0) * sqrtf(kmax + 1.5f));
 }
+// middle and half-length of a narrow range of widths.  The middle is rounded, so over a range of
+// a few roundings the ends would lie outside [-1, 1] (at 2 for two neighbouring floats, where the
+// highest polynomials reach 1e3 and their rounding 1e-5 of the result): at least 1e-5 of the
+// middle, and 1e-30 for the widths next to zero, whose kernels are all the constant one
+__device__ __forceinline__ void pxy_lin_range(float kmin, float kmax, float &kc, float &kh)
+{
+    kc = 0.5f * (kmin + kmax);
+    kh = fmaxf(0.5f * (kmax - kmin), fmaxf(1e-5f * kc, 1e-30f));
+}
 __device__ __forceinline__ void pxy_box_width(PxyBox &B, float kmin, float kmax)
 {
     B.lin = kmax - kmin <= PXY_LIN_R * (kmax + kmin);
@@ -107,8 +116,7 @@ __device__ __forceinline__ void pxy_box_width(PxyBox &B, float kmin, float kmax)
         B.kh = B.inv_kh = 0.f;
     } else if (B.lin) {
         B.Q = 6;
-        B.kc = 0.5f * (kmin + kmax);
-        B.kh = 0.5f * (kmax - kmin);
+        pxy_lin_range(kmin, kmax, B.kc, B.kh);
         B.inv_kh = 1.f / B.kh;
     } else {
         const float l0 = logf(kmin), l1 = logf(kmax);

@@ -185,3 +185,21 @@ def test_deposit_of_nearly_equal_widths(ctx, lo):
     one = ctx.deposit(ud, Ng, L, kappa_uniform=float(k[0])).cpu().numpy()
     ctx.sync()
     assert np.all(np.isfinite(rho)) and rel_l2(rho, one) <= 2 * TOL
+
+
+@pytest.mark.parametrize("lo,ulps", [(1e-39, 1), (1e-30, 1), (14.0, 1), (14.0, 3), (300.0, 1), (300.0, 2)])
+def test_deposit_of_widths_a_few_roundings_apart(ctx, lo, ulps):
+    # the middle of such a range is rounded by a large part of its length.  Against one width for
+    # all, both within TOL of the exact density, whose own difference is below 4e-7
+    N, Ng = 1000003, 4096
+    u = positions(31, N, "box")
+    k = np.full(N, lo, np.float32)
+    hi = k[:1].copy()
+    for _ in range(ulps):
+        hi = np.nextafter(hi, np.float32(1e6))
+    k[::3] = hi
+    ud = to_dev_u(u)
+    rho = ctx.deposit(ud, Ng, L, kappa=to_dev(k)).cpu().numpy()
+    one = ctx.deposit(ud, Ng, L, kappa_uniform=float(k[0])).cpu().numpy()
+    ctx.sync()
+    assert rel_l2(rho, one) <= 2 * TOL
