@@ -105,7 +105,7 @@ enum WsSlot {
 
 // kernels timed by the profiling hook (kde_profile_enable / kde_profile_read)
 enum KdeProfId { PROF_CV_PAIRS = 0, PROF_DEPOSIT, PROF_GATHER, PROF_SORT, PROF_POISSON, PROF_CV_GRID, PROF_CV_LOO,
-                 PROF_SPECTRAL, PROF_AD, PROF_DEPOSIT_ROWS, PROF_NIDS };
+                 PROF_SPECTRAL, PROF_AD, PROF_DEPOSIT_ROWS /* no kernel any more: reads zero */, PROF_NIDS };
 
 struct kde_ctx {
     int device = 0;
@@ -508,8 +508,8 @@ struct DepSums {
     long long *acc, *next;
 };
 kde_status kde_deposit_sums_reset(kde_ctx *ctx);
-kde_status kde_deposit_sums_f32(kde_ctx *ctx, const uint32_t *u, const float *kappa, float kappa_u, const float *norm,
-                                float norm_u, int64_t N, int Ng, double coef, float w_u, double bound, DepSums *out,
+kde_status kde_deposit_sums_f32(kde_ctx *ctx, const uint32_t *u, const float *kappa, float kappa_u, float norm_u,
+                                int64_t N, int Ng, double coef, float w_u, double bound, DepSums *out,
                                 float xcut = 0.f, const unsigned int *krange = nullptr);
 // the PIC step's field from those sums: rho_total = background + charge * rho with its
 // mean removed (so the constant background drops out), E by the spectral or

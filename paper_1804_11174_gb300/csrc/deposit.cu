@@ -37,8 +37,8 @@ template <typename T> struct DepSrc {
     int64_t N;
     const T *kappa;      // per-particle widths, or nullptr
     T kappa_u;           // uniform width
-    T kscale;            // widths are kscale * kappa[j] (CV scale mode), else 1
-    const T *norm;       // per-particle norm, or nullptr (computed from the width when kappa != nullptr)
+    T kscale;            // CV: widths are kscale * kappa[j] in scale mode, else 1
+    const T *norm;       // FP64: per-particle norm, or nullptr (computed from the width when kappa != nullptr)
     const float *lnorm;  // log2 of per-particle norm (CV scale mode), or nullptr
     T norm_u;            // uniform norm
     const T *w;          // per-particle weights, or nullptr
@@ -52,7 +52,7 @@ template <typename T> struct DepSrc {
     double norm_bound;
     unsigned int *status;
     int scale_exp;  // KDE_ES_FROM_BOUND, or the exponent es of the fixed-point scale 2^es
-    const float2 *ntab;  // FP32 norm table (kde_norm_tab) for per-particle widths without norms, or nullptr
+    const float2 *ntab;  // FP32 norm table (kde_norm_tab) for per-particle widths
     float xcut = (float)KDE_XCUT;  // FP32 packed kernels: truncation cut exponent (kde_fp32_cut)
     int nbins = 0;                   // sort bins of the particles: 0 the cells, -1 not sorted at all
     PxyGrid grid;                    // the nodes as position codes
@@ -119,9 +119,9 @@ __device__ __forceinline__ void node_sc(const DepSrc<T> &S, int g, T &s, T &c)
     }
 }
 
-template <typename T, bool UNSORTED = false>
-__device__ void deposit_chunk_body(const DepSrc<T> &S, int64_t chunk, DepRec<T> *rec, T *part, int *red,
-                                   int *cmm = nullptr)
+// a chunk of particles in any order (kde_deposit_noalloc)
+template <typename T>
+__device__ void deposit_chunk_body(const DepSrc<T> &S, int64_t chunk, DepRec<T> *rec, T *part, int *red, int *cmm)
 {
     const int64_t i0 = chunk * DEP_CHUNK;
     if (i0 >= S.N) return;
@@ -134,21 +134,15 @@ __device__ void deposit_chunk_body(const DepSrc<T> &S, int64_t chunk, DepRec<T> 
     for (int t = tid; t < n; t += DEP_THREADS) {
         int64_t j = i0 + t;
         uint32_t uu = S.u[j];
-        if (UNSORTED) {
-            int cc = kde_cell(uu, S.Ng);
-            cmin = cc < cmin ? cc : cmin;
-            cmax = cc > cmax ? cc : cmax;
-        }
-        T k = S.kappa ? S.kscale * S.kappa[j] : S.kappa_u;
+        int cc = kde_cell(uu, S.Ng);
+        cmin = cc < cmin ? cc : cmin;
+        cmax = cc > cmax ? cc : cmax;
+        T k = S.kappa ? S.kappa[j] : S.kappa_u;
         if (!(k > (T)0 && k <= (T)KDE_KAPPA_MAX)) {
             kde_flag(S.status, KDE_DEV_KAPPA_RANGE, (unsigned)j);
             k = (T)KDE_KAPPA_MAX;
         }
-        T nm;
-        if (S.lnorm) nm = (T)exp2f(S.lnorm[j]);
-        else if (S.norm) nm = S.norm[j];
-        else if (S.kappa) nm = (T)kde_norm((double)k);
-        else nm = S.norm_u;
+        const T nm = S.kappa ? (T)kde_norm((double)k) : S.norm_u;
         T wj = S.w ? S.w[j] : S.w_u;
         T sh, ch;
         kde_half_sincos(uu, sh, ch);
@@ -170,30 +164,23 @@ __device__ void deposit_chunk_body(const DepSrc<T> &S, int64_t chunk, DepRec<T> 
     int W = 0;
 #pragma unroll
     for (int k = 0; k < DEP_WARPS; ++k) W = red[k] > W ? red[k] : W;
-    int c_first, c_last;
-    if (UNSORTED) {
-        // particles in any order: the chunk's linear cell range (a range that wraps
-        // around the grid falls back to the whole grid below)
+    // the chunk's linear cell range (a range that wraps around the grid falls back to the whole
+    // grid below)
 #pragma unroll
-        for (int o = 16; o > 0; o >>= 1) {
-            cmin = min(cmin, __shfl_xor_sync(0xffffffffu, cmin, o));
-            cmax = max(cmax, __shfl_xor_sync(0xffffffffu, cmax, o));
-        }
-        if (lane == 0) {
-            cmm[warp] = cmin;
-            cmm[DEP_WARPS + warp] = cmax;
-        }
-        __syncthreads();
-        c_first = cmm[0];
-        c_last = cmm[DEP_WARPS];
+    for (int o = 16; o > 0; o >>= 1) {
+        cmin = min(cmin, __shfl_xor_sync(0xffffffffu, cmin, o));
+        cmax = max(cmax, __shfl_xor_sync(0xffffffffu, cmax, o));
+    }
+    if (lane == 0) {
+        cmm[warp] = cmin;
+        cmm[DEP_WARPS + warp] = cmax;
+    }
+    __syncthreads();
+    int c_first = cmm[0], c_last = cmm[DEP_WARPS];
 #pragma unroll
-        for (int k = 1; k < DEP_WARPS; ++k) {
-            c_first = min(c_first, cmm[k]);
-            c_last = max(c_last, cmm[DEP_WARPS + k]);
-        }
-    } else {
-        c_first = kde_cell(S.u[i0], Ng);
-        c_last = kde_cell(S.u[i0 + n - 1], Ng);
+    for (int k = 1; k < DEP_WARPS; ++k) {
+        c_first = min(c_first, cmm[k]);
+        c_last = max(c_last, cmm[DEP_WARPS + k]);
     }
     int g_lo = c_first - W;
     int R = c_last + W - g_lo + 1;
@@ -259,18 +246,12 @@ __device__ void deposit_chunk_body(const DepSrc<T> &S, int64_t chunk, DepRec<T> 
 }
 
 // ---------------------------------------------------------------------------
-// FP32 chunk body with packed pair arithmetic: each lane owns two nodes (a warp
-// pass covers 64 consecutive nodes) and every particle record is staged
-// pre-duplicated, so that one 128-bit and one 64-bit broadcast load feed the
-// f32x2 multiply-adds of both nodes.  Same node range, slicing and fixed-order
-// combination as the scalar body.  Two forms of the kernel value, chosen per
-// chunk by its largest width:
-//  * half-angle (any width): 2^-(S_g beta c_j - C_g beta s_j)^2 with (s, c) the sine
-//    and cosine of half the angle; records (beta s, beta s, beta c, beta c) and
-//    (w n, w n); four multiply-adds per pair;
-//  * cosine (largest width <= KDE_COSFORM_KMAX, when allowed): 2^(K cos(x_j - x_g))
-//    2^-K with K = kappa log2(e); records (K cos, K cos, K sin, K sin) of the full
-//    angle and (w n 2^-K, w n 2^-K); three multiply-adds per pair.
+// FP32 chunk body of the CV's integral term, with packed pair arithmetic: each lane owns two
+// nodes (a warp pass covers 64 consecutive nodes) and every particle record is staged
+// pre-duplicated, so that one 128-bit and one 64-bit broadcast load feed the f32x2 multiply-adds
+// of both nodes.  Same node range, slicing and fixed-order combination as the scalar body.  The
+// kernel value is 2^-(S_g beta c_j - C_g beta s_j)^2 with (s, c) the sine and cosine of half the
+// angle, records (beta s, beta s, beta c, beta c) and (w n, w n): four multiply-adds per pair.
 // ---------------------------------------------------------------------------
 #define DEP2_PART 512
 #define DEP2_UNROLL_P1 4
@@ -281,7 +262,7 @@ __device__ void deposit_chunk_body(const DepSrc<T> &S, int64_t chunk, DepRec<T> 
 // groups than warps the warps split the particles into slices whose partial sums
 // are combined in a fixed order
 template <int P>
-__device__ __forceinline__ void dep2_nodes(const DepSrc<float> &S, int n, int g_lo, int R, bool cosf, int es,
+__device__ __forceinline__ void dep2_nodes(const DepSrc<float> &S, int n, int g_lo, int R, int es,
                                            const float4 *rsc, const float2 *rwn, float *part)
 {
     constexpr int GW = 64 * P;
@@ -310,42 +291,23 @@ __device__ __forceinline__ void dep2_nodes(const DepSrc<float> &S, int n, int g_
             float sa, ca, sb, cb;
             node_sc(S, ok[2 * q] ? gn[2 * q] : 0, sa, ca);
             node_sc(S, ok[2 * q + 1] ? gn[2 * q + 1] : 0, sb, cb);
-            if (cosf) {
-                // sine and cosine of the full node angle
-                SS[q] = kde_pk(2.f * sa * ca, 2.f * sb * cb);
-                CC[q] = kde_pk((ca - sa) * (ca + sa), (cb - sb) * (cb + sb));
-            } else {
-                SS[q] = kde_pk(sa, sb);
-                CC[q] = kde_pk(-ca, -cb);
-            }
+            SS[q] = kde_pk(sa, sb);
+            CC[q] = kde_pk(-ca, -cb);
         }
     };
     auto sweep = [&](int p0, int p1) {
 #pragma unroll
         for (int q = 0; q < P; ++q) acc[q] = kde_pk(0.f, 0.f);
-        if (cosf) {
 #pragma unroll U
-            for (int p = p0; p < p1; ++p) {
-                const float4 r4 = rsc[p];
-                const float2 w2 = rwn[p];
-                const kde_f2 qs = kde_pk(r4.z, r4.w), qc = kde_pk(r4.x, r4.y), w = kde_pk(w2.x, w2.y);
-                // K cos(x_j - x_g) = sin_g (K sin_j) + cos_g (K cos_j)
+        for (int p = p0; p < p1; ++p) {
+            const float4 r4 = rsc[p];
+            const float2 w2 = rwn[p];
+            const kde_f2 qs = kde_pk(r4.z, r4.w), qc = kde_pk(r4.x, r4.y), w = kde_pk(w2.x, w2.y);
+            // s = S_g (beta cos_j) - C_g (beta sin_j)
 #pragma unroll
-                for (int q = 0; q < P; ++q)
-                    acc[q] = kde_fma2(kde_ex22(kde_fma2(SS[q], qs, kde_mul2(CC[q], qc))), w, acc[q]);
-            }
-        } else {
-#pragma unroll U
-            for (int p = p0; p < p1; ++p) {
-                const float4 r4 = rsc[p];
-                const float2 w2 = rwn[p];
-                const kde_f2 qs = kde_pk(r4.z, r4.w), qc = kde_pk(r4.x, r4.y), w = kde_pk(w2.x, w2.y);
-                // s = S_g (beta cos_j) - C_g (beta sin_j)
-#pragma unroll
-                for (int q = 0; q < P; ++q) {
-                    const kde_f2 sv = kde_fma2(SS[q], qs, kde_mul2(CC[q], qc));
-                    acc[q] = kde_fma2(kde_ex2neg2(kde_mul2(sv, sv)), w, acc[q]);
-                }
+            for (int q = 0; q < P; ++q) {
+                const kde_f2 sv = kde_fma2(SS[q], qs, kde_mul2(CC[q], qc));
+                acc[q] = kde_fma2(kde_ex2neg2(kde_mul2(sv, sv)), w, acc[q]);
             }
         }
     };
@@ -408,7 +370,7 @@ __device__ void deposit_chunk_body_x2(const DepSrc<float> &S, int64_t chunk, flo
     // chunk); the smallest width sets the window
     constexpr int PER = DEP_CHUNK / DEP_THREADS;
     uint32_t ru[PER];
-    float rk[PER], rn[PER], rw[PER];
+    float rk[PER], rn[PER];
     float kmin = (float)KDE_KAPPA_MAX;
 #pragma unroll
     for (int p = 0; p < PER; ++p) {
@@ -417,8 +379,7 @@ __device__ void deposit_chunk_body_x2(const DepSrc<float> &S, int64_t chunk, flo
         const int64_t j = i0 + (ok ? t : 0);
         ru[p] = S.u[j];
         float k = S.kappa ? S.kscale * S.kappa[j] : S.kappa_u;
-        rn[p] = S.lnorm ? S.lnorm[j] : (S.norm ? S.norm[j] : 0.f);
-        rw[p] = S.w ? S.w[j] : S.w_u;
+        rn[p] = S.lnorm ? S.lnorm[j] : 0.f;
         if (ok && !(k > 0.f && k <= (float)KDE_KAPPA_MAX)) {
             kde_flag(S.status, KDE_DEV_KAPPA_RANGE, (unsigned)j);
             k = (float)KDE_KAPPA_MAX;
@@ -429,20 +390,8 @@ __device__ void deposit_chunk_body_x2(const DepSrc<float> &S, int64_t chunk, flo
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) kmin = fminf(kmin, __shfl_xor_sync(0xffffffffu, kmin, o));
     if (lane == 0) red[warp] = __float_as_int(kmin);
-    // the fixed-point scale 2^es, worked out by one thread: FP64 stays off the other threads
-    __shared__ int s_es;
-    if (tid == 0) {
-        int es = S.scale_exp;
-        if (es == KDE_ES_FROM_BOUND) {
-            double bound = S.bound;
-            if (S.wmax_bits)
-                bound = (double)S.N * (double)S.coef * S.norm_bound * (double)__uint_as_float(*S.wmax_bits);
-            es = acc_scale_exp(bound);
-        }
-        s_es = es;
-    }
     __syncthreads();
-    const int es = s_es;
+    const int es = S.scale_exp;
 #pragma unroll
     for (int k = 0; k < DEP_WARPS; ++k) kmin = fminf(kmin, __int_as_float(red[k]));
     // the window shrinks as the width grows: the smallest width's window covers all
@@ -454,12 +403,8 @@ __device__ void deposit_chunk_body_x2(const DepSrc<float> &S, int64_t chunk, flo
         if (t >= n) break;
         const uint32_t uu = ru[p];
         const float k = rk[p];
-        float nm;
-        if (S.lnorm) nm = exp2f(rn[p]);
-        else if (S.norm) nm = rn[p];
-        else if (S.kappa) nm = S.ntab ? kde_norm_tab(S.ntab, k) : (float)kde_norm((double)k);
-        else nm = S.norm_u;
-        const float wn = rw[p] * S.coef * nm;
+        const float nm = S.lnorm ? exp2f(rn[p]) : S.norm_u;
+        const float wn = S.w_u * S.coef * nm;
         float sh, ch;
         kde_half_sincos(uu, sh, ch);
         const float beta = sqrtf((float)(2.0 * KDE_LOG2E) * k);
@@ -478,9 +423,9 @@ __device__ void deposit_chunk_body_x2(const DepSrc<float> &S, int64_t chunk, flo
     // groups compute no extra nodes and their partial sums fit the buffer
     const int n64 = (R + 63) >> 6, n128 = (R + 127) >> 7;
     if (2 * n128 == n64 && (n128 >= DEP_WARPS || n128 * 128 <= DEP2_PART))
-        dep2_nodes<2>(S, n, g_lo, R, false, es, rsc, rwn, part);
+        dep2_nodes<2>(S, n, g_lo, R, es, rsc, rwn, part);
     else
-        dep2_nodes<1>(S, n, g_lo, R, false, es, rsc, rwn, part);
+        dep2_nodes<1>(S, n, g_lo, R, es, rsc, rwn, part);
 }
 
 // ---------------------------------------------------------------------------
@@ -949,14 +894,13 @@ __device__ __forceinline__ void depp_moments_mm(const DepSrc<float> &S, int64_t 
 #pragma unroll 1
     for (int64_t g0 = i0 + warp * PXY_STAGE; g0 < i1; g0 += QB * step) {
         uint32_t ru[QB];
-        float rk[QB], rn[QB], rw[QB];
+        float rk[QB], rw[QB];
 #pragma unroll
         for (int q = 0; q < QB; ++q) {
             const int64_t t = g0 + q * step + row;
             const int64_t j = t < i1 ? t : i0;
             ru[q] = S.u[j];
             rk[q] = S.kappa[j];
-            rn[q] = S.norm ? S.norm[j] : 0.f;
             rw[q] = S.w ? S.w[j] : S.w_u;
         }
 #pragma unroll 1
@@ -971,13 +915,12 @@ __device__ __forceinline__ void depp_moments_mm(const DepSrc<float> &S, int64_t 
             if (ok) {
                 const float k = depp_kappa(S, rk[0], t);
                 z = roleB ? pxy_s(B, k) : pxy_x(B, ru[0]);
-                if (!roleB) y0 = rw[0] * S.coef * (S.norm ? rn[0] : kde_norm_tab(S.ntab, k));
+                if (!roleB) y0 = rw[0] * S.coef * kde_norm_tab(S.ntab, k);
             }
 #pragma unroll
             for (int i = 0; i + 1 < QB; ++i) {
                 ru[i] = ru[i + 1];
                 rk[i] = rk[i + 1];
-                rn[i] = rn[i + 1];
                 rw[i] = rw[i + 1];
             }
             float y1 = y0 * z;
@@ -1353,14 +1296,13 @@ __global__ void __launch_bounds__(DEPP_THREADS, DEPP_MINB) deposit_persist_kerne
 #pragma unroll 1
         for (int p0 = 0; p0 < PER; p0 += QB) {
             uint32_t ru[QB];
-            float rk[QB], rn[QB], rw[QB];
+            float rk[QB], rw[QB];
 #pragma unroll
             for (int q = 0; q < QB; ++q) {
                 const int t = tid + (p0 + q) * DEPP_THREADS;
                 const int64_t j = b0 + (t < n ? t : 0);
                 ru[q] = S.u[j];
-                rk[q] = S.kappa ? S.kscale * S.kappa[j] : S.kappa_u;
-                rn[q] = S.norm ? S.norm[j] : 0.f;
+                rk[q] = S.kappa ? S.kappa[j] : S.kappa_u;
                 rw[q] = S.w ? S.w[j] : S.w_u;
             }
 #pragma unroll
@@ -1372,10 +1314,7 @@ __global__ void __launch_bounds__(DEPP_THREADS, DEPP_MINB) deposit_persist_kerne
                     kde_flag(S.status, KDE_DEV_KAPPA_RANGE, (unsigned)(b0 + t));
                     k = (float)KDE_KAPPA_MAX;
                 }
-                float nm;
-                if (S.norm) nm = rn[q];
-                else if (S.kappa) nm = S.ntab ? kde_norm_tab(S.ntab, k) : (float)kde_norm((double)k);
-                else nm = S.norm_u;
+                const float nm = S.kappa ? kde_norm_tab(S.ntab, k) : S.norm_u;
                 const float wn = rw[q] * S.coef * nm;
                 float sh, ch;
                 kde_half_sincos(ru[q], sh, ch);
@@ -1599,8 +1538,8 @@ kde_status kde_deposit_sorted_f64(kde_ctx *ctx, const uint32_t *u, const double 
                                        norm_bound);
 }
 
-kde_status kde_deposit_sums_f32(kde_ctx *ctx, const uint32_t *u, const float *kappa, float kappa_u, const float *norm,
-                                float norm_u, int64_t N, int Ng, double coef, float w_u, double bound, DepSums *out,
+kde_status kde_deposit_sums_f32(kde_ctx *ctx, const uint32_t *u, const float *kappa, float kappa_u, float norm_u,
+                                int64_t N, int Ng, double coef, float w_u, double bound, DepSums *out,
                                 float xcut, const unsigned int *krange)
 {
     if (N < 1) return kde_fail(ctx, KDE_EINVAL, "deposit sums: need N >= 1");
@@ -1609,7 +1548,7 @@ kde_status kde_deposit_sums_f32(kde_ctx *ctx, const uint32_t *u, const float *ka
     out->acc = s + (ctx->sums_flip ? KDE_MAX_NG : 0);
     out->next = s + (ctx->sums_flip ? 0 : KDE_MAX_NG);
     ctx->sums_flip = !ctx->sums_flip;
-    return deposit_sorted_impl<float>(ctx, u, kappa, kappa_u, norm, norm_u, nullptr, w_u, N, Ng, coef, out->acc, bound,
+    return deposit_sorted_impl<float>(ctx, u, kappa, kappa_u, nullptr, norm_u, nullptr, w_u, N, Ng, coef, out->acc, bound,
                                       nullptr, 0.0, xcut, krange);
 }
 
@@ -1669,7 +1608,9 @@ __global__ void cv_grid_par_kernel(CandList cl, const unsigned int *krmax_bits, 
     par[c] = p;
 }
 
-__global__ void __launch_bounds__(DEP_THREADS)
+// four CTAs an SM (62 registers): left to itself the compiler goes for five at 48 registers, with fewer
+// records in flight (20,000 particles, 3 factors on widths of 1e-5 to 1e5: 291 us, 234 with four)
+__global__ void __launch_bounds__(DEP_THREADS, 4)
     cv_grid_deposit_kernel(const uint32_t *u, int64_t N, const float *kappa_rel, const float *lnorm, int scale_mode,
                            const GridPar *par, long long *acc, unsigned int *status)
 {
@@ -1908,7 +1849,7 @@ __global__ void __launch_bounds__(DEP_THREADS) deposit_chunk_unsorted_kernel(Dep
     __shared__ T part[DEP_WARPS * 32 * DEP_WARPS];
     __shared__ int red[DEP_WARPS];
     __shared__ int cmm[2 * DEP_WARPS];
-    deposit_chunk_body<T, true>(S, blockIdx.x, rec, part, red, cmm);
+    deposit_chunk_body<T>(S, blockIdx.x, rec, part, red, cmm);
 }
 
 template <typename T2>

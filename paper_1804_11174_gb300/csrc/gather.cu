@@ -26,7 +26,7 @@ template <typename T> struct GatherArgs {
     const uint32_t *u;
     const T *kappa;
     T kappa_u;
-    const T *norm;
+    const T *norm;  // FP64: norms of the particles, or null
     T norm_u;
     int64_t N;
     const T *field;
@@ -40,7 +40,7 @@ template <typename T> struct GatherArgs {
     uint32_t *u_out;
     T *v_out;
     T *kappa_out;
-    const T *norm_in;
+    const T *norm_in;  // FP64
     T *norm_out;
     const uint32_t *id_in;
     uint32_t *id_out;
@@ -51,7 +51,7 @@ template <typename T> struct GatherArgs {
     double *kstar_out;
     double dx;
     unsigned int *status;
-    const float2 *ntab;  // FP32 norm table (kde_norm_tab): per-particle widths without norms
+    const float2 *ntab;  // FP32 norm table (kde_norm_tab) for per-particle widths
     // push only: count table of the next step's cell sort, or null (counts of the new
     // positions are added with one atomic per warp and distinct cell)
     unsigned int *counts;
@@ -241,7 +241,7 @@ __device__ __forceinline__ void gat_finish(const GatherArgs<float> &A, int64_t b
         constexpr int HB = NP % 4 == 0 ? 4 : (NP % 3 == 0 ? 3 : 2);
 #pragma unroll
         for (int h0 = 0; h0 < NP; h0 += HB) {
-            float vin[HB], kin[HB], nin[HB];
+            float vin[HB], kin[HB];
             uint32_t idin[HB];
 #pragma unroll
             for (int hh = 0; hh < HB; ++hh) {
@@ -249,7 +249,6 @@ __device__ __forceinline__ void gat_finish(const GatherArgs<float> &A, int64_t b
                 const bool ok = j < A.N;
                 vin[hh] = VIN ? vpre[h0 + hh] : (ok ? A.v_in[j] : 0.f);
                 kin[hh] = (ok && A.kappa_out) ? (A.kappa ? A.kappa[j] : A.kappa_u) : 0.f;
-                nin[hh] = (ok && A.norm_out && A.norm_in) ? A.norm_in[j] : 0.f;
                 idin[hh] = (ok && A.id_out) ? A.id_in[j] : 0u;
             }
 #pragma unroll
@@ -265,7 +264,7 @@ __device__ __forceinline__ void gat_finish(const GatherArgs<float> &A, int64_t b
                     if (A.kappa_out) {
                         const float k = (kin[hh] > 0.f && kin[hh] <= (float)KDE_KAPPA_MAX) ? kin[hh] : (float)KDE_KAPPA_MAX;
                         A.kappa_out[j] = k;
-                        if (A.norm_out) A.norm_out[j] = A.norm_in ? nin[hh] : kde_norm_tab(A.ntab, k);
+                        if (A.norm_out) A.norm_out[j] = kde_norm_tab(A.ntab, k);
                     }
                     if (A.id_out) A.id_out[j] = idin[hh];
                     key = kde_cell(nu, Ng);
@@ -316,7 +315,7 @@ __global__ void __launch_bounds__(GAT2_WARPS * 32, MINB) gather2_kernel(GatherAr
             k = (float)KDE_KAPPA_MAX;
         }
         kap[h] = k;
-        nm[h] = A.norm ? (valid ? A.norm[j] : 0.f) : (A.kappa ? kde_norm_tab(A.ntab, k) : A.norm_u);
+        nm[h] = A.kappa ? kde_norm_tab(A.ntab, k) : A.norm_u;
         if (valid) {
             kmax = fmaxf(kmax, k);
             kmin = fminf(kmin, k);
@@ -704,7 +703,7 @@ __device__ __forceinline__ void gatt_direct(const GatherArgs<float> &A, const fl
             if (valid) kde_flag(A.status, KDE_DEV_KAPPA_RANGE, (unsigned)j);
             k = (float)KDE_KAPPA_MAX;
         }
-        nm[h] = A.norm ? (valid ? A.norm[j] : 0.f) : (A.kappa ? kde_norm_tab(A.ntab, k) : A.norm_u);
+        nm[h] = A.kappa ? kde_norm_tab(A.ntab, k) : A.norm_u;
         if (valid) {
             kmin = fminf(kmin, k);
             const int cell = kde_cell(uu[h], Ng);
@@ -1069,7 +1068,6 @@ static kde_status launch_gather2(kde_ctx *ctx, GatherArgs<float> &A)
         cudaStreamIsCapturing(ctx->stream, &cap);
         auto apart = [](const void *out, const void *in) { return !out || out != in; };
         const bool idem = !A.u_out || (apart(A.u_out, A.u) && apart(A.v_out, A.v_in) && apart(A.kappa_out, A.kappa) &&
-                                       apart(A.norm_out, A.norm_in) && apart(A.norm_out, A.norm) &&
                                        apart(A.id_out, A.id_in));
         tune = cap == cudaStreamCaptureStatusNone && idem;
     }

@@ -94,8 +94,8 @@ static kde_status tune_err(kde_ctx *ctx, const float *a, const float *b, int64_t
     return KDE_OK;
 }
 
-static kde_status tune_cut(kde_ctx *ctx, const uint32_t *us, const float *ks, float kappa_u, const float *ns,
-                           float norm_u, int64_t N, int Ng, double L, double coef, float w_u, double bound,
+static kde_status tune_cut(kde_ctx *ctx, const uint32_t *us, const float *ks, float kappa_u, float norm_u,
+                           int64_t N, int Ng, double L, double coef, float w_u, double bound,
                            double charge, bool fd, const unsigned int *gat_range,
                            const unsigned int *krange, float &cut)
 {
@@ -113,9 +113,9 @@ static kde_status tune_cut(kde_ctx *ctx, const uint32_t *us, const float *ks, fl
     // one candidate: deposit + field into E, and a gather of the reference field into g
     auto run = [&](int c, float *E, float *g) -> kde_status {
         DepSums ds{};
-        KDE_TRY(kde_deposit_sums_f32(ctx, us, ks, kappa_u, ns, norm_u, N, Ng, coef, w_u, bound, &ds, kCutCand[c], krange));
+        KDE_TRY(kde_deposit_sums_f32(ctx, us, ks, kappa_u, norm_u, N, Ng, coef, w_u, bound, &ds, kCutCand[c], krange));
         KDE_TRY(kde_field_from_sums(ctx, ds, Ng, L, 1.0 / kde_acc_scale(bound), charge, fd, E));
-        return kde_gather_sorted<float>(ctx, us, ks, kappa_u, ns, norm_u, N, Eref, Ng, KDE_TWO_PI / Ng, g, nullptr,
+        return kde_gather_sorted<float>(ctx, us, ks, kappa_u, nullptr, norm_u, N, Eref, Ng, KDE_TWO_PI / Ng, g, nullptr,
                                         nullptr, kCutCand[c], gat_range);
     };
     // the reference first (its field feeds every candidate's gather), then rounds in which
@@ -351,8 +351,8 @@ static kde_status pic_run(kde_ctx *ctx, pic_state *st, int n_steps)
                     cudaStreamIsCapturing(ctx->stream, &cap);
                     if (cap == cudaStreamCaptureStatusNone) {
                         KdeRange r_("kdepic truncation tuner");
-                        KDE_TRY(tune_cut(ctx, us, (const float *)ks, (float)st->kappa_uniform, (const float *)ns,
-                                         (float)norm_u, N, Ng, L, coef, (float)w_u, bound, st->charge, fd,
+                        KDE_TRY(tune_cut(ctx, us, (const float *)ks, (float)st->kappa_uniform, (float)norm_u,
+                                         N, Ng, L, coef, (float)w_u, bound, st->charge, fd,
                                          sched ? krange : nullptr, krange, cut));
                         ctx->cut_tuned[key] = cut;
                     }
@@ -362,7 +362,7 @@ static kde_status pic_run(kde_ctx *ctx, pic_state *st, int n_steps)
             DepSums ds{};
             {
                 KdeRange r_("kdepic deposit");
-                KDE_TRY(kde_deposit_sums_f32(ctx, us, ks, (float)st->kappa_uniform, ns, (float)norm_u, N, Ng, coef,
+                KDE_TRY(kde_deposit_sums_f32(ctx, us, ks, (float)st->kappa_uniform, (float)norm_u, N, Ng, coef,
                                              (float)w_u, bound, &ds, cut, krange));
             }
             {
