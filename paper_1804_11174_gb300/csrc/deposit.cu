@@ -772,87 +772,113 @@ template <int PM, int QM, bool TRI> __host__ __device__ constexpr int depp_count
     return n;
 }
 
+// FP32 sums of particles run over PXY_SEG particles of the CTA at most, 16 a thread; beyond, sums
+// are pairs of floats (FP64, slow on this part, took 4 us a launch for the same).  One weight for
+// all makes the zeroth moment add the same number every time, so that its rounding is a bias
+// which all threads and CTAs share: over a thread's whole share it was 2.7e-7 (rms) of the
+// density at 2^22 particles, 4e-6 at 2^26 and growing with N.  Four particles are added up first,
+// so the segment's chain of equal terms is four long, which loses nothing.
+#define PXY_SEG 4096
+
+// (s.x + s.y) + v with s.x the rounded sum and s.y what it lost (Knuth's two-sum)
+__device__ __forceinline__ float2 depp_add2(float2 s, float v)
+{
+    const float t = s.x + v, b = t - s.x;
+    return make_float2(t, s.y + ((s.x - (t - b)) + (v - b)));
+}
+
 template <int PM, int QM, bool TRI>
 __device__ __forceinline__ void depp_moments_reg(const DepSrc<float> &S, int64_t i0, int n, const PxyBox &B,
                                                  float *part, float *M)
 {
     constexpr int NM = depp_count<PM, QM, TRI>(PM * QM), QB = 4;
     constexpr int NR = (NM + 31) / 32;
+    static_assert(PXY_SEG % (QB * DEPP_THREADS) == 0, "whole rounds a segment");
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const uint32_t *u = S.u + i0;
     const float *kap = S.kappa ? S.kappa + i0 : nullptr, *w = S.w ? S.w + i0 : nullptr;
-    float acc[NM];
+    float2 *tot = (float2 *)part + warp * 64;  // the warp's sums, moments lane and lane + 32 a lane's own
 #pragma unroll
-    for (int i = 0; i < NM; ++i) acc[i] = 0.f;
+    for (int h = 0; h < NR; ++h) tot[h * 32 + lane] = make_float2(0.f, 0.f);
 #pragma unroll 1
-    for (int b0 = tid; b0 < n; b0 += QB * DEPP_THREADS) {
-        uint32_t ru[QB];
-        float rk[QB], rw[QB];
+    for (int s0 = 0; s0 < n; s0 += PXY_SEG) {
+        const int s1 = min(n, s0 + PXY_SEG);
+        float acc[NM];
 #pragma unroll
-        for (int q = 0; q < QB; ++q) {
-            const int t = b0 + q * DEPP_THREADS;
-            const int j = t < n ? t : 0;
-            ru[q] = u[j];
-            rk[q] = QM > 1 ? kap[j] : 0.f;
-            rw[q] = t < n ? (w ? w[j] : S.w_u) : 0.f;
-        }
+        for (int i = 0; i < NM; ++i) acc[i] = 0.f;
+#pragma unroll 1
+        for (int b0 = s0 + tid; b0 < s1; b0 += QB * DEPP_THREADS) {
+            uint32_t ru[QB];
+            float rk[QB], rw[QB], sum[PM];
 #pragma unroll
-        for (int q = 0; q < QB; ++q) {
-            if (b0 - tid + q * DEPP_THREADS >= n) break;  // the CTA has no particle left
-            const float x = pxy_x(B, ru[q]), x2 = x + x;
-            float tp[PM];
-            tp[0] = rw[q];
-            tp[1] = tp[0] * x;
+            for (int q = 0; q < QB; ++q) {
+                const int t = b0 + q * DEPP_THREADS;
+                const int j = t < s1 ? t : 0;
+                ru[q] = u[j];
+                rk[q] = QM > 1 ? kap[j] : 0.f;
+                rw[q] = t < s1 ? (w ? w[j] : S.w_u) : 0.f;
+            }
 #pragma unroll
-            for (int p = 2; p < PM; ++p) tp[p] = fmaf(x2, tp[p - 1], -tp[p - 2]);
-            if constexpr (QM == 1) {
+            for (int p = 0; p < PM; ++p) sum[p] = 0.f;
 #pragma unroll
-                for (int p = 0; p < PM; ++p) acc[p] += tp[p];
-            } else {
-                float k = rk[q];
-                if (!(k > 0.f && k <= (float)KDE_KAPPA_MAX)) k = depp_kappa(S, k, i0 + b0 + q * DEPP_THREADS);
-                const float sv = (k - B.kc) * B.inv_kh, s2 = sv + sv;
-                // t0 = T_{r-1}(s), t1 = T_r(s)
-                float t0 = 1.f, t1 = sv;
+            for (int q = 0; q < QB; ++q) {
+                if (b0 - tid + q * DEPP_THREADS >= s1) break;  // the CTA has no particle left
+                const float x = pxy_x(B, ru[q]), x2 = x + x;
+                float tp[PM];
+                tp[0] = rw[q];
+                tp[1] = tp[0] * x;
 #pragma unroll
-                for (int p = 0; p < PM; ++p) acc[depp_count<PM, QM, TRI>(p * QM)] += tp[p];
+                for (int p = 2; p < PM; ++p) tp[p] = fmaf(x2, tp[p - 1], -tp[p - 2]);
 #pragma unroll
-                for (int r = 1; r < QM; ++r) {
+                for (int p = 0; p < PM; ++p) sum[p] += tp[p];
+                if constexpr (QM > 1) {
+                    float k = rk[q];
+                    if (!(k > 0.f && k <= (float)KDE_KAPPA_MAX)) k = depp_kappa(S, k, i0 + b0 + q * DEPP_THREADS);
+                    const float sv = (k - B.kc) * B.inv_kh, s2 = sv + sv;
+                    // t0 = T_{r-1}(s), t1 = T_r(s)
+                    float t0 = 1.f, t1 = sv;
 #pragma unroll
-                    for (int p = 0; p < PM; ++p)
-                        if (depp_kept<PM, QM, TRI>(p, r)) {
-                            const int m = depp_count<PM, QM, TRI>(p * QM + r);
-                            acc[m] = fmaf(tp[p], t1, acc[m]);
-                        }
-                    const float t2 = fmaf(s2, t1, -t0);
-                    t0 = t1;
-                    t1 = t2;
+                    for (int r = 1; r < QM; ++r) {
+#pragma unroll
+                        for (int p = 0; p < PM; ++p)
+                            if (depp_kept<PM, QM, TRI>(p, r)) {
+                                const int m = depp_count<PM, QM, TRI>(p * QM + r);
+                                acc[m] = fmaf(tp[p], t1, acc[m]);
+                            }
+                        const float t2 = fmaf(s2, t1, -t0);
+                        t0 = t1;
+                        t1 = t2;
+                    }
                 }
+            }
+#pragma unroll
+            for (int p = 0; p < PM; ++p) acc[depp_count<PM, QM, TRI>(p * QM)] += sum[p];
+        }
+        // lane l has the warp's sums of moments l, l + 32
+        if (NM <= 8) {
+            float mine = 0.f;
+#pragma unroll
+            for (int i = 0; i < NM; ++i) {
+                float v = acc[i];
+#pragma unroll
+                for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+                if (lane == i) mine = v;
+            }
+            tot[lane] = depp_add2(tot[lane], mine);
+        } else {
+#pragma unroll
+            for (int h = 0; h < NR; ++h) {
+                float v[32];
+#pragma unroll
+                for (int i = 0; i < 32; ++i) v[i] = h * 32 + i < NM ? acc[h * 32 + i < NM ? h * 32 + i : 0] : 0.f;
+                tot[h * 32 + lane] = depp_add2(tot[h * 32 + lane], warp_transpose_sum32(v, lane));
             }
         }
     }
-    // lane l of a warp ends with the warp's sums of moments l, l + 32, ...
-    float *pw = part + warp * 64;
-    if (NM <= 8) {
-#pragma unroll
-        for (int i = 0; i < NM; ++i) {
-            float v = acc[i];
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-            if (lane == 0) pw[i] = v;
-        }
-    } else {
-#pragma unroll
-        for (int h = 0; h < NR; ++h) {
-            float v[32];
-#pragma unroll
-            for (int i = 0; i < 32; ++i) v[i] = h * 32 + i < NM ? acc[h * 32 + i < NM ? h * 32 + i : 0] : 0.f;
-            pw[h * 32 + lane] = warp_transpose_sum32(v, lane);
-        }
-    }
+    const float2 *wsum = (const float2 *)part;
     __syncthreads();
     for (int i = tid; i < PM * QM; i += DEPP_THREADS) {
-        float a = 0.f;
+        float2 a = make_float2(0.f, 0.f);
         int m = i;  // position of moment (p, q) among the kept ones
         bool kept = true;
         if (TRI) {
@@ -863,20 +889,35 @@ __device__ __forceinline__ void depp_moments_reg(const DepSrc<float> &S, int64_t
         }
         if (kept) {
 #pragma unroll
-            for (int k = 0; k < DEPP_WARPS; ++k) a += part[k * 64 + m];
+            for (int k = 0; k < DEPP_WARPS; ++k) {
+                const float2 v = wsum[k * 64 + m];
+                a = depp_add2(a, v.x);
+                a.y += v.y;
+            }
         }
-        M[i] = a * S.coef;
+        M[i] = (a.x + a.y) * S.coef;
     }
 }
 
-// moments of any degrees (P <= 16, Q <= 40) as a matrix product; stage: the warp's rows of
-// RS = 4 (LP + LQ) floats (an odd number of 16-byte words)
-__device__ __forceinline__ void depp_moments_mm(const DepSrc<float> &S, int64_t i0, int64_t i1, const PxyBox &B,
-                                                float *stage, float *part, float *M)
+// moments of any degrees (P <= 16, Q <= 40) as a matrix product; mem: the CTA's DEPP_SUB float4.
+// A lane's chain in registers is 64 / KS particles long (half that at KS <= 2), then part adds up
+// those of a segment of PXY_MMSEG particles, and the segments are added up in pairs of floats (the
+// request-size deposit below 472 -> 491 us for the whole call)
+#define PXY_MMSEG 4096
+#define PXY_ROWS (PXY_STAGE * 60)  // floats of a warp's staged rows, RS <= 60 each
+
+__device__ __forceinline__ void depp_moments_mm(const DepSrc<float> &S, int64_t i0, int n, const PxyBox &B,
+                                                float *mem, float *part, float *M)
 {
+    static_assert(DEPP_WARPS * PXY_ROWS + 2 * PXY_MAXP * PXY_MAXQ <= 4 * DEPP_SUB, "rows and sums fit");
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const uint32_t *u = S.u + i0;
+    const float *kap = S.kappa + i0, *w = S.w ? S.w + i0 : nullptr;
+    float *stage = mem + warp * PXY_ROWS;
+    float2 *tot = (float2 *)(mem + DEPP_WARPS * PXY_ROWS);  // the moments of the segments so far
+    float4 *pw = (float4 *)part + warp * 128 + lane;          // part[warp][row of the tile][lane][4]
     const int LP = (B.P + 3) >> 2, LQ = (B.Q + 3) >> 2;
-    const int RS = 4 * ((LP + LQ) | 1);
+    const int RS = 4 * ((LP + LQ) | 1);  // an odd number of 16-byte words
     const int tiles = LP * LQ;
     int KS = 1;  // particles taken at once (power of two, KS tiles <= 32)
     while (2 * KS * tiles <= 32 && 2 * KS <= PXY_STAGE) KS *= 2;
@@ -884,83 +925,102 @@ __device__ __forceinline__ void depp_moments_mm(const DepSrc<float> &S, int64_t 
     const bool on = ks < KS;
     const int row = lane & (PXY_STAGE - 1);  // the particle this lane stages
     const bool roleB = lane >= PXY_STAGE;    // lanes 0..15 the T_p, lanes 16..31 the T_q
-    float acc[4][4];
-#pragma unroll
-    for (int a = 0; a < 4; ++a)
-#pragma unroll
-        for (int b = 0; b < 4; ++b) acc[a][b] = 0.f;
     constexpr int QB = 4;
-    const int64_t step = (int64_t)DEPP_WARPS * PXY_STAGE;
+    constexpr int step = DEPP_WARPS * PXY_STAGE;
+    for (int i = tid; i < B.P * B.Q; i += DEPP_THREADS) tot[i] = make_float2(0.f, 0.f);
 #pragma unroll 1
-    for (int64_t g0 = i0 + warp * PXY_STAGE; g0 < i1; g0 += QB * step) {
-        uint32_t ru[QB];
-        float rk[QB], rw[QB];
+    for (int s0 = 0; s0 < n; s0 += PXY_MMSEG) {
+        const int s1 = min(n, s0 + PXY_MMSEG);
+        float acc[4][4];
 #pragma unroll
-        for (int q = 0; q < QB; ++q) {
-            const int64_t t = g0 + q * step + row;
-            const int64_t j = t < i1 ? t : i0;
-            ru[q] = S.u[j];
-            rk[q] = S.kappa[j];
-            rw[q] = S.w ? S.w[j] : S.w_u;
+        for (int a = 0; a < 4; ++a) {
+            pw[a * 32] = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+            for (int b = 0; b < 4; ++b) acc[a][b] = 0.f;
         }
+        auto fold = [&]() {
+#pragma unroll
+            for (int a = 0; a < 4; ++a) {
+                const float4 v = pw[a * 32];
+                pw[a * 32] = make_float4(v.x + acc[a][0], v.y + acc[a][1], v.z + acc[a][2], v.w + acc[a][3]);
+#pragma unroll
+                for (int b = 0; b < 4; ++b) acc[a][b] = 0.f;
+            }
+        };
 #pragma unroll 1
-        for (int q = 0; q < QB; ++q) {
-            const int64_t t0 = g0 + q * step;
-            if (t0 >= i1) break;
-            const int64_t t = t0 + row;
-            const bool ok = t < i1;
-            // the first of the recurrence: the weight or 1; rows past the end have no weight and sit
-            // in the middle of the box (values far outside it would overflow, and 0 inf is no 0)
-            float z = 0.f, y0 = roleB ? 1.f : 0.f;
-            if (ok) {
-                const float k = depp_kappa(S, rk[0], t);
-                z = roleB ? pxy_s(B, k) : pxy_x(B, ru[0]);
-                if (!roleB) y0 = rw[0] * S.coef * kde_norm_tab(S.ntab, k);
-            }
+        for (int g0 = s0 + warp * PXY_STAGE; g0 < s1; g0 += QB * step) {
+            uint32_t ru[QB];
+            float rk[QB], rw[QB];
 #pragma unroll
-            for (int i = 0; i + 1 < QB; ++i) {
-                ru[i] = ru[i + 1];
-                rk[i] = rk[i + 1];
-                rw[i] = rw[i + 1];
+            for (int q = 0; q < QB; ++q) {
+                const int t = g0 + q * step + row;
+                const int j = t < s1 ? t : 0;
+                ru[q] = u[j];
+                rk[q] = kap[j];
+                rw[q] = w ? w[j] : S.w_u;
             }
-            float y1 = y0 * z;
-            const float z2 = z + z;
-            float4 *dst = (float4 *)(stage + row * RS) + (roleB ? LP : 0);
-            const int n4 = roleB ? LQ : LP;
-            for (int i = 0; i < n4; ++i) {
-                const float y2 = fmaf(z2, y1, -y0), y3 = fmaf(z2, y2, -y1);
-                dst[i] = make_float4(y0, y1, y2, y3);
-                y0 = fmaf(z2, y3, -y2);
-                y1 = fmaf(z2, y0, -y3);
-            }
-            __syncwarp();
-            if (on) {
-#pragma unroll 4
-                for (int r = ks; r < PXY_STAGE; r += KS) {
-                    const float4 A = *(const float4 *)(stage + r * RS + 4 * lp);
-                    const float4 Q4 = *(const float4 *)(stage + r * RS + 4 * (LP + lq));
-                    const float av[4] = {A.x, A.y, A.z, A.w}, bv[4] = {Q4.x, Q4.y, Q4.z, Q4.w};
-#pragma unroll
-                    for (int a = 0; a < 4; ++a)
-#pragma unroll
-                        for (int b = 0; b < 4; ++b) acc[a][b] = fmaf(av[a], bv[b], acc[a][b]);
+#pragma unroll 1
+            for (int q = 0; q < QB; ++q) {
+                const int t0 = g0 + q * step;
+                if (t0 >= s1) break;
+                const bool ok = t0 + row < s1;
+                // the first of the recurrence: the weight or 1; rows past the end have no weight and sit
+                // in the middle of the box (values far outside it would overflow, and 0 inf is no 0)
+                float z = 0.f, y0 = roleB ? 1.f : 0.f;
+                if (ok) {
+                    const float k = depp_kappa(S, rk[0], i0 + t0 + row);
+                    z = roleB ? pxy_s(B, k) : pxy_x(B, ru[0]);
+                    if (!roleB) y0 = rw[0] * S.coef * kde_norm_tab(S.ntab, k);
                 }
-            }
-            __syncwarp();
-        }
-    }
-    // part[warp][lane][16], then moment (p, q) over the warps and their particle groups
-    float4 *pw = (float4 *)part + (warp * 32 + lane) * 4;
 #pragma unroll
-    for (int a = 0; a < 4; ++a) pw[a] = make_float4(acc[a][0], acc[a][1], acc[a][2], acc[a][3]);
-    __syncthreads();
-    for (int i = tid; i < B.P * B.Q; i += DEPP_THREADS) {
-        const int p = i / B.Q, q = i - p * B.Q;
-        const int off = ((p >> 2) * LQ + (q >> 2)) * 16 + (p & 3) * 4 + (q & 3);
-        float a = 0.f;
-        for (int w = 0; w < DEPP_WARPS; ++w)
-            for (int g = 0; g < KS; ++g) a += part[(w * 32 + g * tiles) * 16 + off];
-        M[i] = a;
+                for (int i = 0; i + 1 < QB; ++i) {
+                    ru[i] = ru[i + 1];
+                    rk[i] = rk[i + 1];
+                    rw[i] = rw[i + 1];
+                }
+                float y1 = y0 * z;
+                const float z2 = z + z;
+                float4 *dst = (float4 *)(stage + row * RS) + (roleB ? LP : 0);
+                const int n4 = roleB ? LQ : LP;
+                for (int i = 0; i < n4; ++i) {
+                    const float y2 = fmaf(z2, y1, -y0), y3 = fmaf(z2, y2, -y1);
+                    dst[i] = make_float4(y0, y1, y2, y3);
+                    y0 = fmaf(z2, y3, -y2);
+                    y1 = fmaf(z2, y0, -y3);
+                }
+                __syncwarp();
+                if (on) {
+#pragma unroll 4
+                    for (int r = ks; r < PXY_STAGE; r += KS) {
+                        const float4 A = *(const float4 *)(stage + r * RS + 4 * lp);
+                        const float4 Q4 = *(const float4 *)(stage + r * RS + 4 * (LP + lq));
+                        const float av[4] = {A.x, A.y, A.z, A.w}, bv[4] = {Q4.x, Q4.y, Q4.z, Q4.w};
+#pragma unroll
+                        for (int a = 0; a < 4; ++a)
+#pragma unroll
+                            for (int b = 0; b < 4; ++b) acc[a][b] = fmaf(av[a], bv[b], acc[a][b]);
+                    }
+                }
+                if (KS <= 2 && q == 1) fold();
+                __syncwarp();
+            }
+            fold();
+        }
+        // moment (p, q) over the warps and their particle groups
+        __syncthreads();
+        for (int i = tid; i < B.P * B.Q; i += DEPP_THREADS) {
+            const int p = i / B.Q, q = i - p * B.Q;
+            const int off = ((p & 3) * 32 + (p >> 2) * LQ + (q >> 2)) * 4 + (q & 3);
+            float2 m = tot[i];
+            for (int v = 0; v < DEPP_WARPS; ++v) {
+                float a = 0.f;
+                for (int g = 0; g < KS; ++g) a += part[v * 512 + g * tiles * 4 + off];
+                m = depp_add2(m, a);
+            }
+            tot[i] = m;
+            M[i] = m.x + m.y;
+        }
+        __syncthreads();
     }
 }
 
@@ -1278,7 +1338,7 @@ __global__ void __launch_bounds__(DEPP_THREADS, DEPP_MINB) deposit_persist_kerne
                 depp_moments_reg<8, 6, false>(S, i0, n, B, part, M);
                 depp_proxies_reg<8, 6>(S, B, g_lo, R, M, tabs, mem, part, flush);
             } else {
-                depp_moments_mm(S, i0, i1, B, (float *)rec + warp * (DEPP_SUB * 4 / DEPP_WARPS), part, M);
+                depp_moments_mm(S, i0, n, B, (float *)rec, part, M);
                 depp_proxies(S, B, g_lo, R, M, (float *)rec, part, flush);
             }
             return;

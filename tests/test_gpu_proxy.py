@@ -203,3 +203,27 @@ def test_deposit_of_widths_a_few_roundings_apart(ctx, lo, ulps):
     one = ctx.deposit(ud, Ng, L, kappa_uniform=float(k[0])).cpu().numpy()
     ctx.sync()
     assert rel_l2(rho, one) <= 2 * TOL
+
+
+@pytest.mark.parametrize("N,kap", [(60000000, 14.0), (60000000, "narrow"), (30000000, "wide"), (1 << 24, "outliers")])
+def test_deposit_mass_of_large_samples(ctx, N, kap):
+    # one weight for all: the zeroth moment adds the same number N / (CTAs x threads) times, and
+    # its rounding would be one factor on the whole density.  The grid's mean is exactly 1 (the
+    # kernels' modes beyond the grid are below 1e-17); TOL covers norms (5e-7) and interpolation
+    import torch
+    Ng = 1024 if kap == "wide" else 256
+    g = torch.Generator(device="cuda:0")
+    g.manual_seed(3)
+    u = torch.randint(-(1 << 31), 1 << 31, (N,), generator=g, device="cuda:0", dtype=torch.int64).to(torch.int32)
+    if kap == "outliers":  # one width but for a few
+        k = torch.full((N,), 40.0, device="cuda:0")
+        k[::1000] = 400.0
+        kw = dict(kappa=k)
+    elif isinstance(kap, str):
+        lo, hi = {"narrow": (13.0, 16.0), "wide": (5.0, 2e3)}[kap]
+        kw = dict(kappa=lo * torch.exp(math.log(hi / lo) * torch.rand(N, generator=g, device="cuda:0")))
+    else:
+        kw = dict(kappa_uniform=kap)
+    rho = ctx.deposit(u, Ng, L, **kw)
+    ctx.sync()
+    assert abs(float(rho.double().mean()) - 1) <= TOL
