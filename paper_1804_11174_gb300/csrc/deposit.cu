@@ -1207,7 +1207,7 @@ template <bool COMP>
 __global__ void __launch_bounds__(DEPP_THREADS, DEPP_MINB) deposit_persist_kernel(DepSrc<float> S, DepPlan Pl)
 {
     __shared__ float4 rec[DEPP_SUB];
-    __shared__ float part[DEPP_WARPS * DEPP_PART];
+    __shared__ __align__(16) float part[DEPP_WARPS * DEPP_PART];  // also read as float2 and float4
     __shared__ float sred[2 * DEPP_WARPS];
     __shared__ int s_es;
     constexpr int PER = DEPP_SUB / DEPP_THREADS;  // particles of a sub-chunk per thread

@@ -775,7 +775,7 @@ __global__ void __launch_bounds__(GATT_THREADS, 3) gather_tile_kernel(GatherArgs
     __shared__ uint32_t cd[PXY_MAXP];
     __shared__ float fr[PXY_MAXP], k2[8], nk[8];
     __shared__ float tabs[PXY_MAXP * PXY_MAXP + 8], part[GATT_WARPS * 49], F[2 * 49];
-    __shared__ float s2a[PXY_MAXP * GATT_THREADS];
+    __shared__ __align__(16) float s2a[PXY_MAXP * GATT_THREADS];  // also the energy sum's doubles
     __shared__ __align__(16) float2 C[50];
     __shared__ float kred[2 * GATT_WARPS];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, Ng = A.Ng;
