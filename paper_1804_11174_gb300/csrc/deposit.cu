@@ -1107,7 +1107,7 @@ __device__ __forceinline__ void depp_proxies(const DepSrc<float> &S, const PxyBo
 // norms); mem: 2 PM QM + 2 PM + QM + PM PM + QM QM floats
 template <int PM, int QM, typename F>
 __device__ __forceinline__ void depp_proxies_reg(const DepSrc<float> &S, const PxyBox &B, int g_lo, int R, const float *M,
-                                                 const float *tabs, float *mem, float *part, F &&flush)
+                                                 const float *tabs, bool shared_range, float *mem, float *part, F &&flush)
 {
     constexpr int PQ = PM * QM;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, Ng = S.Ng;
@@ -1126,7 +1126,7 @@ __device__ __forceinline__ void depp_proxies_reg(const DepSrc<float> &S, const P
         const float k = QM > 1 ? pxy_lin_kappa(B.kc, B.kh, cq[QM + b], QM) : B.kc;
         k2[b] = (float)(-2.0 * KDE_LOG2E) * k;
         if (!S.kappa) nk[b] = S.norm_u;
-        else if (QM > 1 && S.krange) nk[b] = __uint_as_float(S.krange[(QM == 7 ? PXY_NORM7 : PXY_NORM6) + b]);
+        else if (QM > 1 && shared_range) nk[b] = __uint_as_float(S.krange[(QM == 7 ? PXY_NORM7 : PXY_NORM6) + b]);
         else nk[b] = kde_norm_tab(S.ntab, k);
     }
     __syncthreads();  // also: the moments are written
@@ -1218,29 +1218,39 @@ __global__ void __launch_bounds__(DEPP_THREADS, DEPP_MINB) deposit_persist_kerne
     kde_pdl_wait();  // everything read below comes from the sort before
     kde_pdl_trigger();
 
-    // smallest and largest width of the CTA's particles (the window and the form): a pass
-    // over the widths, PER loads in flight per thread
+    // smallest and largest width of the CTA's particles (the window and the form): the range of all
+    // where it is known and narrow, else a pass over the CTA's widths, PER loads in flight per
+    // thread -- a few wide kernels among narrow ones, or widths that follow the density, would
+    // otherwise give every CTA the widest one's window (one width in 1e5 5 and the others 2000, a run
+    // of 10 steps: 2^18 particles on 256 nodes 445 us with the range of all, 397 with the CTAs',
+    // 2^20 on 1024 nodes 1587 and 1297)
     float kmin = (float)KDE_KAPPA_MAX, kmax = 0.f;
+    bool shared_range = false;
     if (S.krange) {
-        kmax = __uint_as_float(S.krange[0]);
-        kmin = __uint_as_float(S.krange[1]);
-    } else if (!S.kappa) {
-        kmin = kmax = S.kappa_u;
-    } else
-    for (int64_t j0 = i0; j0 < i1; j0 += (int64_t)PER * DEPP_THREADS) {
-        float kk[PER];
-#pragma unroll
-        for (int p = 0; p < PER; ++p) {
-            const int64_t j = j0 + tid + p * DEPP_THREADS;
-            kk[p] = j < i1 ? S.kappa[j] : -1.f;
+        const float hi = __uint_as_float(S.krange[0]), lo = __uint_as_float(S.krange[1]);
+        shared_range = pxy_narrow(lo, hi);
+        if (shared_range) {
+            kmax = hi;
+            kmin = lo;
         }
+    }
+    if (!S.kappa) {
+        kmin = kmax = S.kappa_u;
+    } else if (!shared_range) {
+        for (int64_t j0 = i0; j0 < i1; j0 += (int64_t)PER * DEPP_THREADS) {
+            float kk[PER];
 #pragma unroll
-        for (int p = 0; p < PER; ++p)
-            if (kk[p] != -1.f) {
+            for (int p = 0; p < PER; ++p) {
+                const int64_t j = j0 + tid + p * DEPP_THREADS;
+                kk[p] = S.kappa[j < i1 ? j : i0];
+            }
+#pragma unroll
+            for (int p = 0; p < PER; ++p) {
                 const float k = (kk[p] > 0.f && kk[p] <= (float)KDE_KAPPA_MAX) ? kk[p] : (float)KDE_KAPPA_MAX;
                 kmin = fminf(kmin, k);
                 kmax = fmaxf(kmax, k);
             }
+        }
     }
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) {
@@ -1324,19 +1334,19 @@ __global__ void __launch_bounds__(DEPP_THREADS, DEPP_MINB) deposit_persist_kerne
             if (B.Q == 1 && B.P <= 8) {
                 load_tabs(8, 1);
                 depp_moments_reg<8, 1, false>(S, i0, n, B, part, M);
-                depp_proxies_reg<8, 1>(S, B, g_lo, R, M, tabs, mem, part, flush);
+                depp_proxies_reg<8, 1>(S, B, g_lo, R, M, tabs, shared_range, mem, part, flush);
             } else if (B.Q == 1) {
                 load_tabs(16, 1);
                 depp_moments_reg<16, 1, false>(S, i0, n, B, part, M);
-                depp_proxies_reg<16, 1>(S, B, g_lo, R, M, tabs, mem, part, flush);
+                depp_proxies_reg<16, 1>(S, B, g_lo, R, M, tabs, shared_range, mem, part, flush);
             } else if (B.lin && B.P <= 6) {
                 load_tabs(7, 7);
                 depp_moments_reg<7, 7, true>(S, i0, n, B, part, M);
-                depp_proxies_reg<7, 7>(S, B, g_lo, R, M, tabs, mem, part, flush);
+                depp_proxies_reg<7, 7>(S, B, g_lo, R, M, tabs, shared_range, mem, part, flush);
             } else if (B.lin && B.P <= 8) {
                 load_tabs(8, 6);
                 depp_moments_reg<8, 6, false>(S, i0, n, B, part, M);
-                depp_proxies_reg<8, 6>(S, B, g_lo, R, M, tabs, mem, part, flush);
+                depp_proxies_reg<8, 6>(S, B, g_lo, R, M, tabs, shared_range, mem, part, flush);
             } else {
                 depp_moments_mm(S, i0, n, B, (float *)rec, part, M);
                 depp_proxies(S, B, g_lo, R, M, (float *)rec, part, flush);

@@ -98,6 +98,8 @@ __device__ __forceinline__ void pxy_box_pos(PxyBox &B, const PxyGrid &G, int c_f
     B.inv_hw = 1.f / B.hw;
     B.P = pxy_degree_pos(B.hw * (float)(KDE_TWO_PI / 4294967296.0) * sqrtf(kmax + 1.5f));
 }
+// a range of widths narrow enough for the linear map
+__device__ __forceinline__ bool pxy_narrow(float kmin, float kmax) { return kmax - kmin <= PXY_LIN_R * (kmax + kmin); }
 // middle and half-length of a narrow range of widths.  The middle is rounded, so over a range of
 // a few roundings the ends would lie outside [-1, 1] (at 2 for two neighbouring floats, where the
 // highest polynomials reach 1e3 and their rounding 1e-5 of the result): at least 1e-5 of the
@@ -109,7 +111,7 @@ __device__ __forceinline__ void pxy_lin_range(float kmin, float kmax, float &kc,
 }
 __device__ __forceinline__ void pxy_box_width(PxyBox &B, float kmin, float kmax)
 {
-    B.lin = kmax - kmin <= PXY_LIN_R * (kmax + kmin);
+    B.lin = pxy_narrow(kmin, kmax);
     if (kmin == kmax) {
         B.Q = 1;
         B.kc = kmin;
