@@ -1053,28 +1053,28 @@ __global__ void adapt_apply_kernel(const float *loo, int64_t N, const AdaptPar *
                                    unsigned int *krange)
 {
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= N) {
-        if (krange) kde_krange_add(krange, 3.0e38f, 0.f);
-        return;
-    }
+    const bool in = i < N;
+    const float lo_i = in ? loo[i] : 1.f;
     // lambda = (f/g)^-alpha, kappa = kappa* / lambda^2; FP32 widths in FP32 with base-2
     // logarithms (the log-mean of adapt_logsum_dev_kernel<true> is in the same base), FP64
     // widths in FP64 with natural ones
     T k;
     if constexpr (sizeof(T) == 4) {
-        const float f = fmaf(P->a, loo[i], P->b);
+        const float f = fmaf(P->a, lo_i, P->b);
         float kf = P->ks_f * exp2f((float)(2.0 * alpha) * (log2f(f) - P->logg_f));
         kf = kf < (float)kmin ? (float)kmin : (kf > (float)kmax ? (float)kmax : kf);
         k = kf;
     } else {
         const double n = (double)N;
-        const double f = ((n - 1.0) * (double)loo[i] + P->K0) / n;
+        const double f = ((n - 1.0) * (double)lo_i + P->K0) / n;
         double kd = P->ks * exp(2.0 * alpha * (log(f) - P->logg));
         kd = kd < kmin ? kmin : (kd > kmax ? kmax : kd);
         k = kd;
     }
+    // all lanes of a warp together
+    if (krange) kde_krange_add(krange, in ? (float)k : 3.0e38f, in ? (float)k : 0.f);
+    if (!in) return;
     kappa_out[i] = k;
-    if (krange) kde_krange_add(krange, (float)k, (float)k);
     if (norm_out) {
         // FP32 widths take the tabulated norm, FP64 widths the FP64 Bessel series
         if constexpr (sizeof(T) == 4) norm_out[i] = (T)kde_norm_tab(ntab, (float)k);

@@ -18,17 +18,15 @@ __global__ void norm_from_kappa_kernel(const T *kappa, int64_t N, T *norm, unsig
                                        unsigned int *krange)
 {
     int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= N) {
-        if (krange) kde_krange_add(krange, 3.0e38f, 0.f);
-        return;
-    }
-    double k = (double)kappa[i];
+    const bool in = i < N;
+    double k = in ? (double)kappa[i] : 1.0;
     if (!(k > 0 && k <= KDE_KAPPA_MAX)) {
         kde_flag(status, KDE_DEV_KAPPA_RANGE, (unsigned)i);
         k = KDE_KAPPA_MAX;
     }
-    // the range of the widths as the deposit and the gather use them
-    if (krange) kde_krange_add(krange, (float)k, (float)k);
+    // the range of the widths as the deposit and the gather use them (all lanes of a warp together)
+    if (krange) kde_krange_add(krange, in ? (float)k : 3.0e38f, in ? (float)k : 0.f);
+    if (!in) return;
     // FP32 state: the tabulated norm; FP64 state: the FP64 Bessel series
     if constexpr (sizeof(T) == 4) norm[i] = (T)kde_norm_tab(ntab, (float)k);
     else norm[i] = (T)f64_norm(k);
