@@ -549,7 +549,7 @@ __global__ void __launch_bounds__(DEP_THREADS) deposit64_kernel(DepSrc<double> S
 struct DepPlan {
     int G;            // CTAs
     long long *acc;   // [Ng] node sums, zero before
-    float fixed;      // cost of the compressed form's fixed steps (depp_compress_pays)
+    float inv_share;  // 1 / CTAs an SM, at most DEPP_MINB of them (depp_compress_pays)
 };
 // node pairs of the persistent deposit: each lane owns P pairs of nodes (64 P
 // consecutive nodes a warp pass) of the window [g_lo, g_lo + R); the n records of
@@ -1184,22 +1184,48 @@ __device__ __forceinline__ void depp_proxies_reg(const DepSrc<float> &S, const P
     }
 }
 
-// whether the compressed form costs less than the direct sweep: instructions of a lane,
-// direct about 3.2 a (particle, node) pair and 48 a particle; compressed 55 a particle plus
-// its Chebyshev values and moments (shared by the lanes of a warp), then 16 a (node, proxy
-// position), 3 a (node, proxy), the interpolation matrices and the fixed steps -- barriers and
-// table loads, which other CTAs cover where an SM has three but not where it has one.  Near
-// the lines: 658 particles a CTA in windows of 27 nodes with P = 11 (300,007 particles, 512
-// nodes, width 2000) take 10.5 us direct and 13.5 compressed; a PIC step of 3202 particles on
-// 118 nodes 39 us direct and 44 compressed
-__device__ __forceinline__ bool depp_compress_pays(const PxyBox &B, int n, int R, float fixed)
+// the register forms: 1, 2 one width with P <= 8 or 16, 3, 4 a narrow range of widths with P <= 6 or 8;
+// 5 the matrix product, 0 degrees beyond it (its moment tiles have to fit a warp)
+__device__ __forceinline__ int depp_form(const PxyBox &B)
 {
-    // the moment tiles of the matrix product have to fit a warp
-    if (B.P > PXY_MAXP || B.Q > PXY_MAXQ || ((B.P + 3) >> 2) * ((B.Q + 3) >> 2) > 32) return false;
-    const float fn = (float)n, fR = (float)R, P = (float)B.P, Q = (float)B.Q, PQ = P * Q;
-    const float direct = fn * (3.2f * fR + 48.f);
-    const float comp = fn * (55.f + 3.f * (P + Q) + 1.6f * PQ) + fR * P * (16.f + 3.f * Q) + PQ * (P + Q) * 4.f + fixed;
-    return comp < direct;
+    if (B.P > PXY_MAXP || B.Q > PXY_MAXQ || ((B.P + 3) >> 2) * ((B.Q + 3) >> 2) > 32) return 0;
+    if (B.Q == 1) return B.P <= 8 ? 1 : 2;
+    return B.lin && B.P <= 8 ? (B.P <= 6 ? 3 : 4) : 5;
+}
+
+// Costs of the forms in ns of an SM, per CTA, fitted to 867 launches with either form forced (40,000 to
+// 4,000,037 particles, 64 to 4096 nodes, uniform widths and ranges from 0.5 to 20,000; 5 to 9% off).
+// What a launch waits for once (barriers, table loads, the chain of small steps), /share of it a
+// CTA, is beyond the sweep's.  Deposits of a PIC step, swept and compressed: widths of 7 to 20 on 256
+// nodes, 65,536 particles 12.9 and 18.3 us, 2^20 48.7 and 44.7, on 1024 nodes 20.5 and 24.2, 152 and
+// 51 (form 5); widths near 315, 1024 nodes, 131,072 particles 12.2 and 12.5, 4,000,037 121 and 35
+// (form 4); width 5000 on 256 nodes, 2^20 particles 14.2 and 16.3 (form 2); width 14 on 512 nodes,
+// 524,288 particles 37.9 and 11.2 (form 1)
+__host__ __device__ inline float depp_sweep_ns(float n, float R, bool cosf, float inv_share)
+{
+    return n * fmaf(cosf ? 0.0196f : 0.0229f, R, 0.82f) + 4.5f * R * inv_share;
+}
+// cost c.x n + c.y R + (c.z + c.w R) / share of the register forms
+__host__ __device__ inline float4 depp_reg_cost(int form)
+{
+    return form == 1 ? make_float4(0.47f, 0.7f, 180.f, 0.8f)
+                     : (form == 2 ? make_float4(0.53f, 2.0f, 500.f, 0.f)
+                                  : (form == 3 ? make_float4(0.61f, 1.03f, 1450.f, 1.45f) : make_float4(0.89f, 2.1f, 2300.f, 0.f)));
+}
+__device__ __forceinline__ bool depp_compress_pays(const PxyBox &B, int form, int n, int R, bool cosf, float inv_share)
+{
+    // nodes as the sweep's warps take them
+    const int Rs = R > 128 ? (R + 63) & ~63 : (R > 64 ? 128 : (R > 32 ? 64 : (R > 16 ? 32 : (R > 8 ? 16 : 8))));
+    const float direct = depp_sweep_ns((float)n, (float)Rs, cosf, inv_share);
+    float4 c = depp_reg_cost(form);
+    if (form == 5) {
+        const float P = (float)B.P, Q = (float)B.Q;
+        const int LP = (B.P + 3) >> 2, LQ = (B.Q + 3) >> 2, tiles = LP * LQ;
+        const float iKS = tiles > 16 ? 1.f : (tiles > 8 ? 0.5f : (tiles > 4 ? 0.25f : 0.125f));  // 1 / particles taken at once
+        c = make_float4(2.9f + 4.4f * iKS + 0.04f * (float)max(LP, LQ), P * (0.615f + 0.0022f * Q),
+                        4150.f + 0.53f * P * Q * (P + Q), 0.f);
+    }
+    return form && (float)n * c.x + (float)R * c.y + fmaf(c.w, (float)R, c.z) * inv_share < direct;
 }
 
 // COMP: with the compressed form, chosen per CTA; without it where no CTA would take it
@@ -1322,7 +1348,8 @@ __global__ void __launch_bounds__(DEPP_THREADS, DEPP_MINB) deposit_persist_kerne
         pxy_box_pos(B, S.grid, c_first, c_last, kmax);
         pxy_box_width(B, kmin, kmax);
         const int n = (int)(i1 - i0);
-        if (depp_compress_pays(B, n, R, Pl.fixed)) {
+        const int form = depp_form(B);
+        if (depp_compress_pays(B, form, n, R, cosf, Pl.inv_share)) {
             __shared__ float M[PXY_MAXP * PXY_MAXQ];
             // the register forms' interpolation matrices, beside the records' space
             float *tabs = (float *)rec, *mem = tabs + PXY_MAXP * PXY_MAXP + 64;
@@ -1331,19 +1358,19 @@ __global__ void __launch_bounds__(DEPP_THREADS, DEPP_MINB) deposit_persist_kerne
                 for (int i = tid; i < P * P; i += DEPP_THREADS) tabs[i] = cp[i];
                 if (tid < Q * Q) tabs[P * P + tid] = cq[tid];
             };
-            if (B.Q == 1 && B.P <= 8) {
+            if (form == 1) {
                 load_tabs(8, 1);
                 depp_moments_reg<8, 1, false>(S, i0, n, B, part, M);
                 depp_proxies_reg<8, 1>(S, B, g_lo, R, M, tabs, shared_range, mem, part, flush);
-            } else if (B.Q == 1) {
+            } else if (form == 2) {
                 load_tabs(16, 1);
                 depp_moments_reg<16, 1, false>(S, i0, n, B, part, M);
                 depp_proxies_reg<16, 1>(S, B, g_lo, R, M, tabs, shared_range, mem, part, flush);
-            } else if (B.lin && B.P <= 6) {
+            } else if (form == 3) {
                 load_tabs(7, 7);
                 depp_moments_reg<7, 7, true>(S, i0, n, B, part, M);
                 depp_proxies_reg<7, 7>(S, B, g_lo, R, M, tabs, shared_range, mem, part, flush);
-            } else if (B.lin && B.P <= 8) {
+            } else if (form == 4) {
                 load_tabs(8, 6);
                 depp_moments_reg<8, 6, false>(S, i0, n, B, part, M);
                 depp_proxies_reg<8, 6>(S, B, g_lo, R, M, tabs, shared_range, mem, part, flush);
@@ -1569,17 +1596,32 @@ static kde_status deposit_sorted_impl(kde_ctx *ctx, const uint32_t *u, const T *
         const int64_t gn = nbins < 0 ? (N + 63) / 64 : (N + 255) / 256;
         Pl.G = (int)(gn < gmax ? gn : gmax);
         Pl.acc = acc;
-        Pl.fixed = Pl.G <= ctx->sm_count ? 3.0e5f : 6.0e4f;
+        const float share = std::max(1.f, std::min((float)DEPP_MINB, (float)Pl.G / (float)(ctx->sm_count > 0 ? ctx->sm_count : 1)));
+        Pl.inv_share = 1.f / share;
         {
             KdeProfScope _ps(ctx, PROF_DEPOSIT);
             // the compressed form is for the default cut (one the caller has set keeps the sweep
-            // over the particles that it is defined for), and for CTAs whose sweep of the whole
-            // grid would cost more than its fixed steps
-            // A width schedule's few CTAs sweep too: their proxies share seven widths, whose rounding
-            // few CTAs average (66 CTAs, 16,832 particles: field energies 1.0 to 1.6e-6 off, swept
-            // 0.3 to 1.0e-6; 157 CTAs: 0.1 to 1.0e-6 against 0.4 to 1.6e-6)
-            const double n = (double)N / Pl.G;
-            const bool comp = nbins >= 0 && !(krange && Pl.G < 128) && S.xcut == (float)KDE_XCUT && n * (3.2 * Ng + 48.0) > (double)Pl.fixed;
+            // over the particles that it is defined for), and where the best that can be expected of
+            // it spares 0.3 us (the kernel that chooses takes up to 2 us longer when it then sweeps:
+            // particle-wise widths, 2^20 particles on 64 nodes 26.7 against 24.8 us).  One width has a form
+            // by the positions of an average CTA; particle-wise widths form 3 at best, with P <= 6 on
+            // fewer than 80 nodes only for widths below 15.
+            // The few CTAs of a PIC run with particle-wise widths sweep too: their proxies share
+            // seven widths, whose rounding few CTAs average (66 CTAs, 16,832 particles: field energies
+            // 1.0 to 1.6e-6 off, swept 0.3 to 1.0e-6; 157 CTAs: 0.1 to 1.0e-6 against 0.4 to 1.6e-6)
+            const float n = (float)((double)N / Pl.G);
+            int form = Ng < 80 ? 0 : 3;
+            double Rw = Ng;
+            if (!kappa) {
+                const double cells = std::min((double)Ng, (double)Ng / Pl.G + 1.0);
+                const double y = KDE_PI * cells / Ng * sqrt((double)kappa_u + 1.5);
+                form = y <= 0.388 ? 1 : (y <= 1.65 ? 2 : 0);
+                Rw = std::min(Rw, 2.0 * kde_window_nodes((double)kappa_u, Ng) + cells);
+            }
+            const float4 c = depp_reg_cost(form);
+            const float gain = depp_sweep_ns(n, (float)Rw, true, Pl.inv_share) - n * c.x - (float)Rw * c.y -
+                               (c.z + c.w * (float)Rw) * Pl.inv_share;
+            const bool comp = nbins >= 0 && !(krange && Pl.G < 128) && S.xcut == (float)KDE_XCUT && form && gain * share > 300.f;
             KDE_CUDA(ctx,
                      kde_launch(ctx, true, comp ? deposit_persist_kernel<true> : deposit_persist_kernel<false>,
                                 dim3(Pl.G), dim3(DEPP_THREADS), 0, S, Pl),
