@@ -514,8 +514,12 @@ kde_status kde_deposit_sums_f32(kde_ctx *ctx, const uint32_t *u, const float *ka
 // the PIC step's field from those sums: rho_total = background + charge * rho with its
 // mean removed (so the constant background drops out), E by the spectral or
 // finite-difference Green's function (FP32 output)
+// late: with a smallest width (krange) of at most this the kernel lets the next one start when it
+// is done instead of at once
 kde_status kde_field_from_sums(kde_ctx *ctx, const DepSums &ds, int Ng, double L, double acc_inv, double charge, bool fd,
-                               float *E_out);
+                               float *E_out, float late = 0.f, const unsigned int *krange = nullptr);
+// that width for a step's gather (gather.cu)
+float kde_gather_crowds(kde_ctx *ctx, int64_t N, int Ng, bool per_particle, const unsigned int *krange, float xcut);
 
 // Poisson solve of rho_total = background + charge * rho, rho given as a real
 // array or as int64 accumulators (value = acc * acc_inv; in FP64 with the remainders of the

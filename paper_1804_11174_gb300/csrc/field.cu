@@ -72,17 +72,19 @@ __global__ void __launch_bounds__(POI_THREADS)
 
 __global__ void __launch_bounds__(FIELD_THREADS)
     field_sums_kernel(const long long *__restrict__ acc, long long *__restrict__ next, int Ng, int per, float scale62,
-                      float inv_ng, const float *__restrict__ Gf, float *E)
+                      float inv_ng, const float *__restrict__ Gf, float *E, float late,
+                      const unsigned int *krange)
 {
     __shared__ float rt[KDE_MAX_NG];
     __shared__ float gs[KDE_MAX_NG];
     __shared__ long long red[2 * FIELD_WARPS];
     constexpr int PT = KDE_MAX_NG / FIELD_THREADS;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const bool at_end = late > 0.f && __uint_as_float(krange[1]) <= late;  // written before the sort
     // the sums come from the deposit before, and on a grid's first use the Green's function from
     // a kernel launched between the two
     kde_pdl_wait();
-    kde_pdl_trigger();
+    if (!at_end) kde_pdl_trigger();  // else the CTA's end triggers
     long long n[PT];
     float gv[PT];
     long long hi = 0, lo = 0;
@@ -144,7 +146,7 @@ __global__ void __launch_bounds__(FIELD_THREADS)
 }
 
 kde_status kde_field_from_sums(kde_ctx *ctx, const DepSums &ds, int Ng, double L, double acc_inv, double charge, bool fd,
-                               float *E_out)
+                               float *E_out, float late, const unsigned int *krange)
 {
     const float *Gf = (const float *)kde_green_table(ctx, Ng, L, fd, false);
     if (!Gf) return KDE_ENOMEM;
@@ -156,7 +158,7 @@ kde_status kde_field_from_sums(kde_ctx *ctx, const DepSums &ds, int Ng, double L
         KdeProfScope _ps(ctx, PROF_POISSON);
         KDE_CUDA(ctx, kde_launch(ctx, true, field_sums_kernel, dim3((Ng + per - 1) / per), dim3(FIELD_THREADS), 0,
                                  (const long long *)ds.acc, ds.next, Ng, per, (float)(charge * acc_inv * 0x1p62),
-                                 1.f / (float)Ng, Gf, E_out),
+                                 1.f / (float)Ng, Gf, E_out, krange ? late : 0.f, krange),
                  "field_sums_kernel");
     }
     KDE_LAUNCHED(ctx, "field_sums_kernel");

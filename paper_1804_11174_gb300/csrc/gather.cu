@@ -1018,6 +1018,28 @@ static bool gatt_applies(kde_ctx *ctx, GatherArgs<float> &A)
     return y < 1.6 && n * (y < 0.38 ? 26.0 : 33.0) + R * (y < 0.38 ? 40.0 : 80.0) + 60000.0 < n * 2.6 * R;
 }
 
+// Whether the step's gather is gather2_kernel with few blocks for the chip: launched while the field
+// kernel's CTAs hold some SMs, its blocks crowd on the others, and where the windows are long that
+// kernel should let it start only at its end: where the smallest width is at most the value returned (0:
+// never).  Steps with widths over three decades (windows of the whole grid), started at once and at
+// the end: 65,536 particles, 4096 nodes 215 and 181 us; 131,072, 1024 nodes 97 and 74; 262,144, 1024
+// nodes 139 and 121; 131,072, 512 nodes 52.6 and 47.9, 256 nodes 36.5 and 35.2.  With blocks for less than half or for most
+// of the chip, or shorter windows, it costs the 1 to 3 us of overlap: 16,384, 1024 nodes 50.0 and 52.0,
+// 131,072, 4096 nodes 246 and 247, 262,144, 256 nodes 45.2 and 46.5; 60,000, 512 nodes 41 and 43;
+// widths near 315 (windows of 55 nodes), 60,000, 512 nodes 26.3 and 29.2.
+float kde_gather_crowds(kde_ctx *ctx, int64_t N, int Ng, bool per_particle, const unsigned int *krange, float xcut)
+{
+    if (!per_particle) return 0.f;  // one width: short windows, the others take tiles
+    if (krange && xcut == (float)KDE_XCUT && N >= 64 * GATT_UNIT) return 0.f;
+    const int64_t sms = ctx->sm_count > 0 ? ctx->sm_count : 1, blocks = (N + 511) / 512;
+    const int64_t fit = std::min<int64_t>(7, 227 * 1024 / ((int64_t)Ng * (sizeof(float4) + sizeof(float2)) + 2064));
+    if (2 * blocks <= sms || 2 * blocks > fit * sms) return 0.f;
+    const int nodes = blocks < sms ? 768 : (blocks <= 2 * sms ? 256 : 384);  // the shortest window it is for
+    if (Ng < nodes) return 0.f;
+    const double s = sin(KDE_PI * nodes / (2.0 * Ng));
+    return (float)((double)xcut * KDE_LN2 / (2.0 * s * s));
+}
+
 static kde_status gatt_launch(kde_ctx *ctx, GatherArgs<float> &A)
 {
     static bool attr = false;

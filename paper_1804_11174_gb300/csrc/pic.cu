@@ -365,7 +365,8 @@ static kde_status pic_run(kde_ctx *ctx, pic_state *st, int n_steps)
             }
             {
                 KdeRange r_("kdepic field (Poisson)");
-                KDE_TRY(kde_field_from_sums(ctx, ds, Ng, L, 1.0 / kde_acc_scale(bound), st->charge, fd, (float *)E));
+                KDE_TRY(kde_field_from_sums(ctx, ds, Ng, L, 1.0 / kde_acc_scale(bound), st->charge, fd, (float *)E,
+                                            kde_gather_crowds(ctx, N, Ng, per, sched ? krange : nullptr, cut), krange));
             }
         } else {
             {

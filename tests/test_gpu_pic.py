@@ -447,3 +447,21 @@ def test_first_step_on_a_new_grid(kp):
                 assert np.array_equal(a, b), (Ng, i)
     finally:
         c.close()
+
+
+@pytest.mark.parametrize("N, Ng, lo", [(131072, 1024, 5.0), (70001, 4096, 5.0), (131072, 512, 2000.0)])
+def test_gather_started_late_is_bitwise_neutral(ctx, kp, N, Ng, lo):
+    # wide kernels on few blocks: the field kernel lets the gather start at its end; narrow ones, at
+    # once.  Either way as in plain stream order
+    u, v = I.landau_load(45, N, 4 * math.pi, 0.05, 1.0)
+    k = I.log_uniform(5, I.STREAM_KAPPA, N, lo, 5e3).astype(np.float32)
+    states = [make_state(kp, u, v.astype(np.float32), 4 * math.pi, Ng, 0.1, 6, kappa=k) for _ in range(2)]
+    try:
+        for st, on in zip(states, (True, False)):
+            ctx.set_launch_overlap(on)
+            ctx.pic_step(st, 6)
+            ctx.sync()
+    finally:
+        ctx.set_launch_overlap(True)
+    for t in ("u", "v", "id", "energy"):
+        assert torch.equal(getattr(states[0], t), getattr(states[1], t)), t
