@@ -999,10 +999,14 @@ static kde_status gat2_variant(kde_ctx *ctx, const GatherArgs<float> &A, int v)
 static int gatt_tile(kde_ctx *ctx, const GatherArgs<float> &A)
 {
     // one wave of three CTAs an SM, whole rounds of 1024 particles, which spread the tile's
-    // fixed steps (a warp's 128 particles stay in one tile of the sort)
+    // fixed steps (a warp's 128 particles stay in one tile of the sort).  Particle-wise widths,
+    // whose tiles may sweep their nodes: shares of whole warps above 1024 particles, since whole rounds left
+    // a quarter of the slots empty at 2^20 (50 steps with widths over a factor of three: 256 nodes 4.37
+    // -> 4.18 ms, 1024 nodes 6.66 -> 6.08; one width on 512 nodes, which interpolates, 0.36 -> 0.38)
     const int64_t slots = 3LL * (ctx->sm_count > 0 ? ctx->sm_count : 1);
-    const int64_t units = (A.N + GATT_UNIT - 1) / GATT_UNIT;
-    return (int)((units + slots - 1) / slots * GATT_UNIT);
+    const int64_t step = A.kappa && A.N > slots * GATT_UNIT ? 128 : GATT_UNIT;
+    const int64_t units = (A.N + step - 1) / step;
+    return (int)((units + slots - 1) / slots * step);
 }
 static bool gatt_applies(kde_ctx *ctx, GatherArgs<float> &A)
 {

@@ -247,3 +247,42 @@ def test_width_range_of_a_partial_warp(ctx, kp, oracle, N, low):
     r = oracle.pic_run(I.from_fixed(u, L), v.astype(np.float32), L, Ng, dt, 1, kappa=k.astype(np.float64))
     np.testing.assert_allclose(st.energy.cpu().numpy()[:1], r["energy"], rtol=1e-5)
     assert rel_l2(st.v.cpu().numpy()[np.argsort(st.id.cpu().numpy())], r["v"]) <= 1e-5
+
+
+# Scheduled widths of 2^16 particles and more, whose gather takes its tiles' interpolants: Silverman widths of
+# one candidate, so that the widths' law is the oracle's.  The tiles have P <= 6 ("six") or P = 7, 8
+# ("eight"); the widths of the box vary by a few per cent or, with half the density modulated, by a
+# factor of three, and then over a tile by a few per cent; widths of a noisy pilot (alpha = 2) vary
+# by much in every tile, which then sweeps its nodes
+@pytest.mark.parametrize("N,Ng,amp,kstar,alpha", [
+    (131072, 256, 0.05, 14.0, 0.5), (70001, 256, 0.05, 14.0, 0.5), (131072, 256, 0.5, 14.0, 0.5),
+    (70001, 256, 0.5, 14.0, 0.5), (131077, 1000, 0.5, 40.0, 0.5), (70001, 1024, 0.5, 14.0, 0.5),
+    (70001, 256, 0.5, 3000.0, 2.0), (65537, 4096, 0.5, 300.0, 2.0)],
+    ids=["narrow six", "narrow eight", "tile six", "tile eight", "tile, odd grid", "tile eight, fine grid", "noisy",
+         "noisy, fine grid"])
+def test_scheduled_step_against_oracle(ctx, kp, oracle, N, Ng, amp, kstar, alpha):
+    # particles at rest: the velocity after a step is half a kick, the field at the particle.
+    # Tolerance: deposit and gather within TOL of the density's norm and the field's; the density's
+    # modulated part, whose field this is, is a 28th (5%) or a third (50%) of that norm, and noise
+    # of the kernels' widths adds about as much as the modulation at alpha = 2
+    import torch
+    dt = 1.0
+    u, _ = I.landau_load(N + Ng, N, L, amp, 1.0)
+    v = np.zeros(N, np.float32)
+    cand = np.array([kstar])
+    kw = dict(width_every=10, alpha=alpha, kappa_min=1.0, kappa_max=1e5)
+    st = kp.PicState(to_dev_u(u), to_dev(v), L, Ng, dt, kappa=torch.ones(N, device="cuda:0"), cand=cand, max_steps=1,
+                     ids=torch.arange(N, dtype=torch.int32, device="cuda:0"), **kw)
+    ctx.pic_step(st, 1)
+    ctx.sync()
+    r = oracle.pic_run(I.from_fixed(u, L), v, L, Ng, dt, 1, kappa=np.ones(N), cands=cand, width_every=10, alpha=alpha,
+                       kmin=1.0, kmax=1e5)
+    at = np.argsort(st.id.cpu().numpy())
+    k = st.kappa.double().cpu().numpy()[at]
+    print("widths from %g to %g" % (k.min(), k.max()))
+    tol = TOL * (28 if amp < 0.1 else 3)
+    assert rel_l2(k, r["kappa"]) <= 4 * TOL
+    np.testing.assert_allclose(st.energy.cpu().numpy()[:1], r["energy"], rtol=2 * tol)
+    vg = st.v.double().cpu().numpy()[at]
+    assert rel_l2(vg, r["v"]) <= tol
+    assert np.max(np.abs(vg - r["v"])) <= 3 * tol * np.max(np.abs(r["v"]))
