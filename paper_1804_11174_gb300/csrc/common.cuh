@@ -130,6 +130,7 @@ struct kde_ctx {
     double *f64_tab = nullptr;   // 2^(j / 2048) for the FP64 kernels (fp64.cuh), built at creation
     float *pxy_tab = nullptr;    // interpolation matrices (proxy.cuh), built at creation
     unsigned wait_polls = 1u << 26;         // polls of a bounded device wait (kde_set_wait_limit)
+    bool range_reset = false;               // the gathering words of WS_PIC_RANGE are reset
     bool sums_zero = false;                 // kde_deposit's grid of node sums is zero
     bool sums_flip = false;                 // which grid of node sums the next FP32 deposit adds to
     bool count_flip = false;                // which sort count table the next counted sort reads (sort.cu)
@@ -611,11 +612,9 @@ kde_status kde_adapt_device(kde_ctx *ctx, const float *loo, int64_t N, double L,
                             double kstar_host, double alpha, double kmin, double kmax, void *kappa_out,
                             void *norm_out, bool f64, unsigned int *krange = nullptr);
 
-// the norms of the proxy widths (proxy.cuh) of a finished range, behind its two words
-kde_status kde_krange_norms(kde_ctx *ctx, unsigned int *krange);
-// float bits of the largest and smallest of many widths: kde_krange_reset on the stream,
-// then kde_krange_add by every warp of the kernel that writes the widths (all lanes; a lane
-// without a width passes lo = 3e38, hi = 0)
+// float bits of the largest and smallest of many widths, by kde_krange_add from every warp of the
+// kernel that looks at them (all lanes; a lane without a width passes lo = 3e38, hi = 0) after
+// kde_krange_reset on the stream
 inline cudaError_t kde_krange_reset(unsigned int *krange, cudaStream_t stream)
 {
     const cudaError_t e = cudaMemsetAsync(krange, 0, 4, stream);
@@ -631,3 +630,16 @@ __device__ __forceinline__ void kde_krange_add(unsigned int *krange, float lo, f
         if (l < __ldcg(&krange[1])) atomicMin(&krange[1], l);
     }
 }
+// The range of the widths of an FP32 PIC state, in the workspace: the words krange[0 .. 1] (largest,
+// smallest) and the proxies' norms of a narrow one behind them (proxy.cuh), read by the step's
+// kernels.  A kernel that writes the widths gathers it in krange[KDE_KRANGE_ACC ..] by
+// kde_krange_block (proxy.cuh); kde_krange_begin comes before that kernel
+#define KDE_KRANGE_ACC 32
+// Runs on which no kernel gains by it do without, and the deposit's CTAs sweep their particles and look
+// for their widths themselves.  Those are: fewer than 80 nodes without a width schedule, and samples
+// of fewer than 128 CTAs of the deposit -- compressed, their proxies share seven widths, whose rounding
+// few CTAs average (66 CTAs, 16,832 particles: field energies 1.0 to 1.6e-6 off, swept 0.3 to
+// 1.0e-6; 157 CTAs: 0.1 to 1.0e-6 against 0.4 to 1.6e-6)
+inline bool kde_pic_range(int64_t N, int Ng, bool sched) { return N > 127 * 256 && (sched || Ng >= 80); }
+kde_status kde_krange_begin(kde_ctx *ctx, unsigned int *krange);
+void kde_krange_end(kde_ctx *ctx);  // after it

@@ -23,6 +23,7 @@
 // enough for each candidate (deposit.cu).  Combination and argmin in FP64.
 #include "common.cuh"
 #include "fp64.cuh"
+#include "proxy.cuh"
 
 #define CV_T 256
 #define CV_WARPS (CV_T / 32)
@@ -1048,38 +1049,40 @@ __global__ void __launch_bounds__(256) adapt_mean_kernel(const double *part, int
 }
 
 template <typename T>
-__global__ void adapt_apply_kernel(const float *loo, int64_t N, const AdaptPar *__restrict__ P, double alpha,
-                                   double kmin, double kmax, T *kappa_out, T *norm_out, const float2 *ntab,
-                                   unsigned int *krange)
+__global__ void __launch_bounds__(256)
+    adapt_apply_kernel(const float *loo, int64_t N, const AdaptPar *__restrict__ P, double alpha, double kmin, double kmax,
+                       T *kappa_out, T *norm_out, const float2 *ntab, unsigned int *krange, const float *pxt)
 {
-    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    const bool in = i < N;
-    const float lo_i = in ? loo[i] : 1.f;
-    // lambda = (f/g)^-alpha, kappa = kappa* / lambda^2; FP32 widths in FP32 with base-2
-    // logarithms (the log-mean of adapt_logsum_dev_kernel<true> is in the same base), FP64
-    // widths in FP64 with natural ones
-    T k;
-    if constexpr (sizeof(T) == 4) {
-        const float f = fmaf(P->a, lo_i, P->b);
-        float kf = P->ks_f * exp2f((float)(2.0 * alpha) * (log2f(f) - P->logg_f));
-        kf = kf < (float)kmin ? (float)kmin : (kf > (float)kmax ? (float)kmax : kf);
-        k = kf;
-    } else {
-        const double n = (double)N;
-        const double f = ((n - 1.0) * (double)lo_i + P->K0) / n;
-        double kd = P->ks * exp(2.0 * alpha * (log(f) - P->logg));
-        kd = kd < kmin ? kmin : (kd > kmax ? kmax : kd);
-        k = kd;
+    float lo = 3.0e38f, hi = 0.f;
+    for (int64_t i = (int64_t)blockIdx.x * 256 + threadIdx.x; i < N; i += (int64_t)gridDim.x * 256) {
+        // lambda = (f/g)^-alpha, kappa = kappa* / lambda^2; FP32 widths in FP32 with base-2
+        // logarithms (the log-mean of adapt_logsum_dev_kernel<true> is in the same base), FP64
+        // widths in FP64 with natural ones
+        T k;
+        if constexpr (sizeof(T) == 4) {
+            const float f = fmaf(P->a, loo[i], P->b);
+            float kf = P->ks_f * exp2f((float)(2.0 * alpha) * (log2f(f) - P->logg_f));
+            kf = kf < (float)kmin ? (float)kmin : (kf > (float)kmax ? (float)kmax : kf);
+            k = kf;
+        } else {
+            const double n = (double)N;
+            const double f = ((n - 1.0) * (double)loo[i] + P->K0) / n;
+            double kd = P->ks * exp(2.0 * alpha * (log(f) - P->logg));
+            kd = kd < kmin ? kmin : (kd > kmax ? kmax : kd);
+            k = kd;
+        }
+        kappa_out[i] = k;
+        // of the widths as the deposit and the gather use them
+        const float c = (float)k > 0.f && (float)k <= (float)KDE_KAPPA_MAX ? (float)k : (float)KDE_KAPPA_MAX;
+        lo = fminf(lo, c);
+        hi = fmaxf(hi, c);
+        if (norm_out) {
+            // FP32 widths take the tabulated norm, FP64 widths the FP64 Bessel series
+            if constexpr (sizeof(T) == 4) norm_out[i] = (T)kde_norm_tab(ntab, (float)k);
+            else norm_out[i] = (T)f64_norm((double)k);
+        }
     }
-    // all lanes of a warp together
-    if (krange) kde_krange_add(krange, in ? (float)k : 3.0e38f, in ? (float)k : 0.f);
-    if (!in) return;
-    kappa_out[i] = k;
-    if (norm_out) {
-        // FP32 widths take the tabulated norm, FP64 widths the FP64 Bessel series
-        if constexpr (sizeof(T) == 4) norm_out[i] = (T)kde_norm_tab(ntab, (float)k);
-        else norm_out[i] = (T)f64_norm((double)k);
-    }
+    if (krange) kde_krange_block(krange, pxt, lo, hi);
 }
 
 // block partials of the pilot's log-sum.  F32: base-2 logarithms of the FP32 pilot,
@@ -1130,20 +1133,17 @@ kde_status kde_adapt_device(kde_ctx *ctx, const float *loo, int64_t N, double L,
     KDE_LAUNCHED(ctx, "adapt_logsum_dev_kernel");
     adapt_mean_kernel<<<1, AD_BLOCKS, 0, ctx->stream>>>(part, N, P);
     KDE_LAUNCHED(ctx, "adapt_mean_kernel");
-    unsigned grid = (unsigned)((N + 255) / 256);
+    const int64_t want = (N + 255) / 256, most = 8LL * (ctx->sm_count > 0 ? ctx->sm_count : 1);
+    const unsigned grid = (unsigned)(want < most ? want : most);
+    if (krange) KDE_TRY(kde_krange_begin(ctx, krange));
     if (f64)
         adapt_apply_kernel<double><<<grid, 256, 0, ctx->stream>>>(loo, N, P, alpha, kmin, kmax, (double *)kappa_out,
-                                                                   (double *)norm_out, ctx->norm_tab, nullptr);
-    else {
-        if (krange) KDE_CUDA(ctx, kde_krange_reset(krange, ctx->stream), "width range memset");
+                                                                   (double *)norm_out, ctx->norm_tab, nullptr, nullptr);
+    else
         adapt_apply_kernel<float><<<grid, 256, 0, ctx->stream>>>(loo, N, P, alpha, kmin, kmax, (float *)kappa_out,
-                                                                  (float *)norm_out, ctx->norm_tab, krange);
-        if (krange) {
-            KDE_LAUNCHED(ctx, "adapt_apply_kernel");
-            return kde_krange_norms(ctx, krange);
-        }
-    }
+                                                                  (float *)norm_out, ctx->norm_tab, krange, ctx->pxy_tab);
     KDE_LAUNCHED(ctx, "adapt_apply_kernel");
+    if (krange) kde_krange_end(ctx);
     return KDE_OK;
 }
 

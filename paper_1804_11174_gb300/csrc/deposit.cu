@@ -1494,22 +1494,25 @@ __global__ void wmax_kernel(const T *w, int64_t N, unsigned int *wmax_bits, unsi
 }
 
 // ---------------------------------------------------------------------------
-__global__ void krange_norms_kernel(unsigned int *krange, const float *pxt)
+kde_status kde_krange_begin(kde_ctx *ctx, unsigned int *krange)
 {
-    const float kmax = __uint_as_float(krange[0]), kmin = __uint_as_float(krange[1]);
-    float kc, kh;
-    pxy_lin_range(kmin, kmax, kc, kh);
-    const int i = threadIdx.x, Q = i < 16 ? 7 : 6, b = i & 15;
-    if (b >= Q) return;
-    const float k = pxy_lin_kappa(kc, kh, pxt[pxy_tab_off(Q) + Q + b], Q);
-    krange[(Q == 7 ? PXY_NORM7 : PXY_NORM6) + b] = __float_as_uint((float)f64_norm((double)k));
+    // reset by the pass before, unless that failed half-way; a captured pass, whose replays may come
+    // after such a one, resets them itself
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    cudaStreamIsCapturing(ctx->stream, &cap);
+    if (!ctx->range_reset || cap != cudaStreamCaptureStatusNone) {
+        KDE_CUDA(ctx, kde_krange_reset(krange + KDE_KRANGE_ACC, ctx->stream), "width range memset");
+        KDE_CUDA(ctx, cudaMemsetAsync(krange + KDE_KRANGE_ACC + 2, 0, 4, ctx->stream), "width range memset");
+    }
+    ctx->range_reset = false;
+    return KDE_OK;
 }
 
-kde_status kde_krange_norms(kde_ctx *ctx, unsigned int *krange)
+void kde_krange_end(kde_ctx *ctx)
 {
-    krange_norms_kernel<<<1, 32, 0, ctx->stream>>>(krange, ctx->pxy_tab);
-    KDE_LAUNCHED(ctx, "krange_norms_kernel");
-    return KDE_OK;
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    cudaStreamIsCapturing(ctx->stream, &cap);
+    ctx->range_reset = cap == cudaStreamCaptureStatusNone;
 }
 
 // grids of int64 node sums: two for the PIC step's deposits (see DepSums), and one for
@@ -1549,7 +1552,7 @@ template <typename T>
 static kde_status deposit_sorted_impl(kde_ctx *ctx, const uint32_t *u, const T *kappa, T kappa_u, const T *norm,
                                       T norm_u, const T *w, T w_u, int64_t N, int Ng, double coef, long long *acc,
                                       double bound, const unsigned int *wmax_bits, double norm_bound,
-                                      float xcut = 0.f, const unsigned int *krange = nullptr, int nbins = 0)
+                                      float xcut = 0.f, const unsigned int *krange = nullptr, int nbins = 0, bool sweep = false)
 {
     // (the FP32 callers zero their sums)
     if (sizeof(T) == 8)
@@ -1606,9 +1609,6 @@ static kde_status deposit_sorted_impl(kde_ctx *ctx, const uint32_t *u, const T *
             // particle-wise widths, 2^20 particles on 64 nodes 26.7 against 24.8 us).  One width has a form
             // by the positions of an average CTA; particle-wise widths form 3 at best, with P <= 6 on
             // fewer than 80 nodes only for widths below 15.
-            // The few CTAs of a PIC run with particle-wise widths sweep too: their proxies share
-            // seven widths, whose rounding few CTAs average (66 CTAs, 16,832 particles: field energies
-            // 1.0 to 1.6e-6 off, swept 0.3 to 1.0e-6; 157 CTAs: 0.1 to 1.0e-6 against 0.4 to 1.6e-6)
             const float n = (float)((double)N / Pl.G);
             int form = Ng < 80 ? 0 : 3;
             double Rw = Ng;
@@ -1621,7 +1621,7 @@ static kde_status deposit_sorted_impl(kde_ctx *ctx, const uint32_t *u, const T *
             const float4 c = depp_reg_cost(form);
             const float gain = depp_sweep_ns(n, (float)Rw, true, Pl.inv_share) - n * c.x - (float)Rw * c.y -
                                (c.z + c.w * (float)Rw) * Pl.inv_share;
-            const bool comp = nbins >= 0 && !(krange && Pl.G < 128) && S.xcut == (float)KDE_XCUT && form && gain * share > 300.f;
+            const bool comp = nbins >= 0 && !sweep && S.xcut == (float)KDE_XCUT && form && gain * share > 300.f;
             KDE_CUDA(ctx,
                      kde_launch(ctx, true, comp ? deposit_persist_kernel<true> : deposit_persist_kernel<false>,
                                 dim3(Pl.G), dim3(DEPP_THREADS), 0, S, Pl),
@@ -1661,7 +1661,7 @@ kde_status kde_deposit_sums_f32(kde_ctx *ctx, const uint32_t *u, const float *ka
     out->next = s + (ctx->sums_flip ? 0 : KDE_MAX_NG);
     ctx->sums_flip = !ctx->sums_flip;
     return deposit_sorted_impl<float>(ctx, u, kappa, kappa_u, nullptr, norm_u, nullptr, w_u, N, Ng, coef, out->acc, bound,
-                                      nullptr, 0.0, xcut, krange);
+                                      nullptr, 0.0, xcut, krange, 0, kappa && !krange);
 }
 
 template <typename T>

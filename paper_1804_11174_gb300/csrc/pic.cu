@@ -12,24 +12,26 @@
 //   gather + leap-frog push + write-back + field energy (one kernel)
 #include "common.cuh"
 #include "fp64.cuh"
+#include "proxy.cuh"
 
 template <typename T>
-__global__ void norm_from_kappa_kernel(const T *kappa, int64_t N, T *norm, unsigned int *status, const float2 *ntab,
-                                       unsigned int *krange)
+__global__ void __launch_bounds__(256) norm_from_kappa_kernel(const T *kappa, int64_t N, T *norm, unsigned int *status,
+                                                              const float2 *ntab, unsigned int *krange, const float *pxt)
 {
-    int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    const bool in = i < N;
-    double k = in ? (double)kappa[i] : 1.0;
-    if (!(k > 0 && k <= KDE_KAPPA_MAX)) {
-        kde_flag(status, KDE_DEV_KAPPA_RANGE, (unsigned)i);
-        k = KDE_KAPPA_MAX;
+    float lo = 3.0e38f, hi = 0.f;  // of the widths as the deposit and the gather use them
+    for (int64_t i = (int64_t)blockIdx.x * 256 + threadIdx.x; i < N; i += (int64_t)gridDim.x * 256) {
+        double k = (double)kappa[i];
+        if (!(k > 0 && k <= KDE_KAPPA_MAX)) {
+            kde_flag(status, KDE_DEV_KAPPA_RANGE, (unsigned)i);
+            k = KDE_KAPPA_MAX;
+        }
+        lo = fminf(lo, (float)k);
+        hi = fmaxf(hi, (float)k);
+        // FP32 state: the tabulated norm; FP64 state: the FP64 Bessel series
+        if constexpr (sizeof(T) == 4) norm[i] = (T)kde_norm_tab(ntab, (float)k);
+        else norm[i] = (T)f64_norm(k);
     }
-    // the range of the widths as the deposit and the gather use them (all lanes of a warp together)
-    if (krange) kde_krange_add(krange, in ? (float)k : 3.0e38f, in ? (float)k : 0.f);
-    if (!in) return;
-    // FP32 state: the tabulated norm; FP64 state: the FP64 Bessel series
-    if constexpr (sizeof(T) == 4) norm[i] = (T)kde_norm_tab(ntab, (float)k);
-    else norm[i] = (T)f64_norm(k);
+    if (krange) kde_krange_block(krange, pxt, lo, hi);
 }
 
 // ---------------------------------------------------------------------------
@@ -240,16 +242,18 @@ static kde_status pic_run(kde_ctx *ctx, pic_state *st, int n_steps)
 
     // FP32 particle-wise widths: their range, kept on the device beside them
     unsigned int *krange = nullptr;
-    if (per && sizeof(T) == 4) {
+    if (per && sizeof(T) == 4 && kde_pic_range(N, Ng, sched)) {
+        if (ctx->ws_bytes[WS_PIC_RANGE] == 0) ctx->range_reset = false;
         krange = (unsigned int *)kde_ws(ctx, WS_PIC_RANGE, 256);
         if (!krange) return KDE_ENOMEM;
-        KDE_CUDA(ctx, kde_krange_reset(krange, ctx->stream), "width range memset");
+        KDE_TRY(kde_krange_begin(ctx, krange));
     }
     if (per) {
-        norm_from_kappa_kernel<T><<<(unsigned)((N + 255) / 256), 256, 0, ctx->stream>>>(
-            (const T *)st->kappa, N, norm_arr, ctx->d_status, ctx->norm_tab, krange);
+        const int64_t want = (N + 255) / 256, most = 8LL * (ctx->sm_count > 0 ? ctx->sm_count : 1);
+        norm_from_kappa_kernel<T><<<(unsigned)(want < most ? want : most), 256, 0, ctx->stream>>>(
+            (const T *)st->kappa, N, norm_arr, ctx->d_status, ctx->norm_tab, krange, ctx->pxy_tab);
         KDE_LAUNCHED(ctx, "norm_from_kappa_kernel");
-        if (krange) KDE_TRY(kde_krange_norms(ctx, krange));
+        if (krange) kde_krange_end(ctx);
     }
     if (sizeof(T) == 4 && n_steps > 0) KDE_TRY(kde_deposit_sums_reset(ctx));
     const double coef = KDE_TWO_PI / L;

@@ -130,7 +130,7 @@ __device__ __forceinline__ void pxy_box_width(PxyBox &B, float kmin, float kmax)
 }
 
 // norms of the proxy widths of a narrow range, behind the range's two words: PXY_NORM7 + b for
-// Q = 7, PXY_NORM6 + b for Q = 6, in FP64 and rounded (kde_krange_norms).  The proxies' norms
+// Q = 7, PXY_NORM6 + b for Q = 6, in FP64 and rounded (kde_krange_block).  The proxies' norms
 // are a factor on the whole density, so the table's 5e-7 would be the field's.
 #define PXY_NORM7 4
 #define PXY_NORM6 12
@@ -138,6 +138,104 @@ __device__ __forceinline__ void pxy_box_width(PxyBox &B, float kmin, float kmax)
 __device__ __forceinline__ float pxy_lin_kappa(float kc, float kh, float c, int Q)
 {
     return fmaf(kh, c * (0.5f * (float)Q), kc);
+}
+
+// 1 / k!^2 and the coefficients of Hankel's series, prod_{j <= k} (2j - 1)^2 / (8j)
+struct PxySeries {
+    double inv_fact_sq[64], hankel[32];
+    constexpr PxySeries() : inv_fact_sq(), hankel()
+    {
+        inv_fact_sq[0] = hankel[0] = 1.0;
+        for (int k = 1; k < 64; ++k) inv_fact_sq[k] = inv_fact_sq[k - 1] / ((double)k * k);
+        for (int k = 1; k < 32; ++k) hankel[k] = hankel[k - 1] * ((2.0 * k - 1.0) * (2.0 * k - 1.0) / (8.0 * k));
+    }
+};
+static __device__ const PxySeries pxy_series{};
+
+// 1 / (2 pi I0e(x)) in FP64 of two values by a warp, lane 0 the first's and lane 1 the second's: the
+// series of kde_i0e with a term or two a lane, below 30 sum (x^2 / 4)^k / k!^2 (64 terms), above sum
+// hankel_k / x^k (32 terms, still falling there).  A dependent FP64 operation takes some 40 clocks
+// here: term by term, on a lane a value, the series took 5 us
+__device__ __forceinline__ double pxy_norm_warp(const double (&x)[2], int lane)
+{
+    double z[2], p[2] = {1.0, 1.0}, t[2];
+#pragma unroll
+    for (int v = 0; v < 2; ++v) z[v] = x[v] < 30.0 ? 0.25 * x[v] * x[v] : 1.0 / x[v];
+#pragma unroll
+    for (int b = 0; b < 5; ++b)  // p = z^lane, z = z^32 at the end
+#pragma unroll
+        for (int v = 0; v < 2; ++v) {
+            if (lane >> b & 1) p[v] *= z[v];
+            z[v] *= z[v];
+        }
+#pragma unroll
+    for (int v = 0; v < 2; ++v)
+        t[v] = x[v] < 30.0 ? p[v] * fma(z[v], pxy_series.inv_fact_sq[lane + 32], pxy_series.inv_fact_sq[lane])
+                           : p[v] * pxy_series.hankel[lane];
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1)
+#pragma unroll
+        for (int v = 0; v < 2; ++v) t[v] += __shfl_xor_sync(0xffffffffu, t[v], o);
+    const double y = lane ? x[1] : x[0], s = KDE_TWO_PI * (lane ? t[1] : t[0]);
+    return (y < 30.0 ? exp(y) : sqrt(KDE_TWO_PI * y)) / s;
+}
+
+// the range of the widths that a kernel writes (KDE_KRANGE_ACC): called once by all 256 threads of every
+// block with the extremes of the thread's own (lo = 3e38, hi = 0 without any).  One pair of atomics a
+// block (the first blocks all find the range unset, and a pair a warp queued up on the one
+// address); the last block moves the range to its place, adds the norms of the proxy widths of a
+// narrow one and leaves the gathering words reset: a kernel of its own for that, and memsets before
+// every pass, took 8 us of a call
+__device__ __forceinline__ void kde_krange_block(unsigned int *krange, const float *pxt, float lo, float hi)
+{
+    __shared__ unsigned int rl[8], rh[8], last;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    unsigned int *acc = krange + KDE_KRANGE_ACC;
+    const unsigned int h = __reduce_max_sync(0xffffffffu, __float_as_uint(hi));
+    const unsigned int l = __reduce_min_sync(0xffffffffu, __float_as_uint(lo));
+    if (lane == 0) {
+        rh[warp] = h;
+        rl[warp] = l;
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        unsigned int a = rh[0], b = rl[0];
+#pragma unroll
+        for (int w = 1; w < 8; ++w) {
+            a = max(a, rh[w]);
+            b = min(b, rl[w]);
+        }
+        if (a > __ldcg(&acc[0])) atomicMax(&acc[0], a);
+        if (b < __ldcg(&acc[1])) atomicMin(&acc[1], b);
+        __threadfence();
+        last = atomicAdd(&acc[2], 1u) == gridDim.x - 1 ? 1u : 0u;
+    }
+    __syncthreads();
+    if (!last) return;
+    __threadfence();
+    const unsigned int bh = __ldcg(&acc[0]), bl = __ldcg(&acc[1]);
+    const float kmax = __uint_as_float(bh), kmin = __uint_as_float(bl);
+    __syncthreads();  // read by all before the reset
+    if (threadIdx.x == 0) {
+        krange[0] = bh;
+        krange[1] = bl;
+        acc[0] = 0u;
+        acc[1] = 0x7f7f7f7fu;
+        acc[2] = 0u;
+    }
+    if (!pxy_narrow(kmin, kmax)) return;
+    float kc, kh;
+    pxy_lin_range(kmin, kmax, kc, kh);
+    // values 0 .. 6 are those of Q = 7, 7 .. 12 those of Q = 6
+    const int i0 = min(2 * warp, 12), i1 = min(2 * warp + 1, 12);
+    auto width = [&](int i) {
+        const int Q = i < 7 ? 7 : 6;
+        return (double)pxy_lin_kappa(kc, kh, pxt[pxy_tab_off(Q) + Q + (i < 7 ? i : i - 7)], Q);
+    };
+    const double x[2] = {width(i0), width(i1)};
+    const double n = pxy_norm_warp(x, lane);
+    const int i = lane ? i1 : i0;
+    if (lane < 2) krange[i < 7 ? PXY_NORM7 + i : PXY_NORM6 + i - 7] = __float_as_uint((float)n);
 }
 
 // position in the box, [-1, 1]: the code difference is exact

@@ -120,7 +120,8 @@ static void ctx_trim(kde_ctx *c)
             c->ws[i] = nullptr;
             c->ws_bytes[i] = 0;
         }
-    c->sp_atab = nullptr;  // held in a workspace slot
+    c->sp_atab = nullptr;  // held in workspace slots, as is the range
+    c->range_reset = false;
     c->sp_atab_cands.clear();
 }
 

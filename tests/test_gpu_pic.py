@@ -465,3 +465,26 @@ def test_gather_started_late_is_bitwise_neutral(ctx, kp, N, Ng, lo):
         ctx.set_launch_overlap(True)
     for t in ("u", "v", "id", "energy"):
         assert torch.equal(getattr(states[0], t), getattr(states[1], t)), t
+
+
+@pytest.mark.parametrize("N, Ng", [(40001, 512), (32512, 512), (32513, 80)])
+def test_width_range_is_each_calls_own(ctx, kp, N, Ng):
+    # one-step calls on states with other widths between: wide, narrow, all one, narrow elsewhere.
+    # Nothing of a call's range of widths is left for the next: bitwise as on a context of its own
+    u, v = I.landau_load(46, N, 4 * math.pi, 0.05, 1.0)
+    ws = [I.log_uniform(3, I.STREAM_KAPPA, N, lo, hi).astype(np.float32)
+          for lo, hi in ((5.0, 5e3), (13.0, 16.0), (14.0, 14.0), (29.0, 36.0), (300.0, 330.0))]
+    mk = lambda w: make_state(kp, u, v.astype(np.float32), 4 * math.pi, Ng, 0.1, 2, kappa=w)
+    together, alone = [mk(w) for w in ws], [mk(w) for w in ws]
+    for _ in range(2):
+        for st in together:
+            ctx.pic_step(st, 1)
+    ctx.sync()
+    for st, other in zip(alone, together):
+        own = kp.Context(0)
+        own.pic_step(st, 1)
+        own.pic_step(st, 1)
+        own.sync()
+        own.close()
+        for t in ("u", "v", "id", "kappa", "kappa_norm", "energy"):
+            assert torch.equal(getattr(st, t), getattr(other, t)), t
