@@ -130,6 +130,8 @@ struct kde_ctx {
     double *f64_tab = nullptr;   // 2^(j / 2048) for the FP64 kernels (fp64.cuh), built at creation
     float *pxy_tab = nullptr;    // interpolation matrices (proxy.cuh), built at creation
     unsigned wait_polls = 1u << 26;         // polls of a bounded device wait (kde_set_wait_limit)
+    int sums_ng = 0;                        // nodes of the step whose field kernel zeroed the next grid of node sums
+    bool sums_captured = false;             // a captured call uses those grids
     bool range_reset = false;               // the gathering words of WS_PIC_RANGE are reset
     bool sums_zero = false;                 // kde_deposit's grid of node sums is zero
     bool sums_flip = false;                 // which grid of node sums the next FP32 deposit adds to
@@ -502,13 +504,13 @@ kde_status kde_deposit_reserve(kde_ctx *ctx);
 // the FP32 deposit of cell-sorted particles (uniform weight w_u, N >= 1) left as int64 node sums
 // (fixed-point scale kde_acc_scale(bound)) for the field kernel.  Two grids of sums are used in
 // turn: the field kernel that reads one zeroes the other, which the next deposit adds to.
-// kde_deposit_sums_reset zeroes both and comes before the first deposit of a call; every deposit
+// kde_deposit_sums_reset makes the next deposit's grid zero, before the first of a call; every deposit
 // is followed by one kde_field_from_sums.  krange: float bits of the largest and smallest width
 // on the device, which spare the kernel a pass over the widths
 struct DepSums {
     long long *acc, *next;
 };
-kde_status kde_deposit_sums_reset(kde_ctx *ctx);
+kde_status kde_deposit_sums_reset(kde_ctx *ctx, int Ng);
 kde_status kde_deposit_sums_f32(kde_ctx *ctx, const uint32_t *u, const float *kappa, float kappa_u, float norm_u,
                                 int64_t N, int Ng, double coef, float w_u, double bound, DepSums *out,
                                 float xcut = 0.f, const unsigned int *krange = nullptr);

@@ -1519,7 +1519,10 @@ void kde_krange_end(kde_ctx *ctx)
 // kde_deposit, which every call leaves zero
 static long long *depp_sums(kde_ctx *ctx)
 {
-    if (ctx->ws_bytes[WS_DEP_SUMS] == 0) ctx->sums_zero = false;
+    if (ctx->ws_bytes[WS_DEP_SUMS] == 0) {
+        ctx->sums_zero = false;
+        ctx->sums_ng = 0;
+    }
     return (long long *)kde_ws(ctx, WS_DEP_SUMS, (size_t)3 * KDE_MAX_NG * 8);
 }
 
@@ -1539,10 +1542,18 @@ __global__ void __launch_bounds__(256) sums_to_real_kernel(long long *acc, int N
 
 kde_status kde_deposit_reserve(kde_ctx *ctx) { return depp_sums(ctx) ? KDE_OK : KDE_ENOMEM; }
 
-kde_status kde_deposit_sums_reset(kde_ctx *ctx)
+kde_status kde_deposit_sums_reset(kde_ctx *ctx, int Ng)
 {
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    cudaStreamIsCapturing(ctx->stream, &cap);
+    if (cap != cudaStreamCaptureStatusNone) ctx->sums_captured = true;
     long long *s = depp_sums(ctx);
     if (!s) return KDE_ENOMEM;
+    // the grid whose turn it is was zeroed by the last field kernel, if that had as many nodes and
+    // every deposit its field kernel.  Replays of a captured call use the grids in the turn they had
+    // then: a context with one zeroes them always
+    if (ctx->sums_ng == Ng && !ctx->sums_captured) return KDE_OK;
+    ctx->sums_ng = 0;
     ctx->sums_flip = false;
     KDE_CUDA(ctx, cudaMemsetAsync(s, 0, (size_t)2 * KDE_MAX_NG * 8, ctx->stream), "node sums memset");
     return KDE_OK;
@@ -1660,6 +1671,7 @@ kde_status kde_deposit_sums_f32(kde_ctx *ctx, const uint32_t *u, const float *ka
     out->acc = s + (ctx->sums_flip ? KDE_MAX_NG : 0);
     out->next = s + (ctx->sums_flip ? 0 : KDE_MAX_NG);
     ctx->sums_flip = !ctx->sums_flip;
+    ctx->sums_ng = 0;  // known again after the field kernel
     return deposit_sorted_impl<float>(ctx, u, kappa, kappa_u, nullptr, norm_u, nullptr, w_u, N, Ng, coef, out->acc, bound,
                                       nullptr, 0.0, xcut, krange, 0, kappa && !krange);
 }

@@ -162,6 +162,7 @@ kde_status kde_field_from_sums(kde_ctx *ctx, const DepSums &ds, int Ng, double L
                  "field_sums_kernel");
     }
     KDE_LAUNCHED(ctx, "field_sums_kernel");
+    ctx->sums_ng = Ng;
     return KDE_OK;
 }
 

@@ -255,7 +255,7 @@ static kde_status pic_run(kde_ctx *ctx, pic_state *st, int n_steps)
         KDE_LAUNCHED(ctx, "norm_from_kappa_kernel");
         if (krange) kde_krange_end(ctx);
     }
-    if (sizeof(T) == 4 && n_steps > 0) KDE_TRY(kde_deposit_sums_reset(ctx));
+    if (sizeof(T) == 4 && n_steps > 0) KDE_TRY(kde_deposit_sums_reset(ctx, Ng));
     const double coef = KDE_TWO_PI / L;
     const double w_u = L / (double)N;
     // the FP32 gather + push adds the next step's sort counts; a step whose table was

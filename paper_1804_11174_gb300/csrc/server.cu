@@ -120,8 +120,8 @@ static void ctx_trim(kde_ctx *c)
             c->ws[i] = nullptr;
             c->ws_bytes[i] = 0;
         }
-    c->sp_atab = nullptr;  // held in workspace slots, as is the range
-    c->range_reset = false;
+    c->sp_atab = nullptr;  // held in workspace slots, as are the sums and the range
+    c->sums_zero = c->range_reset = false;
     c->sp_atab_cands.clear();
 }
 

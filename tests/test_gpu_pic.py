@@ -488,3 +488,51 @@ def test_width_range_is_each_calls_own(ctx, kp, N, Ng):
         own.close()
         for t in ("u", "v", "id", "kappa", "kappa_norm", "energy"):
             assert torch.equal(getattr(st, t), getattr(other, t)), t
+
+
+def test_node_sums_between_calls(ctx, kp):
+    # the grids of node sums are handed from call to call: other grid sizes, other forms and replays of
+    # a captured call between leave every call what it is on a context of its own, bit for bit
+    u, v = I.landau_load(47, 5000, 4 * math.pi, 0.05, 1.0)
+    mk = lambda Ng: make_state(kp, u, v.astype(np.float32), 4 * math.pi, Ng, 0.1, 8, kappa_uniform=20.0)
+    grids = (64, 64, 1000, 64, 33, 33, 1000, 256)
+    ref = []
+    for Ng in grids:
+        own = kp.Context(0)
+        st = mk(Ng)
+        own.pic_step(st, 1)
+        own.pic_step(st, 2)
+        own.sync()
+        own.close()
+        ref.append(st)
+
+    def check(c):
+        for Ng, r in zip(grids, ref):
+            st = mk(Ng)
+            c.pic_step(st, 1)
+            c.deposit(st.u, Ng, 4 * math.pi, kappa_uniform=20.0)
+            c.pic_step(st, 2)
+            c.sync()
+            assert torch.equal(st.u, r.u) and torch.equal(st.v, r.v) and torch.equal(st.energy, r.energy), Ng
+
+    check(ctx)
+    side = torch.cuda.Stream()
+    with torch.cuda.stream(side):
+        c = kp.Context(0, stream=side)
+        c.reserve(5000, 64, 1)
+        st = mk(64)
+        snap = st.snapshot()
+        c.pic_step(st, 3)  # tables, and an odd number of turns
+        c.sync()
+        st.restore(snap)
+        torch.cuda.synchronize()
+        graph = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(graph, stream=side):
+            c.pic_step(st, 1)
+        for _ in range(2):
+            st.restore(snap)
+            graph.replay()
+            side.synchronize()
+            assert torch.equal(st.energy[:1], ref[0].energy[:1])
+            check(c)
+        c.close()
