@@ -65,24 +65,25 @@ __global__ void __launch_bounds__(256) sc_key_kernel(const float *kr, int64_t N,
 }
 
 // first particle of every band in the sorted order
-__global__ void __launch_bounds__(256) sc_starts_kernel(const uint32_t *key, int64_t N, int *starts)
+__global__ void __launch_bounds__(256) sc_starts_kernel(const uint32_t *key, int64_t N, int64_t *starts)
 {
     const int64_t j = (int64_t)blockIdx.x * 256 + threadIdx.x;
     if (j >= N) return;
     const int b = (int)(key[j] >> 28), a = j ? (int)(key[j - 1] >> 28) : -1;
-    for (int k = a + 1; k <= b; ++k) starts[k] = (int)j;
+    for (int k = a + 1; k <= b; ++k) starts[k] = j;
     if (j == N - 1)
-        for (int k = b + 1; k <= SC_MAXB; ++k) starts[k] = (int)N;
+        for (int k = b + 1; k <= SC_MAXB; ++k) starts[k] = N;
 }
 
 // the chunk x of the bands' chunk lists: its band and particles, or false past the end
-__device__ __forceinline__ bool sc_chunk(const ScBands &B, const int *starts, int x, int &b, int &j0, int &j1)
+__device__ __forceinline__ bool sc_chunk(const ScBands &B, const int64_t *starts, int x, int &b, int64_t &j0, int64_t &j1)
 {
     for (b = 0; b < B.nb; ++b) {
-        const int s = starts[b], e = starts[b + 1], nc = (e - s + B.chunk - 1) / B.chunk;
+        const int64_t s = starts[b], e = starts[b + 1];
+        const int nc = (int)((e - s + B.chunk - 1) / B.chunk);
         if (x < nc) {
-            j0 = s + x * B.chunk;
-            j1 = min(e, j0 + B.chunk);
+            j0 = s + (int64_t)x * B.chunk;
+            j1 = e < j0 + B.chunk ? e : j0 + B.chunk;
             return true;
         }
         x -= nc;
@@ -92,20 +93,21 @@ __device__ __forceinline__ bool sc_chunk(const ScBands &B, const int *starts, in
 
 // partial sums of T_q(s_j) e^{im theta_j} over a chunk, q < SC_Q, four consecutive modes a thread
 __global__ void __launch_bounds__(SC_THREADS)
-    sc_factor_kernel(const uint32_t *__restrict__ u, const float *__restrict__ kr, ScBands B, const int *starts,
+    sc_factor_kernel(const uint32_t *__restrict__ u, const float *__restrict__ kr, ScBands B, const int64_t *starts,
                      double2 *part)
 {
     __shared__ uint32_t us[SC_SUB];
     __shared__ __align__(16) float tq[SC_SUB][SC_Q];
     __shared__ float2 e1[SC_SUB];
-    int b, j0, j1;
+    int b;
+    int64_t j0, j1;
     if (!sc_chunk(B, starts, blockIdx.x, b, j0, j1)) return;
     const int mb = 1 + blockIdx.y * SC_THREADS * SC_MODES;
     if (mb > B.M[b]) return;
     const int m0 = mb + threadIdx.x * SC_MODES;
     double2 *out = part + (size_t)blockIdx.x * SC_Q * B.Mst + (m0 - 1);
-    for (int s0 = j0; s0 < j1; s0 += SC_SUB) {
-        const int n = min(SC_SUB, j1 - s0);
+    for (int64_t s0 = j0; s0 < j1; s0 += SC_SUB) {
+        const int n = (int)(j1 - s0 < SC_SUB ? j1 - s0 : SC_SUB);
         __syncthreads();
         for (int k = threadIdx.x; k < n; k += SC_THREADS) {
             const uint32_t uk = u[s0 + k];
@@ -171,7 +173,7 @@ __global__ void __launch_bounds__(SC_THREADS)
 
 // G summed over a band's chunks in order, then H_q' = sum_q c_q[q'] G_q (proxy.cuh's matrix in
 // FP64); block (32 modes, band), warp w the sums of q = w, w + 8
-__global__ void __launch_bounds__(256) sc_reduce_kernel(const double2 *part, ScBands B, const int *starts, double2 *H)
+__global__ void __launch_bounds__(256) sc_reduce_kernel(const double2 *part, ScBands B, const int64_t *starts, double2 *H)
 {
     __shared__ double2 G[SC_Q][32];
     __shared__ double cm[4 * SC_Q];
@@ -180,8 +182,8 @@ __global__ void __launch_bounds__(256) sc_reduce_kernel(const double2 *part, ScB
     if ((int)(blockIdx.x * 32) >= B.M[b]) return;
     if (threadIdx.x < 4 * SC_Q) cm[threadIdx.x] = cospi((double)threadIdx.x / (2.0 * SC_Q));
     int x0 = 0;
-    for (int k = 0; k < b; ++k) x0 += (starts[k + 1] - starts[k] + B.chunk - 1) / B.chunk;
-    const int nc = (starts[b + 1] - starts[b] + B.chunk - 1) / B.chunk;
+    for (int k = 0; k < b; ++k) x0 += (int)((starts[k + 1] - starts[k] + B.chunk - 1) / B.chunk);
+    const int nc = (int)((starts[b + 1] - starts[b] + B.chunk - 1) / B.chunk);
     for (int q = warp; q < SC_Q; q += 8) {
         double2 s = make_double2(0.0, 0.0);
         if (m < B.M[b])
@@ -420,7 +422,7 @@ kde_status kde_cv_scale_fourier(kde_ctx *ctx, const uint32_t *u, const float *kr
     double2 *H = (double2 *)w, *F = H + nH, *psum = F + nF;
     double *inv = (double *)(psum + nP), *pself = inv + (size_t)B.nb * ns;
     size_t *aoff = (size_t *)(pself + (size_t)n_cand * nself);
-    int *starts = (int *)(aoff + SC_MAXB);
+    int64_t *starts = (int64_t *)(aoff + SC_MAXB);
     KDE_CUDA(ctx, cudaMemcpyAsync(aoff, aoff_h, sizeof(size_t) * B.nb, cudaMemcpyHostToDevice, ctx->stream), "offsets copy");
 
     KdeProfScope _ps(ctx, PROF_SPECTRAL);

@@ -327,3 +327,47 @@ def test_cv_structure_factor_from_moments(ctx, oracle, N, kmax, where):
     _, _, _, lref = oracle.cv_fourier(x, L, cand[am], want_loo=True)
     idx = np.arange(0, N, 97)
     np.testing.assert_allclose(loo.cpu().numpy()[idx], lref[idx], rtol=1e-5, atol=1e-7 * np.max(lref))
+
+
+def test_cv_scale_fourier_form_beyond_31_bits(kp):
+    # more particles than a 31-bit index holds: a sample of 4096 points and widths, repeated.  Its
+    # sums are the sample's times the repetitions; tolerance as for the Fourier form above
+    import torch
+    from scipy import special as sp
+    L, n0 = 2 * math.pi, 4096
+    reps = (1 << 31) // n0 + 1
+    if torch.cuda.mem_get_info()[0] < 100e9:
+        pytest.skip("needs 100 GB of device memory")
+    u0 = I.cv_sweep_load(3, n0)
+    k0 = I.log_uniform(3, I.STREAM_KAPPA, n0, 5.0, 50.0).astype(np.float32)
+    scales = [0.5, 1.0, 2.0]
+    c = kp.Context(0)
+    try:
+        cv, am, _ = c.cv(to_dev_u(u0).repeat(reps), L, scales, kappa_rel=to_dev(k0).repeat(reps))
+    finally:
+        c.close()
+        torch.cuda.empty_cache()
+    n, x, kd = float(reps) * n0, I.from_fixed(u0, L), k0.astype(np.float64)
+    for s, got in zip(scales, cv):
+        f2 = pr = n * n
+        for m in range(1, 160):
+            e = np.exp(1j * m * x)
+            S, F = reps * e.sum(), reps * ((sp.ive(m, s * kd) / sp.ive(0, s * kd)) * e).sum()
+            f2 += 2 * abs(F) ** 2
+            pr += 2 * (S.conjugate() * F).real
+        pairs = pr / (2 * math.pi) - reps * (1 / (2 * math.pi * sp.ive(0, s * kd))).sum()
+        ref = f2 / (2 * math.pi * n * n) - 2 * pairs / (n * (n - 1))
+        assert abs(got - ref) <= 1e-7 * np.max(np.abs(cv)), s
+
+
+@pytest.mark.parametrize("bad", [-1.0, 0.0, float("nan"), 2e6])
+def test_cv_scale_fourier_form_reports_widths_out_of_range(ctx, kp, bad):
+    # a sample large enough for the Fourier form's pass over the widths (2 candidates, 25,000^2 pairs)
+    N = 25000
+    u, _ = I.landau_load(1, N, 4 * math.pi, 0.05, 1.0)
+    kr = np.full(N, 50.0, np.float32)
+    kr[N - 3] = bad
+    with pytest.raises(kp.KdeError):
+        ctx.cv(to_dev_u(u), 4 * math.pi, [0.5, 1.0], kappa_rel=to_dev(kr))
+    kr[N - 3] = 50.0
+    ctx.cv(to_dev_u(u), 4 * math.pi, [0.5, 1.0], kappa_rel=to_dev(kr))
