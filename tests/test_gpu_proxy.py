@@ -286,3 +286,24 @@ def test_scheduled_step_against_oracle(ctx, kp, oracle, N, Ng, amp, kstar, alpha
     vg = st.v.double().cpu().numpy()[at]
     assert rel_l2(vg, r["v"]) <= tol
     assert np.max(np.abs(vg - r["v"])) <= 3 * tol * np.max(np.abs(r["v"]))
+
+
+@pytest.mark.parametrize("weights", [False, True])
+@pytest.mark.parametrize("kap", [0.3, 3.0, 14.0, 60.0, 300.0, 800.0, "one", "narrow", "hundred", "ten"])
+def test_deposit_of_every_compressed_form(ctx, oracle, kap, weights):
+    # more pairs than the unsorted sweep takes, and particles enough for the compressed forms to
+    # pay: one width with P <= 8 (up to 60) and <= 16, narrow ranges with P <= 6 and P = 7, 8
+    # ("hundred"), and the matrix product ("ten")
+    N, Ng = 500009, 256
+    u = positions(N, N, "box")
+    k = None
+    if kap == "hundred":
+        k = I.log_uniform(Ng, I.STREAM_KAPPA, N, 100.0, 115.0).astype(np.float32)
+    elif isinstance(kap, str):
+        k = widths(kap, Ng, N)
+    w = (0.5 + I.uniforms(7, 9, N)).astype(np.float32) if weights else None
+    kw = dict(kappa=to_dev(k)) if k is not None else dict(kappa_uniform=kap)
+    okw = dict(kappa=k.astype(np.float64)) if k is not None else dict(kappa_u=kap)
+    rho = ctx.deposit(to_dev_u(u), Ng, L, weight=None if w is None else to_dev(w), **kw).cpu().numpy()
+    ctx.sync()
+    assert rel_l2(rho, oracle.deposit(I.from_fixed(u, L), Ng, L, w=None if w is None else w.astype(np.float64), **okw)) <= TOL
