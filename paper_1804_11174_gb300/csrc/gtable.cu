@@ -13,8 +13,8 @@
 // or 128 bytes of coefficients from the L1 / L2 caches; the table costs about 40 Ng (node,
 // interval) pairs a band.  Only the bands that hold widths are built (a pass over the widths
 // finds their range).  Measured, whole calls: 1,000,003 particles, 1024 nodes, widths in
-// [5, 5e3] 215 -> 63 us (sorted sweep before: 50 us of it the sort, 174 the sweep; now range 5,
-// bands 30, particles 30); 5000 particles, 256 nodes, one width 21.5 -> 11.8 us.
+// [5, 5e3] 215 -> 61 us (sorted sweep before: 50 us of it the sort, 174 the sweep; now range 5,
+// bands 26, particles 30); 5000 particles, 256 nodes, one width 21.5 -> 11.8 us.
 #include "common.cuh"
 #include "proxy.cuh"
 
@@ -121,6 +121,59 @@ __global__ void __launch_bounds__(GT_THREADS) gt_range_kernel(GtArgs A, float2 *
     }
 }
 
+// coefficients of one interval from the field at its proxies, f[a QM + b], by a warp
+template <int PM, int QM>
+__device__ __forceinline__ void gt_coefs(float *f, const float *nk, const float *cp, const float *cq, float *row)
+{
+    constexpr int PQ = PM * QM;
+    const int lane = threadIdx.x & 31;
+    constexpr int PL = (PQ + 31) / 32;
+    // U[p][b] = sum_a c_p[a] f[a][b], in place
+    float U[PL];
+#pragma unroll
+    for (int h = 0; h < PL; ++h) {
+        const int m = h * 32 + lane, p = m / QM, b = m - p * QM;
+        U[h] = 0.f;
+        if (m < PQ) {
+#pragma unroll
+            for (int a = 0; a < PM; ++a) U[h] = fmaf(cp[p * PM + a], f[a * QM + b], U[h]);
+            U[h] *= nk[b];
+        }
+    }
+    __syncwarp();
+#pragma unroll
+    for (int h = 0; h < PL; ++h)
+        if (h * 32 + lane < PQ) f[h * 32 + lane] = U[h];
+    __syncwarp();
+    constexpr int NC = QM == 1 ? PM : GT_NC;
+    if (lane < NC) {
+        float t = 0.f;
+        if (QM == 1) {
+            t = f[lane];
+        } else {
+            int p = 0, q = lane;  // coefficient `lane` of the triangle p + q < PM
+            while (p < PM && q >= PM - p) q -= PM - p++;
+            if (p < PM) {
+#pragma unroll
+                for (int b = 0; b < QM; ++b) t = fmaf(cq[q * QM + b], f[p * QM + b], t);
+            }
+        }
+        row[lane] = t;
+    }
+    __syncwarp();
+}
+
+// nodes of interval i: the first of R
+__device__ __forceinline__ int gt_nodes(int Ng, int C, int i, int W, int &R)
+{
+    const int c0 = (int)((uint32_t)i * (uint32_t)Ng / (uint32_t)C);
+    const int c1 = (int)(((uint32_t)(i + 1) * (uint32_t)Ng - 1u) / (uint32_t)C);
+    R = c1 + W - (c0 - W) + 1;
+    if (R < Ng) return c0 - W;
+    R = Ng;
+    return 0;
+}
+
 // coefficients of one interval i < C by a group of wpi warps (warp w of the group): the
 // field at the PM x QM proxies, every lane a node with all the proxies' values in registers
 // (PM sines and PM QM exponentials that do not depend on one another), summed over the lanes
@@ -143,13 +196,8 @@ __device__ __forceinline__ void gt_interval(const GtArgs &A, bool on, int C, uin
         uint32_t mid;
         float mfrac;
         pxy_node(G2, 2 * i + 1, mid, mfrac);
-        const int c0 = (int)((uint32_t)i * (uint32_t)Ng / (uint32_t)C);
-        const int c1 = (int)(((uint32_t)(i + 1) * (uint32_t)Ng - 1u) / (uint32_t)C);
-        int g_lo = c0 - W, R = c1 + W - g_lo + 1;
-        if (R >= Ng) {
-            g_lo = 0;
-            R = Ng;
-        }
+        int R;
+        const int g_lo = gt_nodes(Ng, C, i, W, R);
         float acc[NR * 32], kk[QM];
 #pragma unroll
         for (int m = 0; m < NR * 32; ++m) acc[m] = 0.f;
@@ -195,44 +243,60 @@ __device__ __forceinline__ void gt_interval(const GtArgs &A, bool on, int C, uin
             }
     }
     __syncwarp();
-    if (on && w == 0) {
-        float *f = part + warp * PQ;
-        constexpr int PL = (PQ + 31) / 32;
-        // U[p][b] = sum_a c_p[a] f[a][b], in place
-        float U[PL];
-#pragma unroll
-        for (int h = 0; h < PL; ++h) {
-            const int m = h * 32 + lane, p = m / QM, b = m - p * QM;
-            U[h] = 0.f;
-            if (m < PQ) {
-#pragma unroll
-                for (int a = 0; a < PM; ++a) U[h] = fmaf(cp[p * PM + a], f[a * QM + b], U[h]);
-                U[h] *= nk[b];
-            }
-        }
-        __syncwarp();
-#pragma unroll
-        for (int h = 0; h < PL; ++h)
-            if (h * 32 + lane < PQ) f[h * 32 + lane] = U[h];
-        __syncwarp();
-        constexpr int NC = QM == 1 ? PM : GT_NC;
-        if (lane < NC) {
-            float t = 0.f;
-            if (QM == 1) {
-                t = f[lane];
-            } else {
-                int p = 0, q = lane;  // coefficient `lane` of the triangle p + q < PM
-                while (p < PM && q >= PM - p) q -= PM - p++;
-                if (p < PM) {
-#pragma unroll
-                    for (int b = 0; b < QM; ++b) t = fmaf(cq[q * QM + b], f[p * QM + b], t);
-                }
-            }
-            tab[(size_t)i * NC + lane] = t;
-        }
-        __syncwarp();
-    }
+    if (on && w == 0) gt_coefs<PM, QM>(part + warp * PQ, nk, cp, cq, tab + (size_t)i * (QM == 1 ? PM : GT_NC));
     if (wpi > 1) __syncthreads();
+}
+
+// the same for a window of at most 32 nodes, a warp an interval: a lane holds a node, the proxies'
+// values are the lanes' own sums over the nodes.  200,003 particles on 256 nodes, whole calls, before
+// with the window's nodes over the lanes and butterflies over 49 values: widths of 2000 to 20,000
+// (13,000 intervals) 42 -> 35 us, of 5 to 5000 45 -> 39
+#define GT_SHORT 32
+template <int PM, int QM>
+__device__ __forceinline__ void gt_interval_short(const GtArgs &A, int C, uint32_t step, int i, int W, const float *k2,
+                                                  const float *nk, const float *cp, const float *cq, const float2 *scd,
+                                                  float *part, float *tab)
+{
+    constexpr int PQ = PM * QM, H = (PQ + 31) / 32;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, Ng = A.grid.Ng;
+    PxyGrid G2;
+    G2.Ng = 2 * C;
+    G2.step = step;
+    G2.rem = 0u - step * (uint32_t)(2 * C);
+    uint32_t mid, nc;
+    float mfrac, nf, sn, cn;
+    pxy_node(G2, 2 * i + 1, mid, mfrac);
+    int R;
+    int g = gt_nodes(Ng, C, i, W, R) + (lane < GT_SHORT ? lane : 0);
+    g = g < 0 ? g + Ng : (g >= Ng ? g - Ng : g);
+    g = lane < R ? g : 0;
+    const float e = lane < R ? A.field[g] : 0.f;
+    pxy_node(A.grid, g, nc, nf);
+    pxy_sincos(nc, nf, mid, mfrac, sn, cn);
+    float2 d[H];
+    float kk[H], f[H];
+#pragma unroll
+    for (int h = 0; h < H; ++h) {
+        const int m = min(h * 32 + lane, PQ - 1);
+        d[h] = scd[m / QM];
+        kk[h] = k2[m % QM];
+        f[h] = 0.f;
+    }
+#pragma unroll 4
+    for (int r = 0; r < R; ++r) {
+        const float s = __shfl_sync(0xffffffffu, sn, r), c = __shfl_sync(0xffffffffu, cn, r);
+        const float er = __shfl_sync(0xffffffffu, e, r);
+#pragma unroll
+        for (int h = 0; h < H; ++h) {
+            const float sa = fmaf(s, d[h].y, -c * d[h].x);
+            f[h] = fmaf(kde_ex2(sa * sa * kk[h]), er, f[h]);
+        }
+    }
+#pragma unroll
+    for (int h = 0; h < H; ++h)
+        if (h * 32 + lane < PQ) part[warp * PQ + h * 32 + lane] = f[h];
+    __syncwarp();
+    gt_coefs<PM, QM>(part + warp * PQ, nk, cp, cq, tab + (size_t)i * (QM == 1 ? PM : GT_NC));
 }
 
 // warps that share an interval's window: about eight nodes a lane and more
@@ -266,7 +330,7 @@ __global__ void __launch_bounds__(GT_THREADS) gt_table_one_kernel(GtArgs A, int 
     }
 }
 
-__global__ void __launch_bounds__(GT_THREADS) gt_table_bands_kernel(GtArgs A, GtBands T)
+__global__ void __launch_bounds__(GT_THREADS, 2) gt_table_bands_kernel(GtArgs A, GtBands T)
 {
     constexpr int PM = GT_P;
     __shared__ float part[GT_WARPS * PM * PM], cp[PM * PM], xc[PM], k2s[GT_WARPS][PM], nks[GT_WARPS][PM];
@@ -313,8 +377,15 @@ __global__ void __launch_bounds__(GT_THREADS) gt_table_bands_kernel(GtArgs A, Gt
                 sincospif(xc[lane] * (0.5f / (float)C), &scd[lane].x, &scd[lane].y);
             }
             __syncwarp();
+            const bool narrow = 2 * W + A.grid.Ng / C + 2 <= GT_SHORT;  // wpi is 1 then
             for (; turn < items; turn += (int)gridDim.x) {
                 const int i = turn * ipc + warp / wpi;
+                if (narrow) {
+                    if (i < C)
+                        gt_interval_short<PM, PM>(A, C, T.step[b], i, W, k2, nk, cp, cp, scd, part,
+                                                  A.tab + (size_t)T.off[b] * GT_NC);
+                    continue;
+                }
                 gt_interval<PM, PM>(A, i < C, C, T.step[b], i, warp % wpi, wpi, W, k2, nk, cp, cp, scd, part,
                                     A.tab + (size_t)T.off[b] * GT_NC);
             }
@@ -439,13 +510,18 @@ __global__ void __launch_bounds__(GT_THREADS) gt_eval_bands_kernel(GtArgs A, GtB
     }
 }
 
-// small calls: GT_FLAT lanes a particle sweep the particle's own window, node by node
+// small calls: GT_FLAT lanes a particle sweep the particle's own window, node by node.  A warp takes
+// NB rounds of four particles, and what a particle needs first (norm, window, place) is worked
+// out by 32 / (4 NB) lanes, not by all of its eight: more rounds where that leaves the SMs their warps
+// (200,003 particles, widths of 5 to 5000, 64 nodes 30 -> 25 us)
 #define GT_FLAT 8
-__global__ void __launch_bounds__(GT_THREADS) gt_flat_kernel(GtArgs A)
+template <int NB> __global__ void __launch_bounds__(GT_THREADS) gt_flat_kernel(GtArgs A)
 {
-    const int lane = threadIdx.x & (GT_FLAT - 1), Ng = A.grid.Ng;
-    const int64_t j = ((int64_t)blockIdx.x * GT_THREADS + threadIdx.x) / GT_FLAT;
-    const int64_t jj = j < A.N ? j : A.N - 1;
+    constexpr int PW = 32 / GT_FLAT * NB;  // particles a warp
+    const int lane = threadIdx.x & 31, sub = lane & (GT_FLAT - 1), Ng = A.grid.Ng;
+    const int64_t j0 = ((int64_t)blockIdx.x * GT_WARPS + (threadIdx.x >> 5)) * PW;
+    if (j0 >= A.N) return;  // the whole warp
+    const int64_t j = j0 + (lane & (PW - 1)), jj = j < A.N ? j : A.N - 1;
     const uint32_t u = A.u[jj];
     float k = A.kappa_u, nm = A.norm_u;
     if (A.kappa) {
@@ -454,31 +530,41 @@ __global__ void __launch_bounds__(GT_THREADS) gt_flat_kernel(GtArgs A)
     }
     const int W = gt_window(k, Ng), len = min(Ng, 2 * W + 1);
     const float k2 = (float)(-2.0 * KDE_LOG2E) * k;
-    int g = (len == Ng ? 0 : kde_cell(u, Ng) - W) + lane;
-    g = g < 0 ? g + Ng : (g >= Ng ? g - Ng : g);
+    const int g0 = len == Ng ? 0 : kde_cell(u, Ng) - W;
     // the node's code and fraction move on by GT_FLAT nodes at a time (round the circle the
     // codes wrap by themselves)
-    uint32_t nc;
-    float nf;
-    pxy_node(A.grid, g < Ng ? g : 0, nc, nf);
     const uint32_t dn = GT_FLAT * A.grid.step + GT_FLAT * A.grid.rem / (uint32_t)Ng;
     const float df = (float)(GT_FLAT * A.grid.rem % (uint32_t)Ng) / (float)Ng;
-    float e = 0.f;
+    float mine = 0.f;
+#pragma unroll 1
+    for (int b = 0; b < NB; ++b) {
+        const int p = b * (32 / GT_FLAT) + lane / GT_FLAT;  // the lane's particle of this round
+        const uint32_t pu = __shfl_sync(0xffffffffu, u, p);
+        const float pk = __shfl_sync(0xffffffffu, k2, p);
+        const int pl = __shfl_sync(0xffffffffu, len, p);
+        int g = __shfl_sync(0xffffffffu, g0, p) + sub;
+        g = g < 0 ? g + Ng : (g >= Ng ? g - Ng : g);
+        uint32_t nc;
+        float nf, e = 0.f;
+        pxy_node(A.grid, g < Ng ? g : 0, nc, nf);
 #pragma unroll 2
-    for (int r = lane; r < len; r += GT_FLAT) {
-        e = fmaf(kde_ex2(k2 * pxy_sin2(nc, nf, u, 0.f)), A.field[g], e);
-        g += GT_FLAT;
-        while (g >= Ng) g -= Ng;
-        nc += dn;
-        nf += df;
-        if (nf >= 1.f) {
-            nf -= 1.f;
-            ++nc;
+        for (int r = sub; r < pl; r += GT_FLAT) {
+            e = fmaf(kde_ex2(pk * pxy_sin2(nc, nf, pu, 0.f)), A.field[g], e);
+            g += GT_FLAT;
+            while (g >= Ng) g -= Ng;
+            nc += dn;
+            nf += df;
+            if (nf >= 1.f) {
+                nf -= 1.f;
+                ++nc;
+            }
         }
-    }
 #pragma unroll
-    for (int o = GT_FLAT / 2; o > 0; o >>= 1) e += __shfl_xor_sync(0xffffffffu, e, o);
-    if (j < A.N && lane == 0) A.out[j] = e * nm * A.coef;
+        for (int o = GT_FLAT / 2; o > 0; o >>= 1) e += __shfl_xor_sync(0xffffffffu, e, o);
+        const float v = __shfl_sync(0xffffffffu, e, (lane & (32 / GT_FLAT - 1)) * GT_FLAT);
+        if ((lane & (PW - 1)) / (32 / GT_FLAT) == b) mine = v;
+    }
+    if (lane < PW && j < A.N) A.out[j] = mine * nm * A.coef;
 }
 
 // intervals of a width's (or a band's largest width's) table: half-width a = pi / C with
@@ -541,11 +627,21 @@ kde_status kde_gather_table(kde_ctx *ctx, const uint32_t *u, const float *kappa,
     if (!A.tab) return KDE_ENOMEM;
     const int sms = ctx->sm_count > 0 ? ctx->sm_count : 1;
     KdeProfScope _ps(ctx, PROF_GATHER);
-    // few (particle, node) pairs: one launch that sweeps them (at 2^25 pairs about 10 us, where
-    // the two launches of one width's table take 8 and the bands' three 20 to 30)
-    if ((double)N * Ng <= (kappa ? 33554432.0 : 4194304.0)) {
-        const unsigned gf = (unsigned)((N * GT_FLAT + GT_THREADS - 1) / GT_THREADS);
-        gt_flat_kernel<<<gf, GT_THREADS, 0, ctx->stream>>>(A);
+    // few (particle, node) pairs: one launch that sweeps them, for about 0.086 / NB ns a particle and
+    // 1e-3 a pair over 4 us, where the two launches of one width's table take 8 us and the bands' three
+    // 20 (narrow ranges of widths) to 42 (5 to 5000): swept and from tables, 65,536 particles and 512
+    // nodes 31 and 20, 37 and 41; 200,003 and 64 25 and 18, 25 and 41
+    const int64_t full = 64LL * sms * (32 / GT_FLAT);  // particles of a full machine at one round
+    const int nb = N >= 8 * full ? 8 : (N >= 4 * full ? 4 : (N >= 2 * full ? 2 : 1));
+    if (kappa ? (double)N * (0.086 / nb + 1e-3 * Ng) <= 4.0e4 : (double)N * Ng <= 4194304.0) {
+        const int64_t per = (int64_t)GT_WARPS * (32 / GT_FLAT) * nb;
+        const unsigned gf = (unsigned)((N + per - 1) / per);
+        switch (nb) {
+        case 8: gt_flat_kernel<8><<<gf, GT_THREADS, 0, ctx->stream>>>(A); break;
+        case 4: gt_flat_kernel<4><<<gf, GT_THREADS, 0, ctx->stream>>>(A); break;
+        case 2: gt_flat_kernel<2><<<gf, GT_THREADS, 0, ctx->stream>>>(A); break;
+        default: gt_flat_kernel<1><<<gf, GT_THREADS, 0, ctx->stream>>>(A);
+        }
         KDE_LAUNCHED(ctx, "gt_flat_kernel");
         return KDE_OK;
     }
@@ -567,7 +663,7 @@ kde_status kde_gather_table(kde_ctx *ctx, const uint32_t *u, const float *kappa,
     A.kr = kr;
     gt_range_kernel<<<A.nkr, GT_THREADS, 0, ctx->stream>>>(A, kr);
     KDE_LAUNCHED(ctx, "gt_range_kernel");
-    KDE_CUDA(ctx, kde_launch(ctx, true, gt_table_bands_kernel, dim3(4 * sms), dim3(GT_THREADS), 0, A, T),
+    KDE_CUDA(ctx, kde_launch(ctx, true, gt_table_bands_kernel, dim3(2 * sms), dim3(GT_THREADS), 0, A, T),
              "gt_table_bands_kernel");
     KDE_LAUNCHED(ctx, "gt_table_bands_kernel");
     const unsigned ge = (unsigned)((N + 2 * GT_THREADS - 1) / (2 * GT_THREADS));

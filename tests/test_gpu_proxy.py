@@ -307,3 +307,19 @@ def test_deposit_of_every_compressed_form(ctx, oracle, kap, weights):
     rho = ctx.deposit(to_dev_u(u), Ng, L, weight=None if w is None else to_dev(w), **kw).cpu().numpy()
     ctx.sync()
     assert rel_l2(rho, oracle.deposit(I.from_fixed(u, L), Ng, L, w=None if w is None else w.astype(np.float64), **okw)) <= TOL
+
+
+@pytest.mark.parametrize("N,Ng,lo,hi", [(60001, 100, 0.1, 1e5), (80001, 64, 5.0, 5e3), (160003, 65, 2.0, 2e4), (320001, 17, 0.5, 3e3),
+                                        (70001, 700, 1e4, 6e4), (70001, 1001, 100.0, 2e4), (200003, 256, 300.0, 5e3)])
+def test_gather_sweeps_and_short_intervals(ctx, oracle, N, Ng, lo, hi):
+    # calls swept in rounds of four particles a warp (one to eight rounds, with particles past the
+    # end in the last), and tables whose bands' windows are at most 32 nodes, some or all of them
+    u = positions(N, N, "spike")
+    k = I.log_uniform(N, I.STREAM_KAPPA, N, lo, hi).astype(np.float32)
+    g = 2 * math.pi * np.arange(Ng) / Ng
+    f = (np.sin(g) + 0.3 * np.cos(3 * g) + 0.2 * (I.uniforms(5, 3, Ng) - 0.5)).astype(np.float32)
+    out = ctx.gather(to_dev_u(u), to_dev(f), L, kappa=to_dev(k)).cpu().numpy()
+    ctx.sync()
+    ref = oracle.gather(I.from_fixed(u, L), f.astype(np.float64), L, kappa=k.astype(np.float64))
+    assert rel_l2(out, ref) <= TOL
+    assert np.max(np.abs(out - ref)) <= 1e-5 * np.max(np.abs(ref))
