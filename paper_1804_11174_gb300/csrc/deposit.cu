@@ -742,10 +742,9 @@ __device__ __forceinline__ void depp_sweep_pairs(const DepSrc<float> &S, int n, 
 // What bounds it: the direct sweep spends one exp2 and three or four multiply-adds on every
 // (particle, node) pair, 256 a particle for whole-grid windows; here a particle costs the
 // Chebyshev values and 28 to 48 multiply-adds (a few hundred in the matrix form) whatever the
-// window, and is bound by instruction issue and load latency.  Measured (event-free launch
-// times): 2^20 particles, 256 nodes, widths near 14 43.2 -> 12.8 us (16.3 before the register
-// forms' proxies were unrolled); 4,000,037 particles, 4096 nodes, widths log-uniform in [5, 5e3]
-// 2389 -> 306 us.
+// window, and is bound by instruction fetch and issue and load latency.  Measured (by events around
+// the launch): 2^20 particles, 256 nodes, widths near 14 45.0 -> 15.0 us; 4,000,037 particles, 4096
+// nodes, widths log-uniform in [5, 5e3] 2389 -> 315 us.
 // ---------------------------------------------------------------------------
 #define PXY_STAGE 16  // particles a warp stages at a time
 

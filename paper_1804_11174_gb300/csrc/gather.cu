@@ -992,8 +992,8 @@ static kde_status gat2_variant(kde_ctx *ctx, const GatherArgs<float> &A, int v)
 }
 
 // the gather through proxies: at the default truncation, in the PIC step (and its truncation
-// tuner).  The rest -- plain gathers with particle-wise widths and cuts the caller has
-// set -- sweeps the nodes (gather2_kernel)
+// tuner).  The rest -- particle-wise widths outside a schedule and cuts the caller has set -- sweeps
+// the nodes (gather2_kernel)
 // For one width the host knows the outcome: where the tiles would sweep the nodes anyway,
 // gather2_kernel does it.
 static int gatt_tile(kde_ctx *ctx, const GatherArgs<float> &A)
@@ -1013,8 +1013,10 @@ static bool gatt_applies(kde_ctx *ctx, GatherArgs<float> &A)
     if (A.xcut != (float)KDE_XCUT || !(A.kappa ? A.krange != nullptr : A.u_out != nullptr)) return false;
     A.tile = gatt_tile(ctx, A);
     // particle-wise widths: a range is given for those of a width schedule (Silverman's rule
-    // around one width, a narrow range unless the density varies much); a few tiles are
-    // better swept by four times as many blocks
+    // around one width, a narrow range unless the density varies much).  Below 65,536 particles a wide
+    // range's sweep by four times as many blocks would miss more than a narrow range's tiles spare: 50
+    // steps on 256 nodes, tiles and gather2_kernel, narrow 49,152 1194 and 1376 us, 65,536 1224 and
+    // 1466, 262,144 1346 and 1642; over a factor of three 1619 and 1461, 1701 and 1539, 1897 and 1776
     if (A.kappa) return A.N >= 64 * GATT_UNIT;
     const double n = (double)(A.N < A.tile ? A.N : A.tile), share = n / (double)A.N;
     const double a = KDE_PI * std::min(1.0, share + 2.0 / A.Ng), y = a * sqrt((double)A.kappa_u + 1.5);
