@@ -539,7 +539,7 @@ def ad_record(kp, ctx, dev, args, flush):
 # one ncu capture of each on this Landau step (a PIC step after the tuner's runs; the gather
 # with its push on a step that is not a call's last); None once a kernel changes after its
 # capture
-PROFILED_TRAFFIC = {"deposit_persist_kernel": 8459264 + 0, "gather_tile_kernel": 12724224 + 0}
+PROFILED_TRAFFIC = {"deposit_persist_kernel": 8482560 + 0, "gather_tile_kernel": 12726528 + 0}
 
 
 def run_cv_sweep(args, rank, world, local_rank):
