@@ -458,14 +458,16 @@ __host__ __device__ inline double kde_acc_scale(double bound)
 // ---------------------------------------------------------------------------
 // counting sort by bin = floor(u nbins / 2^32), stable.  Moves u and up to four
 // payload arrays (element size 4 or 8 bytes); writes the source index of every
-// output slot to perm_out when not null.
+// output slot to perm_out when not null.  overlap: the count may start while the kernel before it
+// in the stream runs, which neither writes u nor uses the count table
 struct SortPayload {
     const void *src;
     void *dst;
     int elem;
 };
 kde_status kde_sort_by_bin(kde_ctx *ctx, const uint32_t *u, int64_t N, int nbins, uint32_t *u_out,
-                           const SortPayload *pl, int npl, uint32_t *perm_out, bool counted = false);
+                           const SortPayload *pl, int npl, uint32_t *perm_out, bool counted = false,
+                           bool overlap = false);
 // the count table of such a sort (bin-major: entry bin * nblk + tile, tile = index >>
 // tile_shift), for a kernel that adds the counts of the keys it writes; with
 // counted = true kde_sort_by_bin uses the table as it stands (every sort leaves it zero)

@@ -18,6 +18,7 @@ template <typename T>
 __global__ void __launch_bounds__(256) norm_from_kappa_kernel(const T *kappa, int64_t N, T *norm, unsigned int *status,
                                                               const float2 *ntab, unsigned int *krange, const float *pxt)
 {
+    kde_pdl_trigger();  // the first sort's count needs nothing of this kernel's
     float lo = 3.0e38f, hi = 0.f;  // of the widths as the deposit and the gather use them
     for (int64_t i = (int64_t)blockIdx.x * 256 + threadIdx.x; i < N; i += (int64_t)gridDim.x * 256) {
         double k = (double)kappa[i];
@@ -240,6 +241,7 @@ static kde_status pic_run(kde_ctx *ctx, pic_state *st, int n_steps)
     // the AD schedule smooths h = kappa^{-1/2}, carried across the steps of this call
     double h_ad = adsched ? 1.0 / sqrt(st->kappa_uniform) : 0.0;
 
+    if (sizeof(T) == 4 && n_steps > 0) KDE_TRY(kde_deposit_sums_reset(ctx, Ng));
     // FP32 particle-wise widths: their range, kept on the device beside them
     unsigned int *krange = nullptr;
     if (per && sizeof(T) == 4 && kde_pic_range(N, Ng, sched)) {
@@ -255,7 +257,6 @@ static kde_status pic_run(kde_ctx *ctx, pic_state *st, int n_steps)
         KDE_LAUNCHED(ctx, "norm_from_kappa_kernel");
         if (krange) kde_krange_end(ctx);
     }
-    if (sizeof(T) == 4 && n_steps > 0) KDE_TRY(kde_deposit_sums_reset(ctx, Ng));
     const double coef = KDE_TWO_PI / L;
     const double w_u = L / (double)N;
     // the FP32 gather + push adds the next step's sort counts; a step whose table was
@@ -334,7 +335,9 @@ static kde_status pic_run(kde_ctx *ctx, pic_state *st, int n_steps)
         if (st->id) pl[npl++] = SortPayload{id_cur, ids, 4};
         {
             KdeRange r_("kdepic sort by cell");
-            KDE_TRY(kde_sort_by_bin(ctx, st->u, N, Ng, us, pl, npl, nullptr, counted));
+            // the call's first count overlaps the pass over the widths (a one-step call on 131,072
+            // particles with widths of 13 to 16 and 256 nodes 43.7 -> 39.7 us)
+            KDE_TRY(kde_sort_by_bin(ctx, st->u, N, Ng, us, pl, npl, nullptr, counted, s == 0 && per && !update));
         }
 
         const double norm_u = per ? 0.0 : kde_norm(st->kappa_uniform);

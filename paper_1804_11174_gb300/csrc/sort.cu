@@ -74,6 +74,7 @@ __global__ void sort_count_kernel(const uint32_t *__restrict__ u, int64_t N, int
         }
     }
     __syncthreads();
+    kde_pdl_wait();  // (a count that overlaps the kernel before, see kde_sort_by_bin)
     for (int b = threadIdx.x; b < nbins; b += blockDim.x) counts[(size_t)b * nblk + blockIdx.x] = hist[b];
 }
 
@@ -353,7 +354,8 @@ kde_status kde_sort_counts_table(kde_ctx *ctx, int64_t N, int nbins, SortCounts 
 
 template <bool DIGIT>
 static kde_status sort_pass(kde_ctx *ctx, const uint32_t *u, int64_t N, int nbins, int shift, uint32_t *u_out,
-                            const SortPayload *pl, int npl, uint32_t *perm_out, bool counted = false)
+                            const SortPayload *pl, int npl, uint32_t *perm_out, bool counted = false,
+                            bool overlap = false)
 {
     int wpb, unit, nblk;
     sort_geometry(N, nbins, wpb, unit, nblk);
@@ -387,8 +389,9 @@ static kde_status sort_pass(kde_ctx *ctx, const uint32_t *u, int64_t N, int nbin
     if (smem > 100 * 1024) return kde_fail(ctx, KDE_ENOTSUP, "sort: %d tiles of counts exceed shared memory", ntiles);
     KdeProfScope _ps(ctx, PROF_SORT);  // the whole pass: count, scan and scatter
     if (!counted) {
-        sort_count_kernel<DIGIT><<<nblk, wpb * 32, (size_t)nbins * 4, ctx->stream>>>(u, N, nbins, shift, unit, nblk,
-                                                                                    counts);
+        KDE_CUDA(ctx, kde_launch(ctx, overlap, sort_count_kernel<DIGIT>, dim3(nblk), dim3(wpb * 32), (size_t)nbins * 4, u, N,
+                                 nbins, shift, unit, nblk, counts),
+                 "sort_count_kernel");
         KDE_LAUNCHED(ctx, "sort_count_kernel");
     }
     KDE_CUDA(ctx, kde_launch(ctx, true, sort_scan_kernel, dim3(ntiles), dim3(SCAN_THREADS), 0, counts, ncounts, tiles,
@@ -432,12 +435,12 @@ static kde_status sort_pass(kde_ctx *ctx, const uint32_t *u, int64_t N, int nbin
 }
 
 kde_status kde_sort_by_bin(kde_ctx *ctx, const uint32_t *u, int64_t N, int nbins, uint32_t *u_out,
-                           const SortPayload *pl, int npl, uint32_t *perm_out, bool counted)
+                           const SortPayload *pl, int npl, uint32_t *perm_out, bool counted, bool overlap)
 {
     if (N <= 0) return KDE_OK;
     if (nbins < 1 || nbins > 8192 || npl > 4 || N > 0xFFFFFFFFll)
         return kde_fail(ctx, KDE_EINVAL, "sort: unsupported sizes");
-    return sort_pass<false>(ctx, u, N, nbins, 0, u_out, pl, npl, perm_out, counted);
+    return sort_pass<false>(ctx, u, N, nbins, 0, u_out, pl, npl, perm_out, counted, overlap);
 }
 
 kde_status kde_radix_sort_u32(kde_ctx *ctx, const uint32_t *u, int64_t N, uint32_t *out, uint32_t *tmp)

@@ -536,3 +536,21 @@ def test_node_sums_between_calls(ctx, kp):
             assert torch.equal(st.energy[:1], ref[0].energy[:1])
             check(c)
         c.close()
+
+
+@pytest.mark.parametrize("N, Ng, dtype", [(70001, 300, torch.float32), (5000, 64, torch.float32), (5000, 64, torch.float64)])
+def test_one_step_calls_overlap_bitwise(ctx, kp, N, Ng, dtype):
+    # calls of one step on particle-wise widths, whose first count overlaps the pass over the widths
+    u, v = I.landau_load(48, N, 4 * math.pi, 0.05, 1.0)
+    k = I.log_uniform(5, I.STREAM_KAPPA, N, 13.0, 16.0)
+    states = [make_state(kp, u, v, 4 * math.pi, Ng, 0.1, 6, dtype=dtype, kappa=k) for _ in range(2)]
+    try:
+        for st, on in zip(states, (True, False)):
+            ctx.set_launch_overlap(on)
+            for _ in range(6):
+                ctx.pic_step(st, 1)
+            ctx.sync()
+    finally:
+        ctx.set_launch_overlap(True)
+    for n in ("u", "v", "id", "kappa", "kappa_norm", "energy"):
+        assert torch.equal(getattr(states[0], n), getattr(states[1], n)), n
