@@ -64,26 +64,31 @@ __global__ void __launch_bounds__(256) sc_key_kernel(const float *kr, int64_t N,
     key[j] = (uint32_t)b << 28;
 }
 
-// first particle of every band in the sorted order
-__global__ void __launch_bounds__(256) sc_starts_kernel(const uint32_t *key, int64_t N, int64_t *starts)
+// first particle of every band in the sorted order (N < 2^32)
+__global__ void __launch_bounds__(256) sc_starts_kernel(const uint32_t *key, int64_t N, uint32_t *starts)
 {
     const int64_t j = (int64_t)blockIdx.x * 256 + threadIdx.x;
     if (j >= N) return;
     const int b = (int)(key[j] >> 28), a = j ? (int)(key[j - 1] >> 28) : -1;
-    for (int k = a + 1; k <= b; ++k) starts[k] = j;
+    for (int k = a + 1; k <= b; ++k) starts[k] = (uint32_t)j;
     if (j == N - 1)
-        for (int k = b + 1; k <= SC_MAXB; ++k) starts[k] = N;
+        for (int k = b + 1; k <= SC_MAXB; ++k) starts[k] = (uint32_t)N;
 }
 
-// the chunk x of the bands' chunk lists: its band and particles, or false past the end
-__device__ __forceinline__ bool sc_chunk(const ScBands &B, const int64_t *starts, int x, int &b, int64_t &j0, int64_t &j1)
+// chunks of a band
+__device__ __forceinline__ int sc_chunks(const ScBands &B, const uint32_t *starts, int b)
+{
+    const uint32_t n = starts[b + 1] - starts[b], c = (uint32_t)B.chunk;
+    return (int)(n / c + (n % c ? 1u : 0u));
+}
+// the chunk x of the bands' chunk lists: its band, first particle and number, or false past the end
+__device__ __forceinline__ bool sc_chunk(const ScBands &B, const uint32_t *starts, int x, int &b, uint32_t &j0, int &nj)
 {
     for (b = 0; b < B.nb; ++b) {
-        const int64_t s = starts[b], e = starts[b + 1];
-        const int nc = (int)((e - s + B.chunk - 1) / B.chunk);
+        const int nc = sc_chunks(B, starts, b);
         if (x < nc) {
-            j0 = s + (int64_t)x * B.chunk;
-            j1 = e < j0 + B.chunk ? e : j0 + B.chunk;
+            j0 = starts[b] + (uint32_t)x * (uint32_t)B.chunk;
+            nj = (int)min(starts[b + 1] - j0, (uint32_t)B.chunk);
             return true;
         }
         x -= nc;
@@ -93,21 +98,23 @@ __device__ __forceinline__ bool sc_chunk(const ScBands &B, const int64_t *starts
 
 // partial sums of T_q(s_j) e^{im theta_j} over a chunk, q < SC_Q, four consecutive modes a thread
 __global__ void __launch_bounds__(SC_THREADS)
-    sc_factor_kernel(const uint32_t *__restrict__ u, const float *__restrict__ kr, ScBands B, const int64_t *starts,
+    sc_factor_kernel(const uint32_t *__restrict__ u, const float *__restrict__ kr, ScBands B, const uint32_t *starts,
                      double2 *part)
 {
     __shared__ uint32_t us[SC_SUB];
     __shared__ __align__(16) float tq[SC_SUB][SC_Q];
     __shared__ float2 e1[SC_SUB];
-    int b;
-    int64_t j0, j1;
-    if (!sc_chunk(B, starts, blockIdx.x, b, j0, j1)) return;
+    int b, nj;
+    uint32_t j0;
+    if (!sc_chunk(B, starts, blockIdx.x, b, j0, nj)) return;
+    u += j0;
+    kr += j0;
     const int mb = 1 + blockIdx.y * SC_THREADS * SC_MODES;
     if (mb > B.M[b]) return;
     const int m0 = mb + threadIdx.x * SC_MODES;
     double2 *out = part + (size_t)blockIdx.x * SC_Q * B.Mst + (m0 - 1);
-    for (int64_t s0 = j0; s0 < j1; s0 += SC_SUB) {
-        const int n = (int)(j1 - s0 < SC_SUB ? j1 - s0 : SC_SUB);
+    for (int s0 = 0; s0 < nj; s0 += SC_SUB) {
+        const int n = min(SC_SUB, nj - s0);
         __syncthreads();
         for (int k = threadIdx.x; k < n; k += SC_THREADS) {
             const uint32_t uk = u[s0 + k];
@@ -160,7 +167,7 @@ __global__ void __launch_bounds__(SC_THREADS)
             for (int q = 0; q < SC_Q; ++q) {
                 double2 *o = out + (size_t)q * B.Mst + h;
                 double2 v = make_double2((double)ar[h][q], (double)ai[h][q]);
-                if (s0 > j0) {
+                if (s0 > 0) {
                     const double2 w = *o;
                     v.x += w.x;
                     v.y += w.y;
@@ -173,7 +180,7 @@ __global__ void __launch_bounds__(SC_THREADS)
 
 // G summed over a band's chunks in order, then H_q' = sum_q c_q[q'] G_q (proxy.cuh's matrix in
 // FP64); block (32 modes, band), warp w the sums of q = w, w + 8
-__global__ void __launch_bounds__(256) sc_reduce_kernel(const double2 *part, ScBands B, const int64_t *starts, double2 *H)
+__global__ void __launch_bounds__(256) sc_reduce_kernel(const double2 *part, ScBands B, const uint32_t *starts, double2 *H)
 {
     __shared__ double2 G[SC_Q][32];
     __shared__ double cm[4 * SC_Q];
@@ -182,8 +189,8 @@ __global__ void __launch_bounds__(256) sc_reduce_kernel(const double2 *part, ScB
     if ((int)(blockIdx.x * 32) >= B.M[b]) return;
     if (threadIdx.x < 4 * SC_Q) cm[threadIdx.x] = cospi((double)threadIdx.x / (2.0 * SC_Q));
     int x0 = 0;
-    for (int k = 0; k < b; ++k) x0 += (int)((starts[k + 1] - starts[k] + B.chunk - 1) / B.chunk);
-    const int nc = (int)((starts[b + 1] - starts[b] + B.chunk - 1) / B.chunk);
+    for (int k = 0; k < b; ++k) x0 += sc_chunks(B, starts, k);
+    const int nc = sc_chunks(B, starts, b);
     for (int q = warp; q < SC_Q; q += 8) {
         double2 s = make_double2(0.0, 0.0);
         if (m < B.M[b])
@@ -422,7 +429,7 @@ kde_status kde_cv_scale_fourier(kde_ctx *ctx, const uint32_t *u, const float *kr
     double2 *H = (double2 *)w, *F = H + nH, *psum = F + nF;
     double *inv = (double *)(psum + nP), *pself = inv + (size_t)B.nb * ns;
     size_t *aoff = (size_t *)(pself + (size_t)n_cand * nself);
-    int64_t *starts = (int64_t *)(aoff + SC_MAXB);
+    uint32_t *starts = (uint32_t *)(aoff + SC_MAXB);
     KDE_CUDA(ctx, cudaMemcpyAsync(aoff, aoff_h, sizeof(size_t) * B.nb, cudaMemcpyHostToDevice, ctx->stream), "offsets copy");
 
     KdeProfScope _ps(ctx, PROF_SPECTRAL);
